@@ -113,7 +113,8 @@ def draw(rng):
         n = _log_int(rng, 2000, 200000)
         return {"op": op, "points": "surface", "n": n, "r": round(0.015 * math.sqrt(35947.0 / n), 6), "f_in": rng.choice((1, 5, 8, 13)),
                 "hidden": rng.choice((8, 16, 32)), "f_out": rng.choice((1, 3, 4))}
-    return {"op": op, "points": rng.choice(("uniform", "uniform", "surface", "clustered")), "n": _log_int(rng, 1000, 1000000),
+    points = rng.choice(("uniform", "uniform", "surface", "clustered"))
+    return {"op": op, "points": points, "n": _log_int(rng, 1000, 100000 if points == "clustered" else 1000000),
             "F": rng.choice((1, 1, 3, 8, 16)), "k": rng.choice((4, 8, 16, 16, 32))}
 
 
