@@ -22,7 +22,7 @@
 // coordinates; a cell whose stencil wraps around a periodic face moves the points next to the
 // upper face down by the box length, which is exact in fp32, so every displacement is one
 // rounded subtraction of two stored coordinates, for wrapped pairs as for interior ones.
-#include "radius_shared.cuh"
+#include "radius_test.cuh"
 #include <type_traits>
 
 namespace tiga {
@@ -281,7 +281,7 @@ template <int MODE> struct TravSmem {
     static constexpr int QSTRIDE = QCAP + 5;                       // room for four padding entries; odd, so the lists of different queries fall in different banks
     static constexpr int STAGE_BYTES = (STAGE_CAP + STAGE_PAD) * 16;
     static constexpr int LIST_BYTES = (TQB * QSTRIDE * 8 + 15) / 16 * 16;
-    static constexpr int MISC_BYTES = TQB * 16 + 3 * TQB * 4 + TQB * 4 * 2 + 32;   // queries, their coordinates by component, counts, totals, the cell's frame
+    static constexpr int MISC_BYTES = TQB * 16 + 3 * TQB * 4 + TQB * 4 * 2 + 32 + 80;   // queries, their coordinates by component, counts, totals, the frame, range offsets
     static constexpr int PER_WARP = STAGE_BYTES + LIST_BYTES + MISC_BYTES;
     static_assert(PER_WARP % 16 == 0 && LIST_BYTES % 16 == 0, "the stage and the queries are accessed as 16-byte vectors");
 };
@@ -291,7 +291,7 @@ template <int MODE> struct TravSmem {
 // VEC: 0 = scalar feature accesses (F % 4 != 0, forward only); 1 = 128-bit accesses, F % 4 == 0;
 // 2 = additionally F == 4 LF exactly, so the row stride is a compile-time constant.
 template <int MODE, int LF, bool DIST, bool MI, int VEC>
-__device__ __forceinline__ void traverse_slice(const RadiusParams& p, const int cellid, const int qs0, const int qe0, unsigned char* s_raw) {
+__device__ __forceinline__ void traverse_slice(const RadiusParams& p, const int cellid, const int run, const int qs0, const int qe0, unsigned char* s_raw) {
     using SM = TravSmem<MODE>;
     constexpr int STAGE_CAP = SM::STAGE_CAP, QCAP = SM::QCAP, QSTRIDE = SM::QSTRIDE, TQB = SM::TQB;
     constexpr unsigned FULL = 0xffffffffu;
@@ -306,14 +306,17 @@ __device__ __forceinline__ void traverse_slice(const RadiusParams& p, const int 
     int* s_n = reinterpret_cast<int*>(s_qc + 3 * TQB);                                  // list lengths of the drain in progress
     int* s_tot = s_n + TQB;                                                              // neighbours found so far in this chunk
     float* s_frame = reinterpret_cast<float*>(s_tot + TQB);                              // thresholds [3], shifts [3]
+    int* s_delta = reinterpret_cast<int*>(s_frame + 8);                                  // source minus flattened position of every range
 
     const int c[3] = {cellid % p.nc[0], (cellid / p.nc[0]) % p.nc[1], cellid / (p.nc[0] * p.nc[1])};
     const int F = VEC == 2 ? 4 * LF : p.F;
     const float neg_c2 = !DIST ? -1.4426950408889634f / (2.f * p.p0 * p.p0) : 0.f;   // exp(-d2/(2 s^2)) = 2^(d2 * neg_c2)
-    const int fl = lane % LF, grp = lane / LF;
     // a periodic dimension with three cells or fewer has no consistent shifted frame: explicit minimum image
     const bool mi0 = MI && p.periodic[0] && p.nc[0] <= 3, mi1 = MI && p.periodic[1] && p.nc[1] <= 3, mi2 = MI && p.periodic[2] && p.nc[2] <= 3;
-    constexpr int QP = 32 / LF;
+    constexpr int QP = 32 / LF;                        // groups of LF lanes
+    constexpr int SUB = QP > TQB ? QP / TQB : 1;       // groups that share a list (narrow rows: more groups than queries)
+    constexpr int QPASS = QP / SUB;                    // queries per pass (F = 8, n = 1M: forward 632 -> 566, backward 941 -> 770 us)
+    const int fl = lane % LF, grp = lane / LF / SUB, gsub = lane / LF % SUB;
     const bool fvalid = VEC == 2 ? true : fl * 4 < F;
     const unsigned lt_mask = (1u << lane) - 1u;
 
@@ -330,9 +333,10 @@ __device__ __forceinline__ void traverse_slice(const RadiusParams& p, const int 
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
         float thr = FAR_AWAY;
+        const int last = d == 0 ? c[0] + run - 1 : c[d];
         if (p.periodic[d] && p.nc[d] >= 4) {
-            if (c[d] == 0) { thr = 2.5f * p.hcell[d]; face = true; }
-            else if (c[d] == p.nc[d] - 1) { thr = 1.5f * p.hcell[d]; face = true; }
+            if (c[d] == 0) { thr = ((float)(last - c[d]) + 2.5f) * p.hcell[d]; face = true; }
+            else if (last == p.nc[d] - 1) { thr = 1.5f * p.hcell[d]; face = true; }
         }
         if (lane == d) { s_frame[d] = thr; s_frame[3 + d] = p.len[d]; }
     }
@@ -390,8 +394,8 @@ __device__ __forceinline__ void traverse_slice(const RadiusParams& p, const int 
                 if (lane < TQB * 4) list[(lane >> 2) * QSTRIDE + s_n[lane >> 2] + (lane & 3)] = make_float2(__int_as_float(0), 0.f);
                 __syncwarp();
                 {
-                    for (int pass = 0; pass * QP < nq; ++pass) {
-                        const int qq = pass * QP + grp;
+                    for (int pass = 0; pass * QPASS < nq; ++pass) {
+                        const int qq = pass * QPASS + grp;
                         const bool valid = qq < nq && fvalid;
                         float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
                         float px = 0.f, py = 0.f, pz = 0.f;
@@ -402,7 +406,7 @@ __device__ __forceinline__ void traverse_slice(const RadiusParams& p, const int 
                             const int n = s_n[qq];
                             const float2* lq = list + qq * QSTRIDE;
                             if (MODE == 0) {
-                                for (int t = 0; t < n; t += 4) {
+                                for (int t = gsub * 4; t < n; t += 4 * SUB) {
                                     float2 e[4];
                                     float4 x[4];
 #pragma unroll
@@ -423,7 +427,7 @@ __device__ __forceinline__ void traverse_slice(const RadiusParams& p, const int 
                                 const float4 xk = __ldg(reinterpret_cast<const float4*>(p.feat + (size_t)oqq * F) + fl);
                                 const float4 gk = __ldg(reinterpret_cast<const float4*>(p.gy + (size_t)oqq * F) + fl);
                                 constexpr int BU = 4;      // pairs in flight per lane
-                                for (int t = 0; t < n; t += BU) {
+                                for (int t = gsub * BU; t < n; t += BU * SUB) {
                                     float4 e[BU], xj[BU], gj[BU];
                                     float g[BU];
 #pragma unroll
@@ -451,6 +455,13 @@ __device__ __forceinline__ void traverse_slice(const RadiusParams& p, const int 
                                     }
                                 }
                             }
+                        }
+#pragma unroll
+                        for (int o = LF; o < LF * SUB; o <<= 1) {
+                            acc.x += __shfl_xor_sync(FULL, acc.x, o); acc.y += __shfl_xor_sync(FULL, acc.y, o);
+                            acc.z += __shfl_xor_sync(FULL, acc.z, o); acc.w += __shfl_xor_sync(FULL, acc.w, o);
+                        }
+                        if (valid && gsub == 0) {
                             float* orow = (MODE == 0 ? p.out : p.gfeat);
                             if (orow && VEC) {
                                 float4* o = reinterpret_cast<float4*>(orow + (size_t)oqq * F) + fl;
@@ -466,12 +477,12 @@ __device__ __forceinline__ void traverse_slice(const RadiusParams& p, const int 
                         }
                         if (MODE == 2) {
 #pragma unroll
-                            for (int o = LF / 2; o > 0; o >>= 1) {
+                            for (int o = LF * SUB / 2; o > 0; o >>= 1) {
                                 px += __shfl_xor_sync(FULL, px, o);
                                 py += __shfl_xor_sync(FULL, py, o);
                                 pz += __shfl_xor_sync(FULL, pz, o);
                             }
-                            if (p.gpos && qq < nq && fl == 0) {
+                            if (p.gpos && qq < nq && fl == 0 && gsub == 0) {
                                 const float sc = -1.f / (p.p0 * p.p0);
                                 float* o = p.gpos + 3 * (size_t)oqq;
                                 if (first) { o[0] = sc * px; o[1] = sc * py; o[2] = sc * pz; }
@@ -565,45 +576,12 @@ __device__ __forceinline__ void traverse_slice(const RadiusParams& p, const int 
         __syncwarp();
     };
 
-    // ---- the 27-cell stencil as candidate ranges: lane r < 27 resolves neighbour offset r
-    int r_cs = 0, r_ce = 0;
-    {
-        const int off[3] = {lane % 3 - 1, (lane / 3) % 3 - 1, lane / 9 - 1};
-        bool ok = lane < 27;
-        int q[3] = {0, 0, 0};
-        bool merged = false;
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            if (p.nc[d] == 1) { ok = ok && off[d] == 0; continue; }
-            if (d == 0 && c[0] >= 1 && c[0] <= p.nc[0] - 2) {
-                // away from the x faces the three x-adjacent cells are one contiguous range
-                merged = true; ok = ok && off[0] == 0; q[0] = c[0] - 1;
-                continue;
-            }
-            int v = c[d] + off[d];
-            if (v < 0) { if (p.periodic[d]) v += p.nc[d]; else ok = false; }
-            else if (v >= p.nc[d]) { if (p.periodic[d]) v -= p.nc[d]; else ok = false; }
-            q[d] = v;
-        }
-        if (ok) {
-            const int id = (q[2] * p.nc[1] + q[1]) * p.nc[0] + q[0];
-            r_cs = p.cell_start[id];
-            r_ce = p.cell_start[id + (merged ? 3 : 1)];
-        }
-    }
-    // flat copy: staged slot v belongs to the range whose inclusive prefix of lengths first exceeds v
-    const int r_len = r_ce - r_cs;
-    int r_incl = r_len;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(FULL, r_incl, o);
-        if (lane >= o) r_incl += t;
-    }
-    const int total = __shfl_sync(FULL, r_incl, 31);
+    const RunStencil sten(p, c, run, s_delta);
+    const int total = sten.total;
 
-    // bounding box of the cell's own points (in the cell's frame): a candidate farther than the
-    // cutoff from this box cannot be a neighbour of any of them and is not staged at all, which
-    // removes about 40 % of the stencil's candidates before any pair is tested
+    // bounding box of the queries (in the frame): a candidate farther than the cutoff from this box cannot be a
+    // neighbour of any of them and is not staged at all, which removes about 40 % of a cell's stencil
+    // candidates before any pair is tested
     float blo[3] = {FAR_AWAY, FAR_AWAY, FAR_AWAY}, bhi[3] = {-FAR_AWAY, -FAR_AWAY, -FAR_AWAY};
     for (int q = qs0 + lane; q < qe0; q += 32) {
         const float4 pq = to_frame(p.spos[q]);
@@ -612,12 +590,7 @@ __device__ __forceinline__ void traverse_slice(const RadiusParams& p, const int 
         for (int d = 0; d < 3; ++d) { blo[d] = fminf(blo[d], l[d]); bhi[d] = fmaxf(bhi[d], l[d]); }
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            blo[d] = fminf(blo[d], __shfl_xor_sync(FULL, blo[d], o));
-            bhi[d] = fmaxf(bhi[d], __shfl_xor_sync(FULL, bhi[d], o));
-        }
+    for (int d = 0; d < 3; ++d) { blo[d] = warp_min(blo[d]); bhi[d] = warp_max(bhi[d]); }
     // the box lives in one register per lane (lane d: low bound of dimension d, lane 3 + d: high bound) and is
     // broadcast where it is used, so that it costs the pair loops below one register instead of six
     float bb = lane == 0 ? blo[0] : lane == 1 ? blo[1] : lane == 2 ? blo[2] : lane == 3 ? bhi[0] : lane == 4 ? bhi[1] : bhi[2];
@@ -628,6 +601,7 @@ __device__ __forceinline__ void traverse_slice(const RadiusParams& p, const int 
     // candidates might not fit, so the chunks are as full as the pruning allows (one chunk for all but dense cells).
     bool first_chunk = true;
     int nst = 0;                                                             // candidates staged (warp uniform)
+    int before = -1;                                                         // ranges that began before the step, minus one
     constexpr int SU = 4;                                                    // staging groups in flight
     for (int k0 = 0;; k0 += 32 * SU) {
         const bool done = k0 >= total;
@@ -642,16 +616,10 @@ __device__ __forceinline__ void traverse_slice(const RadiusParams& p, const int 
         float4 c4[SU];
 #pragma unroll
         for (int u = 0; u < SU; ++u) {                                       // all loads of the step first
-            const int v = k0 + 32 * u + lane;
-            int r = 0;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const int probe = __shfl_sync(FULL, r_incl, r + o - 1);
-                if (probe <= v) r += o;
-            }
-            r = r > 31 ? 31 : r;
-            const int src = __shfl_sync(FULL, r_cs, r) + (v - (__shfl_sync(FULL, r_incl, r) - __shfl_sync(FULL, r_len, r)));
-            c4[u] = v < total ? __ldg(p.spos + checked(src, p.n, CHECK_SLOT)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            c4[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (32 * u >= step) continue;
+            const int src = sten.source(k0 + 32 * u, before, s_delta);
+            if (k0 + 32 * u + lane < total) c4[u] = __ldg(p.spos + checked(src, p.n, CHECK_SLOT));
         }
         const float lx = __shfl_sync(FULL, bb, 0), ly = __shfl_sync(FULL, bb, 1), lz = __shfl_sync(FULL, bb, 2);
         const float hx = __shfl_sync(FULL, bb, 3), hy = __shfl_sync(FULL, bb, 4), hz = __shfl_sync(FULL, bb, 5);
@@ -670,27 +638,232 @@ __device__ __forceinline__ void traverse_slice(const RadiusParams& p, const int 
     }
 }
 
-// CTAs [0, cell_blocks): warp w takes cell w (of a cell with more than QDENSE points its first QSLICE
-// queries).  The CTAs behind them walk the queue of the remaining slices.
-template <int MODE, int LF, bool DIST, bool MI, int VEC = 1>
-__global__ void __launch_bounds__(TRAV_THREADS, (MODE == 0 ? 7 : 0)) radius_traverse_kernel(const __grid_constant__ RadiusParams p) {
-    extern __shared__ __align__(16) unsigned char s_raw[];
+// CTAs [0, cell_blocks): warp w takes the w-th run of p.run cells along x; the cells are joined as long as they hold at
+// most RUN_QUERIES points together (of a cell with more than QDENSE points the first QSLICE queries).  The CTAs behind
+// them walk the queue of the remaining slices.
+template <typename Work>
+__device__ __forceinline__ void walk_slices(const RadiusParams& p, Work work) {
     if ((int)blockIdx.x < p.cell_blocks) {
         const int w = blockIdx.x * TRAV_WARPS + (threadIdx.x >> 5);
-        if (w >= p.ncells) return;
-        const int qs0 = p.cell_start[w], qe0 = p.cell_start[w + 1];
-        if (qs0 == qe0) return;
-        traverse_slice<MODE, LF, DIST, MI, VEC>(p, w, qs0, qe0 - qs0 > QDENSE ? qs0 + QSLICE : qe0, s_raw);
+        const int lane = threadIdx.x & 31;
+        const int per_row = (p.nc[0] + p.run - 1) / p.run;
+        const int row = w / per_row, x0 = (w - row * per_row) * p.run;
+        if (row >= p.nc[1] * p.nc[2]) return;
+        const int cells = p.nc[0] - x0 < p.run ? p.nc[0] - x0 : p.run, cell0 = row * p.nc[0] + x0;
+        const int start = p.cell_start[cell0 + (lane < cells ? lane : cells)];          // lane k: first point of cell k of the run
+        const int len = __shfl_down_sync(0xffffffffu, start, 1) - start;
+        unsigned left = __ballot_sync(0xffffffffu, lane < cells && len > 0);            // occupied cells not done yet
+        while (left) {
+            const int a = __ffs(left) - 1, qs = __shfl_sync(0xffffffffu, start, a), first = __shfl_sync(0xffffffffu, len, a);
+            int qe = qs + (first > QDENSE ? QSLICE : first), last = a;
+            left &= left - 1u;
+            while (left) {
+                const int b = __ffs(left) - 1, more = __shfl_sync(0xffffffffu, start + len, b);
+                if (first > QDENSE || more - qs > RUN_QUERIES) break;
+                qe = more; last = b;
+                left &= left - 1u;
+            }
+            work(cell0 + a, last - a + 1, qs, qe);
+            __syncwarp();
+        }
     } else {
         const int n = *p.q_count;
         const int w = (blockIdx.x - p.cell_blocks) * TRAV_WARPS + (threadIdx.x >> 5);
         for (int it = w; it < n; it += (gridDim.x - p.cell_blocks) * TRAV_WARPS) {
             const int2 item = p.q_items[it];
             const int qs0 = p.cell_start[item.x] + item.y, end = p.cell_start[item.x + 1];
-            traverse_slice<MODE, LF, DIST, MI, VEC>(p, item.x, qs0, slice_end(qs0, end), s_raw);
+            work(item.x, 1, qs0, slice_end(qs0, end));
             __syncwarp();
         }
     }
+}
+
+template <int MODE, int LF, bool DIST, bool MI, int VEC = 1>
+__global__ void __launch_bounds__(TRAV_THREADS, (MODE == 0 ? 7 : 0)) radius_traverse_kernel(const __grid_constant__ RadiusParams p) {
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    walk_slices(p, [&](const int cell, const int run, const int qs, const int qe) { traverse_slice<MODE, LF, DIST, MI, VEC>(p, cell, run, qs, qe, s_raw); });
+}
+
+// ------------------------------------------------------------------------------ at most four features
+// Forward with NF <= 4 features per point (the distance-weighted scalar sum among them).  A gather by groups of
+// lanes would leave most of the warp idle on such rows, so nothing is gathered: the features are staged with
+// the candidates, every query has its own lanes, and a lane adds weight * features of its accepted candidates in
+// registers (test and expansion: radius_test.cuh).  One warp per run of cells, slices of dense cells from the queue.
+// Bound by instruction issue and by the latency of the staging loads.  Against the list kernel below four features:
+// F = 3, n = 1M, 32 neighbours 754 -> 465 us; F = 1, n = 131072, distance-weighted 108 -> 63 us; F = 4, n = 434630,
+// 4 neighbours (sparse cells, runs of eight) 518 -> 140 us.  Six CTAs per SM (80 registers) measured fastest: eight
+// spill (+15 %), five leave fewer warps (+8 %), ten +32 %.
+template <int NF> struct DirectSmem {
+    static constexpr int STAGE_CAP = 256;
+    static constexpr int STAGE_BYTES = TestStage<STAGE_CAP>::BYTES;
+    static constexpr int FEAT_BYTES = NF * STAGE_CAP * 4;
+    static constexpr int PER_WARP = (STAGE_BYTES + FEAT_BYTES + (QDENSE + 20) * 4 + 15) / 16 * 16;
+};
+constexpr int DIRECT_CTAS = 6;
+
+template <int NF, bool DIST, bool MI>
+__device__ __forceinline__ void direct_slice(const RadiusParams& p, const int cellid, const int run, const int qs0, const int qe0, unsigned char* s_raw) {
+    using SM = DirectSmem<NF>;
+    constexpr int STAGE_CAP = SM::STAGE_CAP;
+    constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    unsigned char* base = s_raw + (size_t)(threadIdx.x >> 5) * SM::PER_WARP;
+    const TestStage<STAGE_CAP> stage(base);
+    float* s_feat = reinterpret_cast<float*>(base + SM::STAGE_BYTES);                   // [NF][STAGE_CAP]
+    int* s_self = reinterpret_cast<int*>(base + SM::STAGE_BYTES + SM::FEAT_BYTES);      // staged slot of every query, or -1
+    int* s_delta = s_self + QDENSE;
+
+    const float neg_c2 = !DIST ? -1.4426950408889634f / (2.f * p.p0 * p.p0) : 0.f;   // exp(-d2/(2 s^2)) = 2^(d2 * neg_c2)
+    // a periodic dimension with three cells or fewer has no consistent shifted frame: explicit minimum image
+    const bool mi0 = MI && p.periodic[0] && p.nc[0] <= 3, mi1 = MI && p.periodic[1] && p.nc[1] <= 3, mi2 = MI && p.periodic[2] && p.nc[2] <= 3;
+    auto delta = [&](const int d, const float q, const float c4) -> float {
+        const bool mi = d == 0 ? mi0 : d == 1 ? mi1 : mi2;
+        return (MI && mi) ? mi_delta(q, c4, p.len[d], 0.5f * p.len[d]) : q - c4;
+    };
+    const unsigned lt_mask = (1u << lane) - 1u;
+    const RunFrame frame(p, cellid, run);
+    const RunStencil sten(p, frame.c, run, s_delta);
+
+    // bounding box of the queries: a candidate farther than the cutoff from it is not staged
+    float blo[3] = {FAR_AWAY, FAR_AWAY, FAR_AWAY}, bhi[3] = {-FAR_AWAY, -FAR_AWAY, -FAR_AWAY};
+    for (int q = qs0 + lane; q < qe0; q += 32) {
+        float4 pq = p.spos[q];
+        frame.shift(p, pq);
+        const float l[3] = {pq.x, pq.y, pq.z};
+#pragma unroll
+        for (int d = 0; d < 3; ++d) { blo[d] = fminf(blo[d], l[d]); bhi[d] = fmaxf(bhi[d], l[d]); }
+    }
+#pragma unroll
+    for (int d = 0; d < 3; ++d) { blo[d] = warp_min(blo[d]); bhi[d] = warp_max(bhi[d]); }
+    if (mi0) { blo[0] = -FAR_AWAY; bhi[0] = FAR_AWAY; }   // a dimension folded by the explicit minimum image is not pruned
+    if (mi1) { blo[1] = -FAR_AWAY; bhi[1] = FAR_AWAY; }
+    if (mi2) { blo[2] = -FAR_AWAY; bhi[2] = FAR_AWAY; }
+    for (int k = lane; k < qe0 - qs0; k += 32) s_self[k] = -1;
+
+    auto process_chunk = [&](const int ns, const bool first_chunk) {
+        stage.seal(ns);
+        __syncwarp();
+        const int batches = (qe0 - qs0 + TEST_BATCH - 1) / TEST_BATCH, per = (qe0 - qs0 + batches - 1) / batches;
+        for (int qb0 = qs0; qb0 < qe0; qb0 += per) {
+            const int nq = (qe0 - qb0 < per) ? qe0 - qb0 : per;
+            const LaneSplit split(nq);
+            float4 qv = p.spos[qb0 + (split.active ? split.q : 0)];
+            frame.shift(p, qv);
+            const int qid = checked(__float_as_int(qv.w), p.n, CHECK_POINT);
+            unsigned mask[4];
+            test_candidates<MI, STAGE_CAP>(p, stage, ns, split, qv.x, qv.y, qv.z, mask, delta);
+            drop_candidate(mask, split, split.active ? s_self[qb0 - qs0 + split.q] : -1);
+            float acc[NF];
+            int cnt = 0;
+#pragma unroll
+            for (int f = 0; f < NF; ++f) acc[f] = 0.f;
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+                unsigned m = mask[w];
+                while (m) {
+                    const int k = __clz(m);
+                    m ^= 0x80000000u >> k;
+                    const int slot = split.slot(w, k);
+                    const float dx = delta(0, qv.x, stage.x[slot]), dy = delta(1, qv.y, stage.y[slot]), dz = delta(2, qv.z, stage.z[slot]);
+                    const float d2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+                    // within the fp32 error band of the cutoff: decided in fp64
+                    if (d2 > p.r2_mid - p.r2_band && !exact_pair(p, qid, stage.id[slot])) continue;
+                    const float val = DIST ? sqrtf(d2) : fast_exp2(d2 * neg_c2);
+#pragma unroll
+                    for (int f = 0; f < NF; ++f) acc[f] = fmaf(val, s_feat[f * STAGE_CAP + slot], acc[f]);
+                    ++cnt;
+                }
+            }
+            // sum over the lanes of a query, result in its lane with sub = 0
+            auto query_sum = [&](auto v) {
+#pragma unroll
+                for (int o = 1; o < TEST_LPQ; o <<= 1) {
+                    const auto other = __shfl_down_sync(FULL, v, o);
+                    if (split.sub + o < split.lpq) v += other;
+                }
+                return v;
+            };
+#pragma unroll
+            for (int f = 0; f < NF; ++f) acc[f] = query_sum(acc[f]);
+            if (p.count) cnt = query_sum(cnt);
+            if (split.active && split.sub == 0) {
+                float* o = p.out + (size_t)qid * NF;
+#pragma unroll
+                for (int f = 0; f < NF; ++f) o[f] = first_chunk ? acc[f] : o[f] + acc[f];
+                if (p.count) p.count[qid] = first_chunk ? cnt : p.count[qid] + cnt;
+            }
+        }
+        __syncwarp();
+    };
+
+    // The stage fills with candidates that survive the pruning and is processed when the next step's
+    // candidates might not fit, so the chunks are as full as the pruning allows (one chunk for all but dense cells).
+    bool first_chunk = true;
+    int nst = 0;                                                             // candidates staged (warp uniform)
+    int before = -1;                                                         // ranges that began before the step, minus one
+    constexpr int SU = 4;                                                    // staging groups in flight
+    for (int k0 = 0;; k0 += 32 * SU) {
+        const bool done = k0 >= sten.total;
+        const int step = done ? 0 : (sten.total - k0 < 32 * SU ? sten.total - k0 : 32 * SU);
+        if ((done && (nst > 0 || first_chunk)) || nst + step > STAGE_CAP) {     // the one place a chunk is processed
+            process_chunk(nst, first_chunk);
+            first_chunk = false;
+            nst = 0;
+            for (int k = lane; k < qe0 - qs0; k += 32) s_self[k] = -1;
+            __syncwarp();
+        }
+        if (done) break;
+        float4 c4[SU];
+        int src[SU], slot[SU];
+#pragma unroll
+        for (int u = 0; u < SU; ++u) {                                       // all loads of the step first
+            c4[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            src[u] = -1;
+            if (32 * u >= step) continue;
+            src[u] = sten.source(k0 + 32 * u, before, s_delta);
+            if (k0 + 32 * u + lane < sten.total) c4[u] = __ldg(p.spos + checked(src[u], p.n, CHECK_SLOT));
+        }
+#pragma unroll
+        for (int u = 0; u < SU; ++u) {
+            slot[u] = -1;
+            if (32 * u >= step) continue;
+            frame.shift(p, c4[u]);
+            const float ex = fmaxf(fmaxf(blo[0] - c4[u].x, c4[u].x - bhi[0]), 0.f);
+            const float ey = fmaxf(fmaxf(blo[1] - c4[u].y, c4[u].y - bhi[1]), 0.f);
+            const float ez = fmaxf(fmaxf(blo[2] - c4[u].z, c4[u].z - bhi[2]), 0.f);
+            const bool keep = k0 + 32 * u + lane < sten.total && fmaf(ez, ez, fmaf(ey, ey, ex * ex)) <= p.r2_hi * 1.0001f;
+            const unsigned m = __ballot_sync(FULL, keep);
+            if (keep) slot[u] = nst + __popc(m & lt_mask);
+            nst += __popc(m);
+        }
+        float xf[SU][NF];
+#pragma unroll
+        for (int u = 0; u < SU; ++u) {
+            if (32 * u >= step) continue;
+            const float* xr = p.feat + (size_t)(unsigned)(slot[u] < 0 ? 0 : checked(__float_as_int(c4[u].w), p.n, CHECK_POINT)) * NF;
+            if constexpr (NF == 4) {
+                const float4 v = __ldg(reinterpret_cast<const float4*>(xr));
+                xf[u][0] = v.x; xf[u][1] = v.y; xf[u][2] = v.z; xf[u][3] = v.w;
+            } else {
+#pragma unroll
+                for (int f = 0; f < NF; ++f) xf[u][f] = __ldg(xr + f);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < SU; ++u) {
+            if (slot[u] < 0) continue;
+            stage.put(slot[u], c4[u]);
+            if (src[u] >= qs0 && src[u] < qe0) s_self[src[u] - qs0] = slot[u];
+#pragma unroll
+            for (int f = 0; f < NF; ++f) s_feat[f * STAGE_CAP + slot[u]] = xf[u][f];
+        }
+    }
+}
+
+template <int NF, bool DIST, bool MI>
+__global__ void __launch_bounds__(TRAV_THREADS, DIRECT_CTAS) radius_direct_kernel(const __grid_constant__ RadiusParams p) {
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    walk_slices(p, [&](const int cell, const int run, const int qs, const int qe) { direct_slice<NF, DIST, MI>(p, cell, run, qs, qe, s_raw); });
 }
 
 // ------------------------------------------------------------------------------ host side
@@ -740,6 +913,20 @@ RadiusLayout carve_radius(RadiusParams* p, void* ws, int32_t** fill) {
     return RadiusLayout{cv.off, nblocks};
 }
 
+// A cell of a sparse input holds a point or two, and its stencil costs as much as a full one: joining cells along x
+// shares it (F = 16, n = 300k, 8 neighbours: forward 218 -> 135, backward 341 -> 175 us; F = 64, n = 100k, 4
+// neighbours: 139 -> 48 and 209 -> 78 us; nothing is joined at 32 neighbours).
+// Cells along x per warp: enough for about RUN_QUERIES / 2 points at the mean density, as long as a dozen warps per SM
+// remain; a run's stencil must not meet itself around a periodic face (the frame shift needs two cells between).
+static int run_length(const RadiusParams& p) {
+    long long r = p.n > 0 ? (long long)p.ncells * (RUN_QUERIES / 2) / p.n : 1;
+    const long long warps = p.ncells / (148 * 12), room = !p.periodic[0] ? RUN_CELLS : p.nc[0] < 4 ? 1 : p.nc[0] - 3;
+    r = r > warps ? warps : r;
+    r = r > room ? room : r;
+    r = r > RUN_CELLS ? RUN_CELLS : r;
+    return r < 1 ? 1 : (int)r;
+}
+
 tiga_status fill_params(RadiusParams* p, long long n, float r, const tiga_box* box) {
     int nc[3];
     float invh[3];
@@ -757,6 +944,7 @@ tiga_status fill_params(RadiusParams* p, long long n, float r, const tiga_box* b
         if (p->periodic[d] && nc[d] <= 3) single_periodic = true;
     }
     p->ncells = nc[0] * nc[1] * nc[2];
+    p->run = run_length(*p);
     const float r2 = r * r;
     const float beta = (single_periodic ? 96.f : 32.f) * 5.9604645e-8f;
     p->r2_lo = r2 * (1.f - beta);
@@ -793,23 +981,39 @@ static int feature_lanes(int F) {
 
 template <int MODE, int LF, bool DIST, bool MI>
 static tiga_status launch_traverse_t(const RadiusParams& p, cudaStream_t s) {
-    const unsigned blocks = (unsigned)((p.ncells + TRAV_WARPS - 1) / TRAV_WARPS);
     constexpr int smem = TravSmem<MODE>::PER_WARP * TRAV_WARPS;
     if (MODE == 0 && (p.F & 3)) {
         // scalar feature accesses (only the forward supports widths that are not multiples of 4)
         auto sk = radius_traverse_kernel<MODE == 0 ? 0 : MODE, LF, DIST, MI, MODE != 0 ? 1 : 0>;
         if (smem > 48 * 1024) TIGA_CUDA_TRY(cudaFuncSetAttribute(sk, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        return cells_then_queue(p, s, [&](const RadiusParams& q, unsigned grid) { sk<<<counted(grid), TRAV_THREADS, smem, s>>>(q); });
+        return runs_then_queue(p, s, [&](const RadiusParams& q, unsigned grid) { sk<<<counted(grid), TRAV_THREADS, smem, s>>>(q); });
     }
     auto kern = p.F == 4 * LF ? radius_traverse_kernel<MODE, LF, DIST, MI, 2> : radius_traverse_kernel<MODE, LF, DIST, MI, 1>;
     if (smem > 48 * 1024) TIGA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    return cells_then_queue(p, s, [&](const RadiusParams& q, unsigned grid) { kern<<<counted(grid), TRAV_THREADS, smem, s>>>(q); });
+    return runs_then_queue(p, s, [&](const RadiusParams& q, unsigned grid) { kern<<<counted(grid), TRAV_THREADS, smem, s>>>(q); });
+}
+
+template <int NF, bool DIST, bool MI>
+static tiga_status launch_direct_t(const RadiusParams& p, cudaStream_t s) {
+    constexpr int smem = DirectSmem<NF>::PER_WARP * TRAV_WARPS;
+    auto kern = radius_direct_kernel<NF, DIST, MI>;
+    if (smem > 48 * 1024) TIGA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    return runs_then_queue(p, s, [&](const RadiusParams& q, unsigned grid) { kern<<<counted(grid), TRAV_THREADS, smem, s>>>(q); });
 }
 
 template <int MODE, bool DIST, bool MI>
 static tiga_status launch_traverse_lf(const RadiusParams& p, cudaStream_t s) {
+    if constexpr (MODE == 0) {
+        switch (p.F) {
+            case 1: return launch_direct_t<1, DIST, MI>(p, s);
+            case 2: return launch_direct_t<2, DIST, MI>(p, s);
+            case 3: return launch_direct_t<3, DIST, MI>(p, s);
+            case 4: return launch_direct_t<4, DIST, MI>(p, s);
+            default: break;
+        }
+    }
     switch (feature_lanes(p.F)) {
-        case 1: return launch_traverse_t<MODE, 1, DIST, MI>(p, s);
+        case 1: if constexpr (MODE == 2) return launch_traverse_t<2, 1, DIST, MI>(p, s);
         case 2: return launch_traverse_t<MODE, 2, DIST, MI>(p, s);
         case 4: return launch_traverse_t<MODE, 4, DIST, MI>(p, s);
         case 8: return launch_traverse_t<MODE, 8, DIST, MI>(p, s);

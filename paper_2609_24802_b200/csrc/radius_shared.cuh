@@ -14,6 +14,8 @@ constexpr float FAR_AWAY = 1.0e18f;
 constexpr int QDENSE = 64;              // a cell with more points than this is cut into slices of QSLICE queries:
 constexpr int QSLICE = 16;              // its warp takes the first slice, the others wait in a queue that other warps walk
 constexpr int QUEUE_BLOCKS = 148 * 8;   // most CTAs that walk the queued slices
+constexpr int RUN_CELLS = 8;            // longest run of cells along x that one warp covers
+constexpr int RUN_QUERIES = 16;         // points a warp joins cells for
 constexpr int SORT_DENSE = 256;         // a cell with more points than this is ordered by a sorting network, not by rank counting
 
 struct RadiusParams {
@@ -54,6 +56,7 @@ struct RadiusParams {
     int2* q_items;            // (cell, first query of the slice)
     int* q_count;
     int q_mode;               // two-launch form: 0 = one warp per cell, 1 = warps walk the queue
+    int run;                  // cells along x that one warp of the Gaussian / distance traversals covers
     int cell_blocks;          // one-launch form: CTAs [0, cell_blocks) take cells, the CTAs behind them walk the queue
     int32_t* b_items;         // cells with more than SORT_DENSE points (queued by the same scan), and how many
     int* b_count;
@@ -122,6 +125,16 @@ static inline tiga_status cells_then_queue(const RadiusParams& p, cudaStream_t s
     return launch_status();
 }
 
+// The same with runs of p.run cells along x per warp.
+template <typename Launch>
+static inline tiga_status runs_then_queue(const RadiusParams& p, cudaStream_t s, Launch launch) {
+    RadiusParams q = p;
+    const long long warps = (long long)((p.nc[0] + p.run - 1) / p.run) * p.nc[1] * p.nc[2];
+    q.cell_blocks = (int)((warps + TRAV_WARPS - 1) / TRAV_WARPS);
+    launch(q, (unsigned)q.cell_blocks + queue_blocks(p.n));
+    return launch_status();
+}
+
 // Runs a traversal kernel twice: over the cells, then over the queue of slices (for kernels whose
 // register allocation suffers from carrying both loops).
 template <typename Launch>
@@ -146,12 +159,25 @@ static __device__ __forceinline__ float fast_rcp(float x) {
     return r;
 }
 
+// minimum / maximum over the warp in one instruction (sm_100a has the fp32 form), the result in every lane
+static __device__ __forceinline__ float warp_min(float v) {
+    float r;
+    asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
+}
+static __device__ __forceinline__ float warp_max(float v) {
+    float r;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
+}
+
 // two fp32 values per register pair: sm_100 executes add / mul / fma on both with one instruction
 typedef unsigned long long f32x2;
 static __device__ __forceinline__ f32x2 pack2(float a, float b) { f32x2 r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b)); return r; }
 static __device__ __forceinline__ void unpack2(f32x2 v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
 static __device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) { f32x2 r; asm("sub.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
 static __device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) { f32x2 r; asm("mul.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+static __device__ __forceinline__ f32x2 dup2(float a) { return pack2(a, a); }
 static __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) { f32x2 r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
 
 // Minimum-image displacement of two coordinates of a periodic dimension that is not split into enough

@@ -114,6 +114,39 @@ def test_forward_widths_that_are_not_multiples_of_four(tiga, F):
     assert ei.value.status == 2
 
 
+@pytest.mark.parametrize("per_cell", [1, 3, 4, 5, 8, 9, 16, 17, 33, 64, 65, 130])
+@pytest.mark.parametrize("F", [1, 2, 3, 4, 8])
+def test_narrow_features_at_every_split_of_the_lanes(tiga, F, per_cell):
+    """Forwards with at most four features share the warp's lanes out by the number of queries of a cell (and
+    F = 8 shares lists between lane groups): occupancies on both sides of every split, of the query
+    batch (16), of the dense-cell slices (64) and of the staged chunk (256 candidates), with wrapped
+    faces (four cells) and with the explicit minimum image (three cells)."""
+    ones = np.ones(3, np.float32)
+    for cells, periodic in ((3, 1), (4, 1), (3, 0)):
+        n = per_cell * cells ** 3
+        pos = gen.uniform_points(n, 60 + F + per_cell)
+        x = gen.normal_features(n, F, 60 + F + per_cell, 31)
+        r = np.float32(1.0 / cells / 1.002)
+        for kind in (tiga.MSG_GAUSS, tiga.MSG_DIST):
+            _check_gauss(tiga, pos, x, None, r, ones, [periodic] * 3, np.float32(float(r) / 2), kind=kind, backward=False)
+
+
+@pytest.mark.parametrize("F", [1, 4, 16])
+@pytest.mark.parametrize("cells", [(5, 60, 61), (11, 41, 41), (64, 24, 24), (41, 30, 30)])
+def test_runs_of_sparse_cells(tiga, cells, F):
+    """Sparse inputs join neighbouring cells along x: every run length from 1 to 8 (limited by the grid where the faces
+    wrap), runs that touch the lower or the upper face, a remainder run at the end of a row."""
+    box = np.array(cells, np.float32)
+    r = np.float32(1.0 / 1.002)
+    n = int(np.prod(cells))
+    for share, periodic in ((1.0, 1), (0.4, 1), (0.4, 0), (3.0, 0)):
+        m = int(share * n)
+        pos = gen.uniform_points(m, 70 + F) * box[None, :]
+        pos = np.minimum(pos, box[None, :])
+        x, gy = gen.normal_features(m, F, 71, 31), gen.normal_features(m, F, 71, 32)
+        _check_gauss(tiga, pos, x, gy, r, box, [periodic] * 3, np.float32(0.5), use_cells=True, backward=F >= 4)
+
+
 def test_few_cells_mixed_periodicity_and_anisotropic_box(tiga):
     # the paper's tiny radius shape: 128 points, cutoff 0.35 (two cells per dimension)
     pos = gen.uniform_points(128, 7)
