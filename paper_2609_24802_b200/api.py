@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 
 import torch
 
@@ -151,34 +152,39 @@ def load_library() -> ctypes.CDLL:
     return lib
 
 
-load_library()      # fail at import time, loudly, when the CUDA library is not there
+_L = load_library()      # fail at import time, loudly, when the CUDA library is not there
+
+# A call on a small relation is bound by its marshalling, so the calls below avoid what costs a microsecond each:
+# the message structs of the stored relation are built once, a stream is looked up by its handle (no Stream object),
+# pointers are passed as plain integers, outputs are allocated with new_empty.
+_current_device = torch._C._cuda_getDevice
+_raw_stream = torch._C._cuda_getCurrentRawStream
 
 
 def checked_status(reset: bool = True) -> int:
     """Bits of the checked build's status word (0 in the normal build): 1 source index, 2 edge position,
     4 point id, 8 slot.  Synchronises the device."""
-    return int(load_library().tiga_checked_status(int(reset)))
+    return int(_L.tiga_checked_status(int(reset)))
 
 
 def is_checked_build() -> bool:
-    return bool(load_library().tiga_is_checked_build())
+    return bool(_L.tiga_is_checked_build())
 
 
 def launch_count() -> int:
     """Kernels launched by the library so far in this process (counted inside the library)."""
-    return int(load_library().tiga_kernel_launches())
+    return int(_L.tiga_kernel_launches())
 
 
 def _ptr(t):
     if t is None:
-        return ctypes.c_void_p(0)
+        return None
     assert t.is_cuda and t.is_contiguous(), "device arrays must be contiguous CUDA tensors"
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _stream(stream):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    return _raw_stream(_current_device()) if stream is None else stream.cuda_stream
 
 
 def _ok(st, where):
@@ -190,6 +196,14 @@ def _ws(nbytes, like):
     return torch.empty(max(int(nbytes), 256), dtype=torch.uint8, device=like.device)
 
 
+def _new(like, shape, dtype=torch.float32):
+    """Uninitialised fp32 (or `dtype`) array on the device of `like`."""
+    return like.new_empty(shape) if like.dtype is dtype else like.new_empty(shape, dtype=dtype)
+
+
+_ARG_DTYPE = {MAX: torch.int32, MAX64: torch.int64}
+
+
 def _dt(t):
     if t.dtype == torch.float32:
         return F32
@@ -199,7 +213,7 @@ def _dt(t):
 
 
 def tiga_status_string(status: int) -> str:
-    return load_library().tiga_status_string(int(status)).decode()
+    return _L.tiga_status_string(int(status)).decode()
 
 
 class CsrRelation:
@@ -214,32 +228,32 @@ class CsrRelation:
         self.c = _Csr(rowptr.data_ptr(), I32 if rowptr.dtype == torch.int32 else I64,
                       col.data_ptr() if col.numel() else 0, self.n_dst, self.n_src, self.n_edges)
 
-    @property
-    def ref(self):
-        return ctypes.byref(self.c)
+        self.ref = ctypes.byref(self.c)
+
+
+_MSG_REF = {False: ctypes.byref(_Msg(MSG_COPY, 0.0, 0.0)), True: ctypes.byref(_Msg(MSG_WEIGHTED, 0.0, 0.0))}     # by "has weights"
 
 
 def tiga_csr_workspace_bytes(g: CsrRelation, F: int, x_dtype: int = F32, reducer: int = SUM,
                              backward: bool = False) -> int:
-    return int(load_library().tiga_csr_workspace_bytes(g.ref, F, x_dtype, reducer, int(backward)))
+    return int(_L.tiga_csr_workspace_bytes(g.ref, F, x_dtype, reducer, int(backward)))
 
 
 def tiga_validate_csr(g: CsrRelation, level: int = 1, stream=None) -> None:
     ws = _ws(256, g.rowptr)
-    _ok(load_library().tiga_validate_csr(g.ref, level, _ptr(ws), ws.numel(), _stream(stream)), "tiga_validate_csr")
+    _ok(_L.tiga_validate_csr(g.ref, level, _ptr(ws), ws.numel(), _stream(stream)), "tiga_validate_csr")
 
 
 def tiga_apply_csr(g: CsrRelation, x, w=None, reducer: int = SUM, out=None, argmax=None, ws=None, stream=None):
     """out[i,:] = reduce over the row's edges of w[e] * x[col[e],:].  Returns (out, argmax)."""
     F = x.shape[1]
     if out is None:
-        out = torch.empty((g.n_dst, F), dtype=torch.float32, device=x.device)
-    if reducer in (MAX, MAX64) and argmax is None:
-        argmax = torch.empty((g.n_dst, F), dtype=torch.int32 if reducer == MAX else torch.int64, device=x.device)
+        out = _new(x, (g.n_dst, F))
+    if reducer in _ARG_DTYPE and argmax is None:
+        argmax = _new(x, (g.n_dst, F), _ARG_DTYPE[reducer])
     if ws is None:
         ws = _ws(tiga_csr_workspace_bytes(g, F, _dt(x), reducer, False), x)
-    msg = _Msg(MSG_COPY if w is None else MSG_WEIGHTED, 0.0, 0.0)
-    _ok(load_library().tiga_apply_csr(g.ref, _ptr(x), _dt(x), F, _ptr(w), ctypes.byref(msg), reducer, _ptr(out),
+    _ok(_L.tiga_apply_csr(g.ref, _ptr(x), _dt(x), F, _ptr(w), _MSG_REF[w is not None], reducer, _ptr(out),
                                       _ptr(argmax), _ptr(ws), ws.numel(), _stream(stream)), "tiga_apply_csr")
     return out, argmax
 
@@ -255,11 +269,10 @@ def tiga_apply_csr_builtin_ws(g: CsrRelation, x, w=None, reducer: int = SUM, out
     as a convenience when omitted.  Returns (out, argmax)."""
     F = x.shape[1]
     if out is None:
-        out = torch.empty((g.n_dst, F), dtype=torch.float32, device=x.device)
-    if reducer in (MAX, MAX64) and argmax is None:
-        argmax = torch.empty((g.n_dst, F), dtype=torch.int32 if reducer == MAX else torch.int64, device=x.device)
-    msg = _Msg(MSG_COPY if w is None else MSG_WEIGHTED, 0.0, 0.0)
-    _ok(load_library().tiga_apply_csr_builtin_ws(g.ref, _ptr(x), _dt(x), F, _ptr(w), ctypes.byref(msg), reducer,
+        out = _new(x, (g.n_dst, F))
+    if reducer in _ARG_DTYPE and argmax is None:
+        argmax = _new(x, (g.n_dst, F), _ARG_DTYPE[reducer])
+    _ok(_L.tiga_apply_csr_builtin_ws(g.ref, _ptr(x), _dt(x), F, _ptr(w), _MSG_REF[w is not None], reducer,
                                                  _ptr(out), _ptr(argmax), _stream(stream)), "tiga_apply_csr_builtin_ws")
     return out, argmax
 
@@ -269,13 +282,12 @@ def tiga_apply_csr_backward(g: CsrRelation, x, w, grad_out, reducer: int = SUM, 
     """Returns (grad_x, grad_w); either is None when not requested."""
     F = x.shape[1]
     if want_x and grad_x is None:
-        grad_x = torch.empty((g.n_src, F), dtype=torch.float32, device=x.device)
+        grad_x = _new(x, (g.n_src, F))
     if want_w and grad_w is None:
-        grad_w = torch.empty((g.n_edges,), dtype=torch.float32, device=x.device)
+        grad_w = _new(x, (g.n_edges,))
     if ws is None:
         ws = _ws(tiga_csr_workspace_bytes(g, F, _dt(x), reducer, True), x)
-    msg = _Msg(MSG_COPY if w is None else MSG_WEIGHTED, 0.0, 0.0)
-    _ok(load_library().tiga_apply_csr_backward(g.ref, _ptr(x), _dt(x), F, _ptr(w), ctypes.byref(msg), reducer, _ptr(grad_out),
+    _ok(_L.tiga_apply_csr_backward(g.ref, _ptr(x), _dt(x), F, _ptr(w), _MSG_REF[w is not None], reducer, _ptr(grad_out),
                                                _ptr(argmax), _ptr(grad_x), _ptr(grad_w), _ptr(ws), ws.numel(),
                                                _stream(stream)), "tiga_apply_csr_backward")
     return grad_x, grad_w
@@ -303,7 +315,7 @@ def tiga_csr_plan_build(g: CsrRelation, max_hot_rows: int = None, row_bytes: int
                         stream=None) -> CsrPlan:
     """Builds the hot-source plan of a relation (one-time, synchronises).  ``max_hot_rows`` defaults to
     as many rows as fit ``hot_bytes`` of compact feature table."""
-    lib = load_library()
+    lib = _L
     if max_hot_rows is None:
         max_hot_rows = max(1, hot_bytes // row_bytes)
     max_hot_rows = int(min(max_hot_rows, g.n_src))
@@ -320,7 +332,7 @@ def tiga_csr_plan_build(g: CsrRelation, max_hot_rows: int = None, row_bytes: int
 
 
 def tiga_csr_planned_workspace_bytes(plan: CsrPlan, F: int, x_dtype: int = F32, reducer: int = SUM) -> int:
-    return int(load_library().tiga_csr_planned_workspace_bytes(plan.g.ref, ctypes.byref(plan.c), F, x_dtype, reducer))
+    return int(_L.tiga_csr_planned_workspace_bytes(plan.g.ref, ctypes.byref(plan.c), F, x_dtype, reducer))
 
 
 def tiga_apply_csr_planned(plan: CsrPlan, x, w=None, reducer: int = SUM, out=None, argmax=None, ws=None, stream=None):
@@ -328,33 +340,31 @@ def tiga_apply_csr_planned(plan: CsrPlan, x, w=None, reducer: int = SUM, out=Non
     F = x.shape[1]
     g = plan.g
     if out is None:
-        out = torch.empty((g.n_dst, F), dtype=torch.float32, device=x.device)
-    if reducer in (MAX, MAX64) and argmax is None:
-        argmax = torch.empty((g.n_dst, F), dtype=torch.int32 if reducer == MAX else torch.int64, device=x.device)
+        out = _new(x, (g.n_dst, F))
+    if reducer in _ARG_DTYPE and argmax is None:
+        argmax = _new(x, (g.n_dst, F), _ARG_DTYPE[reducer])
     if ws is None:
         ws = _ws(tiga_csr_planned_workspace_bytes(plan, F, _dt(x), reducer), x)
-    msg = _Msg(MSG_COPY if w is None else MSG_WEIGHTED, 0.0, 0.0)
-    _ok(load_library().tiga_apply_csr_planned(g.ref, ctypes.byref(plan.c), _ptr(plan.buf), _ptr(x), _dt(x), F, _ptr(w),
-                                              ctypes.byref(msg), reducer, _ptr(out), _ptr(argmax), _ptr(ws), ws.numel(),
+    _ok(_L.tiga_apply_csr_planned(g.ref, ctypes.byref(plan.c), _ptr(plan.buf), _ptr(x), _dt(x), F, _ptr(w),
+                                              _MSG_REF[w is not None], reducer, _ptr(out), _ptr(argmax), _ptr(ws), ws.numel(),
                                               _stream(stream)), "tiga_apply_csr_planned")
     return out, argmax
 
 
 def tiga_csr_degree_histogram(g: CsrRelation, nbins: int = 4096, stream=None):
     """Returns (hist int64[nbins], max_degree int64[1]) as device tensors."""
-    hist = torch.empty(nbins, dtype=torch.int64, device=g.rowptr.device)
-    mx = torch.empty(1, dtype=torch.int64, device=g.rowptr.device)
-    _ok(load_library().tiga_csr_degree_histogram(g.ref, _ptr(hist), nbins, _ptr(mx), _stream(stream)),
+    hist, mx = _new(g.rowptr, (nbins,), torch.int64), _new(g.rowptr, (1,), torch.int64)
+    _ok(_L.tiga_csr_degree_histogram(g.ref, _ptr(hist), nbins, _ptr(mx), _stream(stream)),
         "tiga_csr_degree_histogram")
     return hist, mx
 
 
+_BOX_BYTES = struct.Struct("=3f3i")
+_BOX_OF = _Box.from_buffer_copy
+
+
 def _box(box, periodic):
-    b = _Box()
-    for d in range(3):
-        b.len[d] = float(box[d])
-        b.periodic[d] = int(periodic[d])
-    return b
+    return _BOX_OF(_BOX_BYTES.pack(box[0], box[1], box[2], int(periodic[0]), int(periodic[1]), int(periodic[2])))
 
 
 def tiga_radius_grid(n: int, r: float, box, periodic):
@@ -362,7 +372,7 @@ def tiga_radius_grid(n: int, r: float, box, periodic):
     b = _box(box, periodic)
     nc = (ctypes.c_int32 * 3)()
     ih = (ctypes.c_float * 3)()
-    _ok(load_library().tiga_radius_grid(n, float(r), ctypes.byref(b), nc, ih), "tiga_radius_grid")
+    _ok(_L.tiga_radius_grid(n, float(r), ctypes.byref(b), nc, ih), "tiga_radius_grid")
     return list(nc), list(ih)
 
 
@@ -370,13 +380,13 @@ def tiga_validate_points(pos, box, periodic=(0, 0, 0), level: int = 1, stream=No
     """Raises TigaError (status 7) when a coordinate is not finite or lies outside [0, len]."""
     b = _box(box, periodic)
     ws = _ws(256, pos)
-    _ok(load_library().tiga_validate_points(_ptr(pos), pos.shape[0], ctypes.byref(b), level, _ptr(ws), ws.numel(),
+    _ok(_L.tiga_validate_points(_ptr(pos), pos.shape[0], ctypes.byref(b), level, _ptr(ws), ws.numel(),
                                             _stream(stream)), "tiga_validate_points")
 
 
 def tiga_radius_workspace_bytes(n: int, F: int, r: float, box, periodic, backward: bool = False) -> int:
     b = _box(box, periodic)
-    return int(load_library().tiga_radius_workspace_bytes(n, F, float(r), ctypes.byref(b), int(backward)))
+    return int(_L.tiga_radius_workspace_bytes(n, F, float(r), ctypes.byref(b), int(backward)))
 
 
 def tiga_radius_bin(pos, r: float, box, periodic, ws=None, stream=None):
@@ -390,7 +400,7 @@ def tiga_radius_bin(pos, r: float, box, periodic, ws=None, stream=None):
     order = torch.empty(n, dtype=torch.int32, device=pos.device)
     if ws is None:
         ws = _ws(tiga_radius_workspace_bytes(n, 0, r, box, periodic), pos)
-    _ok(load_library().tiga_radius_bin(_ptr(pos), n, float(r), ctypes.byref(b), _ptr(cell), _ptr(start),
+    _ok(_L.tiga_radius_bin(_ptr(pos), n, float(r), ctypes.byref(b), _ptr(cell), _ptr(start),
                                        _ptr(order), _ptr(ws), ws.numel(), _stream(stream)), "tiga_radius_bin")
     return dict(cell=cell, cell_start=start, order=order, ncell=ncell, ws=ws)
 
@@ -402,12 +412,12 @@ def tiga_apply_radius(pos, feat, r: float, box, periodic, kind: int = MSG_GAUSS,
     F = 4 if kind == MSG_LJ else feat.shape[1]
     b = _box(box, periodic)
     if out is None:
-        out = torch.empty((n, F), dtype=torch.float32, device=pos.device)
+        out = _new(pos, (n, F))
     if want_count and count is None:
-        count = torch.empty(n, dtype=torch.int32, device=pos.device)
+        count = _new(pos, (n,), torch.int32)
     if ws is None:
         ws = _ws(tiga_radius_workspace_bytes(n, F, r, box, periodic), pos)
-    _ok(load_library().tiga_apply_radius(_ptr(pos), _ptr(feat), n, F, float(r), ctypes.byref(b),
+    _ok(_L.tiga_apply_radius(_ptr(pos), _ptr(feat), n, F, float(r), ctypes.byref(b),
                                          ctypes.byref(_Msg(kind, float(p0), float(p1))), _ptr(out), _ptr(count), _ptr(ws),
                                          ws.numel(), _stream(stream)), "tiga_apply_radius")
     return out, count, ws
@@ -420,13 +430,13 @@ def tiga_apply_radius_backward(pos, feat, grad_out, r: float, box, periodic, sig
     n, F = feat.shape
     b = _box(box, periodic)
     if want_feat and grad_feat is None:
-        grad_feat = torch.empty((n, F), dtype=torch.float32, device=pos.device)
+        grad_feat = _new(pos, (n, F))
     if want_pos and grad_pos is None:
-        grad_pos = torch.empty((n, 3), dtype=torch.float32, device=pos.device)
+        grad_pos = _new(pos, (n, 3))
     if ws is None:
         assert not reuse_plan
         ws = _ws(tiga_radius_workspace_bytes(n, F, r, box, periodic, True), pos)
-    _ok(load_library().tiga_apply_radius_backward(_ptr(pos), _ptr(feat), n, F, float(r), ctypes.byref(b),
+    _ok(_L.tiga_apply_radius_backward(_ptr(pos), _ptr(feat), n, F, float(r), ctypes.byref(b),
                                                   ctypes.byref(_Msg(MSG_GAUSS, float(sigma), 0.0)), _ptr(grad_out),
                                                   _ptr(grad_feat), _ptr(grad_pos), _ptr(ws), ws.numel(),
                                                   int(bool(reuse_plan)), _stream(stream)),
@@ -448,12 +458,12 @@ def tiga_apply_radius_mlp(pos, feat, r: float, box, periodic, W1, b1, W2, b2, ou
     m = _edge_mlp(W1, b1, W2, b2)
     bx = _box(box, periodic)
     if out is None:
-        out = torch.empty((n, m.f_out), dtype=torch.float32, device=pos.device)
+        out = _new(pos, (n, m.f_out))
     if want_count and count is None:
-        count = torch.empty(n, dtype=torch.int32, device=pos.device)
+        count = _new(pos, (n,), torch.int32)
     if ws is None:
         ws = _ws(tiga_radius_workspace_bytes(n, m.f_in, r, box, periodic), pos)
-    _ok(load_library().tiga_apply_radius_mlp(_ptr(pos), _ptr(feat), n, float(r), ctypes.byref(bx), ctypes.byref(m),
+    _ok(_L.tiga_apply_radius_mlp(_ptr(pos), _ptr(feat), n, float(r), ctypes.byref(bx), ctypes.byref(m),
                                              _ptr(out), _ptr(count), _ptr(ws), ws.numel(), _stream(stream)),
         "tiga_apply_radius_mlp")
     return out, count, ws
@@ -465,14 +475,12 @@ def tiga_apply_radius_mlp_backward(pos, feat, grad_out, r: float, box, periodic,
     n = pos.shape[0]
     m = _edge_mlp(W1, b1, W2, b2)
     bx = _box(box, periodic)
-    dev = pos.device
-    g = dict(grad_feat=torch.empty((n, m.f_in), device=dev), grad_pos=torch.empty((n, 3), device=dev),
-             grad_W1=torch.empty_like(W1), grad_b1=torch.empty_like(b1), grad_W2=torch.empty_like(W2),
-             grad_b2=torch.empty_like(b2))
+    g = dict(grad_feat=_new(pos, (n, m.f_in)), grad_pos=_new(pos, (n, 3)), grad_W1=torch.empty_like(W1),
+             grad_b1=torch.empty_like(b1), grad_W2=torch.empty_like(W2), grad_b2=torch.empty_like(b2))
     if ws is None:
         assert not reuse_plan
         ws = _ws(tiga_radius_workspace_bytes(n, m.f_in, r, box, periodic, True), pos)
-    _ok(load_library().tiga_apply_radius_mlp_backward(_ptr(pos), _ptr(feat), n, float(r), ctypes.byref(bx), ctypes.byref(m),
+    _ok(_L.tiga_apply_radius_mlp_backward(_ptr(pos), _ptr(feat), n, float(r), ctypes.byref(bx), ctypes.byref(m),
                                                       _ptr(grad_out), _ptr(g["grad_feat"]), _ptr(g["grad_pos"]),
                                                       _ptr(g["grad_W1"]), _ptr(g["grad_b1"]), _ptr(g["grad_W2"]),
                                                       _ptr(g["grad_b2"]), _ptr(ws), ws.numel(), int(bool(reuse_plan)),
@@ -482,7 +490,7 @@ def tiga_apply_radius_mlp_backward(pos, feat, grad_out, r: float, box, periodic,
 
 def tiga_knn_workspace_bytes(n: int, k: int, box) -> int:
     b = _box(box, (0, 0, 0))
-    return int(load_library().tiga_knn_workspace_bytes(n, k, ctypes.byref(b)))
+    return int(_L.tiga_knn_workspace_bytes(n, k, ctypes.byref(b)))
 
 
 def tiga_apply_knn(pos, feat, k: int, box, periodic=(0, 0, 0), out=None, nbr=None, nbr_d2=None,
@@ -491,22 +499,21 @@ def tiga_apply_knn(pos, feat, k: int, box, periodic=(0, 0, 0), out=None, nbr=Non
     Returns (out, nbr int32 [n,k] or None, nbr_d2 fp32 [n,k] or None, ws)."""
     n, F = feat.shape
     b = _box(box, periodic)
-    dev = pos.device
     if out is None:
-        out = torch.empty((n, F), dtype=torch.float32, device=dev)
+        out = _new(pos, (n, F))
     if want_nbr and nbr is None:
-        nbr = torch.empty((n, k), dtype=torch.int32, device=dev)
+        nbr = _new(pos, (n, k), torch.int32)
     if want_nbr and nbr_d2 is None:
-        nbr_d2 = torch.empty((n, k), dtype=torch.float32, device=dev)
+        nbr_d2 = _new(pos, (n, k))
     if ws is None:
         ws = _ws(tiga_knn_workspace_bytes(n, k, box), pos)
-    _ok(load_library().tiga_apply_knn(_ptr(pos), _ptr(feat), n, F, int(k), ctypes.byref(b), _ptr(out), _ptr(nbr),
+    _ok(_L.tiga_apply_knn(_ptr(pos), _ptr(feat), n, F, int(k), ctypes.byref(b), _ptr(out), _ptr(nbr),
                                       _ptr(nbr_d2), _ptr(ws), ws.numel(), _stream(stream)), "tiga_apply_knn")
     return out, nbr, nbr_d2, ws
 
 
 def tiga_csr_attention_workspace_bytes(g: CsrRelation, D: int) -> int:
-    return int(load_library().tiga_csr_attention_workspace_bytes(g.ref, int(D)))
+    return int(_L.tiga_csr_attention_workspace_bytes(g.ref, int(D)))
 
 
 def tiga_apply_csr_attention(g: CsrRelation, q, key, value, scale: float, out=None, lse=None, want_lse=True,
@@ -515,11 +522,11 @@ def tiga_apply_csr_attention(g: CsrRelation, q, key, value, scale: float, out=No
     (online-softmax reducer).  Returns (out, lse, ws)."""
     D = q.shape[1]
     if out is None:
-        out = torch.empty((g.n_dst, D), dtype=torch.float32, device=q.device)
+        out = _new(q, (g.n_dst, D))
     if want_lse and lse is None:
-        lse = torch.empty(g.n_dst, dtype=torch.float32, device=q.device)
+        lse = _new(q, (g.n_dst,))
     if ws is None:
         ws = _ws(tiga_csr_attention_workspace_bytes(g, D), q)
-    _ok(load_library().tiga_apply_csr_attention(g.ref, _ptr(q), _ptr(key), _ptr(value), D, float(scale), _ptr(out),
+    _ok(_L.tiga_apply_csr_attention(g.ref, _ptr(q), _ptr(key), _ptr(value), D, float(scale), _ptr(out),
                                                 _ptr(lse), _ptr(ws), ws.numel(), _stream(stream)), "tiga_apply_csr_attention")
     return out, lse, ws
