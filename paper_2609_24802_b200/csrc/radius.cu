@@ -22,7 +22,7 @@
 // coordinates; a cell whose stencil wraps around a periodic face moves the points next to the
 // upper face down by the box length, which is exact in fp32, so every displacement is one
 // rounded subtraction of two stored coordinates, for wrapped pairs as for interior ones.
-#include "radius_test.cuh"
+#include "radius_direct.cuh"
 #include <type_traits>
 
 namespace tiga {
@@ -263,8 +263,8 @@ __global__ void validate_points_kernel(const float* __restrict__ pos, long long 
 //             (staged slot, d^2 or weight) where the displacement is needed again.
 //   phase B : MODE 0 (Gaussian / distance forward) and MODE 2 (Gaussian backward): LF lanes
 //             span one feature row with 128-bit accesses and 32 / LF queries advance together,
-//             four gathered rows in flight per lane.  (The Lennard-Jones message has its own
-//             kernel in radius_lj.cu, which visits every unordered pair once.)
+//             four gathered rows in flight per lane.  (Lennard-Jones and rows of at most four
+//             features: radius_direct.cuh.)
 // Lists hold QCAP entries per query and the stage STAGE_CAP candidates; when either fills up
 // the warp drains / processes and goes on, so any density works.  A cell with more than QDENSE
 // points is cut into slices of QSLICE queries: its warp takes the first, the others wait in a queue (filled
@@ -291,7 +291,7 @@ template <int MODE> struct TravSmem {
 // VEC: 0 = scalar feature accesses (F % 4 != 0, forward only); 1 = 128-bit accesses, F % 4 == 0;
 // 2 = additionally F == 4 LF exactly, so the row stride is a compile-time constant.
 template <int MODE, int LF, bool DIST, bool MI, int VEC>
-__device__ __forceinline__ void traverse_slice(const RadiusParams& p, const int cellid, const int run, const int qs0, const int qe0, unsigned char* s_raw) {
+__device__ __forceinline__ void traverse_slice(const RadiusParams& p, const int (&c)[3], const int run, const int qs0, const int qe0, unsigned char* s_raw) {
     using SM = TravSmem<MODE>;
     constexpr int STAGE_CAP = SM::STAGE_CAP, QCAP = SM::QCAP, QSTRIDE = SM::QSTRIDE, TQB = SM::TQB;
     constexpr unsigned FULL = 0xffffffffu;
@@ -308,7 +308,6 @@ __device__ __forceinline__ void traverse_slice(const RadiusParams& p, const int 
     float* s_frame = reinterpret_cast<float*>(s_tot + TQB);                              // thresholds [3], shifts [3]
     int* s_delta = reinterpret_cast<int*>(s_frame + 8);                                  // source minus flattened position of every range
 
-    const int c[3] = {cellid % p.nc[0], (cellid / p.nc[0]) % p.nc[1], cellid / (p.nc[0] * p.nc[1])};
     const int F = VEC == 2 ? 4 * LF : p.F;
     const float neg_c2 = !DIST ? -1.4426950408889634f / (2.f * p.p0 * p.p0) : 0.f;   // exp(-d2/(2 s^2)) = 2^(d2 * neg_c2)
     // a periodic dimension with three cells or fewer has no consistent shifted frame: explicit minimum image
@@ -638,233 +637,33 @@ __device__ __forceinline__ void traverse_slice(const RadiusParams& p, const int 
     }
 }
 
-// CTAs [0, cell_blocks): warp w takes the w-th run of p.run cells along x; the cells are joined as long as they hold at
-// most RUN_QUERIES points together (of a cell with more than QDENSE points the first QSLICE queries).  The CTAs behind
-// them walk the queue of the remaining slices.
-template <typename Work>
-__device__ __forceinline__ void walk_slices(const RadiusParams& p, Work work) {
-    if ((int)blockIdx.x < p.cell_blocks) {
-        const int w = blockIdx.x * TRAV_WARPS + (threadIdx.x >> 5);
-        const int lane = threadIdx.x & 31;
-        const int per_row = (p.nc[0] + p.run - 1) / p.run;
-        const int row = w / per_row, x0 = (w - row * per_row) * p.run;
-        if (row >= p.nc[1] * p.nc[2]) return;
-        const int cells = p.nc[0] - x0 < p.run ? p.nc[0] - x0 : p.run, cell0 = row * p.nc[0] + x0;
-        const int start = p.cell_start[cell0 + (lane < cells ? lane : cells)];          // lane k: first point of cell k of the run
-        const int len = __shfl_down_sync(0xffffffffu, start, 1) - start;
-        unsigned left = __ballot_sync(0xffffffffu, lane < cells && len > 0);            // occupied cells not done yet
-        while (left) {
-            const int a = __ffs(left) - 1, qs = __shfl_sync(0xffffffffu, start, a), first = __shfl_sync(0xffffffffu, len, a);
-            int qe = qs + (first > QDENSE ? QSLICE : first), last = a;
-            left &= left - 1u;
-            while (left) {
-                const int b = __ffs(left) - 1, more = __shfl_sync(0xffffffffu, start + len, b);
-                if (first > QDENSE || more - qs > RUN_QUERIES) break;
-                qe = more; last = b;
-                left &= left - 1u;
-            }
-            work(cell0 + a, last - a + 1, qs, qe);
-            __syncwarp();
-        }
-    } else {
-        const int n = *p.q_count;
-        const int w = (blockIdx.x - p.cell_blocks) * TRAV_WARPS + (threadIdx.x >> 5);
-        for (int it = w; it < n; it += (gridDim.x - p.cell_blocks) * TRAV_WARPS) {
-            const int2 item = p.q_items[it];
-            const int qs0 = p.cell_start[item.x] + item.y, end = p.cell_start[item.x + 1];
-            work(item.x, 1, qs0, slice_end(qs0, end));
-            __syncwarp();
-        }
-    }
-}
-
 template <int MODE, int LF, bool DIST, bool MI, int VEC = 1>
 __global__ void __launch_bounds__(TRAV_THREADS, (MODE == 0 ? 7 : 0)) radius_traverse_kernel(const __grid_constant__ RadiusParams p) {
     extern __shared__ __align__(16) unsigned char s_raw[];
-    walk_slices(p, [&](const int cell, const int run, const int qs, const int qe) { traverse_slice<MODE, LF, DIST, MI, VEC>(p, cell, run, qs, qe, s_raw); });
+    walk_slices(p, [&](const int (&cell)[3], const int run, const int qs, const int qe) { traverse_slice<MODE, LF, DIST, MI, VEC>(p, cell, run, qs, qe, s_raw); });
 }
 
 // ------------------------------------------------------------------------------ at most four features
 // Forward with NF <= 4 features per point (the distance-weighted scalar sum among them).  A gather by groups of
 // lanes would leave most of the warp idle on such rows, so nothing is gathered: the features are staged with
-// the candidates, every query has its own lanes, and a lane adds weight * features of its accepted candidates in
-// registers (test and expansion: radius_test.cuh).  One warp per run of cells, slices of dense cells from the queue.
+// the candidates and summed where a pair is accepted (radius_direct.cuh).
 // Bound by instruction issue and by the latency of the staging loads.  Against the list kernel below four features:
-// F = 3, n = 1M, 32 neighbours 754 -> 465 us; F = 1, n = 131072, distance-weighted 108 -> 63 us; F = 4, n = 434630,
-// 4 neighbours (sparse cells, runs of eight) 518 -> 140 us.  Six CTAs per SM (80 registers) measured fastest: eight
-// spill (+15 %), five leave fewer warps (+8 %), ten +32 %.
-template <int NF> struct DirectSmem {
-    static constexpr int STAGE_CAP = 256;
-    static constexpr int STAGE_BYTES = TestStage<STAGE_CAP>::BYTES;
-    static constexpr int FEAT_BYTES = NF * STAGE_CAP * 4;
-    static constexpr int PER_WARP = (STAGE_BYTES + FEAT_BYTES + (QDENSE + 20) * 4 + 15) / 16 * 16;
+// F = 3, n = 1M, 32 neighbours 754 -> 405 us; F = 1, n = 131072, distance-weighted 108 -> 53 us; F = 4, n = 434630,
+// 4 neighbours (sparse cells, runs of eight) 518 -> 126 us.
+template <int NF, bool DIST>
+struct SumMsg {
+    static constexpr int CAP = 256, STAGED = NF, OUT = NF, CTAS = 6;
+    static constexpr float OUTSIDE = DIST ? 0.f : 1.0e30f;
+    float neg_c2;
+    // exp(-d2/(2 s^2)) = 2^(d2 * neg_c2)
+    __device__ __forceinline__ explicit SumMsg(const RadiusParams& p) : neg_c2(!DIST ? -1.4426950408889634f / (2.f * p.p0 * p.p0) : 0.f) {}
+    __device__ __forceinline__ void pair(f32x2 (&acc)[NF], const float da, const float db, f32x2, f32x2, f32x2, const float* xa, const float* xb) const {
+        const f32x2 val = DIST ? pack2(sqrtf(da), sqrtf(db)) : pack2(fast_exp2(da * neg_c2), fast_exp2(db * neg_c2));
+#pragma unroll
+        for (int f = 0; f < NF; ++f) acc[f] = fma2(val, pack2(xa[f * CAP], xb[f * CAP]), acc[f]);
+    }
+    __device__ __forceinline__ float scale(int, const float v) const { return v; }
 };
-constexpr int DIRECT_CTAS = 6;
-
-template <int NF, bool DIST, bool MI>
-__device__ __forceinline__ void direct_slice(const RadiusParams& p, const int cellid, const int run, const int qs0, const int qe0, unsigned char* s_raw) {
-    using SM = DirectSmem<NF>;
-    constexpr int STAGE_CAP = SM::STAGE_CAP;
-    constexpr unsigned FULL = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    unsigned char* base = s_raw + (size_t)(threadIdx.x >> 5) * SM::PER_WARP;
-    const TestStage<STAGE_CAP> stage(base);
-    float* s_feat = reinterpret_cast<float*>(base + SM::STAGE_BYTES);                   // [NF][STAGE_CAP]
-    int* s_self = reinterpret_cast<int*>(base + SM::STAGE_BYTES + SM::FEAT_BYTES);      // staged slot of every query, or -1
-    int* s_delta = s_self + QDENSE;
-
-    const float neg_c2 = !DIST ? -1.4426950408889634f / (2.f * p.p0 * p.p0) : 0.f;   // exp(-d2/(2 s^2)) = 2^(d2 * neg_c2)
-    // a periodic dimension with three cells or fewer has no consistent shifted frame: explicit minimum image
-    const bool mi0 = MI && p.periodic[0] && p.nc[0] <= 3, mi1 = MI && p.periodic[1] && p.nc[1] <= 3, mi2 = MI && p.periodic[2] && p.nc[2] <= 3;
-    auto delta = [&](const int d, const float q, const float c4) -> float {
-        const bool mi = d == 0 ? mi0 : d == 1 ? mi1 : mi2;
-        return (MI && mi) ? mi_delta(q, c4, p.len[d], 0.5f * p.len[d]) : q - c4;
-    };
-    const unsigned lt_mask = (1u << lane) - 1u;
-    const RunFrame frame(p, cellid, run);
-    const RunStencil sten(p, frame.c, run, s_delta);
-
-    // bounding box of the queries: a candidate farther than the cutoff from it is not staged
-    float blo[3] = {FAR_AWAY, FAR_AWAY, FAR_AWAY}, bhi[3] = {-FAR_AWAY, -FAR_AWAY, -FAR_AWAY};
-    for (int q = qs0 + lane; q < qe0; q += 32) {
-        float4 pq = p.spos[q];
-        frame.shift(p, pq);
-        const float l[3] = {pq.x, pq.y, pq.z};
-#pragma unroll
-        for (int d = 0; d < 3; ++d) { blo[d] = fminf(blo[d], l[d]); bhi[d] = fmaxf(bhi[d], l[d]); }
-    }
-#pragma unroll
-    for (int d = 0; d < 3; ++d) { blo[d] = warp_min(blo[d]); bhi[d] = warp_max(bhi[d]); }
-    if (mi0) { blo[0] = -FAR_AWAY; bhi[0] = FAR_AWAY; }   // a dimension folded by the explicit minimum image is not pruned
-    if (mi1) { blo[1] = -FAR_AWAY; bhi[1] = FAR_AWAY; }
-    if (mi2) { blo[2] = -FAR_AWAY; bhi[2] = FAR_AWAY; }
-    for (int k = lane; k < qe0 - qs0; k += 32) s_self[k] = -1;
-
-    auto process_chunk = [&](const int ns, const bool first_chunk) {
-        stage.seal(ns);
-        __syncwarp();
-        const int batches = (qe0 - qs0 + TEST_BATCH - 1) / TEST_BATCH, per = (qe0 - qs0 + batches - 1) / batches;
-        for (int qb0 = qs0; qb0 < qe0; qb0 += per) {
-            const int nq = (qe0 - qb0 < per) ? qe0 - qb0 : per;
-            const LaneSplit split(nq);
-            float4 qv = p.spos[qb0 + (split.active ? split.q : 0)];
-            frame.shift(p, qv);
-            const int qid = checked(__float_as_int(qv.w), p.n, CHECK_POINT);
-            unsigned mask[4];
-            test_candidates<MI, STAGE_CAP>(p, stage, ns, split, qv.x, qv.y, qv.z, mask, delta);
-            drop_candidate(mask, split, split.active ? s_self[qb0 - qs0 + split.q] : -1);
-            float acc[NF];
-            int cnt = 0;
-#pragma unroll
-            for (int f = 0; f < NF; ++f) acc[f] = 0.f;
-#pragma unroll
-            for (int w = 0; w < 4; ++w) {
-                unsigned m = mask[w];
-                while (m) {
-                    const int k = __clz(m);
-                    m ^= 0x80000000u >> k;
-                    const int slot = split.slot(w, k);
-                    const float dx = delta(0, qv.x, stage.x[slot]), dy = delta(1, qv.y, stage.y[slot]), dz = delta(2, qv.z, stage.z[slot]);
-                    const float d2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-                    // within the fp32 error band of the cutoff: decided in fp64
-                    if (d2 > p.r2_mid - p.r2_band && !exact_pair(p, qid, stage.id[slot])) continue;
-                    const float val = DIST ? sqrtf(d2) : fast_exp2(d2 * neg_c2);
-#pragma unroll
-                    for (int f = 0; f < NF; ++f) acc[f] = fmaf(val, s_feat[f * STAGE_CAP + slot], acc[f]);
-                    ++cnt;
-                }
-            }
-            // sum over the lanes of a query, result in its lane with sub = 0
-            auto query_sum = [&](auto v) {
-#pragma unroll
-                for (int o = 1; o < TEST_LPQ; o <<= 1) {
-                    const auto other = __shfl_down_sync(FULL, v, o);
-                    if (split.sub + o < split.lpq) v += other;
-                }
-                return v;
-            };
-#pragma unroll
-            for (int f = 0; f < NF; ++f) acc[f] = query_sum(acc[f]);
-            if (p.count) cnt = query_sum(cnt);
-            if (split.active && split.sub == 0) {
-                float* o = p.out + (size_t)qid * NF;
-#pragma unroll
-                for (int f = 0; f < NF; ++f) o[f] = first_chunk ? acc[f] : o[f] + acc[f];
-                if (p.count) p.count[qid] = first_chunk ? cnt : p.count[qid] + cnt;
-            }
-        }
-        __syncwarp();
-    };
-
-    // The stage fills with candidates that survive the pruning and is processed when the next step's
-    // candidates might not fit, so the chunks are as full as the pruning allows (one chunk for all but dense cells).
-    bool first_chunk = true;
-    int nst = 0;                                                             // candidates staged (warp uniform)
-    int before = -1;                                                         // ranges that began before the step, minus one
-    constexpr int SU = 4;                                                    // staging groups in flight
-    for (int k0 = 0;; k0 += 32 * SU) {
-        const bool done = k0 >= sten.total;
-        const int step = done ? 0 : (sten.total - k0 < 32 * SU ? sten.total - k0 : 32 * SU);
-        if ((done && (nst > 0 || first_chunk)) || nst + step > STAGE_CAP) {     // the one place a chunk is processed
-            process_chunk(nst, first_chunk);
-            first_chunk = false;
-            nst = 0;
-            for (int k = lane; k < qe0 - qs0; k += 32) s_self[k] = -1;
-            __syncwarp();
-        }
-        if (done) break;
-        float4 c4[SU];
-        int src[SU], slot[SU];
-#pragma unroll
-        for (int u = 0; u < SU; ++u) {                                       // all loads of the step first
-            c4[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-            src[u] = -1;
-            if (32 * u >= step) continue;
-            src[u] = sten.source(k0 + 32 * u, before, s_delta);
-            if (k0 + 32 * u + lane < sten.total) c4[u] = __ldg(p.spos + checked(src[u], p.n, CHECK_SLOT));
-        }
-#pragma unroll
-        for (int u = 0; u < SU; ++u) {
-            slot[u] = -1;
-            if (32 * u >= step) continue;
-            frame.shift(p, c4[u]);
-            const float ex = fmaxf(fmaxf(blo[0] - c4[u].x, c4[u].x - bhi[0]), 0.f);
-            const float ey = fmaxf(fmaxf(blo[1] - c4[u].y, c4[u].y - bhi[1]), 0.f);
-            const float ez = fmaxf(fmaxf(blo[2] - c4[u].z, c4[u].z - bhi[2]), 0.f);
-            const bool keep = k0 + 32 * u + lane < sten.total && fmaf(ez, ez, fmaf(ey, ey, ex * ex)) <= p.r2_hi * 1.0001f;
-            const unsigned m = __ballot_sync(FULL, keep);
-            if (keep) slot[u] = nst + __popc(m & lt_mask);
-            nst += __popc(m);
-        }
-        float xf[SU][NF];
-#pragma unroll
-        for (int u = 0; u < SU; ++u) {
-            if (32 * u >= step) continue;
-            const float* xr = p.feat + (size_t)(unsigned)(slot[u] < 0 ? 0 : checked(__float_as_int(c4[u].w), p.n, CHECK_POINT)) * NF;
-            if constexpr (NF == 4) {
-                const float4 v = __ldg(reinterpret_cast<const float4*>(xr));
-                xf[u][0] = v.x; xf[u][1] = v.y; xf[u][2] = v.z; xf[u][3] = v.w;
-            } else {
-#pragma unroll
-                for (int f = 0; f < NF; ++f) xf[u][f] = __ldg(xr + f);
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < SU; ++u) {
-            if (slot[u] < 0) continue;
-            stage.put(slot[u], c4[u]);
-            if (src[u] >= qs0 && src[u] < qe0) s_self[src[u] - qs0] = slot[u];
-#pragma unroll
-            for (int f = 0; f < NF; ++f) s_feat[f * STAGE_CAP + slot[u]] = xf[u][f];
-        }
-    }
-}
-
-template <int NF, bool DIST, bool MI>
-__global__ void __launch_bounds__(TRAV_THREADS, DIRECT_CTAS) radius_direct_kernel(const __grid_constant__ RadiusParams p) {
-    extern __shared__ __align__(16) unsigned char s_raw[];
-    walk_slices(p, [&](const int cell, const int run, const int qs, const int qe) { direct_slice<NF, DIST, MI>(p, cell, run, qs, qe, s_raw); });
-}
 
 // ------------------------------------------------------------------------------ host side
 static long long icbrt_floor(long long v) {
@@ -993,22 +792,14 @@ static tiga_status launch_traverse_t(const RadiusParams& p, cudaStream_t s) {
     return runs_then_queue(p, s, [&](const RadiusParams& q, unsigned grid) { kern<<<counted(grid), TRAV_THREADS, smem, s>>>(q); });
 }
 
-template <int NF, bool DIST, bool MI>
-static tiga_status launch_direct_t(const RadiusParams& p, cudaStream_t s) {
-    constexpr int smem = DirectSmem<NF>::PER_WARP * TRAV_WARPS;
-    auto kern = radius_direct_kernel<NF, DIST, MI>;
-    if (smem > 48 * 1024) TIGA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    return runs_then_queue(p, s, [&](const RadiusParams& q, unsigned grid) { kern<<<counted(grid), TRAV_THREADS, smem, s>>>(q); });
-}
-
 template <int MODE, bool DIST, bool MI>
 static tiga_status launch_traverse_lf(const RadiusParams& p, cudaStream_t s) {
     if constexpr (MODE == 0) {
         switch (p.F) {
-            case 1: return launch_direct_t<1, DIST, MI>(p, s);
-            case 2: return launch_direct_t<2, DIST, MI>(p, s);
-            case 3: return launch_direct_t<3, DIST, MI>(p, s);
-            case 4: return launch_direct_t<4, DIST, MI>(p, s);
+            case 1: return launch_direct_t<SumMsg<1, DIST>, MI>(p, s);
+            case 2: return launch_direct_t<SumMsg<2, DIST>, MI>(p, s);
+            case 3: return launch_direct_t<SumMsg<3, DIST>, MI>(p, s);
+            case 4: return launch_direct_t<SumMsg<4, DIST>, MI>(p, s);
             default: break;
         }
     }
@@ -1133,7 +924,7 @@ extern "C" tiga_status tiga_apply_radius(const float* pos, const float* feat, in
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     st = run_binning(p, fill, lay.nblocks, s);
     if (st != TIGA_OK) return st;
-    if (msg->kind == TIGA_MSG_LJ) return launch_lj_pairs(p, s);
+    if (msg->kind == TIGA_MSG_LJ) return launch_lj(p, s);
     if (msg->kind == TIGA_MSG_DIST) return launch_traverse<0, true>(p, s);
     return launch_traverse<0, false>(p, s);
 }

@@ -1,0 +1,282 @@
+// Traversal that consumes a pair where it is accepted (test: radius_test.cuh): every query has its own lanes, and a
+// lane adds the messages of its accepted candidates in registers.  No lists, no gathers, no atomics.  One warp per run
+// of cells, slices of dense cells from the queue.
+//
+// Msg supplies the message:
+//   CAP             candidates the stage holds
+//   STAGED          features per point that are staged with the candidates
+//   OUT             sums per query
+//   OUTSIDE         a squared distance whose message is zero
+//   Msg(p)          constants
+//   pair(...)       adds the messages of two accepted candidates to acc[OUT], one per half
+//   scale(f, v)     the stored value of sum f
+#pragma once
+#include "radius_test.cuh"
+
+namespace tiga {
+
+// CTAs [0, cell_blocks): warp w takes the w-th run of p.run cells along x; the cells are joined as long as they hold at
+// most RUN_QUERIES points together (of a cell with more than QDENSE points the first QSLICE queries).  The CTAs behind
+// them walk the queue of the remaining slices.
+template <typename Work>
+__device__ __forceinline__ void walk_slices(const RadiusParams& p, Work work) {
+    if ((int)blockIdx.x < p.cell_blocks) {
+        const int w = blockIdx.x * TRAV_WARPS + (threadIdx.x >> 5);
+        const int lane = threadIdx.x & 31;
+        const int row = w / p.row_runs, x0 = (w - row * p.row_runs) * p.run;
+        const int cz = row / p.nc[1], cy = row - cz * p.nc[1];
+        if (cz >= p.nc[2]) return;
+        const int cells = p.nc[0] - x0 < p.run ? p.nc[0] - x0 : p.run, cell0 = row * p.nc[0] + x0;
+        const int start = p.cell_start[cell0 + (lane < cells ? lane : cells)];          // lane k: first point of cell k of the run
+        const int len = __shfl_down_sync(0xffffffffu, start, 1) - start;
+        unsigned left = __ballot_sync(0xffffffffu, lane < cells && len > 0);            // occupied cells not done yet
+        while (left) {
+            const int a = __ffs(left) - 1, qs = __shfl_sync(0xffffffffu, start, a), first = __shfl_sync(0xffffffffu, len, a);
+            int qe = qs + (first > QDENSE ? QSLICE : first), last = a;
+            left &= left - 1u;
+            while (left) {
+                const int b = __ffs(left) - 1, more = __shfl_sync(0xffffffffu, start + len, b);
+                if (first > QDENSE || more - qs > RUN_QUERIES) break;
+                qe = more; last = b;
+                left &= left - 1u;
+            }
+            const int cell[3] = {x0 + a, cy, cz};
+            work(cell, last - a + 1, qs, qe);
+            __syncwarp();
+        }
+    } else {
+        const int n = *p.q_count;
+        const int w = (blockIdx.x - p.cell_blocks) * TRAV_WARPS + (threadIdx.x >> 5);
+        for (int it = w; it < n; it += (gridDim.x - p.cell_blocks) * TRAV_WARPS) {
+            const int2 item = p.q_items[it];
+            const int qs0 = p.cell_start[item.x] + item.y, end = p.cell_start[item.x + 1];
+            const int row = item.x / p.nc[0], cz = row / p.nc[1];
+            const int cell[3] = {item.x - row * p.nc[0], row - cz * p.nc[1], cz};
+            work(cell, 1, qs0, slice_end(qs0, end));
+            __syncwarp();
+        }
+    }
+}
+
+template <typename Msg> struct DirectSmem {
+    static constexpr int STAGE_CAP = Msg::CAP, STAGED = Msg::STAGED;
+    static constexpr int STAGE_BYTES = TestStage<STAGE_CAP>::BYTES;
+    static constexpr int FEAT_BYTES = STAGED * STAGE_CAP * 4;
+    static constexpr int PER_WARP = (STAGE_BYTES + FEAT_BYTES + (QDENSE + 20) * 4 + 15) / 16 * 16;
+};
+
+// MI: some periodic dimension has three cells or fewer and uses the explicit minimum image.
+template <typename Msg, bool MI>
+__device__ __forceinline__ void direct_slice(const RadiusParams& p, const int (&cell)[3], const int run, const int qs0, const int qe0, unsigned char* s_raw) {
+    using SM = DirectSmem<Msg>;
+    constexpr int STAGE_CAP = SM::STAGE_CAP, OUT = Msg::OUT, NF = Msg::STAGED;
+    constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    unsigned char* base = s_raw + (size_t)(threadIdx.x >> 5) * SM::PER_WARP;
+    const TestStage<STAGE_CAP> stage(base);
+    float* s_feat = reinterpret_cast<float*>(base + SM::STAGE_BYTES);                   // [NF][STAGE_CAP]
+    int* s_self = reinterpret_cast<int*>(base + SM::STAGE_BYTES + SM::FEAT_BYTES);      // staged slot of every query, or -1
+    int* s_delta = s_self + QDENSE;
+
+    const Msg msg(p);
+    const bool mi0 = MI && p.periodic[0] && p.nc[0] <= 3, mi1 = MI && p.periodic[1] && p.nc[1] <= 3, mi2 = MI && p.periodic[2] && p.nc[2] <= 3;
+    auto delta = [&](const int d, const float q, const float c4) -> float {
+        const bool mi = d == 0 ? mi0 : d == 1 ? mi1 : mi2;
+        return (MI && mi) ? mi_delta(q, c4, p.len[d], 0.5f * p.len[d]) : q - c4;
+    };
+    const unsigned lt_mask = (1u << lane) - 1u;
+    const RunFrame frame(p, cell, run);
+    const RunStencil sten(p, frame.c, run, s_delta);
+
+    // bounding box of the queries: a candidate farther than the cutoff from it is not staged
+    float blo[3] = {FAR_AWAY, FAR_AWAY, FAR_AWAY}, bhi[3] = {-FAR_AWAY, -FAR_AWAY, -FAR_AWAY};
+    for (int q = qs0 + lane; q < qe0; q += 32) {
+        float4 pq = p.spos[q];
+        frame.shift(p, pq);
+        const float l[3] = {pq.x, pq.y, pq.z};
+#pragma unroll
+        for (int d = 0; d < 3; ++d) { blo[d] = fminf(blo[d], l[d]); bhi[d] = fmaxf(bhi[d], l[d]); }
+    }
+#pragma unroll
+    for (int d = 0; d < 3; ++d) { blo[d] = warp_min(blo[d]); bhi[d] = warp_max(bhi[d]); }
+    if (mi0) { blo[0] = -FAR_AWAY; bhi[0] = FAR_AWAY; }   // a dimension folded by the explicit minimum image is not pruned
+    if (mi1) { blo[1] = -FAR_AWAY; bhi[1] = FAR_AWAY; }
+    if (mi2) { blo[2] = -FAR_AWAY; bhi[2] = FAR_AWAY; }
+    for (int k = lane; k < qe0 - qs0; k += 32) s_self[k] = -1;
+
+    auto process_chunk = [&](const int ns, const bool first_chunk) {
+        stage.seal(ns);
+        __syncwarp();
+        // batches of one size, at most TEST_BATCH: a short last one would idle as many lanes as a full one keeps busy
+        const int all = qe0 - qs0;
+        const int per = all <= TEST_BATCH ? all : all <= 2 * TEST_BATCH ? (all + 1) >> 1 : TEST_BATCH;
+        for (int qb0 = qs0; qb0 < qe0; qb0 += per) {
+            const int nq = (qe0 - qb0 < per) ? qe0 - qb0 : per;
+            const LaneSplit split(nq);
+            float4 qv = p.spos[qb0 + (split.active ? split.q : 0)];
+            frame.shift(p, qv);
+            const int qid = checked(__float_as_int(qv.w), p.n, CHECK_POINT);
+            unsigned mask[4];
+            test_candidates<MI, STAGE_CAP>(p, stage, ns, split, qv.x, qv.y, qv.z, mask, delta);
+            drop_candidate(mask, split, split.active ? s_self[qb0 - qs0 + split.q] : -1);
+            f32x2 acc2[OUT];
+            int cnt = 0;
+#pragma unroll
+            for (int f = 0; f < OUT; ++f) acc2[f] = 0ull;
+            if (p.count) cnt = __popc(mask[0]) + __popc(mask[1]) + __popc(mask[2]) + __popc(mask[3]);
+            // the lane's accepted candidates, two at a time; a lane moves on to its next word by itself, so the
+            // warp makes as many trips as its busiest lane needs
+            const f32x2 qx2 = dup2(qv.x), qy2 = dup2(qv.y), qz2 = dup2(qv.z);
+            unsigned m = mask[0], m1 = mask[1], m2 = mask[2], m3 = mask[3];
+            int word = 2 * split.sub, next = 1;                         // stage slot of bit 31 of the current word, step to the next
+            while (m | m1 | m2 | m3) {
+                if (m == 0u) { m = m1; m1 = m2; m2 = m3; m3 = 0u; word += next; next = 2 * TEST_GROUP * split.lpq - next; }
+                if (m == 0u) continue;
+                const int ka = __clz(m);
+                m ^= 0x80000000u >> ka;
+                const bool two = m != 0u;
+                const int kb = two ? __clz(m) : ka;
+                m &= 0x7fffffffu >> kb;
+                const int sa = word + 2 * split.lpq * ka, sb = word + 2 * split.lpq * kb;
+                const float *ca = stage.x + sa, *cb = stage.x + sb;
+                constexpr int SL = TestStage<STAGE_CAP>::SLOTS;
+                f32x2 dx, dy, dz;
+                if constexpr (!MI) {
+                    dx = sub2(qx2, pack2(ca[0], cb[0]));
+                    dy = sub2(qy2, pack2(ca[SL], cb[SL]));
+                    dz = sub2(qz2, pack2(ca[2 * SL], cb[2 * SL]));
+                } else {
+                    dx = pack2(delta(0, qv.x, ca[0]), delta(0, qv.x, cb[0]));
+                    dy = pack2(delta(1, qv.y, ca[SL]), delta(1, qv.y, cb[SL]));
+                    dz = pack2(delta(2, qv.z, ca[2 * SL]), delta(2, qv.z, cb[2 * SL]));
+                }
+                float da, db;
+                unpack2(fma2(dz, dz, fma2(dy, dy, mul2(dx, dx))), da, db);
+                if (fmaxf(da, db) > p.r2_mid - p.r2_band) {        // within the fp32 error band of the cutoff: decided in fp64
+                    if (da > p.r2_mid - p.r2_band && !exact_pair(p, qid, stage.id[sa])) { da = Msg::OUTSIDE; --cnt; }
+                    if (two && db > p.r2_mid - p.r2_band && !exact_pair(p, qid, stage.id[sb])) { db = Msg::OUTSIDE; --cnt; }
+                }
+                if (!two) db = Msg::OUTSIDE;
+                msg.pair(acc2, da, db, dx, dy, dz, s_feat + sa, s_feat + sb);
+            }
+            float acc[OUT];
+#pragma unroll
+            for (int f = 0; f < OUT; ++f) { float lo, hi; unpack2(acc2[f], lo, hi); acc[f] = lo + hi; }
+            // sum over the lanes of a query, result in its lane with sub = 0
+            auto query_sum = [&](auto v) {
+#pragma unroll
+                for (int o = 1; o < TEST_LPQ; o <<= 1) {
+                    if (o >= split.lpq) break;
+                    const auto other = __shfl_down_sync(FULL, v, o);
+                    if (split.sub + o < split.lpq) v += other;
+                }
+                return v;
+            };
+#pragma unroll
+            for (int f = 0; f < OUT; ++f) acc[f] = msg.scale(f, query_sum(acc[f]));
+            if (p.count) cnt = query_sum(cnt);
+            if (split.active && split.sub == 0) {
+                float* o = p.out + (size_t)qid * OUT;
+                if constexpr (OUT == 4) {
+                    float4 v = make_float4(acc[0], acc[1], acc[2], acc[3]);
+                    if (!first_chunk) { const float4 old = *reinterpret_cast<float4*>(o); v.x += old.x; v.y += old.y; v.z += old.z; v.w += old.w; }
+                    *reinterpret_cast<float4*>(o) = v;
+                } else {
+#pragma unroll
+                    for (int f = 0; f < OUT; ++f) o[f] = first_chunk ? acc[f] : o[f] + acc[f];
+                }
+                if (p.count) p.count[qid] = first_chunk ? cnt : p.count[qid] + cnt;
+            }
+        }
+        __syncwarp();
+    };
+
+    // The stage fills with candidates that survive the pruning and is processed when the next step's survivors do
+    // not fit (that step is then taken again), so the chunks are as full as the pruning allows: one chunk for all but
+    // dense cells.
+    bool first_chunk = true, full = false;
+    int nst = 0;                                                             // candidates staged (warp uniform)
+    int before = -1;                                                         // ranges that began before the step, minus one
+    constexpr int SU = 4;                                                    // staging groups in flight
+    static_assert(STAGE_CAP >= 32 * SU, "a step fits an empty stage");
+    for (int k0 = 0;;) {
+        const bool done = k0 >= sten.total;
+        if (full || (done && (nst > 0 || first_chunk))) {                    // the one place a chunk is processed
+            process_chunk(nst, first_chunk);
+            first_chunk = false;
+            full = false;
+            nst = 0;
+            for (int k = lane; k < qe0 - qs0; k += 32) s_self[k] = -1;
+            __syncwarp();
+        }
+        if (done) break;
+        const int step = sten.total - k0 < 32 * SU ? sten.total - k0 : 32 * SU, before0 = before;
+        float4 c4[SU];
+        int src[SU];
+        unsigned kept[SU];
+#pragma unroll
+        for (int u = 0; u < SU; ++u) {                                       // all loads of the step first
+            c4[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            src[u] = -1;
+            if (32 * u >= step) continue;
+            src[u] = sten.source(k0 + 32 * u, before, s_delta);
+            if (k0 + 32 * u + lane < sten.total) c4[u] = __ldg(p.spos + checked(src[u], p.n, CHECK_SLOT));
+        }
+        int all = nst;
+#pragma unroll
+        for (int u = 0; u < SU; ++u) {
+            kept[u] = 0u;
+            if (32 * u >= step) continue;
+            frame.shift(p, c4[u]);
+            const float ex = fmaxf(fmaxf(blo[0] - c4[u].x, c4[u].x - bhi[0]), 0.f);
+            const float ey = fmaxf(fmaxf(blo[1] - c4[u].y, c4[u].y - bhi[1]), 0.f);
+            const float ez = fmaxf(fmaxf(blo[2] - c4[u].z, c4[u].z - bhi[2]), 0.f);
+            kept[u] = __ballot_sync(FULL, k0 + 32 * u + lane < sten.total && fmaf(ez, ez, fmaf(ey, ey, ex * ex)) <= p.r2_hi * 1.0001f);
+            all += __popc(kept[u]);
+        }
+        if (all > STAGE_CAP) { full = true; before = before0; continue; }
+        float xf[SU][NF > 0 ? NF : 1];
+        if constexpr (NF > 0) {
+#pragma unroll
+            for (int u = 0; u < SU; ++u) {
+                if (!((kept[u] >> lane) & 1u)) continue;
+                const float* xr = p.feat + (size_t)(unsigned)checked(__float_as_int(c4[u].w), p.n, CHECK_POINT) * NF;
+                if constexpr (NF == 4) {
+                    const float4 v = __ldg(reinterpret_cast<const float4*>(xr));
+                    xf[u][0] = v.x; xf[u][1] = v.y; xf[u][2] = v.z; xf[u][3] = v.w;
+                } else {
+#pragma unroll
+                    for (int f = 0; f < NF; ++f) xf[u][f] = __ldg(xr + f);
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < SU; ++u) {
+            if ((kept[u] >> lane) & 1u) {
+                const int slot = nst + __popc(kept[u] & lt_mask);
+                stage.put(slot, c4[u]);
+                if (src[u] >= qs0 && src[u] < qe0) s_self[src[u] - qs0] = slot;
+#pragma unroll
+                for (int f = 0; f < NF; ++f) s_feat[f * STAGE_CAP + slot] = xf[u][f];
+            }
+            nst += __popc(kept[u]);
+        }
+        k0 += 32 * SU;
+    }
+}
+
+template <typename Msg, bool MI>
+__global__ void __launch_bounds__(TRAV_THREADS, Msg::CTAS) radius_direct_kernel(const __grid_constant__ RadiusParams p) {
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    walk_slices(p, [&](const int (&cell)[3], const int run, const int qs, const int qe) { direct_slice<Msg, MI>(p, cell, run, qs, qe, s_raw); });
+}
+
+template <typename Msg, bool MI>
+static tiga_status launch_direct_t(const RadiusParams& p, cudaStream_t s) {
+    constexpr int smem = DirectSmem<Msg>::PER_WARP * TRAV_WARPS;
+    auto kern = radius_direct_kernel<Msg, MI>;
+    if (smem > 48 * 1024) TIGA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    return runs_then_queue(p, s, [&](const RadiusParams& q, unsigned grid) { kern<<<counted(grid), TRAV_THREADS, smem, s>>>(q); });
+}
+
+}  // namespace tiga

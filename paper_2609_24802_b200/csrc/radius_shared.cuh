@@ -55,8 +55,8 @@ struct RadiusParams {
     // slices of cells with more than QDENSE points, queued by the binning scan
     int2* q_items;            // (cell, first query of the slice)
     int* q_count;
-    int q_mode;               // two-launch form: 0 = one warp per cell, 1 = warps walk the queue
     int run;                  // cells along x that one warp of the Gaussian / distance traversals covers
+    int row_runs;             // runs per row of cells
     int cell_blocks;          // one-launch form: CTAs [0, cell_blocks) take cells, the CTAs behind them walk the queue
     int32_t* b_items;         // cells with more than SORT_DENSE points (queued by the same scan), and how many
     int* b_count;
@@ -75,8 +75,8 @@ struct RadiusLayout {
 tiga_status fill_params(RadiusParams* p, long long n, float r, const tiga_box* box);
 RadiusLayout carve_radius(RadiusParams* p, void* ws, int32_t** fill);
 tiga_status run_binning(RadiusParams& p, int32_t* fill, int nblocks, cudaStream_t s);
-// host side, defined in radius_lj.cu: zeroes out / count, then one launch (pairs visited once, rows summed by atomics)
-tiga_status launch_lj_pairs(const RadiusParams& p, cudaStream_t s);
+// host side, defined in radius_lj.cu
+tiga_status launch_lj(const RadiusParams& p, cudaStream_t s);
 
 // The defining predicate in double precision (same operations as the plain definition).
 static __device__ __noinline__ bool exact_within(const RadiusParams& p, const float4 a, const float4 b) {
@@ -115,35 +115,15 @@ static inline unsigned queue_blocks(long long n) {
     return (unsigned)(need < QUEUE_BLOCKS ? need : QUEUE_BLOCKS);
 }
 
-// One launch over the cells and, in the CTAs appended behind them, over the queue of slices (which the
-// binning filled before the launch).
-template <typename Launch>
-static inline tiga_status cells_then_queue(const RadiusParams& p, cudaStream_t s, Launch launch) {
-    RadiusParams q = p;
-    q.cell_blocks = (p.ncells + TRAV_WARPS - 1) / TRAV_WARPS;
-    launch(q, (unsigned)q.cell_blocks + queue_blocks(p.n));
-    return launch_status();
-}
-
-// The same with runs of p.run cells along x per warp.
+// One launch over the runs of p.run cells along x and, in the CTAs appended behind them, over the queue of slices
+// (which the binning filled before the launch).
 template <typename Launch>
 static inline tiga_status runs_then_queue(const RadiusParams& p, cudaStream_t s, Launch launch) {
     RadiusParams q = p;
-    const long long warps = (long long)((p.nc[0] + p.run - 1) / p.run) * p.nc[1] * p.nc[2];
+    q.row_runs = (p.nc[0] + p.run - 1) / p.run;
+    const long long warps = (long long)q.row_runs * p.nc[1] * p.nc[2];
     q.cell_blocks = (int)((warps + TRAV_WARPS - 1) / TRAV_WARPS);
     launch(q, (unsigned)q.cell_blocks + queue_blocks(p.n));
-    return launch_status();
-}
-
-// Runs a traversal kernel twice: over the cells, then over the queue of slices (for kernels whose
-// register allocation suffers from carrying both loops).
-template <typename Launch>
-static inline tiga_status two_passes(const RadiusParams& p, cudaStream_t s, Launch launch) {
-    RadiusParams q = p;
-    q.q_mode = 0;
-    launch(q, (unsigned)((p.ncells + TRAV_WARPS - 1) / TRAV_WARPS));
-    q.q_mode = 1;
-    launch(q, queue_blocks(p.n));
     return launch_status();
 }
 
@@ -176,6 +156,7 @@ typedef unsigned long long f32x2;
 static __device__ __forceinline__ f32x2 pack2(float a, float b) { f32x2 r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b)); return r; }
 static __device__ __forceinline__ void unpack2(f32x2 v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
 static __device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) { f32x2 r; asm("sub.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+static __device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) { f32x2 r; asm("add.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
 static __device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) { f32x2 r; asm("mul.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
 static __device__ __forceinline__ f32x2 dup2(float a) { return pack2(a, a); }
 static __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) { f32x2 r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }

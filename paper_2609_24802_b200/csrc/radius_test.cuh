@@ -4,14 +4,14 @@
 // The stage holds the candidates' coordinates by component, so that a test reads two candidates with one 64-bit load
 // per component and forms both squared distances with packed instructions.  Every query of the run gets
 // LPQ = 32 / queries lanes.  A lane keeps its query in registers, walks the candidate pairs sub, sub + LPQ, ... and
-// shifts one sign bit per candidate into a mask, which costs about six instructions per 32 tests; only accepted
+// shifts one sign bit per candidate into a mask, which costs about seven instructions per 32 tests; only accepted
 // candidates (one in four at the usual density) are looked at again, one at a time per lane.
 #pragma once
 #include "radius_shared.cuh"
 
 namespace tiga {
 
-constexpr int TEST_BATCH = 16;         // queries tested together: at least two lanes each, so four mask words cover the stage
+constexpr int TEST_BATCH = 16;         // queries tested together: at least two lanes each
 constexpr int TEST_LPQ = 8;            // most lanes per query
 constexpr int TEST_PAD = 40;           // sentinels behind the staged candidates (a test reads up to 4 TEST_LPQ + 1 further)
 
@@ -23,8 +23,8 @@ struct RunFrame {
     int c[3];
     bool face;
     float thr[3];
-    __device__ __forceinline__ RunFrame(const RadiusParams& p, const int cell, const int run) {
-        c[0] = cell % p.nc[0]; c[1] = cell / p.nc[0] % p.nc[1]; c[2] = cell / (p.nc[0] * p.nc[1]);
+    __device__ __forceinline__ RunFrame(const RadiusParams& p, const int (&cell)[3], const int run) {
+        c[0] = cell[0]; c[1] = cell[1]; c[2] = cell[2];
         face = false;
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
@@ -113,77 +113,90 @@ struct TestStage {
         id = reinterpret_cast<int*>(z + SLOTS);
     }
     __device__ __forceinline__ void put(const int slot, const float4& v) const {
-        x[slot] = v.x; y[slot] = v.y; z[slot] = v.z; id[slot] = __float_as_int(v.w);
+        float* s = x + slot;
+        s[0] = v.x; s[SLOTS] = v.y; s[2 * SLOTS] = v.z; s[3 * SLOTS] = v.w;
     }
     __device__ __forceinline__ void seal(const int ns) const {
         for (int k = threadIdx.x & 31; k < TEST_PAD; k += 32) { x[ns + k] = -FAR_AWAY; y[ns + k] = -FAR_AWAY; z[ns + k] = -FAR_AWAY; id[ns + k] = -1; }
     }
 };
 
-// How the lanes of the warp are shared out to a batch of nq queries: lane -> (query q, sub), LPQ lanes per query.
+// How the lanes of the warp are shared out to a batch of nq <= TEST_BATCH queries: lane -> (query q, sub), LPQ lanes per
+// query.
 struct LaneSplit {
     int lpq, q, sub;
+    unsigned inv;                  // ceil(65536 / lpq): x * inv >> 16 is x / lpq for every x that occurs
     bool active;
     __device__ __forceinline__ explicit LaneSplit(const int nq) {
         const int lane = threadIdx.x & 31;
-        lpq = nq <= 4 ? TEST_LPQ : 32 / nq;
-        q = (lane * ((255 + lpq) / lpq)) >> 8;          // lane / lpq, exact for these ranges
+        lpq = nq <= 4 ? 8 : nq == 5 ? 6 : nq == 6 ? 5 : nq <= 8 ? 4 : nq <= 10 ? 3 : 2;      // 32 / nq, at most TEST_LPQ
+        inv = lpq == 8 ? 8192u : lpq == 6 ? 10923u : lpq == 5 ? 13108u : lpq == 4 ? 16384u : lpq == 3 ? 21846u : 32768u;
+        q = (int)(lane * inv >> 16);
         sub = lane - q * lpq;
         active = q < nq;
     }
-    // stage slot of test k of mask word w
-    __device__ __forceinline__ int slot(const int w, const int k) const { return 2 * sub + 32 * w * lpq + lpq * (k & ~1) + (k & 1); }
 };
 
-// Tests query (qx, qy, qz) of every lane against the ns staged candidates: bit 31 - k of mask[w] is set when test k of
-// word w (candidate slot split.slot(w, k)) lies within the cutoff or in the fp32 error band around it.
+// Mask words of a lane: word 2 g + b holds the tests of candidates 2 (sub + lpq (32 g + k)) + b, k = 0..31 from the top bit
+// down, so a set bit is a candidate slot with one multiply-add.  Two groups cover 64 pairs a lane: the whole stage of
+// 256 at two lanes per query.
+constexpr int TEST_GROUP = 32;
+
+// Tests query (qx, qy, qz) of every lane against the ns staged candidates: a bit is set when the candidate lies within
+// the cutoff or in the fp32 error band around it.
 // delta(component, query coordinate, candidate coordinate) is the scalar displacement of the explicit-minimum-image form.
 template <bool MI, int CAP, typename Delta>
 __device__ __forceinline__ void test_candidates(const RadiusParams& p, const TestStage<CAP>& st, const int ns, const LaneSplit& split,
                                                 const float qx, const float qy, const float qz, unsigned (&mask)[4], Delta delta) {
-    const int steps = (((ns + 1) / 2 + split.lpq - 1) / split.lpq + 1) & ~1;      // even
+    static_assert(CAP <= 4 * 2 * TEST_GROUP, "two groups of tests cover the stage");
+    constexpr int NEXT = TestStage<CAP>::SLOTS / 2;                              // next component, in pairs
+    static_assert(TestStage<CAP>::SLOTS % 2 == 0, "pairs");
+    const int steps = ((int)((((ns + 1) >> 1) + split.lpq - 1) * split.inv >> 16) + 1) & ~1;      // even
     const f32x2 qx2 = dup2(qx), qy2 = dup2(qy), qz2 = dup2(qz), neg = dup2(-p.r2_hi);
-    const f32x2* px = reinterpret_cast<const f32x2*>(st.x) + split.sub;
-    const f32x2* py = reinterpret_cast<const f32x2*>(st.y) + split.sub;
-    const f32x2* pz = reinterpret_cast<const f32x2*>(st.z) + split.sub;
+    const f32x2* pc = reinterpret_cast<const f32x2*>(st.x) + split.sub;
 #pragma unroll
-    for (int w = 0; w < 4; ++w) {
-        mask[w] = 0u;
-        const int here = steps - 16 * w < 16 ? steps - 16 * w : 16;
-        if (here <= 0) continue;
-        unsigned m = 0u;
-#pragma unroll 2
-        for (int s = 0; s < here; ++s) {
-            float t0, t1;
-            const f32x2 cx = *px, cy = *py, cz = *pz;
-            px += split.lpq; py += split.lpq; pz += split.lpq;
-            if constexpr (!MI) {
-                const f32x2 dx = sub2(qx2, cx), dy = sub2(qy2, cy), dz = sub2(qz2, cz);
-                unpack2(fma2(dz, dz, fma2(dy, dy, fma2(dx, dx, neg))), t0, t1);
-            } else {
-                float x0, x1, y0, y1, z0, z1;
-                unpack2(cx, x0, x1); unpack2(cy, y0, y1); unpack2(cz, z0, z1);
-                const float ax = delta(0, qx, x0), ay = delta(1, qy, y0), az = delta(2, qz, z0);
-                const float bx = delta(0, qx, x1), by = delta(1, qy, y1), bz = delta(2, qz, z1);
-                t0 = fmaf(az, az, fmaf(ay, ay, fmaf(ax, ax, -p.r2_hi)));
-                t1 = fmaf(bz, bz, fmaf(by, by, fmaf(bx, bx, -p.r2_hi)));
+    for (int g = 0; g < 2; ++g) {
+        const int here = steps - TEST_GROUP * g < TEST_GROUP ? steps - TEST_GROUP * g : TEST_GROUP;
+        unsigned m0 = 0u, m1 = 0u;
+        if (here > 0) {
+            for (int s = 0; s < here; s += 2) {
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    float t0, t1;
+                    const f32x2 cx = pc[0], cy = pc[NEXT], cz = pc[2 * NEXT];
+                    pc += split.lpq;
+                    if constexpr (!MI) {
+                        const f32x2 dx = sub2(qx2, cx), dy = sub2(qy2, cy), dz = sub2(qz2, cz);
+                        unpack2(fma2(dz, dz, fma2(dy, dy, fma2(dx, dx, neg))), t0, t1);
+                    } else {
+                        float x0, x1, y0, y1, z0, z1;
+                        unpack2(cx, x0, x1); unpack2(cy, y0, y1); unpack2(cz, z0, z1);
+                        const float ax = delta(0, qx, x0), ay = delta(1, qy, y0), az = delta(2, qz, z0);
+                        const float bx = delta(0, qx, x1), by = delta(1, qy, y1), bz = delta(2, qz, z1);
+                        t0 = fmaf(az, az, fmaf(ay, ay, fmaf(ax, ax, -p.r2_hi)));
+                        t1 = fmaf(bz, bz, fmaf(by, by, fmaf(bx, bx, -p.r2_hi)));
+                    }
+                    m0 = __funnelshift_l(__float_as_uint(t0), m0, 1);
+                    m1 = __funnelshift_l(__float_as_uint(t1), m1, 1);
+                }
             }
-            m = __funnelshift_l(__float_as_uint(t0), m, 1);
-            m = __funnelshift_l(__float_as_uint(t1), m, 1);
+            m0 = split.active ? m0 << (TEST_GROUP - here) : 0u;
+            m1 = split.active ? m1 << (TEST_GROUP - here) : 0u;
         }
-        mask[w] = split.active ? m << (32 - 2 * here) : 0u;
+        mask[2 * g] = m0;
+        mask[2 * g + 1] = m1;
     }
 }
 
 // clears the bit of staged slot `slot` (the query itself) where this lane tested it
 static __device__ __forceinline__ void drop_candidate(unsigned (&mask)[4], const LaneSplit& split, const int slot) {
-    if (slot < 0) return;
     const int pair = slot >> 1;
-    const int step = (pair * ((65535 + split.lpq) / split.lpq)) >> 16;      // pair / lpq
-    if (pair - step * split.lpq != split.sub) return;
-    const unsigned bit = 0x80000000u >> ((2 * step + (slot & 1)) & 31);
+    const int step = (int)((unsigned)pair * split.inv >> 16);               // pair / lpq
+    if (slot < 0 || pair - step * split.lpq != split.sub) return;
+    const unsigned bit = 0x80000000u >> (step & 31);
+    const int w = (step >> 5) * 2 + (slot & 1);
 #pragma unroll
-    for (int w = 0; w < 4; ++w) if ((step >> 4) == w) mask[w] &= ~bit;
+    for (int k = 0; k < 4; ++k) if (k == w) mask[k] &= ~bit;
 }
 
 }  // namespace tiga
