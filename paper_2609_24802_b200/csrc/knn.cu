@@ -40,6 +40,7 @@ constexpr int KNN_LIST_BYTES = (KQB * KNN_QSTRIDE * 8 + 15) / 16 * 16;
 constexpr int KNN_MISC_BYTES = KQB * 16 + KQB * 4 * 2;
 constexpr int KNN_PER_WARP = KNN_STAGE_BYTES + KNN_LIST_BYTES + KNN_MISC_BYTES;
 static_assert(KNN_PER_WARP % 16 == 0 && KNN_LIST_BYTES % 16 == 0, "the stage and the queries are accessed as 16-byte vectors");
+constexpr int RING_WARPS = 4, RING_THREADS = 32 * RING_WARPS;
 constexpr int KNN_RING_BLOCKS = 148 * 4;
 constexpr double KNN_BALL_FACTOR = 2.0;            // expected points within the search radius, in units of k
 
@@ -160,7 +161,7 @@ static __device__ __forceinline__ void emit_row(const KnnParams& P, const int i,
 
 // ------------------------------------------------------------------------------ cells kernel
 // queries [qs0, qe0) of one cell (the whole cell, or a slice of a dense one)
-__device__ __forceinline__ void knn_cell_slice(const KnnParams& P, const int cellid, const int qs0, const int qe0, unsigned char* s_raw) {
+__device__ __forceinline__ void knn_cell_slice(const KnnParams& P, const int (&c)[3], const int qs0, const int qe0, unsigned char* s_raw) {
     const RadiusParams& p = P.rp;
     constexpr unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
@@ -178,10 +179,9 @@ __device__ __forceinline__ void knn_cell_slice(const KnnParams& P, const int cel
     // ---- the stencil as nine runs of the cell-ordered points: the x neighbours are contiguous
     int r_cs = 0, r_len = 0;
     {
-        const int c0 = cellid % p.nc[0], c1 = (cellid / p.nc[0]) % p.nc[1], c2 = cellid / (p.nc[0] * p.nc[1]);
-        const int y = c1 + lane % 3 - 1, z = c2 + lane / 3 - 1;
+        const int y = c[1] + lane % 3 - 1, z = c[2] + lane / 3 - 1;
         if (lane < 9 && y >= 0 && y < p.nc[1] && z >= 0 && z < p.nc[2]) {
-            const int x0 = c0 > 0 ? c0 - 1 : 0, x1 = c0 + 1 < p.nc[0] ? c0 + 1 : p.nc[0] - 1;
+            const int x0 = c[0] > 0 ? c[0] - 1 : 0, x1 = c[0] + 1 < p.nc[0] ? c[0] + 1 : p.nc[0] - 1;
             const int id0 = (z * p.nc[1] + y) * p.nc[0] + x0;
             r_cs = p.cell_start[id0];
             r_len = p.cell_start[id0 + (x1 - x0 + 1)] - r_cs;
@@ -342,34 +342,18 @@ __device__ __forceinline__ void knn_cell_slice(const KnnParams& P, const int cel
     }
 }
 
-// CTAs [0, cell_blocks): one warp per cell; of a cell with more than QDENSE points it takes the first
-// QSLICE queries.  The CTAs behind them walk the queue of the remaining slices.
-__global__ void __launch_bounds__(TRAV_THREADS) knn_cells_kernel(const __grid_constant__ KnnParams P) {
-    const RadiusParams& p = P.rp;
+// one warp per unit of points; cells are not joined (the search radius already gives a cell about k / 2 points)
+__global__ void __launch_bounds__(TRAV_THREADS, 32 / TRAV_WARPS) knn_cells_kernel(const __grid_constant__ KnnParams P) {
     extern __shared__ __align__(16) unsigned char s_raw[];
-    if ((int)blockIdx.x < p.cell_blocks) {
-        const int w = blockIdx.x * TRAV_WARPS + (threadIdx.x >> 5);
-        if (w >= p.ncells) return;
-        const int qs0 = p.cell_start[w], qe0 = p.cell_start[w + 1];
-        if (qs0 == qe0) return;
-        knn_cell_slice(P, w, qs0, qe0 - qs0 > QDENSE ? qs0 + QSLICE : qe0, s_raw);
-    } else {
-        const int n = *p.q_count;
-        const int w = (blockIdx.x - p.cell_blocks) * TRAV_WARPS + (threadIdx.x >> 5);
-        for (int it = w; it < n; it += (gridDim.x - p.cell_blocks) * TRAV_WARPS) {
-            const int2 item = p.q_items[it];
-            const int qs0 = p.cell_start[item.x] + item.y, end = p.cell_start[item.x + 1];
-            knn_cell_slice(P, item.x, qs0, slice_end(qs0, end), s_raw);
-            __syncwarp();
-        }
-    }
+    auto work = [&](const int (&cell)[3], int, const int qs, const int qe) { knn_cell_slice(P, cell, qs, qe, s_raw); };
+    walk_unit(P.rp, blockIdx.x * TRAV_WARPS + (threadIdx.x >> 5), 1, work);
 }
 
 // ------------------------------------------------------------------------------ rings kernel
-__global__ void __launch_bounds__(TRAV_THREADS) knn_rings_kernel(const __grid_constant__ KnnParams P) {
+__global__ void __launch_bounds__(RING_THREADS) knn_rings_kernel(const __grid_constant__ KnnParams P) {
     const RadiusParams& p = P.rp;
     constexpr unsigned FULL = 0xffffffffu;
-    __shared__ float2 s_list[TRAV_WARPS][KNN_RING_CAP + 32];
+    __shared__ float2 s_list[RING_WARPS][KNN_RING_CAP + 32];
 
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
@@ -377,11 +361,11 @@ __global__ void __launch_bounds__(TRAV_THREADS) knn_rings_kernel(const __grid_co
     const unsigned lt_mask = (1u << lane) - 1u;
     const int k = P.k;
     const int nqueue = *P.queue_n;
-    const int nwarps = gridDim.x * TRAV_WARPS;
+    const int nwarps = gridDim.x * RING_WARPS;
     const int nx = p.nc[0], ny = p.nc[1], nz = p.nc[2];
     const int smax = max(nx, max(ny, nz));
 
-    for (int t = blockIdx.x * TRAV_WARPS + wib; t < nqueue; t += nwarps) {
+    for (int t = blockIdx.x * RING_WARPS + wib; t < nqueue; t += nwarps) {
         const int i = P.queue[t];
         const float qx = p.pos[3 * (size_t)i], qy = p.pos[3 * (size_t)i + 1], qz = p.pos[3 * (size_t)i + 2];
         const int cid = p.cell[i];
@@ -547,12 +531,10 @@ extern "C" tiga_status tiga_apply_knn(const float* pos, const float* feat, int64
     TIGA_CUDA_TRY(cudaMemsetAsync(P.queue_n, 0, sizeof(int32_t), s));
     st = run_binning(P.rp, fill, lay.nblocks, s);
     if (st != TIGA_OK) return st;
-    const unsigned blocks = (unsigned)((P.rp.ncells + TRAV_WARPS - 1) / TRAV_WARPS);
     constexpr int smem = KNN_PER_WARP * TRAV_WARPS;
     TIGA_CUDA_TRY(cudaFuncSetAttribute(knn_cells_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    P.rp.cell_blocks = (int)blocks;
-    knn_cells_kernel<<<counted(blocks + queue_blocks(P.rp.n)), TRAV_THREADS, smem, s>>>(P);
-    knn_rings_kernel<<<counted(KNN_RING_BLOCKS), TRAV_THREADS, 0, s>>>(P);
+    knn_cells_kernel<<<counted(unit_blocks(P.rp)), TRAV_THREADS, smem, s>>>(P);
+    knn_rings_kernel<<<counted(KNN_RING_BLOCKS), RING_THREADS, 0, s>>>(P);
     return launch_status();
 }
 

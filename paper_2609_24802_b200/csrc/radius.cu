@@ -37,13 +37,7 @@ __global__ void bin_count_kernel(const RadiusParams p) {
     if (i >= p.n) return;
     int c[3];
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        const float t = __fmul_rn(p.pos[3 * (size_t)i + d], p.invh[d]);   // one rounded product
-        int k = (int)floorf(t);
-        k = k > p.nc[d] - 1 ? p.nc[d] - 1 : k;
-        k = k < 0 ? 0 : k;
-        c[d] = k;
-    }
+    for (int d = 0; d < 3; ++d) c[d] = cell_coordinate(p, p.pos[3 * (size_t)i + d], d);
     const int id = (c[2] * p.nc[1] + c[1]) * p.nc[0] + c[0];
     p.cell[i] = id;
     if (p.u_cell) p.u_cell[i] = id;
@@ -127,7 +121,7 @@ static __device__ int scan_chunk(const RadiusParams& p, const int chunk, const i
         if (base + k < p.ncells) {
             p.cell_start[base + k] = ex;
             if (p.u_cell_start) p.u_cell_start[base + k] = ex;
-            queue_extra_slices(p, base + k, v[k]);          // a dense cell is cut into slices for the traversals
+            if (v[k] > SORT_DENSE) p.b_items[atomicAdd(p.b_count, 1)] = base + k;
         }
         ex += v[k];
     }
@@ -266,9 +260,7 @@ __global__ void validate_points_kernel(const float* __restrict__ pos, long long 
 //             four gathered rows in flight per lane.  (Lennard-Jones and rows of at most four
 //             features: radius_direct.cuh.)
 // Lists hold QCAP entries per query and the stage STAGE_CAP candidates; when either fills up
-// the warp drains / processes and goes on, so any density works.  A cell with more than QDENSE
-// points is cut into slices of QSLICE queries: its warp takes the first, the others wait in a queue (filled
-// by the binning) that the CTAs appended behind the cells' CTAs walk, so a dense cell spreads over many warps.
+// the warp drains / processes and goes on, so any density works.
 
 template <int MODE> struct TravSmem {
     // queries per batch: the forward runs fastest with short batches and seven CTAs per SM, the
@@ -638,9 +630,10 @@ __device__ __forceinline__ void traverse_slice(const RadiusParams& p, const int 
 }
 
 template <int MODE, int LF, bool DIST, bool MI, int VEC = 1>
-__global__ void __launch_bounds__(TRAV_THREADS, (MODE == 0 ? 7 : 0)) radius_traverse_kernel(const __grid_constant__ RadiusParams p) {
+__global__ void __launch_bounds__(TRAV_THREADS, (MODE == 0 ? 28 : 16) / TRAV_WARPS) radius_traverse_kernel(const __grid_constant__ RadiusParams p) {
     extern __shared__ __align__(16) unsigned char s_raw[];
-    walk_slices(p, [&](const int (&cell)[3], const int run, const int qs, const int qe) { traverse_slice<MODE, LF, DIST, MI, VEC>(p, cell, run, qs, qe, s_raw); });
+    auto work = [&](const int (&cell)[3], const int run, const int qs, const int qe) { traverse_slice<MODE, LF, DIST, MI, VEC>(p, cell, run, qs, qe, s_raw); };
+    walk_unit(p, blockIdx.x * TRAV_WARPS + (threadIdx.x >> 5), p.run, work);
 }
 
 // ------------------------------------------------------------------------------ at most four features
@@ -652,7 +645,7 @@ __global__ void __launch_bounds__(TRAV_THREADS, (MODE == 0 ? 7 : 0)) radius_trav
 // 4 neighbours (sparse cells, runs of eight) 518 -> 126 us.
 template <int NF, bool DIST>
 struct SumMsg {
-    static constexpr int CAP = 256, STAGED = NF, OUT = NF, CTAS = 6;
+    static constexpr int CAP = 256, STAGED = NF, OUT = NF, WARPS = 24;
     static constexpr float OUTSIDE = DIST ? 0.f : 1.0e30f;
     float neg_c2;
     // exp(-d2/(2 s^2)) = 2^(d2 * neg_c2)
@@ -690,16 +683,12 @@ static tiga_status make_grid(long long n, float r, const tiga_box* box, int nc[3
     return TIGA_OK;
 }
 
-// bytes of the queue of extra slices: at most n / QSLICE of them exist
-static size_t queue_items(size_t n) { return n / QSLICE + 2; }
-
 RadiusLayout carve_radius(RadiusParams* p, void* ws, int32_t** fill) {
     Carver cv(ws);
     const size_t n = (size_t)p->n, nc = (size_t)p->ncells;
     const int nblocks = (int)((nc + SCAN_BLOCK - 1) / SCAN_BLOCK);
-    p->cnt = cv.take<int32_t>(2 * nc + 2 + 16);     // counts, then the scatter cursors, then the length of the slice queue
-    p->q_count = p->cnt + 2 * nc + 2;
-    p->b_count = p->q_count + 1;
+    p->cnt = cv.take<int32_t>(2 * nc + 2 + 16);     // counts, then the scatter cursors, then the length of the dense-cell queue
+    p->b_count = p->cnt + 2 * nc + 2;
     *fill = p->cnt + nc;
     p->cell = cv.take<int32_t>(n);
     p->cell_start = cv.take<int32_t>(nc + 1);
@@ -707,7 +696,6 @@ RadiusLayout carve_radius(RadiusParams* p, void* ws, int32_t** fill) {
     p->order = cv.take<int32_t>(n);
     p->spos = cv.take<float4>(n);
     p->blocksum = cv.take<int32_t>((size_t)nblocks + 1);
-    p->q_items = cv.take<int2>(queue_items(n));
     p->b_items = cv.take<int32_t>(n / SORT_DENSE + 2);
     return RadiusLayout{cv.off, nblocks};
 }
@@ -715,15 +703,24 @@ RadiusLayout carve_radius(RadiusParams* p, void* ws, int32_t** fill) {
 // A cell of a sparse input holds a point or two, and its stencil costs as much as a full one: joining cells along x
 // shares it (F = 16, n = 300k, 8 neighbours: forward 218 -> 135, backward 341 -> 175 us; F = 64, n = 100k, 4
 // neighbours: 139 -> 48 and 209 -> 78 us; nothing is joined at 32 neighbours).
-// Cells along x per warp: enough for about RUN_QUERIES / 2 points at the mean density, as long as a dozen warps per SM
-// remain; a run's stencil must not meet itself around a periodic face (the frame shift needs two cells between).
+// Cells along x that are joined at most: enough for about RUN_QUERIES / 2 points at the mean density; a run's stencil must
+// not meet itself around a periodic face (the frame shift needs two cells between).
 static int run_length(const RadiusParams& p) {
     long long r = p.n > 0 ? (long long)p.ncells * (RUN_QUERIES / 2) / p.n : 1;
-    const long long warps = p.ncells / (148 * 12), room = !p.periodic[0] ? RUN_CELLS : p.nc[0] < 4 ? 1 : p.nc[0] - 3;
-    r = r > warps ? warps : r;
+    const long long room = !p.periodic[0] ? RUN_CELLS : p.nc[0] < 4 ? 1 : p.nc[0] - 3;
     r = r > room ? room : r;
     r = r > RUN_CELLS ? RUN_CELLS : r;
     return r < 1 ? 1 : (int)r;
+}
+
+// Points per warp: up to eight while that leaves a warp for each of 4736 slots (eight per scheduler), more once there are
+// four such rounds.  Measured with 4 / 8 / 16 / 32 points: 36 k surface points backward 32 / 28 / 28 / 28 us; 131 k points,
+// scalar sum 67 / 61 / 61 / 70 us; 300 k points, F = 16, forward 134 / 117 / 113 / 120 us; 1 M points, F = 32, backward
+// 1386 / 1168 / 1069 / 1028 us.
+static int unit_length(const RadiusParams& p) {
+    const int slots = 148 * 4 * 8, few = p.n / slots < 8 ? p.n / slots : 8, many = p.n / (4 * slots);
+    const int per = few > many ? few : many;
+    return per > UNIT_MAX ? UNIT_MAX : per < 2 ? 2 : per;
 }
 
 tiga_status fill_params(RadiusParams* p, long long n, float r, const tiga_box* box) {
@@ -744,6 +741,7 @@ tiga_status fill_params(RadiusParams* p, long long n, float r, const tiga_box* b
     }
     p->ncells = nc[0] * nc[1] * nc[2];
     p->run = run_length(*p);
+    p->unit = unit_length(*p);
     const float r2 = r * r;
     const float beta = (single_periodic ? 96.f : 32.f) * 5.9604645e-8f;
     p->r2_lo = r2 * (1.f - beta);
@@ -781,15 +779,12 @@ static int feature_lanes(int F) {
 template <int MODE, int LF, bool DIST, bool MI>
 static tiga_status launch_traverse_t(const RadiusParams& p, cudaStream_t s) {
     constexpr int smem = TravSmem<MODE>::PER_WARP * TRAV_WARPS;
-    if (MODE == 0 && (p.F & 3)) {
-        // scalar feature accesses (only the forward supports widths that are not multiples of 4)
-        auto sk = radius_traverse_kernel<MODE == 0 ? 0 : MODE, LF, DIST, MI, MODE != 0 ? 1 : 0>;
-        if (smem > 48 * 1024) TIGA_CUDA_TRY(cudaFuncSetAttribute(sk, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        return runs_then_queue(p, s, [&](const RadiusParams& q, unsigned grid) { sk<<<counted(grid), TRAV_THREADS, smem, s>>>(q); });
-    }
-    auto kern = p.F == 4 * LF ? radius_traverse_kernel<MODE, LF, DIST, MI, 2> : radius_traverse_kernel<MODE, LF, DIST, MI, 1>;
+    // scalar feature accesses only where the forward has to (F % 4 != 0)
+    auto kern = MODE == 0 && (p.F & 3) ? radius_traverse_kernel<MODE, LF, DIST, MI, MODE != 0 ? 1 : 0>
+              : p.F == 4 * LF ? radius_traverse_kernel<MODE, LF, DIST, MI, 2> : radius_traverse_kernel<MODE, LF, DIST, MI, 1>;
     if (smem > 48 * 1024) TIGA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    return runs_then_queue(p, s, [&](const RadiusParams& q, unsigned grid) { kern<<<counted(grid), TRAV_THREADS, smem, s>>>(q); });
+    kern<<<counted(unit_blocks(p)), TRAV_THREADS, smem, s>>>(p);
+    return launch_status();
 }
 
 template <int MODE, bool DIST, bool MI>

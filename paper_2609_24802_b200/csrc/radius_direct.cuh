@@ -1,6 +1,5 @@
 // Traversal that consumes a pair where it is accepted (test: radius_test.cuh): every query has its own lanes, and a
-// lane adds the messages of its accepted candidates in registers.  No lists, no gathers, no atomics.  One warp per run
-// of cells, slices of dense cells from the queue.
+// lane adds the messages of its accepted candidates in registers.  No lists, no gathers, no atomics.
 //
 // Msg supplies the message:
 //   CAP             candidates the stage holds
@@ -14,49 +13,6 @@
 #include "radius_test.cuh"
 
 namespace tiga {
-
-// CTAs [0, cell_blocks): warp w takes the w-th run of p.run cells along x; the cells are joined as long as they hold at
-// most RUN_QUERIES points together (of a cell with more than QDENSE points the first QSLICE queries).  The CTAs behind
-// them walk the queue of the remaining slices.
-template <typename Work>
-__device__ __forceinline__ void walk_slices(const RadiusParams& p, Work work) {
-    if ((int)blockIdx.x < p.cell_blocks) {
-        const int w = blockIdx.x * TRAV_WARPS + (threadIdx.x >> 5);
-        const int lane = threadIdx.x & 31;
-        const int row = w / p.row_runs, x0 = (w - row * p.row_runs) * p.run;
-        const int cz = row / p.nc[1], cy = row - cz * p.nc[1];
-        if (cz >= p.nc[2]) return;
-        const int cells = p.nc[0] - x0 < p.run ? p.nc[0] - x0 : p.run, cell0 = row * p.nc[0] + x0;
-        const int start = p.cell_start[cell0 + (lane < cells ? lane : cells)];          // lane k: first point of cell k of the run
-        const int len = __shfl_down_sync(0xffffffffu, start, 1) - start;
-        unsigned left = __ballot_sync(0xffffffffu, lane < cells && len > 0);            // occupied cells not done yet
-        while (left) {
-            const int a = __ffs(left) - 1, qs = __shfl_sync(0xffffffffu, start, a), first = __shfl_sync(0xffffffffu, len, a);
-            int qe = qs + (first > QDENSE ? QSLICE : first), last = a;
-            left &= left - 1u;
-            while (left) {
-                const int b = __ffs(left) - 1, more = __shfl_sync(0xffffffffu, start + len, b);
-                if (first > QDENSE || more - qs > RUN_QUERIES) break;
-                qe = more; last = b;
-                left &= left - 1u;
-            }
-            const int cell[3] = {x0 + a, cy, cz};
-            work(cell, last - a + 1, qs, qe);
-            __syncwarp();
-        }
-    } else {
-        const int n = *p.q_count;
-        const int w = (blockIdx.x - p.cell_blocks) * TRAV_WARPS + (threadIdx.x >> 5);
-        for (int it = w; it < n; it += (gridDim.x - p.cell_blocks) * TRAV_WARPS) {
-            const int2 item = p.q_items[it];
-            const int qs0 = p.cell_start[item.x] + item.y, end = p.cell_start[item.x + 1];
-            const int row = item.x / p.nc[0], cz = row / p.nc[1];
-            const int cell[3] = {item.x - row * p.nc[0], row - cz * p.nc[1], cz};
-            work(cell, 1, qs0, slice_end(qs0, end));
-            __syncwarp();
-        }
-    }
-}
 
 template <typename Msg> struct DirectSmem {
     static constexpr int STAGE_CAP = Msg::CAP, STAGED = Msg::STAGED;
@@ -266,9 +222,10 @@ __device__ __forceinline__ void direct_slice(const RadiusParams& p, const int (&
 }
 
 template <typename Msg, bool MI>
-__global__ void __launch_bounds__(TRAV_THREADS, Msg::CTAS) radius_direct_kernel(const __grid_constant__ RadiusParams p) {
+__global__ void __launch_bounds__(TRAV_THREADS, Msg::WARPS / TRAV_WARPS) radius_direct_kernel(const __grid_constant__ RadiusParams p) {
     extern __shared__ __align__(16) unsigned char s_raw[];
-    walk_slices(p, [&](const int (&cell)[3], const int run, const int qs, const int qe) { direct_slice<Msg, MI>(p, cell, run, qs, qe, s_raw); });
+    auto work = [&](const int (&cell)[3], const int run, const int qs, const int qe) { direct_slice<Msg, MI>(p, cell, run, qs, qe, s_raw); };
+    walk_unit(p, blockIdx.x * TRAV_WARPS + (threadIdx.x >> 5), p.run, work);
 }
 
 template <typename Msg, bool MI>
@@ -276,7 +233,8 @@ static tiga_status launch_direct_t(const RadiusParams& p, cudaStream_t s) {
     constexpr int smem = DirectSmem<Msg>::PER_WARP * TRAV_WARPS;
     auto kern = radius_direct_kernel<Msg, MI>;
     if (smem > 48 * 1024) TIGA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    return runs_then_queue(p, s, [&](const RadiusParams& q, unsigned grid) { kern<<<counted(grid), TRAV_THREADS, smem, s>>>(q); });
+    kern<<<counted(unit_blocks(p)), TRAV_THREADS, smem, s>>>(p);
+    return launch_status();
 }
 
 }  // namespace tiga

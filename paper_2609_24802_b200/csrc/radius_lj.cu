@@ -11,7 +11,7 @@
 namespace tiga {
 
 struct LjMsg {
-    static constexpr int CAP = 256, STAGED = 0, OUT = 4, CTAS = 8;
+    static constexpr int CAP = 256, STAGED = 0, OUT = 4, WARPS = 32;
     static constexpr float OUTSIDE = 1.0e30f;
     float s2, force, energy;
     __device__ __forceinline__ explicit LjMsg(const RadiusParams& p) : s2(p.p1 * p.p1), force(24.f * p.p0), energy(2.f * p.p0) {}

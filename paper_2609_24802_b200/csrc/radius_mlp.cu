@@ -1,531 +1,412 @@
 // Edge neural network over the generated radius relation (paper Appendix A):
 //     y_i = sum over j in N(i) of [ W2 ReLU( W1 [p_j - p_i ; x_j] + b1 ) + b2 ]
 // fused with the cell-directory traversal, and its reverse mode with the membership frozen
-// (Section 5), which recomputes the activations per pair instead of storing them and gives
+// (Section 5), which recomputes the pre-activations per pair instead of storing them and gives
 // gradients with respect to node features, positions and the four parameter arrays.
 //
-// Same skeleton as the other radius traversals: one warp per query cell (here in a persistent
-// loop over cells), the 27-cell stencil staged in shared memory in cell-local coordinates,
-// one staged candidate per lane tested against eight queries, ballot compaction into one list
-// per query.  What differs is phase B: every lane takes one accepted pair and evaluates the
-// whole network for it with the weights broadcast from shared memory (input padded to 4 KQ,
-// hidden width HID in registers).  The pairs of all queries of a batch form one flat sequence,
-// 32 per step, so short neighbour lists do not leave lanes idle; per-query sums are segmented
-// shuffle reductions (fixed order: reproducible).
+// Staging and candidate test are those of radius_test.cuh (a run of cells per warp, persistent grid); accepted pairs
+// are compacted into one list of (displacement, staged slot) per query.  A pair is then evaluated by HID lanes, one
+// hidden unit each, with the lane's row of W1 in registers and the pair's inputs broadcast from shared memory, so 32 / HID
+// pairs advance together.  Everything behind the ReLU is linear, so it is applied once per query to sums over the pairs:
+//     S[a] = sum relu(h_a)      c[a] = #(h_a > 0)      D[a] = sum (p_j - p_i) [h_a > 0]
+//     out_i = W2 S + |N(i)| b2
+// Backward, owner computes: with v = W2^T ybar, query k and its neighbours m,
+//     G[a] = sum over m of v_m[a] [h_a of the pair (m <- k) > 0]
+//     xbar_k = W1x^T G,   pbar_k = W1p^T (G - v_k c)          (no atomics, reproducible)
+//     W1bar += [ v_k D ; G x_k ],   b1bar += v_k c,   W2bar += ybar_k S,   b2bar += |N(k)| ybar_k
+// where every lane accumulates the parameter gradients of its hidden unit in registers over all its queries; at the end
+// warps fold into the CTA's shared copy and the CTA adds that to global memory with one atomic per entry.
 //
-// Backward, owner computes: for query k and neighbour m a lane evaluates the pair twice,
-//   (k <- m) gives the parameter gradients and -ubar[0:3] for pbar_k,
-//   (m <- k) gives xbar_k and +ubar[0:3] for pbar_k,
-// so feature and position gradients need no atomics.  Parameter gradients: the 32 pairs of a
-// step park (hbar, u, a, ybar) in shared memory, then every lane accumulates "its" parameter
-// entries over those pairs in registers; at the end warps fold into the CTA's shared copy and
-// the CTA adds that to global memory with one atomic per entry.
-#include "radius_shared.cuh"
-#include <type_traits>
+// Bound by latency and the tail of the work units (36 to 40 % of the issue slots).  35,947 surface points, 15.6 neighbours,
+// 8 features, HID = 32: forward 121 -> 103 us, backward 512 -> 138 us against one lane per pair with the weights read from
+// shared memory (the earlier form, some 600 shared-memory reads per 32 pairs).
+//
+// The displacement is formed from coordinates relative to the corner of the query's cell and the pre-activation as one chain
+// of fused multiply-adds (bias, displacement, features): a ReLU switches on the last bit of that sum.
+#include "radius_direct.cuh"
 
 namespace tiga {
 
-constexpr int MLP_STAGE_CAP = 256;
-constexpr int MLP_QCAP = 80;
-constexpr int MLP_QSTRIDE = MLP_QCAP + 1;
-constexpr int MLP_DIN = 16;             // padded input width (3 + f_in <= 16)
+constexpr int MLP_WARPS = 4, MLP_THREADS = 32 * MLP_WARPS;
 
-template <int HID, bool BWD> struct MlpSmem {
-    static constexpr int W_FLOATS = HID * MLP_DIN + HID + 4 * HID + 4;          // W1 (padded), b1, W2 (4 rows), b2
-    static constexpr int CTA_BYTES = (W_FLOATS * (BWD ? 2 : 1) * 4 + 15) / 16 * 16;   // weights (+ gradient accumulators)
-    static constexpr int STAGE_BYTES = (MLP_STAGE_CAP + STAGE_PAD) * 16;
-    static constexpr int LIST_BYTES = (QB * MLP_QSTRIDE * 4 + 15) / 16 * 16;
-    static constexpr int ACC_W = 16;                                             // per-query accumulator: outputs, or pbar (3) + xbar (13)
-    static constexpr int MISC_BYTES = QB * 16 + QB * 4 * 2 + QB * ACC_W * 4;
-    static constexpr int PAIR_STRIDE = 2 * HID + MLP_DIN + 4 + 1;                // hbar, u, a, ybar (+1: odd stride)
-    static constexpr int PAIR_BYTES = BWD ? (32 * PAIR_STRIDE * 4 + 15) / 16 * 16 : 0;
-    static constexpr int PER_WARP = STAGE_BYTES + LIST_BYTES + MISC_BYTES + PAIR_BYTES;
-    static_assert(PER_WARP % 16 == 0, "the stage and the queries are accessed as 16-byte vectors");
-    static constexpr int TOTAL = CTA_BYTES + TRAV_WARPS * PER_WARP;
+template <int HID, int FQ, bool BWD> struct MlpSmem {
+    static constexpr int NX = 4 * FQ;                                            // staged features per candidate (zero padded)
+    static constexpr int STAGE_CAP = 144, LIST_CAP = 176;
+    static_assert(LIST_CAP >= STAGE_CAP, "a query's whole chunk fits the list");
+    static constexpr int STAGE_BYTES = TestStage<STAGE_CAP>::BYTES;
+    static constexpr int X_BYTES = STAGE_CAP * NX * 4, G_BYTES = BWD ? STAGE_CAP * 16 : 0, LIST_BYTES = LIST_CAP * 16;
+    static constexpr int PER_WARP = STAGE_BYTES + X_BYTES + G_BYTES + LIST_BYTES + ((2 * TEST_BATCH + QDENSE + 20) * 4 + 15) / 16 * 16;
+    static constexpr int K_PAD = 3 + NX;
+    static constexpr int GRAD_FLOATS = HID * (K_PAD + 1 + 4) + 4;                // W1, b1, W2, b2 of the CTA's gradient copy
+    static constexpr int CTA_BYTES = BWD ? (GRAD_FLOATS * 4 + 15) / 16 * 16 : 0;
+    static constexpr int TOTAL = CTA_BYTES + MLP_WARPS * PER_WARP;
 };
 
-template <int HID, int KQ>
-__device__ __forceinline__ void mlp_forward(const float* sW1, const float* sb1, const float* sW2, const float* sb2,
-                                            const float (&u)[4 * KQ], float (&h)[HID], float (&m)[4]) {
-#pragma unroll
-    for (int a = 0; a < HID; ++a) {
-        float s = sb1[a];
-        const float4* w = reinterpret_cast<const float4*>(sW1 + a * MLP_DIN);
-#pragma unroll
-        for (int q = 0; q < KQ; ++q) {
-            const float4 w4 = w[q];
-            s = fmaf(w4.x, u[4 * q], s); s = fmaf(w4.y, u[4 * q + 1], s);
-            s = fmaf(w4.z, u[4 * q + 2], s); s = fmaf(w4.w, u[4 * q + 3], s);
-        }
-        h[a] = s;
-    }
-#pragma unroll
-    for (int o = 0; o < 4; ++o) {
-        float s = sb2[o];
-#pragma unroll
-        for (int a = 0; a < HID; ++a) s = fmaf(sW2[o * HID + a], fmaxf(h[a], 0.f), s);
-        m[o] = s;
-    }
-}
-
-// hbar = (W2^T ybar) * [h > 0],  ubar = W1^T hbar.  hbar is consumed entry by entry (and parked in
-// shared memory where the parameter gradients need it), so it never occupies HID registers.
-template <int HID, int KQ, bool STORE>
-__device__ __forceinline__ void mlp_backward(const float* sW1, const float* sW2, const float (&h)[HID], const float (&gy)[4],
-                                             float* hb_out, float (&ub)[4 * KQ]) {
-#pragma unroll
-    for (int c = 0; c < 4 * KQ; ++c) ub[c] = 0.f;
-#pragma unroll
-    for (int a = 0; a < HID; ++a) {
-        float s = sW2[a] * gy[0];
-        s = fmaf(sW2[HID + a], gy[1], s); s = fmaf(sW2[2 * HID + a], gy[2], s); s = fmaf(sW2[3 * HID + a], gy[3], s);
-        const float hb = h[a] > 0.f ? s : 0.f;
-        if (STORE) hb_out[a] = hb;
-        const float4* w = reinterpret_cast<const float4*>(sW1 + a * MLP_DIN);
-#pragma unroll
-        for (int q = 0; q < KQ; ++q) {
-            const float4 w4 = w[q];
-            ub[4 * q] = fmaf(w4.x, hb, ub[4 * q]); ub[4 * q + 1] = fmaf(w4.y, hb, ub[4 * q + 1]);
-            ub[4 * q + 2] = fmaf(w4.z, hb, ub[4 * q + 2]); ub[4 * q + 3] = fmaf(w4.w, hb, ub[4 * q + 3]);
-        }
-    }
-}
-
 // resident CTAs per SM the kernel is compiled for (register budget) and launched with (persistent grid)
-template <int HID, bool BWD> constexpr int mlp_ctas_per_sm() { return BWD ? (HID <= 16 ? 3 : 2) : (HID <= 16 ? 4 : 3); }
+template <int FQ, bool BWD> __host__ __device__ constexpr int mlp_ctas_per_sm() { return BWD ? (FQ <= 2 ? 4 : 3) : (FQ <= 2 ? 5 : 4); }
 
-template <int HID, int KQ, bool BWD, bool MI>
-__global__ void __launch_bounds__(TRAV_THREADS, mlp_ctas_per_sm<HID, BWD>()) radius_mlp_kernel(const __grid_constant__ RadiusParams p) {
-    using SM = MlpSmem<HID, BWD>;
+// Sums v[0..NV) over the L lanes of an aligned group by a halving exchange; afterwards lane l holds, in v[0..NV / min(NV, L)),
+// the totals of the entries from spread_first<NV, L>(l).
+template <int NV, int L>
+static __device__ __forceinline__ void spread_sum(float* v, const int l) {
+#pragma unroll
+    for (int j = 0; (1 << j) < L; ++j) {
+        const int left = NV >> j;
+        if (left > 1) {
+            const bool up = (l >> j) & 1;
+#pragma unroll
+            for (int k = 0; k < left / 2; ++k) {
+                const float send = up ? v[k] : v[k + left / 2], keep = up ? v[k + left / 2] : v[k];
+                v[k] = keep + __shfl_xor_sync(0xffffffffu, send, 1 << j);
+            }
+        } else {
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1 << j);
+        }
+    }
+}
+template <int NV, int L>
+static __device__ __forceinline__ int spread_first(const int l) {
+    int first = 0;
+#pragma unroll
+    for (int j = 0; (1 << j) < L && (NV >> j) > 1; ++j) first += ((l >> j) & 1) * (NV >> (j + 1));
+    return first;
+}
+
+template <int HID, int FQ, bool BWD, bool MI>
+__global__ void __launch_bounds__(MLP_THREADS, (mlp_ctas_per_sm<FQ, BWD>())) radius_mlp_kernel(const __grid_constant__ RadiusParams p) {
+    using SM = MlpSmem<HID, FQ, BWD>;
+    constexpr int STAGE_CAP = SM::STAGE_CAP, LIST_CAP = SM::LIST_CAP, NX = SM::NX, KP = SM::K_PAD;
+    constexpr int PS = 32 / HID;                       // pairs evaluated together
     constexpr unsigned FULL = 0xffffffffu;
-    constexpr int KU = 4 * KQ;
-    constexpr int PS = SM::PAIR_STRIDE;
     extern __shared__ __align__(16) unsigned char s_raw[];
-
-    const int lane = threadIdx.x & 31;
-    const int wib = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const int a = lane % HID, ps = lane / HID;
     const int Fin = p.Fin, Fout = p.Fout, K = 3 + p.Fin;
 
-    // ---- CTA: weights into shared memory (zero padded), gradient accumulators cleared
-    float* sW1 = reinterpret_cast<float*>(s_raw);
-    float* sb1 = sW1 + HID * MLP_DIN;
-    float* sW2 = sb1 + HID;
-    float* sb2 = sW2 + 4 * HID;
-    float* sG = sb2 + 4;                       // BWD: same layout as the weights
-    for (int e = threadIdx.x; e < HID * MLP_DIN; e += TRAV_THREADS) {
-        const int a = e / MLP_DIN, k = e % MLP_DIN;
-        sW1[e] = k < K ? p.W1[a * K + k] : 0.f;
+    float* sG = reinterpret_cast<float*>(s_raw);       // BWD: W1 [HID][KP], b1 [HID], W2 [4][HID], b2 [4]
+    if constexpr (BWD) {
+        for (int e = threadIdx.x; e < SM::GRAD_FLOATS; e += MLP_THREADS) sG[e] = 0.f;
+        __syncthreads();
     }
-    for (int e = threadIdx.x; e < HID; e += TRAV_THREADS) sb1[e] = p.b1[e];
-    for (int e = threadIdx.x; e < 4 * HID; e += TRAV_THREADS) sW2[e] = (e / HID) < Fout ? p.W2[e] : 0.f;
-    if (threadIdx.x < 4) sb2[threadIdx.x] = threadIdx.x < Fout ? p.b2[threadIdx.x] : 0.f;
-    if (BWD) for (int e = threadIdx.x; e < SM::W_FLOATS; e += TRAV_THREADS) sG[e] = 0.f;
-    __syncthreads();
-
     unsigned char* base = s_raw + SM::CTA_BYTES + (size_t)wib * SM::PER_WARP;
-    float4* stage = reinterpret_cast<float4*>(base);
-    int* list = reinterpret_cast<int*>(base + SM::STAGE_BYTES);
-    float4* s_q = reinterpret_cast<float4*>(base + SM::STAGE_BYTES + SM::LIST_BYTES);
-    int* s_n = reinterpret_cast<int*>(s_q + QB);
-    int* s_tot = s_n + QB;
-    float* s_acc = reinterpret_cast<float*>(s_tot + QB);          // [QB][ACC_W] sums of the drain in progress
-    float* pairbuf = reinterpret_cast<float*>(base + SM::STAGE_BYTES + SM::LIST_BYTES + SM::MISC_BYTES);
+    const TestStage<STAGE_CAP> stage(base);
+    float* s_x = reinterpret_cast<float*>(base + SM::STAGE_BYTES);                       // [slot][NX]
+    float4* s_g = reinterpret_cast<float4*>(base + SM::STAGE_BYTES + SM::X_BYTES);       // [slot] cotangents (BWD)
+    float4* list = reinterpret_cast<float4*>(base + SM::STAGE_BYTES + SM::X_BYTES + SM::G_BYTES);
+    int* s_off = reinterpret_cast<int*>(list + LIST_CAP);                                // list of every query of the batch: start,
+    int* s_end = s_off + TEST_BATCH;                                                     // end
+    int* s_self = s_end + TEST_BATCH;                                                    // staged slot of every query, or -1
+    int* s_delta = s_self + QDENSE;
 
-    const bool mi0 = MI && p.periodic[0] && p.nc[0] == 1, mi1 = MI && p.periodic[1] && p.nc[1] == 1, mi2 = MI && p.periodic[2] && p.nc[2] == 1;
-    const unsigned lt_mask = (1u << lane) - 1u;
-    auto fold = [&](float& dx, float& dy, float& dz) {
-        if (MI) {
-            if (mi0) dx -= p.len[0] * rintf(dx * p.inv_len[0]);
-            if (mi1) dy -= p.len[1] * rintf(dy * p.inv_len[1]);
-            if (mi2) dz -= p.len[2] * rintf(dz * p.inv_len[2]);
-        }
-    };
-
-    // parameter-gradient entries owned by this lane (BWD): W1[a0 + 2 i][k1], W2[o][lane], b1[lane], b2[lane]
-    const int k1 = lane & 15, a0 = lane >> 4;
-    float gW1acc[BWD ? HID / 2 : 1], gW2acc[4] = {0.f, 0.f, 0.f, 0.f}, gb1acc = 0.f, gb2acc = 0.f;
+    // this lane's hidden unit
+    float w[KP], w2[4], b1 = p.b1[a], b2 = lane < Fout ? p.b2[lane] : 0.f;
 #pragma unroll
-    for (int i = 0; i < (BWD ? HID / 2 : 1); ++i) gW1acc[i] = 0.f;
+    for (int k = 0; k < KP; ++k) w[k] = k < K ? p.W1[a * K + k] : 0.f;
+#pragma unroll
+    for (int o = 0; o < 4; ++o) w2[o] = o < Fout ? p.W2[o * HID + a] : 0.f;
+    float gW1[BWD ? KP : 1], gW2[4] = {0.f, 0.f, 0.f, 0.f}, gb1 = 0.f, gb2 = 0.f;
+#pragma unroll
+    for (int k = 0; k < (BWD ? KP : 1); ++k) gW1[k] = 0.f;
 
-    // work items: every cell (of a cell with more than QDENSE points only its first QSLICE queries), then
-    // the queued slices of the dense cells, so that a clustered input spreads over all warps
-    const int nitems = p.ncells + *p.q_count;
-    for (int item = blockIdx.x * TRAV_WARPS + wib; item < nitems; item += gridDim.x * TRAV_WARPS) {
-        int cellid, qs0, qe0;
-        if (item < p.ncells) {
-            cellid = item;
-            qs0 = p.cell_start[cellid]; qe0 = p.cell_start[cellid + 1];
-            if (qe0 - qs0 > QDENSE) qe0 = qs0 + QSLICE;
-        } else {
-            const int2 it = p.q_items[item - p.ncells];
-            cellid = it.x;
-            qs0 = p.cell_start[cellid] + it.y;
-            qe0 = slice_end(qs0, p.cell_start[cellid + 1]);
+    const bool mi0 = MI && p.periodic[0] && p.nc[0] <= 3, mi1 = MI && p.periodic[1] && p.nc[1] <= 3, mi2 = MI && p.periodic[2] && p.nc[2] <= 3;
+    auto delta = [&](const int d, const float q, const float c4) -> float {
+        const bool mi = d == 0 ? mi0 : d == 1 ? mi1 : mi2;
+        return (MI && mi) ? mi_delta(q, c4, p.len[d], 0.5f * p.len[d]) : q - c4;
+    };
+    const unsigned lt_mask = (1u << lane) - 1u;
+
+    auto slice = [&](const int (&cell)[3], const int run, const int qs0, const int qe0) {
+        const RunFrame frame(p, cell, run);
+        const RunStencil sten(p, frame.c, run, s_delta);
+        float blo[3] = {FAR_AWAY, FAR_AWAY, FAR_AWAY}, bhi[3] = {-FAR_AWAY, -FAR_AWAY, -FAR_AWAY};
+        for (int q = qs0 + lane; q < qe0; q += 32) {
+            float4 pq = p.spos[q];
+            frame.shift(p, pq);
+            const float l[3] = {pq.x, pq.y, pq.z};
+#pragma unroll
+            for (int d = 0; d < 3; ++d) { blo[d] = fminf(blo[d], l[d]); bhi[d] = fmaxf(bhi[d], l[d]); }
         }
-        if (qs0 == qe0) continue;
-        const int c[3] = {cellid % p.nc[0], (cellid / p.nc[0]) % p.nc[1], cellid / (p.nc[0] * p.nc[1])};
-        const float org[3] = {(float)c[0] * p.hcell[0], (float)c[1] * p.hcell[1], (float)c[2] * p.hcell[2]};
+#pragma unroll
+        for (int d = 0; d < 3; ++d) { blo[d] = warp_min(blo[d]); bhi[d] = warp_max(bhi[d]); }
+        if (mi0) { blo[0] = -FAR_AWAY; bhi[0] = FAR_AWAY; }   // a dimension folded by the explicit minimum image is not pruned
+        if (mi1) { blo[1] = -FAR_AWAY; bhi[1] = FAR_AWAY; }
+        if (mi2) { blo[2] = -FAR_AWAY; bhi[2] = FAR_AWAY; }
+        for (int k = lane; k < qe0 - qs0; k += 32) s_self[k] = -1;
 
         auto process_chunk = [&](const int ns, const bool first_chunk) {
-            if (lane < STAGE_PAD) stage[ns + lane] = make_float4(FAR_AWAY, FAR_AWAY, FAR_AWAY, __int_as_float(-1));
-            for (int qb0 = qs0; qb0 < qe0; qb0 += QB) {
-                const int nq = (qe0 - qb0 < QB) ? qe0 - qb0 : QB;
-                __syncwarp();
-                if (lane < nq) {
-                    const float4 pq = p.spos[qb0 + lane];
-                    s_q[lane] = make_float4(pq.x - org[0], pq.y - org[1], pq.z - org[2], pq.w);
-                    s_tot[lane] = 0;
+            stage.seal(ns);
+            __syncwarp();
+            const int all = qe0 - qs0;
+            const int per = all <= TEST_BATCH ? all : all <= 2 * TEST_BATCH ? (all + 1) >> 1 : TEST_BATCH;
+            for (int qb0 = qs0; qb0 < qe0; qb0 += per) {
+                const int nq = (qe0 - qb0 < per) ? qe0 - qb0 : per;
+                const LaneSplit split(nq);
+                float4 qv = p.spos[qb0 + (split.active ? split.q : 0)];
+                const int qid = checked(__float_as_int(qv.w), p.n, CHECK_POINT);
+                // corner of the query's cell, in the frame (moved down with its points where a run touches an upper face)
+                float ox = (float)(p.cell[qid] - (cell[2] * p.nc[1] + cell[1]) * p.nc[0]) * p.hcell[0];
+                float oy = (float)cell[1] * p.hcell[1], oz = (float)cell[2] * p.hcell[2];
+                if (frame.face) {
+                    if (ox + 0.5f * p.hcell[0] > frame.thr[0]) ox -= p.len[0];
+                    if (oy + 0.5f * p.hcell[1] > frame.thr[1]) oy -= p.len[1];
+                    if (oz + 0.5f * p.hcell[2] > frame.thr[2]) oz -= p.len[2];
                 }
-                __syncwarp();
-                int qcnt[QB];
-#pragma unroll
-                for (int q = 0; q < QB; ++q) qcnt[q] = 0;
-                bool first = first_chunk;
+                frame.shift(p, qv);
+                unsigned mask[4];
+                test_candidates<MI, STAGE_CAP>(p, stage, ns, split, qv.x, qv.y, qv.z, mask, delta);
+                drop_candidate(mask, split, split.active ? s_self[qb0 - qs0 + split.q] : -1);
 
-                auto drain = [&]() {
-                    constexpr int ACC_W = SM::ACC_W;
-                    __syncwarp();
-                    if (lane == 0) {
+                const int mine = __popc(mask[0]) + __popc(mask[1]) + __popc(mask[2]) + __popc(mask[3]);
+                int cnt = mine;                                    // exact decisions below may take some back
+                int incl = mine;
 #pragma unroll
-                        for (int q = 0; q < QB; ++q) { s_n[q] = qcnt[q]; s_tot[q] += qcnt[q]; }
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int t = __shfl_up_sync(FULL, incl, o);
+                    if (lane >= o) incl += t;
+                }
+                for (int qa = 0; qa < nq;) {
+                    // queries [qa, qb): as many as the list holds
+                    const int e0 = __shfl_sync(FULL, incl - mine, qa * split.lpq);
+                    const int qb = qa + __popc(__ballot_sync(FULL, split.active && split.q >= qa && split.sub == split.lpq - 1 && incl - e0 <= LIST_CAP));
+                    const bool part = split.active && split.q >= qa && split.q < qb;
+                    int at = incl - mine - e0;
+                    if (part && split.sub == 0) s_off[split.q] = at;
+                    if (part && split.sub == split.lpq - 1) s_end[split.q] = at + mine;
+                    if (part) {
+#pragma unroll
+                        for (int wd = 0; wd < 4; ++wd) {
+                            unsigned m = mask[wd];
+                            while (m) {
+                                const int k = __clz(m);
+                                m ^= 0x80000000u >> k;
+                                int slot = 2 * (split.sub + split.lpq * (TEST_GROUP * (wd >> 1) + k)) + (wd & 1);
+                                const float *c4 = stage.x + slot;
+                                constexpr int SL = TestStage<STAGE_CAP>::SLOTS;
+                                const float jx = c4[0], jy = c4[SL], jz = c4[2 * SL];
+                                const float ex = delta(0, qv.x, jx), ey = delta(1, qv.y, jy), ez = delta(2, qv.z, jz);
+                                // within the fp32 error band of the cutoff: decided in fp64
+                                if (fmaf(ez, ez, fmaf(ey, ey, ex * ex)) > p.r2_mid - p.r2_band && !exact_pair(p, qid, stage.id[slot])) { slot = -1; --cnt; }
+                                // source minus destination
+                                list[at++] = make_float4(mi0 ? -ex : (jx - ox) - (qv.x - ox), mi1 ? -ey : (jy - oy) - (qv.y - oy),
+                                                         mi2 ? -ez : (jz - oz) - (qv.z - oz), __int_as_float(slot));
+                            }
+                        }
                     }
-                    for (int e = lane; e < QB * ACC_W; e += 32) s_acc[e] = 0.f;
+                    int nin = cnt;                                 // neighbours of the lane's query: sum over its lanes, in the first
+#pragma unroll
+                    for (int o = 1; o < TEST_LPQ; o <<= 1) {
+                        if (o >= split.lpq) break;
+                        const int other = __shfl_down_sync(FULL, nin, o);
+                        if (split.sub + o < split.lpq) nin += other;
+                    }
                     __syncwarp();
-                    // The accepted pairs of all queries of the batch form one flat sequence, 32 pairs per step
-                    // whatever the list lengths (a query with a dozen neighbours would otherwise leave most of
-                    // a step idle).  Lanes of one query are neighbours in that sequence, so per-query sums are
-                    // segmented reductions; the first lane of a segment adds the sum to the query's accumulator.
-                    int pre[QB + 1];
-                    pre[0] = 0;
+                    for (int q = qa; q < qb; ++q) {                // the warp evaluates one query at a time
+                        const int oq = __shfl_sync(FULL, qid, q * split.lpq), nq_in = __shfl_sync(FULL, nin, q * split.lpq);
+                        const int off = s_off[q], end = s_end[q];
+                        float S = 0.f, cpos = 0.f, D0 = 0.f, D1 = 0.f, D2 = 0.f, G = 0.f, v = 0.f;
+                        float xq[BWD ? NX : 1], gq[4];
+                        if constexpr (BWD) {
 #pragma unroll
-                    for (int q = 0; q < QB; ++q) pre[q + 1] = pre[q] + (q < nq ? s_n[q] : 0);
-                    const int npairs = pre[QB];
-                    for (int t0 = 0; t0 < npairs; t0 += 32) {
-                        const int f = t0 + lane;
-                        const bool valid = f < npairs;
-                        int q = 0;
+                            for (int f = 0; f < NX; ++f) xq[f] = f < Fin ? __ldg(p.feat + (size_t)oq * Fin + f) : 0.f;
 #pragma unroll
-                        for (int j = 1; j < QB; ++j) q += (f >= pre[j]) ? 1 : 0;
-                        q = q < nq ? q : nq - 1;
-                        int tq = 0;
+                            for (int o = 0; o < 4; ++o) gq[o] = o < Fout ? __ldg(p.gy + (size_t)oq * Fout + o) : 0.f;
+                        }
+#pragma unroll 2
+                        for (int t = off + ps; t < end; t += PS) {
+                            const float4 e = list[t];
+                            const int slot = __float_as_int(e.w);
+                            if (slot < 0) continue;
+                            float h = fmaf(w[2], e.z, fmaf(w[1], e.y, fmaf(w[0], e.x, b1)));
+                            const float4* xr = reinterpret_cast<const float4*>(s_x + slot * NX);
 #pragma unroll
-                        for (int j = 0; j < QB; ++j) tq = (j == q) ? f - pre[j] : tq;
-                        const int key = valid ? q : -1 - lane;               // idle lanes form segments of their own
-                        const float4 qv = s_q[q];
-                        const int oq = checked(__float_as_int(qv.w), p.n, CHECK_POINT);
-                        float4 pj = make_float4(0.f, 0.f, 0.f, __int_as_float(0));
-                        if (valid) pj = stage[list[q * MLP_QSTRIDE + tq]];
-                        float dx = pj.x - qv.x, dy = pj.y - qv.y, dz = pj.z - qv.z;      // source minus destination
-                        fold(dx, dy, dz);
-                        constexpr int NV = BWD ? KU : 4;
-                        float red[NV];
+                            for (int i = 0; i < FQ; ++i) {
+                                const float4 x4 = xr[i];
+                                h = fmaf(w[3 + 4 * i], x4.x, h); h = fmaf(w[4 + 4 * i], x4.y, h);
+                                h = fmaf(w[5 + 4 * i], x4.z, h); h = fmaf(w[6 + 4 * i], x4.w, h);
+                            }
+                            S += fmaxf(h, 0.f);
+                            if constexpr (BWD) {
+                                // the pair the other way round: the query as the source
+                                float h2 = fmaf(w[2], -e.z, fmaf(w[1], -e.y, fmaf(w[0], -e.x, b1)));
 #pragma unroll
-                        for (int i = 0; i < NV; ++i) red[i] = 0.f;
+                                for (int f = 0; f < NX; ++f) h2 = fmaf(w[3 + f], xq[f], h2);
+                                const float4 g4 = s_g[slot];
+                                const float vm = fmaf(w2[3], g4.w, fmaf(w2[2], g4.z, fmaf(w2[1], g4.y, w2[0] * g4.x)));
+                                if (h > 0.f) { cpos += 1.f; D0 += e.x; D1 += e.y; D2 += e.z; }
+                                if (h2 > 0.f) G += vm;
+                            }
+                        }
+                        // sums over the groups of HID lanes
+#pragma unroll
+                        for (int o = HID; o < 32; o <<= 1) {
+                            S += __shfl_xor_sync(FULL, S, o);
+                            if constexpr (BWD) {
+                                cpos += __shfl_xor_sync(FULL, cpos, o); G += __shfl_xor_sync(FULL, G, o);
+                                D0 += __shfl_xor_sync(FULL, D0, o); D1 += __shfl_xor_sync(FULL, D1, o); D2 += __shfl_xor_sync(FULL, D2, o);
+                            }
+                        }
                         if constexpr (!BWD) {
-                            if (valid) {
-                                float u[KU], h[HID], m[4];
-                                u[0] = dx; u[1] = dy; u[2] = dz;
-                                const float* xr = p.feat + (size_t)checked(__float_as_int(pj.w), p.n, CHECK_POINT) * Fin;
+                            float y[4];
 #pragma unroll
-                                for (int k = 3; k < KU; ++k) u[k] = (k - 3 < Fin) ? __ldg(xr + k - 3) : 0.f;
-                                mlp_forward<HID, KQ>(sW1, sb1, sW2, sb2, u, h, m);
-#pragma unroll
-                                for (int o = 0; o < 4; ++o) red[o] = m[o];
+                            for (int o = 0; o < 4; ++o) y[o] = w2[o] * S;
+                            spread_sum<4, HID>(y, a);
+                            const int o = spread_first<4, HID>(a);
+                            const float bias = __shfl_sync(FULL, b2, o);
+                            if (lane < 4 && o < Fout) {
+                                float* dst = p.out + (size_t)oq * Fout + o;
+                                const float val = fmaf((float)nq_in, bias, y[0]);
+                                *dst = first_chunk ? val : *dst + val;
                             }
                         } else {
-                            float* mine = pairbuf + lane * PS;
-                            if (valid) {
-                                const int om = checked(__float_as_int(pj.w), p.n, CHECK_POINT);
-                                float gyk[4], gym[4];
+                            v = fmaf(w2[3], gq[3], fmaf(w2[2], gq[2], fmaf(w2[1], gq[1], w2[0] * gq[0])));
+                            const float vc = v * cpos, Y = G - vc;
+                            gW1[0] = fmaf(v, D0, gW1[0]); gW1[1] = fmaf(v, D1, gW1[1]); gW1[2] = fmaf(v, D2, gW1[2]);
 #pragma unroll
-                                for (int o = 0; o < 4; ++o) {
-                                    gyk[o] = o < Fout ? __ldg(p.gy + (size_t)oq * Fout + o) : 0.f;
-                                    gym[o] = o < Fout ? __ldg(p.gy + (size_t)om * Fout + o) : 0.f;
+                            for (int f = 0; f < NX; ++f) gW1[3 + f] = fmaf(G, xq[f], gW1[3 + f]);
+                            gb1 += vc;
+#pragma unroll
+                            for (int o = 0; o < 4; ++o) gW2[o] = fmaf(gq[o], S, gW2[o]);
+                            gb2 = fmaf((float)nq_in, lane == 0 ? gq[0] : lane == 1 ? gq[1] : lane == 2 ? gq[2] : gq[3], gb2);     // lanes 0..3
+                            constexpr int NV = KP <= 8 ? 8 : KP <= 16 ? 16 : 32;
+                            float r[NV];
+#pragma unroll
+                            for (int k = 0; k < NV; ++k) r[k] = k < KP ? w[k < KP ? k : 0] * (k < 3 ? Y : G) : 0.f;
+                            spread_sum<NV, HID>(r, a);
+                            constexpr int LEFT = NV > HID ? NV / HID : 1;
+                            const int first = spread_first<NV, HID>(a);
+                            if (lane < (NV < HID ? NV : HID)) {
+#pragma unroll
+                                for (int k = 0; k < LEFT; ++k) {
+                                    const int c = first + k;
+                                    float* dst = c < 3 ? (p.gpos ? p.gpos + 3 * (size_t)oq + c : nullptr)
+                                                       : (c < K && p.gfeat ? p.gfeat + (size_t)oq * Fin + c - 3 : nullptr);
+                                    if (dst) *dst = first_chunk ? r[k] : *dst + r[k];
                                 }
-                                float u[KU], h[HID], m[4], ub[KU];
-                                // pair (k <- m): parameter gradients and the destination part of pbar_k
-                                u[0] = dx; u[1] = dy; u[2] = dz;
-                                const float* xr = p.feat + (size_t)om * Fin;
-#pragma unroll
-                                for (int k = 3; k < KU; ++k) u[k] = (k - 3 < Fin) ? __ldg(xr + k - 3) : 0.f;
-                                mlp_forward<HID, KQ>(sW1, sb1, sW2, sb2, u, h, m);
-                                mlp_backward<HID, KQ, true>(sW1, sW2, h, gyk, mine, ub);       // hbar goes straight to the pair buffer
-                                red[0] = -ub[0]; red[1] = -ub[1]; red[2] = -ub[2];
-#pragma unroll
-                                for (int a = 0; a < HID; ++a) mine[HID + MLP_DIN + a] = fmaxf(h[a], 0.f);
-#pragma unroll
-                                for (int k = 0; k < MLP_DIN; ++k) mine[HID + k] = k < KU ? u[k < KU ? k : 0] : 0.f;
-#pragma unroll
-                                for (int o = 0; o < 4; ++o) mine[2 * HID + MLP_DIN + o] = gyk[o];
-                                // pair (m <- k): xbar_k and the source part of pbar_k
-                                const float* xq = p.feat + (size_t)oq * Fin;
-                                u[0] = -dx; u[1] = -dy; u[2] = -dz;
-#pragma unroll
-                                for (int k = 3; k < KU; ++k) u[k] = (k - 3 < Fin) ? __ldg(xq + k - 3) : 0.f;
-                                mlp_forward<HID, KQ>(sW1, sb1, sW2, sb2, u, h, m);
-                                mlp_backward<HID, KQ, false>(sW1, sW2, h, gym, nullptr, ub);
-                                red[0] += ub[0]; red[1] += ub[1]; red[2] += ub[2];
-#pragma unroll
-                                for (int k = 3; k < KU; ++k) red[k] = ub[k];
-                            }
-                            __syncwarp();
-                            const int np = npairs - t0 < 32 ? npairs - t0 : 32;
-                            for (int pp = 0; pp < np; ++pp) {
-                                const float* pb = pairbuf + pp * PS;
-                                const float uk = pb[HID + k1];
-#pragma unroll
-                                for (int i = 0; i < HID / 2; ++i) gW1acc[i] = fmaf(pb[a0 + 2 * i], uk, gW1acc[i]);
-                                if (lane < HID) {
-                                    const float act = pb[HID + MLP_DIN + lane];
-#pragma unroll
-                                    for (int o = 0; o < 4; ++o) gW2acc[o] = fmaf(pb[2 * HID + MLP_DIN + o], act, gW2acc[o]);
-                                    gb1acc += pb[lane];
-                                }
-                                if (lane < 4) gb2acc += pb[2 * HID + MLP_DIN + lane];
-                            }
-                        }
-                        // segmented sums over the lanes of one query
-#pragma unroll
-                        for (int d = 1; d < 32; d <<= 1) {
-                            const int kd = __shfl_down_sync(FULL, key, d);
-                            const bool same = lane + d < 32 && kd == key;
-#pragma unroll
-                            for (int i = 0; i < NV; ++i) {
-                                const float vd = __shfl_down_sync(FULL, red[i], d);
-                                if (same) red[i] += vd;
-                            }
-                        }
-                        const int kprev = __shfl_up_sync(FULL, key, 1);
-                        if (valid && (lane == 0 || kprev != key)) {
-#pragma unroll
-                            for (int i = 0; i < NV; ++i) s_acc[q * ACC_W + i] += red[i];     // one first lane per query and step
-                        }
-                        __syncwarp();
-                    }
-                    // the batch's rows
-                    if constexpr (!BWD) {
-                        const int q = lane >> 2, o = lane & 3;
-                        if (q < nq && o < Fout) {
-                            float* dst = p.out + (size_t)__float_as_int(s_q[q].w) * Fout + o;
-                            const float v = s_acc[q * ACC_W + o];
-                            *dst = first ? v : *dst + v;
-                        }
-                    } else {
-                        for (int e = lane; e < nq * ACC_W; e += 32) {
-                            const int q = e / ACC_W, cidx = e % ACC_W;
-                            const int oq = __float_as_int(s_q[q].w);
-                            const float v = s_acc[e];
-                            if (cidx < 3) {
-                                if (p.gpos) { float* o = p.gpos + 3 * (size_t)oq + cidx; *o = first ? v : *o + v; }
-                            } else if (cidx - 3 < Fin && cidx < KU) {
-                                if (p.gfeat) { float* o = p.gfeat + (size_t)oq * Fin + cidx - 3; *o = first ? v : *o + v; }
                             }
                         }
                     }
-#pragma unroll
-                    for (int q = 0; q < QB; ++q) qcnt[q] = 0;
-                    first = false;
                     __syncwarp();
-                };
-
-                auto phase_a = [&](const int cbase) -> bool {
-                    const float4 pj = stage[cbase + lane];
-                    const int idj = __float_as_int(pj.w);
-                    float d2q[QB];
-                    float nearest = FAR_AWAY;
-#pragma unroll
-                    for (int q = 0; q < QB; ++q) {
-                        if (q >= nq) break;
-                        const float4 qv = s_q[q];
-                        float dx = qv.x - pj.x, dy = qv.y - pj.y, dz = qv.z - pj.z;
-                        fold(dx, dy, dz);
-                        float d2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-                        if (idj == __float_as_int(qv.w) || (MI && idj < 0)) d2 = FAR_AWAY;
-                        nearest = fminf(nearest, fabsf(d2 - p.r2_mid));
-                        d2q[q] = d2;
-                    }
-                    if (__any_sync(FULL, nearest <= p.r2_band)) {
-#pragma unroll
-                        for (int q = 0; q < QB; ++q) {
-                            if (q >= nq) break;
-                            if (fabsf(d2q[q] - p.r2_mid) <= p.r2_band)
-                                d2q[q] = exact_pair(p, __float_as_int(s_q[q].w), idj) ? fminf(d2q[q], p.r2_lo) : FAR_AWAY;
-                        }
-                    }
-                    int mx = 0;
-#pragma unroll
-                    for (int q = 0; q < QB; ++q) {
-                        if (q >= nq) break;
-                        const bool ok = d2q[q] <= p.r2_lo;
-                        const unsigned m = __ballot_sync(FULL, ok);
-                        if (ok) list[q * MLP_QSTRIDE + qcnt[q] + __popc(m & lt_mask)] = cbase + lane;
-                        qcnt[q] += __popc(m);
-                        mx = qcnt[q] > mx ? qcnt[q] : mx;
-                    }
-                    return mx > MLP_QCAP - 32;
-                };
-                bool need = false;
-                for (int cbase = 0;; cbase += 32) {
-                    const bool done = cbase >= ns;
-                    if (done || need) drain();
-                    if (done) break;
-                    need = phase_a(cbase);
-                }
-                if (!BWD && p.count && lane < nq) {
-                    const int oq = __float_as_int(s_q[lane].w);
-                    p.count[oq] = first_chunk ? s_tot[lane] : p.count[oq] + s_tot[lane];
+                    if (!BWD && p.count && part && split.sub == 0) p.count[qid] = first_chunk ? nin : p.count[qid] + nin;
+                    qa = qb;
                 }
             }
             __syncwarp();
         };
 
-        // the 27-cell stencil as candidate ranges (lane r < 27 resolves neighbour offset r)
-        int r_cs = 0, r_ce = 0;
-        float r_off[3] = {0.f, 0.f, 0.f};
-        {
-            const int off[3] = {lane % 3 - 1, (lane / 3) % 3 - 1, lane / 9 - 1};
-            bool ok = lane < 27;
-            int q[3] = {0, 0, 0};
-            bool merged = false;
-#pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                if (p.nc[d] == 1) { ok = ok && off[d] == 0; r_off[d] = org[d]; continue; }
-                if (d == 0 && c[0] >= 1 && c[0] <= p.nc[0] - 2) {
-                    merged = true; ok = ok && off[0] == 0; q[0] = c[0] - 1; r_off[0] = org[0];
-                    continue;
-                }
-                int v = c[d] + off[d];
-                r_off[d] = org[d];
-                if (v < 0) {
-                    if (p.periodic[d]) { v += p.nc[d]; r_off[d] = org[d] + p.len[d]; }
-                    else ok = false;
-                } else if (v >= p.nc[d]) {
-                    if (p.periodic[d]) { v -= p.nc[d]; r_off[d] = org[d] - p.len[d]; }
-                    else ok = false;
-                }
-                q[d] = v;
+        // the stage fills with candidates that survive the pruning; a step that does not fit is taken again
+        bool first_chunk = true, full = false;
+        int nst = 0, before = -1;
+        constexpr int SU = 4;
+        static_assert(STAGE_CAP >= 32 * SU, "a step fits an empty stage");
+        for (int k0 = 0;;) {
+            const bool done = k0 >= sten.total;
+            if (full || (done && (nst > 0 || first_chunk))) {
+                process_chunk(nst, first_chunk);
+                first_chunk = false;
+                full = false;
+                nst = 0;
+                for (int k = lane; k < qe0 - qs0; k += 32) s_self[k] = -1;
+                __syncwarp();
             }
-            if (ok) {
-                const int id = (q[2] * p.nc[1] + q[1]) * p.nc[0] + q[0];
-                r_cs = p.cell_start[id];
-                r_ce = p.cell_start[id + (merged ? 3 : 1)];
+            if (done) break;
+            const int step = sten.total - k0 < 32 * SU ? sten.total - k0 : 32 * SU, before0 = before;
+            float4 c4[SU];
+            int src[SU];
+            unsigned kept[SU];
+#pragma unroll
+            for (int u = 0; u < SU; ++u) {
+                c4[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                src[u] = -1;
+                if (32 * u >= step) continue;
+                src[u] = sten.source(k0 + 32 * u, before, s_delta);
+                if (k0 + 32 * u + lane < sten.total) c4[u] = __ldg(p.spos + checked(src[u], p.n, CHECK_SLOT));
             }
-        }
-        const int r_len = r_ce - r_cs;
-        int r_incl = r_len;
+            int all = nst;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(FULL, r_incl, o);
-            if (lane >= o) r_incl += t;
-        }
-        const int total = __shfl_sync(FULL, r_incl, 31);
-        // bounding box of the cell's own points (local coordinates), one register per lane: a candidate
-        // farther than the cutoff from it is no neighbour of any of them and is not staged
-        float bb;
-        {
-            float blo[3] = {FAR_AWAY, FAR_AWAY, FAR_AWAY}, bhi[3] = {-FAR_AWAY, -FAR_AWAY, -FAR_AWAY};
-            for (int q = qs0 + lane; q < qe0; q += 32) {
-                const float4 pq = p.spos[q];
-                const float l[3] = {pq.x - org[0], pq.y - org[1], pq.z - org[2]};
-#pragma unroll
-                for (int d = 0; d < 3; ++d) { blo[d] = fminf(blo[d], l[d]); bhi[d] = fmaxf(bhi[d], l[d]); }
+            for (int u = 0; u < SU; ++u) {
+                kept[u] = 0u;
+                if (32 * u >= step) continue;
+                frame.shift(p, c4[u]);
+                const float ex = fmaxf(fmaxf(blo[0] - c4[u].x, c4[u].x - bhi[0]), 0.f);
+                const float ey = fmaxf(fmaxf(blo[1] - c4[u].y, c4[u].y - bhi[1]), 0.f);
+                const float ez = fmaxf(fmaxf(blo[2] - c4[u].z, c4[u].z - bhi[2]), 0.f);
+                kept[u] = __ballot_sync(FULL, k0 + 32 * u + lane < sten.total && fmaf(ez, ez, fmaf(ey, ey, ex * ex)) <= p.r2_hi * 1.0001f);
+                all += __popc(kept[u]);
             }
+            if (all > STAGE_CAP) { full = true; before = before0; continue; }
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1)
+            for (int u = 0; u < SU; ++u) {
+                if ((kept[u] >> lane) & 1u) {
+                    const int slot = nst + __popc(kept[u] & lt_mask);
+                    stage.put(slot, c4[u]);
+                    if (src[u] >= qs0 && src[u] < qe0) s_self[src[u] - qs0] = slot;
+                    const int id = checked(__float_as_int(c4[u].w), p.n, CHECK_POINT);
+                    const float* xr = p.feat + (size_t)id * Fin;
+                    float4* dst = reinterpret_cast<float4*>(s_x + slot * NX);
 #pragma unroll
-                for (int d = 0; d < 3; ++d) {
-                    blo[d] = fminf(blo[d], __shfl_xor_sync(FULL, blo[d], o));
-                    bhi[d] = fmaxf(bhi[d], __shfl_xor_sync(FULL, bhi[d], o));
-                }
-            bb = lane == 0 ? blo[0] : lane == 1 ? blo[1] : lane == 2 ? blo[2] : lane == 3 ? bhi[0] : lane == 4 ? bhi[1] : bhi[2];
-            if (mi0 && (lane == 0 || lane == 3)) bb = lane == 0 ? -FAR_AWAY : FAR_AWAY;   // a dimension folded by the explicit
-            if (mi1 && (lane == 1 || lane == 4)) bb = lane == 1 ? -FAR_AWAY : FAR_AWAY;   // minimum image is not pruned
-            if (mi2 && (lane == 2 || lane == 5)) bb = lane == 2 ? -FAR_AWAY : FAR_AWAY;
-        }
-        bool first_chunk = true;
-        for (int lo = 0; lo < total || first_chunk; lo += MLP_STAGE_CAP) {
-            const int ns = total - lo < MLP_STAGE_CAP ? total - lo : MLP_STAGE_CAP;
-            int nst = 0;                                                     // candidates kept (warp uniform)
-            constexpr int SU = 4;                                            // staging groups in flight
-            for (int k0 = 0; k0 < ns; k0 += 32 * SU) {
-                float4 c4[SU];
-                float ox[SU], oy[SU], oz[SU];
-#pragma unroll
-                for (int u = 0; u < SU; ++u) {                               // all loads of the step first
-                    const int k = k0 + 32 * u + lane;
-                    const int v = lo + k;
-                    int r = 0;
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) {
-                        const int probe = __shfl_sync(FULL, r_incl, r + o - 1);
-                        if (probe <= v) r += o;
+                    for (int i = 0; i < FQ; ++i)
+                        dst[i] = (Fin & 3) == 0 ? __ldg(reinterpret_cast<const float4*>(xr) + i)
+                                                : make_float4(4 * i < Fin ? __ldg(xr + 4 * i) : 0.f, 4 * i + 1 < Fin ? __ldg(xr + 4 * i + 1) : 0.f,
+                                                              4 * i + 2 < Fin ? __ldg(xr + 4 * i + 2) : 0.f, 4 * i + 3 < Fin ? __ldg(xr + 4 * i + 3) : 0.f);
+                    if constexpr (BWD) {
+                        const float* gr = p.gy + (size_t)id * Fout;
+                        s_g[slot] = make_float4(__ldg(gr), Fout > 1 ? __ldg(gr + 1) : 0.f, Fout > 2 ? __ldg(gr + 2) : 0.f, Fout > 3 ? __ldg(gr + 3) : 0.f);
                     }
-                    r = r > 31 ? 31 : r;
-                    const int src = __shfl_sync(FULL, r_cs, r) + (v - (__shfl_sync(FULL, r_incl, r) - __shfl_sync(FULL, r_len, r)));
-                    ox[u] = __shfl_sync(FULL, r_off[0], r); oy[u] = __shfl_sync(FULL, r_off[1], r); oz[u] = __shfl_sync(FULL, r_off[2], r);
-                    c4[u] = k < ns ? __ldg(p.spos + checked(src, p.n, CHECK_SLOT)) : make_float4(0.f, 0.f, 0.f, 0.f);
                 }
-                const float lx = __shfl_sync(FULL, bb, 0), ly = __shfl_sync(FULL, bb, 1), lz = __shfl_sync(FULL, bb, 2);
-                const float hx = __shfl_sync(FULL, bb, 3), hy = __shfl_sync(FULL, bb, 4), hz = __shfl_sync(FULL, bb, 5);
-#pragma unroll
-                for (int u = 0; u < SU; ++u) {
-                    if (k0 + 32 * u >= ns) break;
-                    const float4 val = make_float4(c4[u].x - ox[u], c4[u].y - oy[u], c4[u].z - oz[u], c4[u].w);
-                    const float ex = fmaxf(fmaxf(lx - val.x, val.x - hx), 0.f);
-                    const float ey = fmaxf(fmaxf(ly - val.y, val.y - hy), 0.f);
-                    const float ez = fmaxf(fmaxf(lz - val.z, val.z - hz), 0.f);
-                    const bool keep = k0 + 32 * u + lane < ns && fmaf(ez, ez, fmaf(ey, ey, ex * ex)) <= p.r2_hi * 1.0001f;
-                    const unsigned m = __ballot_sync(FULL, keep);
-                    if (keep) stage[nst + __popc(m & lt_mask)] = val;
-                    nst += __popc(m);
-                }
+                nst += __popc(kept[u]);
             }
-            __syncwarp();
-            process_chunk(nst, first_chunk);
-            first_chunk = false;
+            k0 += 32 * SU;
         }
-    }
+    };
+    const int units = (p.n + p.unit - 1) / p.unit;
+    for (int u = blockIdx.x * MLP_WARPS + wib; u < units; u += gridDim.x * MLP_WARPS) walk_unit(p, u, p.run, slice);
 
     if constexpr (BWD) {
         // warps -> CTA copy in shared memory -> one atomic per parameter entry and CTA
         float* gW1s = sG;
-        float* gb1s = gW1s + HID * MLP_DIN;
+        float* gb1s = gW1s + HID * KP;
         float* gW2s = gb1s + HID;
         float* gb2s = gW2s + 4 * HID;
+        if (ps == 0) {
 #pragma unroll
-        for (int i = 0; i < HID / 2; ++i) atomicAdd(gW1s + (a0 + 2 * i) * MLP_DIN + k1, gW1acc[i]);
-        if (lane < HID) {
+            for (int k = 0; k < KP; ++k) atomicAdd(gW1s + a * KP + k, gW1[k]);
 #pragma unroll
-            for (int o = 0; o < 4; ++o) atomicAdd(gW2s + o * HID + lane, gW2acc[o]);
-            atomicAdd(gb1s + lane, gb1acc);
+            for (int o = 0; o < 4; ++o) atomicAdd(gW2s + o * HID + a, gW2[o]);
+            atomicAdd(gb1s + a, gb1);
         }
-        if (lane < 4) atomicAdd(gb2s + lane, gb2acc);
+        if (lane < 4) atomicAdd(gb2s + lane, gb2);
         __syncthreads();
-        for (int e = threadIdx.x; e < HID * MLP_DIN; e += TRAV_THREADS) {
-            const int a = e / MLP_DIN, k = e % MLP_DIN;
-            if (k < K && p.gW1) atomicAdd(p.gW1 + a * K + k, gW1s[e]);
+        for (int e = threadIdx.x; e < HID * KP; e += MLP_THREADS) {
+            const int i = e / KP, k = e % KP;
+            if (k < K && p.gW1) atomicAdd(p.gW1 + i * K + k, gW1s[e]);
         }
-        for (int e = threadIdx.x; e < HID; e += TRAV_THREADS) if (p.gb1) atomicAdd(p.gb1 + e, gb1s[e]);
-        for (int e = threadIdx.x; e < Fout * HID; e += TRAV_THREADS) if (p.gW2) atomicAdd(p.gW2 + e, gW2s[e]);
+        for (int e = threadIdx.x; e < HID; e += MLP_THREADS) if (p.gb1) atomicAdd(p.gb1 + e, gb1s[e]);
+        for (int e = threadIdx.x; e < Fout * HID; e += MLP_THREADS) if (p.gW2) atomicAdd(p.gW2 + e, gW2s[e]);
         if (threadIdx.x < Fout && p.gb2) atomicAdd(p.gb2 + threadIdx.x, gb2s[threadIdx.x]);
     }
 }
 
-template <int HID, int KQ, bool BWD, bool MI>
+// parameter gradients start from zero (one launch for the four arrays)
+__global__ void mlp_zero_kernel(float* a, int na, float* b, int nb, float* c, int nc, float* d, int nd) {
+    for (int k = threadIdx.x; k < na; k += blockDim.x) a[k] = 0.f;
+    for (int k = threadIdx.x; k < nb; k += blockDim.x) b[k] = 0.f;
+    for (int k = threadIdx.x; k < nc; k += blockDim.x) c[k] = 0.f;
+    for (int k = threadIdx.x; k < nd; k += blockDim.x) d[k] = 0.f;
+}
+
+template <int HID, int FQ, bool BWD, bool MI>
 static tiga_status launch_mlp_t(const RadiusParams& p, cudaStream_t s) {
-    using SM = MlpSmem<HID, BWD>;
-    auto kern = radius_mlp_kernel<HID, KQ, BWD, MI>;
+    using SM = MlpSmem<HID, FQ, BWD>;
+    auto kern = radius_mlp_kernel<HID, FQ, BWD, MI>;
     if (SM::TOTAL > 48 * 1024) TIGA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SM::TOTAL));
-    long long blocks = (p.ncells + TRAV_WARPS - 1) / TRAV_WARPS;
-    const long long cap = 148LL * mlp_ctas_per_sm<HID, BWD>();       // persistent: parameter gradients are folded once per CTA
-    if (blocks > cap) blocks = cap;
-    kern<<<counted((unsigned)blocks), TRAV_THREADS, SM::TOTAL, s>>>(p);
+    const unsigned need = (unit_count(p) + MLP_WARPS - 1) / MLP_WARPS, cap = 148u * mlp_ctas_per_sm<FQ, BWD>();       // persistent: parameter gradients are folded once per CTA
+    kern<<<counted(need < cap ? need : cap), MLP_THREADS, SM::TOTAL, s>>>(p);
     return launch_status();
 }
 
 template <int HID, bool BWD, bool MI>
 static tiga_status launch_mlp_k(const RadiusParams& p, cudaStream_t s) {
-    switch ((3 + p.Fin + 3) / 4) {
+    switch ((p.Fin + 3) / 4) {
         case 1: return launch_mlp_t<HID, 1, BWD, MI>(p, s);
         case 2: return launch_mlp_t<HID, 2, BWD, MI>(p, s);
         case 3: return launch_mlp_t<HID, 3, BWD, MI>(p, s);
@@ -536,7 +417,7 @@ static tiga_status launch_mlp_k(const RadiusParams& p, cudaStream_t s) {
 template <bool BWD>
 static tiga_status launch_mlp(const RadiusParams& p, int hidden, cudaStream_t s) {
     bool mi = false;
-    for (int d = 0; d < 3; ++d) mi = mi || (p.periodic[d] && p.nc[d] == 1);
+    for (int d = 0; d < 3; ++d) mi = mi || (p.periodic[d] && p.nc[d] <= 3);
     if (hidden == 8) return mi ? launch_mlp_k<8, BWD, true>(p, s) : launch_mlp_k<8, BWD, false>(p, s);
     if (hidden == 16) return mi ? launch_mlp_k<16, BWD, true>(p, s) : launch_mlp_k<16, BWD, false>(p, s);
     return mi ? launch_mlp_k<32, BWD, true>(p, s) : launch_mlp_k<32, BWD, false>(p, s);
@@ -591,10 +472,11 @@ extern "C" tiga_status tiga_apply_radius_mlp_backward(const float* pos, const fl
     if (st != TIGA_OK) return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int K = 3 + mlp->f_in;
-    if (grad_W1) TIGA_CUDA_TRY(cudaMemsetAsync(grad_W1, 0, sizeof(float) * mlp->hidden * K, s));
-    if (grad_b1) TIGA_CUDA_TRY(cudaMemsetAsync(grad_b1, 0, sizeof(float) * mlp->hidden, s));
-    if (grad_W2) TIGA_CUDA_TRY(cudaMemsetAsync(grad_W2, 0, sizeof(float) * mlp->f_out * mlp->hidden, s));
-    if (grad_b2) TIGA_CUDA_TRY(cudaMemsetAsync(grad_b2, 0, sizeof(float) * mlp->f_out, s));
+    if (grad_W1 || grad_b1 || grad_W2 || grad_b2) {
+        mlp_zero_kernel<<<counted(1), 256, 0, s>>>(grad_W1, grad_W1 ? mlp->hidden * K : 0, grad_b1, grad_b1 ? mlp->hidden : 0,
+                                                   grad_W2, grad_W2 ? mlp->f_out * mlp->hidden : 0, grad_b2, grad_b2 ? mlp->f_out : 0);
+        if (launch_status() != TIGA_OK) return TIGA_ERR_CUDA;
+    }
     if (n == 0) return TIGA_OK;
     if (!grad_out || !aligned16(grad_out)) return TIGA_ERR_INVALID_ARG;
     p.gy = grad_out; p.gfeat = grad_feat; p.gpos = grad_pos;

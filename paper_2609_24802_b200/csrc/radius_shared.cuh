@@ -6,14 +6,16 @@
 
 namespace tiga {
 
-constexpr int TRAV_WARPS = 4;
+// one warp per CTA: units differ in work (0 to 3 cells), and a CTA holds its place until its last warp is done (four
+// warps: forward of 1 M points, 32 neighbours, 725 instead of 557 us)
+constexpr int TRAV_WARPS = 1;
 constexpr int TRAV_THREADS = TRAV_WARPS * 32;
 constexpr int STAGE_PAD = 32;           // sentinels behind the staged candidates: no bounds checks
 constexpr int QB = 8;                   // queries per batch (kernels that run faster with four define their own width)
 constexpr float FAR_AWAY = 1.0e18f;
-constexpr int QDENSE = 64;              // a cell with more points than this is cut into slices of QSLICE queries:
-constexpr int QSLICE = 16;              // its warp takes the first slice, the others wait in a queue that other warps walk
-constexpr int QUEUE_BLOCKS = 148 * 8;   // most CTAs that walk the queued slices
+constexpr int QDENSE = 64;              // a cell with more points than this is cut into slices
+constexpr int QSLICE = 16;              // of this many queries
+constexpr int UNIT_MAX = 32;            // most points per unit of work (at most 32: a lane each)
 constexpr int RUN_CELLS = 8;            // longest run of cells along x that one warp covers
 constexpr int RUN_QUERIES = 16;         // points a warp joins cells for
 constexpr int SORT_DENSE = 256;         // a cell with more points than this is ordered by a sorting network, not by rank counting
@@ -52,13 +54,9 @@ struct RadiusParams {
     int32_t* order;
     float4* spos;             // positions in cell order, .w = original point id (bit pattern)
     int32_t* blocksum;
-    // slices of cells with more than QDENSE points, queued by the binning scan
-    int2* q_items;            // (cell, first query of the slice)
-    int* q_count;
-    int run;                  // cells along x that one warp of the Gaussian / distance traversals covers
-    int row_runs;             // runs per row of cells
-    int cell_blocks;          // one-launch form: CTAs [0, cell_blocks) take cells, the CTAs behind them walk the queue
-    int32_t* b_items;         // cells with more than SORT_DENSE points (queued by the same scan), and how many
+    int run;                  // cells along x that a warp joins at most
+    int unit;                 // points per warp (walk_unit)
+    int32_t* b_items;         // cells with more than SORT_DENSE points (queued by the scan), and how many
     int* b_count;
     // optional user copies of the plan
     int32_t* u_cell;
@@ -78,6 +76,12 @@ tiga_status run_binning(RadiusParams& p, int32_t* fill, int nblocks, cudaStream_
 // host side, defined in radius_lj.cu
 tiga_status launch_lj(const RadiusParams& p, cudaStream_t s);
 
+// cell coordinate of a point coordinate: one rounded product, clamped to the grid
+static __device__ __forceinline__ int cell_coordinate(const RadiusParams& p, const float v, const int d) {
+    const int k = (int)floorf(__fmul_rn(v, p.invh[d]));
+    return k > p.nc[d] - 1 ? p.nc[d] - 1 : k < 0 ? 0 : k;
+}
+
 // The defining predicate in double precision (same operations as the plain definition).
 static __device__ __noinline__ bool exact_within(const RadiusParams& p, const float4 a, const float4 b) {
     const float pa[3] = {a.x, a.y, a.z}, pb[3] = {b.x, b.y, b.z};
@@ -95,37 +99,55 @@ static __device__ __noinline__ bool exact_within(const RadiusParams& p, const fl
     return d2 <= p.r2_exact;
 }
 
-// A cell with more than QDENSE points: the warp that owns it keeps the first QSLICE queries; the others
-// are queued, QSLICE at a time, for the pass over the queue.  The queue is part of the binning plan
-// (written where the cell offsets are, so the traversals carry no code for it).  (Short slices: a dense cell's queries meet
-// thousands of candidates each, and many short slices fill the machine where a few long ones leave a tail.)
-static __device__ __forceinline__ int slice_end(int qs, int cell_end) { return cell_end - qs > QSLICE ? qs + QSLICE : cell_end; }
-static __device__ __forceinline__ void queue_extra_slices(const RadiusParams& p, int cell, int count) {
-    if (count > QDENSE) {
-        const int extra = (count - 1) / QSLICE;
-        const int at = atomicAdd(p.q_count, extra);
-        for (int k = 0; k < extra; ++k) p.q_items[at + k] = make_int2(cell, (k + 1) * QSLICE);
+// The traversals share the points out by their place in cell order: unit u, one warp's work, is the cells whose first
+// point lies in [u p.unit, (u + 1) p.unit), and of a cell with more than QDENSE points the slices of QSLICE queries that
+// begin there.  So every warp has about p.unit queries whatever the density, empty cells cost nothing and a dense cell
+// spreads over many warps, without a list of work items.  (Short slices: a dense cell's queries meet thousands of
+// candidates each.)  Neighbouring cells along x are joined to runs of at most `run` cells and RUN_QUERIES points.
+// work(first cell of the run, cells, first query, end)
+template <typename Work>
+static __device__ __forceinline__ void walk_unit(const RadiusParams& p, const int u, const int run, Work& work) {
+    constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const int i = u * p.unit + lane;
+    const bool valid = lane < p.unit && i < p.n;
+    int at = 0, qe = 0;                                         // cell of the lane's point, ten bits per coordinate; end of its queries
+    bool dense = false, head = false;
+    if (valid) {
+        const float4 v = p.spos[i];
+        const int x = cell_coordinate(p, v.x, 0), y = cell_coordinate(p, v.y, 1), z = cell_coordinate(p, v.z, 2);
+        at = x | y << 10 | z << 20;
+        const int id = (z * p.nc[1] + y) * p.nc[0] + x;
+        const int cs = p.cell_start[id], ce = p.cell_start[id + 1];
+        dense = ce - cs > QDENSE;
+        head = dense ? (i - cs) % QSLICE == 0 : i == cs;
+        qe = dense && i + QSLICE < ce ? i + QSLICE : ce;
     }
-    if (count > SORT_DENSE) p.b_items[atomicAdd(p.b_count, 1)] = cell;
+    unsigned left = __ballot_sync(FULL, head);                  // cells and slices of the unit not done yet
+    qe |= dense ? 0x80000000 : 0;
+    while (left) {
+        const int a = __ffs(left) - 1;
+        left &= left - 1u;
+        const int first = __shfl_sync(FULL, at, a), qs = u * p.unit + a;
+        int end = __shfl_sync(FULL, qe, a), last = first;
+        if (end >= 0) {                                         // not a slice: join what follows in the row
+            while (left) {
+                const int b = __ffs(left) - 1;
+                const int next = __shfl_sync(FULL, at, b), more = __shfl_sync(FULL, qe, b);
+                if (((next ^ first) >> 10) != 0 || next - first >= run || more - qs > RUN_QUERIES || more < 0) break;
+                end = more; last = next;
+                left &= left - 1u;
+            }
+        }
+        const int cell[3] = {first & 1023, (first >> 10) & 1023, first >> 20};
+        work(cell, last - first + 1, qs, end & 0x7fffffff);
+        __syncwarp();
+    }
 }
 
-// CTAs that walk the queue: no more than the queue can have items for (at most n / QSLICE slices exist)
-static inline unsigned queue_blocks(long long n) {
-    const long long need = n / ((long long)QSLICE * TRAV_WARPS) + 1;
-    return (unsigned)(need < QUEUE_BLOCKS ? need : QUEUE_BLOCKS);
-}
-
-// One launch over the runs of p.run cells along x and, in the CTAs appended behind them, over the queue of slices
-// (which the binning filled before the launch).
-template <typename Launch>
-static inline tiga_status runs_then_queue(const RadiusParams& p, cudaStream_t s, Launch launch) {
-    RadiusParams q = p;
-    q.row_runs = (p.nc[0] + p.run - 1) / p.run;
-    const long long warps = (long long)q.row_runs * p.nc[1] * p.nc[2];
-    q.cell_blocks = (int)((warps + TRAV_WARPS - 1) / TRAV_WARPS);
-    launch(q, (unsigned)q.cell_blocks + queue_blocks(p.n));
-    return launch_status();
-}
+static inline unsigned unit_count(const RadiusParams& p) { return (unsigned)(((long long)p.n + p.unit - 1) / p.unit); }
+// CTAs with one warp per unit
+static inline unsigned unit_blocks(const RadiusParams& p) { return (unit_count(p) + TRAV_WARPS - 1) / TRAV_WARPS; }
 
 static __device__ __forceinline__ float fast_exp2(float x) {
     float r;

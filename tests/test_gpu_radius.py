@@ -278,8 +278,9 @@ def test_lennard_jones_small_grids(tiga, cells, periodic):
 
 
 def test_lennard_jones_dense_cells_span_several_stage_chunks(tiga):
-    """Hundreds of points per cell: the cell's own points alone overflow the stage, so the
-    stencil is processed in several chunks and a query is left out across chunk borders."""
+    """Hundreds of points per cell: the cell's own points alone overflow the stage, so the half
+    stencil is processed in several chunks and the own-cell rule (each pair once, by index) is
+    applied across chunk borders."""
     box = np.array([6.0, 6.0, 6.0], np.float32)
     pos = _separated_points(2600, box, 77, 0.25)
     assert len(pos) > 1800
