@@ -742,6 +742,8 @@ tiga_status fill_params(RadiusParams* p, long long n, float r, const tiga_box* b
     p->ncells = nc[0] * nc[1] * nc[2];
     p->run = run_length(*p);
     p->unit = unit_length(*p);
+    p->dense = QDENSE;
+    p->slice = QSLICE;
     const float r2 = r * r;
     const float beta = (single_periodic ? 96.f : 32.f) * 5.9604645e-8f;
     p->r2_lo = r2 * (1.f - beta);

@@ -56,6 +56,7 @@ struct RadiusParams {
     int32_t* blocksum;
     int run;                  // cells along x that a warp joins at most
     int unit;                 // points per warp (walk_unit)
+    int dense, slice;         // a cell with more than `dense` points is cut into slices of `slice` queries
     int32_t* b_items;         // cells with more than SORT_DENSE points (queued by the scan), and how many
     int* b_count;
     // optional user copies of the plan
@@ -100,7 +101,7 @@ static __device__ __noinline__ bool exact_within(const RadiusParams& p, const fl
 }
 
 // The traversals share the points out by their place in cell order: unit u, one warp's work, is the cells whose first
-// point lies in [u p.unit, (u + 1) p.unit), and of a cell with more than QDENSE points the slices of QSLICE queries that
+// point lies in [u p.unit, (u + 1) p.unit), and of a cell with more than p.dense points the slices of p.slice queries that
 // begin there.  So every warp has about p.unit queries whatever the density, empty cells cost nothing and a dense cell
 // spreads over many warps, without a list of work items.  (Short slices: a dense cell's queries meet thousands of
 // candidates each.)  Neighbouring cells along x are joined to runs of at most `run` cells and RUN_QUERIES points.
@@ -119,9 +120,9 @@ static __device__ __forceinline__ void walk_unit(const RadiusParams& p, const in
         at = x | y << 10 | z << 20;
         const int id = (z * p.nc[1] + y) * p.nc[0] + x;
         const int cs = p.cell_start[id], ce = p.cell_start[id + 1];
-        dense = ce - cs > QDENSE;
-        head = dense ? (i - cs) % QSLICE == 0 : i == cs;
-        qe = dense && i + QSLICE < ce ? i + QSLICE : ce;
+        dense = ce - cs > p.dense;
+        head = dense ? (i - cs) % p.slice == 0 : i == cs;
+        qe = dense && i + p.slice < ce ? i + p.slice : ce;
     }
     unsigned left = __ballot_sync(FULL, head);                  // cells and slices of the unit not done yet
     qe |= dense ? 0x80000000 : 0;
