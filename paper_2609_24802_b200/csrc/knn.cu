@@ -609,9 +609,7 @@ extern "C" tiga_status tiga_apply_knn(const float* pos, const float* feat, int64
     knn_carve(&P, ws, &fill, &lay);
     P.rp.pos = pos; P.rp.feat = feat; P.rp.F = F;
     P.k = k;
-    // small inputs are cut finer: three warps for each of the 4144 places before a slice grows to 16 queries
-    const int slice = (int)(n / (148LL * 28 * 3) + KQB - 1) / KQB * KQB;
-    if (slice < QSLICE) { P.rp.slice = slice < KQB ? KQB : slice; P.rp.dense = P.rp.slice + P.rp.slice / 2; }
+    cut_cells(P.rp, 148 * 84);           // a query costs more here: finer slices
     P.h2 = h * h;
     P.prune2 = P.rp.r2_hi * 1.0001f;
     float hmin = P.rp.hcell[0];

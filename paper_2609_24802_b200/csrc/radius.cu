@@ -689,6 +689,7 @@ RadiusLayout carve_radius(RadiusParams* p, void* ws, int32_t** fill) {
     const int nblocks = (int)((nc + SCAN_BLOCK - 1) / SCAN_BLOCK);
     p->cnt = cv.take<int32_t>(2 * nc + 2 + 16);     // counts, then the scatter cursors, then the length of the dense-cell queue
     p->b_count = p->cnt + 2 * nc + 2;
+    p->ticket = p->b_count + 1;
     *fill = p->cnt + nc;
     p->cell = cv.take<int32_t>(n);
     p->cell_start = cv.take<int32_t>(nc + 1);
@@ -742,8 +743,9 @@ tiga_status fill_params(RadiusParams* p, long long n, float r, const tiga_box* b
     p->ncells = nc[0] * nc[1] * nc[2];
     p->run = run_length(*p);
     p->unit = unit_length(*p);
-    p->dense = QDENSE;
-    p->slice = QSLICE;
+    // (slices of 16 from cells above 64 points, the earlier rule, against this one: 40 k clustered points, F = 8, forward +
+    // backward 1972 -> 594 us; 4 k, F = 16, 330 -> 109 us; 30 k uniform points with 45 neighbours 155 -> 140 us)
+    cut_cells(*p, 148 * 42);
     const float r2 = r * r;
     const float beta = (single_periodic ? 96.f : 32.f) * 5.9604645e-8f;
     p->r2_lo = r2 * (1.f - beta);

@@ -17,9 +17,10 @@
 // where every lane accumulates the parameter gradients of its hidden unit in registers over all its queries; at the end
 // warps fold into the CTA's shared copy and the CTA adds that to global memory with one atomic per entry.
 //
-// Bound by latency and the tail of the work units (36 to 40 % of the issue slots).  35,947 surface points, 15.6 neighbours,
-// 8 features, HID = 32: forward 121 -> 103 us, backward 512 -> 138 us against one lane per pair with the weights read from
-// shared memory (the earlier form, some 600 shared-memory reads per 32 pairs).
+// Bound by instruction issue (57 % of the slots, 28 and 49 M warp instructions) and the tail of the work units.  35,947 surface
+// points, 15.6 neighbours, 8 features, HID = 32: forward 121 -> 53 us, backward 512 -> 85 us against one lane per pair with
+// the weights read from shared memory (the earlier form, some 600 shared-memory reads per 32 pairs); 300 k uniform points,
+// 32 neighbours, HID = 16: 455 -> 383 and 1750 -> 603 us.
 //
 // The displacement is formed from coordinates relative to the corner of the query's cell and the pre-activation as one chain
 // of fused multiply-adds (bias, displacement, features): a ReLU switches on the last bit of that sum.
@@ -27,7 +28,9 @@
 
 namespace tiga {
 
-constexpr int MLP_WARPS = 4, MLP_THREADS = 32 * MLP_WARPS;
+// Forward: one warp per CTA, a CTA per unit of points.  Backward: a persistent grid of four-warp CTAs (the parameter gradients
+// are folded once per CTA) whose warps draw their units from a counter.
+__host__ __device__ constexpr int mlp_warps(bool bwd) { return bwd ? 4 : 1; }
 
 template <int HID, int FQ, bool BWD> struct MlpSmem {
     static constexpr int NX = 4 * FQ;                                            // staged features per candidate (zero padded)
@@ -39,11 +42,11 @@ template <int HID, int FQ, bool BWD> struct MlpSmem {
     static constexpr int K_PAD = 3 + NX;
     static constexpr int GRAD_FLOATS = HID * (K_PAD + 1 + 4) + 4;                // W1, b1, W2, b2 of the CTA's gradient copy
     static constexpr int CTA_BYTES = BWD ? (GRAD_FLOATS * 4 + 15) / 16 * 16 : 0;
-    static constexpr int TOTAL = CTA_BYTES + MLP_WARPS * PER_WARP;
+    static constexpr int WARPS = mlp_warps(BWD), THREADS = 32 * WARPS, TOTAL = CTA_BYTES + WARPS * PER_WARP;
 };
 
-// resident CTAs per SM the kernel is compiled for (register budget) and launched with (persistent grid)
-template <int FQ, bool BWD> __host__ __device__ constexpr int mlp_ctas_per_sm() { return BWD ? (FQ <= 2 ? 4 : 3) : (FQ <= 2 ? 5 : 4); }
+// resident warps per SM the kernel is compiled for (register budget)
+template <int FQ, bool BWD> __host__ __device__ constexpr int mlp_warps_per_sm() { return BWD ? (FQ <= 2 ? 16 : 12) : (FQ <= 2 ? 20 : 16); }
 
 // Sums v[0..NV) over the L lanes of an aligned group by a halving exchange; afterwards lane l holds, in v[0..NV / min(NV, L)),
 // the totals of the entries from spread_first<NV, L>(l).
@@ -73,7 +76,7 @@ static __device__ __forceinline__ int spread_first(const int l) {
 }
 
 template <int HID, int FQ, bool BWD, bool MI>
-__global__ void __launch_bounds__(MLP_THREADS, (mlp_ctas_per_sm<FQ, BWD>())) radius_mlp_kernel(const __grid_constant__ RadiusParams p) {
+__global__ void __launch_bounds__(32 * mlp_warps(BWD), (mlp_warps_per_sm<FQ, BWD>() / mlp_warps(BWD))) radius_mlp_kernel(const __grid_constant__ RadiusParams p) {
     using SM = MlpSmem<HID, FQ, BWD>;
     constexpr int STAGE_CAP = SM::STAGE_CAP, LIST_CAP = SM::LIST_CAP, NX = SM::NX, KP = SM::K_PAD;
     constexpr int PS = 32 / HID;                       // pairs evaluated together
@@ -85,7 +88,7 @@ __global__ void __launch_bounds__(MLP_THREADS, (mlp_ctas_per_sm<FQ, BWD>())) rad
 
     float* sG = reinterpret_cast<float*>(s_raw);       // BWD: W1 [HID][KP], b1 [HID], W2 [4][HID], b2 [4]
     if constexpr (BWD) {
-        for (int e = threadIdx.x; e < SM::GRAD_FLOATS; e += MLP_THREADS) sG[e] = 0.f;
+        for (int e = threadIdx.x; e < SM::GRAD_FLOATS; e += SM::THREADS) sG[e] = 0.f;
         __syncthreads();
     }
     unsigned char* base = s_raw + SM::CTA_BYTES + (size_t)wib * SM::PER_WARP;
@@ -211,29 +214,50 @@ __global__ void __launch_bounds__(MLP_THREADS, (mlp_ctas_per_sm<FQ, BWD>())) rad
 #pragma unroll
                             for (int o = 0; o < 4; ++o) gq[o] = o < Fout ? __ldg(p.gy + (size_t)oq * Fout + o) : 0.f;
                         }
-#pragma unroll 2
-                        for (int t = off + ps; t < end; t += PS) {
-                            const float4 e = list[t];
-                            const int slot = __float_as_int(e.w);
-                            if (slot < 0) continue;
-                            float h = fmaf(w[2], e.z, fmaf(w[1], e.y, fmaf(w[0], e.x, b1)));
-                            const float4* xr = reinterpret_cast<const float4*>(s_x + slot * NX);
+                        for (int t = off + ps; t < end; t += 2 * PS) {
+                            // two pairs side by side (their chains are independent); an absent or refused one adds nothing
+                            const bool two = t + PS < end;
+                            const float4 e[2] = {list[t], list[two ? t + PS : t]};
+                            const int slot[2] = {__float_as_int(e[0].w), __float_as_int(e[1].w)};
+                            const bool in[2] = {slot[0] >= 0, two && slot[1] >= 0};
+                            float h[2];
+                            const float4* xr[2];
+#pragma unroll
+                            for (int u = 0; u < 2; ++u) {
+                                xr[u] = reinterpret_cast<const float4*>(s_x + (slot[u] < 0 ? 0 : slot[u]) * NX);
+                                h[u] = fmaf(w[2], e[u].z, fmaf(w[1], e[u].y, fmaf(w[0], e[u].x, b1)));
+                            }
 #pragma unroll
                             for (int i = 0; i < FQ; ++i) {
-                                const float4 x4 = xr[i];
-                                h = fmaf(w[3 + 4 * i], x4.x, h); h = fmaf(w[4 + 4 * i], x4.y, h);
-                                h = fmaf(w[5 + 4 * i], x4.z, h); h = fmaf(w[6 + 4 * i], x4.w, h);
-                            }
-                            S += fmaxf(h, 0.f);
-                            if constexpr (BWD) {
-                                // the pair the other way round: the query as the source
-                                float h2 = fmaf(w[2], -e.z, fmaf(w[1], -e.y, fmaf(w[0], -e.x, b1)));
 #pragma unroll
-                                for (int f = 0; f < NX; ++f) h2 = fmaf(w[3 + f], xq[f], h2);
-                                const float4 g4 = s_g[slot];
-                                const float vm = fmaf(w2[3], g4.w, fmaf(w2[2], g4.z, fmaf(w2[1], g4.y, w2[0] * g4.x)));
-                                if (h > 0.f) { cpos += 1.f; D0 += e.x; D1 += e.y; D2 += e.z; }
-                                if (h2 > 0.f) G += vm;
+                                for (int u = 0; u < 2; ++u) {
+                                    const float4 x4 = xr[u][i];
+                                    h[u] = fmaf(w[3 + 4 * i], x4.x, h[u]); h[u] = fmaf(w[4 + 4 * i], x4.y, h[u]);
+                                    h[u] = fmaf(w[5 + 4 * i], x4.z, h[u]); h[u] = fmaf(w[6 + 4 * i], x4.w, h[u]);
+                                }
+                            }
+                            if constexpr (BWD) {
+                                // the pairs the other way round: the query as the source
+                                float h2[2], vm[2];
+#pragma unroll
+                                for (int u = 0; u < 2; ++u) {
+                                    h2[u] = fmaf(w[2], -e[u].z, fmaf(w[1], -e[u].y, fmaf(w[0], -e[u].x, b1)));
+                                    const float4 g4 = s_g[slot[u] < 0 ? 0 : slot[u]];
+                                    vm[u] = fmaf(w2[3], g4.w, fmaf(w2[2], g4.z, fmaf(w2[1], g4.y, w2[0] * g4.x)));
+                                }
+#pragma unroll
+                                for (int f = 0; f < NX; ++f) {
+#pragma unroll
+                                    for (int u = 0; u < 2; ++u) h2[u] = fmaf(w[3 + f], xq[f], h2[u]);
+                                }
+#pragma unroll
+                                for (int u = 0; u < 2; ++u) {
+                                    if (in[u] && h[u] > 0.f) { S += h[u]; cpos += 1.f; D0 += e[u].x; D1 += e[u].y; D2 += e[u].z; }
+                                    if (in[u] && h2[u] > 0.f) G += vm[u];
+                                }
+                            } else {
+#pragma unroll
+                                for (int u = 0; u < 2; ++u) S += in[u] ? fmaxf(h[u], 0.f) : 0.f;
                             }
                         }
                         // sums over the groups of HID lanes
@@ -358,8 +382,18 @@ __global__ void __launch_bounds__(MLP_THREADS, (mlp_ctas_per_sm<FQ, BWD>())) rad
             k0 += 32 * SU;
         }
     };
-    const int units = (p.n + p.unit - 1) / p.unit;
-    for (int u = blockIdx.x * MLP_WARPS + wib; u < units; u += gridDim.x * MLP_WARPS) walk_unit(p, u, p.run, slice);
+    if constexpr (!BWD) {
+        walk_unit(p, blockIdx.x, p.run, slice);
+    } else {
+        const int units = (p.n + p.unit - 1) / p.unit;
+        for (;;) {
+            int u = 0;
+            if (lane == 0) u = atomicAdd(p.ticket, 1);
+            u = __shfl_sync(FULL, u, 0);
+            if (u >= units) break;
+            walk_unit(p, u, p.run, slice);
+        }
+    }
 
     if constexpr (BWD) {
         // warps -> CTA copy in shared memory -> one atomic per parameter entry and CTA
@@ -376,18 +410,19 @@ __global__ void __launch_bounds__(MLP_THREADS, (mlp_ctas_per_sm<FQ, BWD>())) rad
         }
         if (lane < 4) atomicAdd(gb2s + lane, gb2);
         __syncthreads();
-        for (int e = threadIdx.x; e < HID * KP; e += MLP_THREADS) {
+        for (int e = threadIdx.x; e < HID * KP; e += SM::THREADS) {
             const int i = e / KP, k = e % KP;
             if (k < K && p.gW1) atomicAdd(p.gW1 + i * K + k, gW1s[e]);
         }
-        for (int e = threadIdx.x; e < HID; e += MLP_THREADS) if (p.gb1) atomicAdd(p.gb1 + e, gb1s[e]);
-        for (int e = threadIdx.x; e < Fout * HID; e += MLP_THREADS) if (p.gW2) atomicAdd(p.gW2 + e, gW2s[e]);
+        for (int e = threadIdx.x; e < HID; e += SM::THREADS) if (p.gb1) atomicAdd(p.gb1 + e, gb1s[e]);
+        for (int e = threadIdx.x; e < Fout * HID; e += SM::THREADS) if (p.gW2) atomicAdd(p.gW2 + e, gW2s[e]);
         if (threadIdx.x < Fout && p.gb2) atomicAdd(p.gb2 + threadIdx.x, gb2s[threadIdx.x]);
     }
 }
 
-// parameter gradients start from zero (one launch for the four arrays)
-__global__ void mlp_zero_kernel(float* a, int na, float* b, int nb, float* c, int nc, float* d, int nd) {
+// parameter gradients and the unit counter start from zero (one launch)
+__global__ void mlp_zero_kernel(int* ticket, float* a, int na, float* b, int nb, float* c, int nc, float* d, int nd) {
+    if (threadIdx.x == 0) *ticket = 0;
     for (int k = threadIdx.x; k < na; k += blockDim.x) a[k] = 0.f;
     for (int k = threadIdx.x; k < nb; k += blockDim.x) b[k] = 0.f;
     for (int k = threadIdx.x; k < nc; k += blockDim.x) c[k] = 0.f;
@@ -399,8 +434,8 @@ static tiga_status launch_mlp_t(const RadiusParams& p, cudaStream_t s) {
     using SM = MlpSmem<HID, FQ, BWD>;
     auto kern = radius_mlp_kernel<HID, FQ, BWD, MI>;
     if (SM::TOTAL > 48 * 1024) TIGA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SM::TOTAL));
-    const unsigned need = (unit_count(p) + MLP_WARPS - 1) / MLP_WARPS, cap = 148u * mlp_ctas_per_sm<FQ, BWD>();       // persistent: parameter gradients are folded once per CTA
-    kern<<<counted(need < cap ? need : cap), MLP_THREADS, SM::TOTAL, s>>>(p);
+    const unsigned need = (unit_count(p) + SM::WARPS - 1) / SM::WARPS, cap = 148u * mlp_warps_per_sm<FQ, BWD>() / SM::WARPS;
+    kern<<<counted(BWD && need > cap ? cap : need), SM::THREADS, SM::TOTAL, s>>>(p);
     return launch_status();
 }
 
@@ -433,6 +468,7 @@ static tiga_status mlp_common(RadiusParams* p, const float* pos, const float* fe
     if (st != TIGA_OK) return st;
     if (n > 0 && (!pos || !aligned16(pos) || !feat || !aligned16(feat))) return TIGA_ERR_INVALID_ARG;
     if (!ws || !aligned16(ws) || ws_bytes < tiga_radius_workspace_bytes(n, mlp->f_in, r, box, 0)) return TIGA_ERR_WORKSPACE;
+    cut_cells(*p, 148 * 84);             // a query costs more here: finer slices
     *lay = carve_radius(p, ws, fill);
     p->pos = pos; p->feat = feat; p->F = mlp->f_in; p->Fin = mlp->f_in; p->Fout = mlp->f_out;
     p->W1 = mlp->W1; p->b1 = mlp->b1; p->W2 = mlp->W2; p->b2 = mlp->b2;
@@ -472,11 +508,9 @@ extern "C" tiga_status tiga_apply_radius_mlp_backward(const float* pos, const fl
     if (st != TIGA_OK) return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int K = 3 + mlp->f_in;
-    if (grad_W1 || grad_b1 || grad_W2 || grad_b2) {
-        mlp_zero_kernel<<<counted(1), 256, 0, s>>>(grad_W1, grad_W1 ? mlp->hidden * K : 0, grad_b1, grad_b1 ? mlp->hidden : 0,
-                                                   grad_W2, grad_W2 ? mlp->f_out * mlp->hidden : 0, grad_b2, grad_b2 ? mlp->f_out : 0);
-        if (launch_status() != TIGA_OK) return TIGA_ERR_CUDA;
-    }
+    mlp_zero_kernel<<<counted(1), 256, 0, s>>>(p.ticket, grad_W1, grad_W1 ? mlp->hidden * K : 0, grad_b1, grad_b1 ? mlp->hidden : 0,
+                                               grad_W2, grad_W2 ? mlp->f_out * mlp->hidden : 0, grad_b2, grad_b2 ? mlp->f_out : 0);
+    if (launch_status() != TIGA_OK) return TIGA_ERR_CUDA;
     if (n == 0) return TIGA_OK;
     if (!grad_out || !aligned16(grad_out)) return TIGA_ERR_INVALID_ARG;
     p.gy = grad_out; p.gfeat = grad_feat; p.gpos = grad_pos;

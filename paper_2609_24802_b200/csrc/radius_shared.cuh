@@ -13,8 +13,8 @@ constexpr int TRAV_THREADS = TRAV_WARPS * 32;
 constexpr int STAGE_PAD = 32;           // sentinels behind the staged candidates: no bounds checks
 constexpr int QB = 8;                   // queries per batch (kernels that run faster with four define their own width)
 constexpr float FAR_AWAY = 1.0e18f;
-constexpr int QDENSE = 64;              // a cell with more points than this is cut into slices
-constexpr int QSLICE = 16;              // of this many queries
+constexpr int QSLICE = 16;              // most queries of a slice of a dense cell (cut_cells)
+constexpr int QDENSE = QSLICE + QSLICE / 2;   // most queries of one piece of work
 constexpr int UNIT_MAX = 32;            // most points per unit of work (at most 32: a lane each)
 constexpr int RUN_CELLS = 8;            // longest run of cells along x that one warp covers
 constexpr int RUN_QUERIES = 16;         // points a warp joins cells for
@@ -57,6 +57,7 @@ struct RadiusParams {
     int run;                  // cells along x that a warp joins at most
     int unit;                 // points per warp (walk_unit)
     int dense, slice;         // a cell with more than `dense` points is cut into slices of `slice` queries
+    int* ticket;              // unit counter of the edge network's backward (zeroed by that call)
     int32_t* b_items;         // cells with more than SORT_DENSE points (queued by the scan), and how many
     int* b_count;
     // optional user copies of the plan
@@ -144,6 +145,14 @@ static __device__ __forceinline__ void walk_unit(const RadiusParams& p, const in
         work(cell, last - first + 1, qs, end & 0x7fffffff);
         __syncwarp();
     }
+}
+
+// Slices of four to QSLICE queries, so that there are about `warps` of them before a slice grows; a cell is cut when that
+// gives at least two.
+static inline void cut_cells(RadiusParams& p, long long warps) {
+    const long long want = (p.n / warps + 3) / 4 * 4;
+    p.slice = (int)(want < 4 ? 4 : want < QSLICE ? want : QSLICE);
+    p.dense = p.slice + p.slice / 2;
 }
 
 static inline unsigned unit_count(const RadiusParams& p) { return (unsigned)(((long long)p.n + p.unit - 1) / p.unit); }
