@@ -218,6 +218,10 @@ __global__ void __launch_bounds__(CSR_THREADS, 5) csr_forward_kernel(const CsrPa
                     float xf[VW];
 #pragma unroll
                     for (int i = 0; i < VPL; ++i) {
+                        if constexpr (RED == 0 && sizeof(XT) == 2) {
+                            // unit weights: mixed-precision adds, no conversion
+                            if (!p.w) { XTraits<XT>::add_to(xv[u][i], &st.v[i][0]); continue; }
+                        }
                         XTraits<XT>::unpack(xv[u][i], xf);
                         if constexpr (PACKED) {
 #pragma unroll
@@ -626,12 +630,22 @@ __global__ void csr_huge_fold_kernel(const CsrParams p) {
         using AT = ArgT<RED>;
         const AT* carg = static_cast<const AT*>(p.carry_arg);
         AT a = RED ? carg[(size_t)idx * p.F + f] : AT(0);
-        for (int c = 1; c < ent.z; ++c) {
-            const float ov = p.carry_val[(size_t)(idx + c) * p.F + f];
-            if (RED == 0) v += ov;
-            else {
-                const AT oa = carg[(size_t)(idx + c) * p.F + f];
-                if (oa >= 0 && (a < 0 || ov > v)) { v = ov; a = oa; }
+        // eight chunk states are requested at a time (one by one the longest row's chain of loads set the time of the
+        // launch)
+        for (int c0 = 1; c0 < ent.z; c0 += 8) {
+            float ov[8];
+            AT oa[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const size_t at = (size_t)(idx + (c0 + k < ent.z ? c0 + k : 0)) * p.F + f;
+                ov[k] = p.carry_val[at];
+                oa[k] = RED ? carg[at] : AT(0);
+            }
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                if (c0 + k >= ent.z) break;
+                if (RED == 0) v += ov[k];
+                else if (oa[k] >= 0 && (a < 0 || ov[k] > v)) { v = ov[k]; a = oa[k]; }
             }
         }
         p.out[(size_t)ent.x * p.F + f] = v;
@@ -654,13 +668,26 @@ __global__ void csr_fixup_kernel(const CsrParams p) {
     using AT = ArgT<RED>;
     const AT* carg = static_cast<const AT*>(p.carry_arg);
     AT a = RED ? carg[tile * p.F + f] : AT(0);
-    for (long long u = tile + 1; u < p.ntiles && p.carry_row[u] == row; ++u) {
-        const float ov = p.carry_val[u * p.F + f];
-        if (RED == 0) v += ov;
-        else {
-            const AT oa = carg[u * p.F + f];
-            if (oa >= 0 && (a < 0 || ov > v)) { v = ov; a = oa; }
+    for (long long u0 = tile + 1; u0 < p.ntiles; u0 += 8) {      // eight carry-outs are requested at a time
+        int rr[8];
+        float ov[8];
+        AT oa[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const long long u = u0 + k < p.ntiles ? u0 + k : p.ntiles - 1;
+            rr[k] = u0 + k < p.ntiles ? p.carry_row[u] : -1;
+            ov[k] = p.carry_val[u * p.F + f];
+            oa[k] = RED ? carg[u * p.F + f] : AT(0);
         }
+        bool more = true;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            more = more && rr[k] == row;
+            if (!more) continue;
+            if (RED == 0) v += ov[k];
+            else if (oa[k] >= 0 && (a < 0 || ov[k] > v)) { v = ov[k]; a = oa[k]; }
+        }
+        if (!more) break;
     }
     const size_t o = (size_t)row * p.F + f;
     if (RED == 0) {

@@ -29,7 +29,7 @@
 // through the general form, a bitonic network of shuffles over 32 keys at a time and merges, which orders
 // whole keys.  (Sorting every list took 225 of 520 warp instructions per query at k = 16, counting takes about 90; a
 // full list is trimmed for 60 instructions where sorting it took 500.)
-#include "radius_shared.cuh"
+#include "radius_test.cuh"
 #include <type_traits>
 
 namespace tiga {
@@ -43,7 +43,7 @@ constexpr int KNN_COUNT_K = 24;                    // largest k that counting se
 constexpr int KNN_RING_CAP = 128;                  // list entries of the rings kernel
 constexpr int KNN_STAGE_BYTES = (KNN_STAGE_CAP + STAGE_PAD) * 16;
 constexpr int KNN_LIST_BYTES = (KQB * KNN_QSTRIDE * 8 + 15) / 16 * 16;
-constexpr int KNN_MISC_BYTES = KQB * 16 + KQB * 4 * 2;
+constexpr int KNN_MISC_BYTES = KQB * 16 + KQB * 4 * 2 + 80;     // queries, list lengths, thresholds, range offsets of the stencil
 constexpr int KNN_PER_WARP = KNN_STAGE_BYTES + KNN_LIST_BYTES + KNN_MISC_BYTES;
 static_assert(KNN_PER_WARP % 16 == 0 && KNN_LIST_BYTES % 16 == 0, "the stage and the queries are accessed as 16-byte vectors");
 constexpr int RING_WARPS = 4, RING_THREADS = 32 * RING_WARPS;
@@ -63,7 +63,6 @@ struct KnnParams {
     int32_t* nbr;
     float* nbr_d2;
     int32_t* queue;         // queries the cells kernel could not finish
-    int32_t* queue_n;
 };
 
 // the key's squared distance: operation order fixed, nothing contracted
@@ -257,24 +256,10 @@ __device__ __forceinline__ void knn_cell_slice(const KnnParams& P, const int (&c
     const unsigned lt_mask = (1u << lane) - 1u;
     const int k = P.k;
 
-    // ---- the stencil as nine runs of the cell-ordered points: the x neighbours are contiguous
-    int r_cs = 0, r_len = 0;
-    {
-        const int y = c[1] + lane % 3 - 1, z = c[2] + lane / 3 - 1;
-        if (lane < 9 && y >= 0 && y < p.nc[1] && z >= 0 && z < p.nc[2]) {
-            const int x0 = c[0] > 0 ? c[0] - 1 : 0, x1 = c[0] + 1 < p.nc[0] ? c[0] + 1 : p.nc[0] - 1;
-            const int id0 = (z * p.nc[1] + y) * p.nc[0] + x0;
-            r_cs = p.cell_start[id0];
-            r_len = p.cell_start[id0 + (x1 - x0 + 1)] - r_cs;
-        }
-    }
-    int r_incl = r_len;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(FULL, r_incl, o);
-        if (lane >= o) r_incl += v;
-    }
-    const int total = __shfl_sync(FULL, r_incl, 31);
+    // ---- the stencil as nine ranges of the cell-ordered points: the x neighbours are contiguous
+    int* s_delta = reinterpret_cast<int*>(s_tau + KQB);
+    const RunStencil sten(p, c, 1, s_delta);
+    const int total = sten.total;
 
     // ---- bounding box of the cell's points, one register per lane (lane d: low, lane 3 + d: high)
     float bb;
@@ -287,43 +272,47 @@ __device__ __forceinline__ void knn_cell_slice(const KnnParams& P, const int (&c
             blo[2] = fminf(blo[2], pq.z); bhi[2] = fmaxf(bhi[2], pq.z);
         }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                blo[d] = fminf(blo[d], __shfl_xor_sync(FULL, blo[d], o));
-                bhi[d] = fmaxf(bhi[d], __shfl_xor_sync(FULL, bhi[d], o));
-            }
+        for (int d = 0; d < 3; ++d) { blo[d] = warp_min(blo[d]); bhi[d] = warp_max(bhi[d]); }
         bb = lane == 0 ? blo[0] : lane == 1 ? blo[1] : lane == 2 ? blo[2] : lane == 3 ? bhi[0] : lane == 4 ? bhi[1] : bhi[2];
     }
 
-    // ---- stages kept candidates starting at flattened stencil position v0 until the stage is
-    //      full or the stencil ends; returns the next position, the kept count in ns
-    auto stage_from = [&](int v0, int& ns) -> int {
+    // ---- stages kept candidates starting at flattened stencil position v0 until the next step might not fit or the stencil
+    //      ends; returns the next position, the kept count in ns.  `before` counts the ranges that began before v0 (-1 at 0).
+    auto stage_from = [&](int v0, int& before, int& ns) -> int {
+        constexpr int SU = 4;                                 // groups of 32 candidates in flight
+        static_assert(KNN_STAGE_CAP >= 32 * SU, "a step fits an empty stage");
         int nst = 0;
-        for (; v0 < total && nst <= KNN_STAGE_CAP - 32; v0 += 32) {
-            const int v = v0 + lane;
-            int r = 0;
+        while (v0 < total) {
+            const int step = total - v0 < 32 * SU ? total - v0 : 32 * SU, before0 = before;
+            float4 c4[SU];
+            unsigned kept[SU];
 #pragma unroll
-            for (int o = 8; o > 0; o >>= 1) {                 // nine runs: a four-step search
-                const int probe = __shfl_sync(FULL, r_incl, r + o - 1);
-                if (probe <= v) r += o;
+            for (int u = 0; u < SU; ++u) {                    // all loads of the step first
+                c4[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (32 * u >= step) continue;
+                const int src = sten.source(v0 + 32 * u, before, s_delta);
+                if (v0 + 32 * u + lane < total) c4[u] = __ldg(p.spos + checked(src, p.n, CHECK_SLOT));
             }
-            r = r > 8 ? 8 : r;
-            const int src = __shfl_sync(FULL, r_cs, r) + (v - (__shfl_sync(FULL, r_incl, r) - __shfl_sync(FULL, r_len, r)));
             const float lx = __shfl_sync(FULL, bb, 0), ly = __shfl_sync(FULL, bb, 1), lz = __shfl_sync(FULL, bb, 2);
             const float hx = __shfl_sync(FULL, bb, 3), hy = __shfl_sync(FULL, bb, 4), hz = __shfl_sync(FULL, bb, 5);
-            bool keep = false;
-            float4 c4 = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (v < total) {
-                c4 = __ldg(p.spos + checked(src, p.n, CHECK_SLOT));
-                const float ex = fmaxf(fmaxf(lx - c4.x, c4.x - hx), 0.f);
-                const float ey = fmaxf(fmaxf(ly - c4.y, c4.y - hy), 0.f);
-                const float ez = fmaxf(fmaxf(lz - c4.z, c4.z - hz), 0.f);
-                keep = fmaf(ez, ez, fmaf(ey, ey, ex * ex)) <= P.prune2;
+            int all = nst;
+#pragma unroll
+            for (int u = 0; u < SU; ++u) {
+                kept[u] = 0u;
+                if (32 * u >= step) continue;
+                const float ex = fmaxf(fmaxf(lx - c4[u].x, c4[u].x - hx), 0.f);
+                const float ey = fmaxf(fmaxf(ly - c4[u].y, c4[u].y - hy), 0.f);
+                const float ez = fmaxf(fmaxf(lz - c4[u].z, c4[u].z - hz), 0.f);
+                kept[u] = __ballot_sync(FULL, v0 + 32 * u + lane < total && fmaf(ez, ez, fmaf(ey, ey, ex * ex)) <= P.prune2);
+                all += __popc(kept[u]);
             }
-            const unsigned m = __ballot_sync(FULL, keep);
-            if (keep) stage[nst + __popc(m & lt_mask)] = c4;
-            nst += __popc(m);
+            if (all > KNN_STAGE_CAP) { before = before0; break; }     // taken again with an empty stage
+#pragma unroll
+            for (int u = 0; u < SU; ++u) {
+                if ((kept[u] >> lane) & 1u) stage[nst + __popc(kept[u] & lt_mask)] = c4[u];
+                nst += __popc(kept[u]);
+            }
+            v0 += 32 * SU;
         }
         if (lane < STAGE_PAD) stage[nst + lane] = make_float4(FAR_AWAY, FAR_AWAY, FAR_AWAY, __int_as_float(-1));
         __syncwarp();
@@ -331,8 +320,8 @@ __device__ __forceinline__ void knn_cell_slice(const KnnParams& P, const int (&c
         return v0;
     };
 
-    int ns = 0;
-    const bool single = stage_from(0, ns) >= total;           // the whole (pruned) stencil fits: staged once
+    int ns = 0, before = -1;
+    const bool single = stage_from(0, before, ns) >= total;           // the whole (pruned) stencil fits: staged once
 
     for (int qb0 = qs0; qb0 < qe0; qb0 += KQB) {
         const int nq = (qe0 - qb0 < KQB) ? qe0 - qb0 : KQB;
@@ -403,9 +392,10 @@ __device__ __forceinline__ void knn_cell_slice(const KnnParams& P, const int (&c
             if (nq <= KQB / 2) scan(ns, std::integral_constant<int, KQB / 2>{});
             else scan(ns, std::integral_constant<int, KQB>{});
         } else {
+            before = -1;
             for (int v = 0; v < total;) {
                 int ns2;
-                v = stage_from(v, ns2);
+                v = stage_from(v, before, ns2);
                 scan(ns2, std::integral_constant<int, KQB>{});
                 __syncwarp();
             }
@@ -422,7 +412,7 @@ __device__ __forceinline__ void knn_cell_slice(const KnnParams& P, const int (&c
             const int n = s_n[q];
             const int i = __float_as_int(s_q[q].w);
             if (n < k) {
-                if (lane == 0) P.queue[atomicAdd(P.queue_n, 1)] = i;
+                if (lane == 0) P.queue[atomicAdd(p.queue_n, 1)] = i;
             } else {
                 select_and_emit(P, i, list + q * KNN_QSTRIDE, n, s_tau[q], lane);
             }
@@ -448,7 +438,7 @@ __global__ void __launch_bounds__(RING_THREADS) knn_rings_kernel(const __grid_co
     float2* list = s_list[wib];
     const unsigned lt_mask = (1u << lane) - 1u;
     const int k = P.k;
-    const int nqueue = *P.queue_n;
+    const int nqueue = *p.queue_n;
     const int nwarps = gridDim.x * RING_WARPS;
     const int nx = p.nc[0], ny = p.nc[1], nz = p.nc[2];
     const int smax = max(nx, max(ny, nz));
@@ -574,7 +564,6 @@ static size_t knn_carve(KnnParams* P, void* ws, int32_t** fill, RadiusLayout* la
     Carver cv(ws);
     cv.off = lay->bytes;
     P->queue = cv.take<int32_t>((size_t)P->rp.n + 1);
-    P->queue_n = cv.take<int32_t>(64);
     return cv.off;
 }
 
@@ -617,7 +606,6 @@ extern "C" tiga_status tiga_apply_knn(const float* pos, const float* feat, int64
     P.hmin = hmin * (1.f - 1.f / 1024.f);
     P.out = out; P.nbr = nbr; P.nbr_d2 = nbr_d2;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    TIGA_CUDA_TRY(cudaMemsetAsync(P.queue_n, 0, sizeof(int32_t), s));
     st = run_binning(P.rp, fill, lay.nblocks, s);
     if (st != TIGA_OK) return st;
     constexpr int smem = KNN_PER_WARP * TRAV_WARPS;

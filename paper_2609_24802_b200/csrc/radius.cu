@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(SMALL_THREADS) bin_small_kernel(const RadiusPa
     constexpr int PP = SMALL_POINTS / SMALL_THREADS, PC = SMALL_CELLS / SMALL_THREADS;
     const int tid = threadIdx.x;
     for (int k = tid; k < p.ncells; k += SMALL_THREADS) s_start[k] = 0;
-    if (tid == 0) s_ndense = 0;
+    if (tid == 0) { s_ndense = 0; *p.queue_n = 0; }
     __syncthreads();
     float v[PP][3];
     int c[PP], slot[PP];
@@ -768,6 +768,7 @@ RadiusLayout carve_radius(RadiusParams* p, void* ws, int32_t** fill) {
     p->cnt = cv.take<int32_t>(2 * nc + 2 + 16);     // counts, then the scatter cursors, then the length of the dense-cell queue
     p->b_count = p->cnt + 2 * nc + 2;
     p->ticket = p->b_count + 1;
+    p->queue_n = p->b_count + 2;
     *fill = p->cnt + nc;
     p->cell = cv.take<int32_t>(n);
     p->cell_start = cv.take<int32_t>(nc + 1);

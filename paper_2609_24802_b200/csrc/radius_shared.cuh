@@ -57,6 +57,7 @@ struct RadiusParams {
     int run;                  // cells along x that a warp joins at most
     int unit;                 // points per warp (walk_unit)
     int dense, slice;         // a cell with more than `dense` points is cut into slices of `slice` queries
+    int* queue_n;             // length of the kNN queue (zeroed with the counts)
     int* ticket;              // unit counter of the edge network's backward (zeroed by that call)
     int32_t* b_items;         // cells with more than SORT_DENSE points (queued by the scan), and how many
     int* b_count;
@@ -182,16 +183,6 @@ static __device__ __forceinline__ float warp_max(float v) {
     asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
     return r;
 }
-
-// two fp32 values per register pair: sm_100 executes add / mul / fma on both with one instruction
-typedef unsigned long long f32x2;
-static __device__ __forceinline__ f32x2 pack2(float a, float b) { f32x2 r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b)); return r; }
-static __device__ __forceinline__ void unpack2(f32x2 v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
-static __device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) { f32x2 r; asm("sub.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
-static __device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) { f32x2 r; asm("add.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
-static __device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) { f32x2 r; asm("mul.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
-static __device__ __forceinline__ f32x2 dup2(float a) { return pack2(a, a); }
-static __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) { f32x2 r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
 
 // Minimum-image displacement of two coordinates of a periodic dimension that is not split into enough
 // cells for a frame shift: the subtraction that can lose bits (x near 0 against x near len) is replaced
