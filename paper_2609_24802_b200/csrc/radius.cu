@@ -172,14 +172,17 @@ __global__ void __launch_bounds__(256) bin_sort_kernel(const RadiusParams p, con
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= p.n) return;
     const int id = p.order_tmp[t];
-    const int c = p.cell[id];
+    // the cell follows from the position, which is gathered anyway (with a gather of p.cell[id] as well:
+    // 1 M points 17.0 instead of 13.7 us, 4.1 M 59 instead of 53 us)
+    const float x = p.pos[3 * (size_t)id], y = p.pos[3 * (size_t)id + 1], z = p.pos[3 * (size_t)id + 2];
+    const int c = (cell_coordinate(p, z, 2) * p.nc[1] + cell_coordinate(p, y, 1)) * p.nc[0] + cell_coordinate(p, x, 0);
     const int s = p.cell_start[c], e = p.cell_start[c + 1];
     if (e - s > SORT_DENSE) return;        // sort_dense_cells orders this cell
     int rank = 0;
     for (int u = s; u < e; ++u) rank += (p.order_tmp[u] < id) ? 1 : 0;
     p.order[s + rank] = id;
     if (p.u_order) p.u_order[s + rank] = id;
-    p.spos[s + rank] = make_float4(p.pos[3 * (size_t)id], p.pos[3 * (size_t)id + 1], p.pos[3 * (size_t)id + 2], __int_as_float(id));
+    p.spos[s + rank] = make_float4(x, y, z, __int_as_float(id));
 }
 
 // Cells with more than SORT_DENSE points (rank counting is quadratic in the occupancy): one CTA per
@@ -719,11 +722,11 @@ __global__ void __launch_bounds__(TRAV_THREADS, (MODE == 0 ? 28 : 16) / TRAV_WAR
 // lanes would leave most of the warp idle on such rows, so nothing is gathered: the features are staged with
 // the candidates and summed where a pair is accepted (radius_direct.cuh).
 // Bound by instruction issue and by the latency of the staging loads.  Against the list kernel below four features:
-// F = 3, n = 1M, 32 neighbours 754 -> 405 us; F = 1, n = 131072, distance-weighted 108 -> 53 us; F = 4, n = 434630,
-// 4 neighbours (sparse cells, runs of eight) 518 -> 126 us.
+// F = 4, n = 1M, 32 neighbours 616 -> 393 us; F = 1, n = 131072, distance-weighted 108 -> 58 us; F = 2, n = 300k,
+// 8 neighbours 218 -> 100 us.  Warps per SM measured: F = 1 28 / 24 / 20: 57 / 61 / 65 us; F = 3 401 / 394 / 381 us.
 template <int NF, bool DIST>
 struct SumMsg {
-    static constexpr int CAP = 256, STAGED = NF, OUT = NF, WARPS = 24;
+    static constexpr int CAP = 256, STAGED = NF, OUT = NF, WARPS = NF <= 2 ? 28 : 20;
     static constexpr float OUTSIDE = DIST ? 0.f : 1.0e30f;
     float neg_c2;
     // exp(-d2/(2 s^2)) = 2^(d2 * neg_c2)

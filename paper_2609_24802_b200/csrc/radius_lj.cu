@@ -4,14 +4,14 @@
 // Every row walks its full neighbourhood, which forms each unordered pair twice but needs no atomics, no memset and no
 // list, and is reproducible.  Bound by instruction issue (75 % of the slots): per cell of 12.6 particles 1430 warp
 // instructions stage 340 candidates (195 survive the pruning), 760 test them, 1280 form the forces, 300 add up and store.
-// 4.1 M particles 1467 -> 1385 us against the earlier form (every unordered pair once through per-query lists, the
-// opposite force added with a vector atomic); eight CTAs per SM measured fastest (six 1451, seven 1398 us).
+// 4.1 M particles 1467 -> 1321 us against the earlier form (every unordered pair once through per-query lists, the
+// opposite force added with a vector atomic); 28 warps per SM measured fastest (24 1350, 32 1343 us).
 #include "radius_direct.cuh"
 
 namespace tiga {
 
 struct LjMsg {
-    static constexpr int CAP = 256, STAGED = 0, OUT = 4, WARPS = 32;
+    static constexpr int CAP = 256, STAGED = 0, OUT = 4, WARPS = 28;
     static constexpr float OUTSIDE = 1.0e30f;
     float s2, force, energy;
     __device__ __forceinline__ explicit LjMsg(const RadiusParams& p) : s2(p.p1 * p.p1), force(24.f * p.p0), energy(2.f * p.p0) {}
