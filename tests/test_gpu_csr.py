@@ -407,3 +407,20 @@ def test_row_gather_probe_runs_and_checks_its_arguments(tiga):
         bench_probe.row_gather(torch.randn((16, 3), device="cuda"), idx[:4] % 16, sink)      # 12-byte rows
     with pytest.raises(ValueError, match="status 2"):
         bench_probe.row_gather(torch.randn((16, 12), device="cuda"), idx[:4] % 16, sink)     # 48-byte rows: not a power of two
+
+
+@pytest.mark.parametrize("items", [255, 256, 257, 592 * 256 - 1, 592 * 256 + 1, 592 * 512 + 600])
+def test_tile_lengths_of_small_relations(tiga, items):
+    """Tiles have 256, 512, ... items by the relation's size: sizes on both sides of the steps, with one row across
+    many tiles (more than the eight carry-outs that are folded at a time), empty rows and short ones."""
+    n = max(items // 9, 20)
+    E = items - n
+    rng = np.random.default_rng(items)
+    deg = np.zeros(n, np.int64)
+    deg[n // 2] = E // 3
+    np.add.at(deg, rng.integers(0, n, E - E // 3), 1)
+    rowptr = np.concatenate([[0], np.cumsum(deg)])
+    col = rng.integers(0, n, E).astype(np.int32)
+    x, w, gy = gen.normal_features(n, 12, 5, 31), gen.edge_weights(E, 6), gen.normal_features(n, 12, 5, 32)
+    g, xd, wd, res = _check_forward(tiga, rowptr, col, x, w)
+    _check_backward(tiga, rowptr, col, x, w, gy, g, xd, wd, res)

@@ -148,3 +148,19 @@ def test_paper_size_131072_points(tiga):
     assert nb.min() >= 0 and np.all(nb != np.arange(n)[:, None])
     assert np.all(np.sort(nb, 1)[:, 1:] != np.sort(nb, 1)[:, :-1])          # k distinct neighbours per row
     assert np.allclose(host(out)[:, 0], x[nb, 0].sum(1), rtol=1e-4, atol=1e-4)
+
+
+@pytest.mark.parametrize("k", [23, 24, 25, 31, 32])
+def test_both_forms_of_selection(tiga, k):
+    """Rows are counted up to k = 24 and sorted above; lists of 32 / 33 entries are on either side of the trimming, and
+    coincident points leave no distance that trims a list."""
+    n = 5000
+    pos = gen.clustered_points(n, 15 + k)
+    pos[::7] = pos[3]
+    _check(tiga, pos, gen.normal_features(n, 9, 94, 31), k)
+    _check(tiga, gen.uniform_points(n, 16), gen.normal_features(n, 8, 95, 31), k)
+
+
+@pytest.mark.parametrize("n", [4095, 4096, 4097, 12500, 25000])
+def test_sizes_at_the_limits_of_slices_and_one_launch_binning(tiga, n):
+    _check(tiga, gen.clustered_points(n, 17), gen.normal_features(n, 1, 96, 31), 8)

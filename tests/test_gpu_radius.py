@@ -83,6 +83,16 @@ def test_binning_is_bit_exact(tiga):
     _check_bin(tiga, c["pos"], c["r"], c["box"], c["periodic"])
 
 
+@pytest.mark.parametrize("n,r", [(1, 0.3), (4096, 0.06), (4096, 0.049), (4096, 0.047), (4095, 0.051), (4097, 0.06), (4096, 0.4), (1024, 0.2)])
+def test_one_launch_binning_at_its_limits(tiga, n, r):
+    """At most 4096 points and 8192 cells are binned by one CTA: both limits, and cells fuller than the ranking limit."""
+    ones = np.ones(3, np.float32)
+    pos = gen.uniform_points(n, 18)
+    _check_bin(tiga, pos, np.float32(r), ones, [0, 0, 0])
+    pos[n // 3:] = pos[n // 3:] * np.float32(0.04) + np.float32(0.3)
+    _check_bin(tiga, pos, np.float32(r), ones, [0, 1, 0])
+
+
 # ------------------------------------------------------------------------------ Gaussian
 def test_cfg0_tiny_forward_and_backward(tiga):
     c = gen.config("cfg0")
