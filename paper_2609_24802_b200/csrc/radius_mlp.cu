@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(32 * mlp_warps(BWD), (mlp_warps_per_sm<FQ, BWD
                     for (int q = qa; q < qb; ++q) {                // the warp evaluates one query at a time
                         const int oq = __shfl_sync(FULL, qid, q * split.lpq), nq_in = __shfl_sync(FULL, nin, q * split.lpq);
                         const int off = s_off[q], end = s_end[q];
-                        float S = 0.f, cpos = 0.f, D0 = 0.f, D1 = 0.f, D2 = 0.f, G = 0.f, v = 0.f;
+                        float S = 0.f, comp = 0.f, cpos = 0.f, D0 = 0.f, D1 = 0.f, D2 = 0.f, G = 0.f, v = 0.f;
                         float xq[BWD ? NX : 1], gq[4];
                         if constexpr (BWD) {
 #pragma unroll
@@ -256,8 +256,12 @@ __global__ void __launch_bounds__(32 * mlp_warps(BWD), (mlp_warps_per_sm<FQ, BWD
                                     if (in[u] && h2[u] > 0.f) G += vm[u];
                                 }
                             } else {
-#pragma unroll
-                                for (int u = 0; u < 2; ++u) S += in[u] ? fmaxf(h[u], 0.f) : 0.f;
+                                // compensated: W2 S + |N| b2 cancels where the messages do, and a sum of hundreds of positive
+                                // terms must not lose more there than summing the messages one by one would
+                                const float y = (in[0] ? fmaxf(h[0], 0.f) : 0.f) + (in[1] ? fmaxf(h[1], 0.f) : 0.f) - comp;
+                                const float sum = S + y;
+                                comp = (sum - S) - y;
+                                S = sum;
                             }
                         }
                         // sums over the groups of HID lanes
