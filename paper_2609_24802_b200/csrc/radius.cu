@@ -841,7 +841,11 @@ tiga_status fill_params(RadiusParams* p, long long n, float r, const tiga_box* b
 tiga_status run_binning(RadiusParams& p, int32_t* fill, int nblocks, cudaStream_t s) {
     if (p.n == 0) return TIGA_OK;
     if (p.n <= SMALL_POINTS && p.ncells <= SMALL_CELLS) {
-        bin_small_kernel<<<counted(1), SMALL_THREADS, (size_t)(p.ncells + p.n) * sizeof(int), s>>>(p);
+        // counts and ids take up to 48 KB, which the kernel's static arrays push past what a launch gets without asking
+        const int smem = (p.ncells + p.n) * (int)sizeof(int);
+        if (smem > 47 * 1024)
+            TIGA_CUDA_TRY(cudaFuncSetAttribute(bin_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (SMALL_POINTS + SMALL_CELLS) * (int)sizeof(int)));
+        bin_small_kernel<<<counted(1), SMALL_THREADS, smem, s>>>(p);
         return launch_status();
     }
     TIGA_CUDA_TRY(cudaMemsetAsync(p.cnt, 0, (2 * (size_t)p.ncells + 2 + 16) * sizeof(int32_t), s));

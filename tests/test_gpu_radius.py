@@ -94,6 +94,22 @@ def test_one_launch_binning_at_its_limits(tiga, n, r):
 
 
 # ------------------------------------------------------------------------------ Gaussian
+@pytest.mark.parametrize("n,r,box,cells", [(4046, 0.99, (31, 24, 11), 8184), (4095, 0.99, (31, 24, 11), 8184), (4096, 0.06, (2, 1, 1), 8192),
+                                           (4096, 0.99, (32, 32, 8), 8192), (4096, 0.99, (32, 16, 16), 8192), (4096, 0.96, (32, 16, 17), 8704)])
+def test_one_launch_binning_of_anisotropic_boxes(tiga, n, r, box, cells):
+    """Grids of up to 8192 cells, the most that one CTA bins (no cubic grid comes nearer than 8000), with point counts
+    around what fits the default 48 KB of shared memory, and one grid beyond them."""
+    box = np.array(box, np.float32)
+    assert np.prod(tiga.tiga_radius_grid(n, r, box, [0, 0, 0])[0]) == cells
+    pos = gen.uniform_points(n, 7) * box
+    _check_bin(tiga, pos, np.float32(r), box, [0, 0, 0])
+    x = gen.normal_features(n, 4, 8)
+    _check_gauss(tiga, pos, x, x, np.float32(r), box, [0, 0, 0], np.float32(r / 2), backward=False)
+    idx, d2, y, A = oracle.knn(pos, x, 1)
+    out, nbr, nd2, _ = tiga.tiga_apply_knn(dev(pos, torch), dev(x, torch), 1, box)
+    assert np.array_equal(host(nbr), idx) and np.array_equal(host(nd2), d2) and rel_err(host(out), y, A) <= SUM_TOL
+
+
 def test_cfg0_tiny_forward_and_backward(tiga):
     c = gen.config("cfg0")
     _check_gauss(tiga, c["pos"], c["x"], c["gy"], c["r"], c["box"], c["periodic"], c["sigma"])
