@@ -135,6 +135,7 @@ __global__ void __launch_bounds__(32 * mlp_warps(BWD), (mlp_warps_per_sm<FQ, BWD
         if (mi1) { blo[1] = -FAR_AWAY; bhi[1] = FAR_AWAY; }
         if (mi2) { blo[2] = -FAR_AWAY; bhi[2] = FAR_AWAY; }
         for (int k = lane; k < qe0 - qs0; k += 32) s_self[k] = -1;
+        __syncwarp();                        // staging sets the slot of a query from whichever lane holds its point
 
         auto process_chunk = [&](const int ns, const bool first_chunk) {
             stage.seal(ns);
