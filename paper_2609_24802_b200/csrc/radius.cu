@@ -727,14 +727,15 @@ __global__ void __launch_bounds__(TRAV_THREADS, (MODE == 0 ? 28 : 16) / TRAV_WAR
 template <int NF, bool DIST>
 struct SumMsg {
     static constexpr int CAP = 256, STAGED = NF, OUT = NF, WARPS = NF <= 2 ? 28 : 20;
-    static constexpr float OUTSIDE = DIST ? 0.f : 1.0e30f;
+    static constexpr float OUTSIDE = 1.f;                  // any weight that is finite for every sigma
+    static constexpr int FEAT_STRIDE = CAP + 4;
     float neg_c2;
     // exp(-d2/(2 s^2)) = 2^(d2 * neg_c2)
     __device__ __forceinline__ explicit SumMsg(const RadiusParams& p) : neg_c2(!DIST ? -1.4426950408889634f / (2.f * p.p0 * p.p0) : 0.f) {}
     __device__ __forceinline__ void pair(f32x2 (&acc)[NF], const float da, const float db, f32x2, f32x2, f32x2, const float* xa, const float* xb) const {
         const f32x2 val = DIST ? pack2(sqrtf(da), sqrtf(db)) : pack2(fast_exp2(da * neg_c2), fast_exp2(db * neg_c2));
 #pragma unroll
-        for (int f = 0; f < NF; ++f) acc[f] = fma2(val, pack2(xa[f * CAP], xb[f * CAP]), acc[f]);
+        for (int f = 0; f < NF; ++f) acc[f] = fma2(val, pack2(xa[f * FEAT_STRIDE], xb[f * FEAT_STRIDE]), acc[f]);
     }
     __device__ __forceinline__ float scale(int, const float v) const { return v; }
 };

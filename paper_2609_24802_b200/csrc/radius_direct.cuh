@@ -5,7 +5,9 @@
 //   CAP             candidates the stage holds
 //   STAGED          features per point that are staged with the candidates
 //   OUT             sums per query
-//   OUTSIDE         a squared distance whose message is zero
+//   OUTSIDE         squared distance given to a half that adds nothing (an absent or refused candidate); its features read as
+//                   zero, and the message of that distance times zero must be zero (no decay with the distance is assumed:
+//                   a Gaussian as wide as fp32 allows gives every distance the weight one)
 //   Msg(p)          constants
 //   pair(...)       adds the messages of two accepted candidates to acc[OUT], one per half
 //   scale(f, v)     the stored value of sum f
@@ -17,7 +19,8 @@ namespace tiga {
 template <typename Msg> struct DirectSmem {
     static constexpr int STAGE_CAP = Msg::CAP, STAGED = Msg::STAGED;
     static constexpr int STAGE_BYTES = TestStage<STAGE_CAP>::BYTES;
-    static constexpr int FEAT_BYTES = STAGED * STAGE_CAP * 4;
+    static constexpr int FEAT_STRIDE = STAGE_CAP + 4;                       // the entry behind the stage stays zero
+    static constexpr int FEAT_BYTES = STAGED * FEAT_STRIDE * 4;
     static constexpr int PER_WARP = (STAGE_BYTES + FEAT_BYTES + (QDENSE + 20) * 4 + 15) / 16 * 16;
 };
 
@@ -30,7 +33,7 @@ __device__ __forceinline__ void direct_slice(const RadiusParams& p, const int (&
     const int lane = threadIdx.x & 31;
     unsigned char* base = s_raw + (size_t)(threadIdx.x >> 5) * SM::PER_WARP;
     const TestStage<STAGE_CAP> stage(base);
-    float* s_feat = reinterpret_cast<float*>(base + SM::STAGE_BYTES);                   // [NF][STAGE_CAP]
+    float* s_feat = reinterpret_cast<float*>(base + SM::STAGE_BYTES);                   // [NF][FEAT_STRIDE]
     int* s_self = reinterpret_cast<int*>(base + SM::STAGE_BYTES + SM::FEAT_BYTES);      // staged slot of every query, or -1
     int* s_delta = s_self + QDENSE;
 
@@ -59,6 +62,7 @@ __device__ __forceinline__ void direct_slice(const RadiusParams& p, const int (&
     if (mi1) { blo[1] = -FAR_AWAY; bhi[1] = FAR_AWAY; }
     if (mi2) { blo[2] = -FAR_AWAY; bhi[2] = FAR_AWAY; }
     for (int k = lane; k < qe0 - qs0; k += 32) s_self[k] = -1;
+    if (lane < NF) s_feat[lane * SM::FEAT_STRIDE + STAGE_CAP] = 0.f;
     __syncwarp();                            // staging sets the slot of a query from whichever lane holds its point
 
     auto process_chunk = [&](const int ns, const bool first_chunk) {
@@ -109,12 +113,13 @@ __device__ __forceinline__ void direct_slice(const RadiusParams& p, const int (&
                 }
                 float da, db;
                 unpack2(fma2(dz, dz, fma2(dy, dy, mul2(dx, dx))), da, db);
+                int fa = sa, fb = two ? sb : STAGE_CAP;              // where the halves read their features
                 if (fmaxf(da, db) > p.r2_mid - p.r2_band) {        // within the fp32 error band of the cutoff: decided in fp64
-                    if (da > p.r2_mid - p.r2_band && !exact_pair(p, qid, stage.id[sa])) { da = Msg::OUTSIDE; --cnt; }
-                    if (two && db > p.r2_mid - p.r2_band && !exact_pair(p, qid, stage.id[sb])) { db = Msg::OUTSIDE; --cnt; }
+                    if (da > p.r2_mid - p.r2_band && !exact_pair(p, qid, stage.id[sa])) { da = Msg::OUTSIDE; fa = STAGE_CAP; --cnt; }
+                    if (two && db > p.r2_mid - p.r2_band && !exact_pair(p, qid, stage.id[sb])) { db = Msg::OUTSIDE; fb = STAGE_CAP; --cnt; }
                 }
                 if (!two) db = Msg::OUTSIDE;
-                msg.pair(acc2, da, db, dx, dy, dz, s_feat + sa, s_feat + sb);
+                msg.pair(acc2, da, db, dx, dy, dz, s_feat + fa, s_feat + fb);
             }
             float acc[OUT];
 #pragma unroll
@@ -214,7 +219,7 @@ __device__ __forceinline__ void direct_slice(const RadiusParams& p, const int (&
                 stage.put(slot, c4[u]);
                 if (src[u] >= qs0 && src[u] < qe0) s_self[src[u] - qs0] = slot;
 #pragma unroll
-                for (int f = 0; f < NF; ++f) s_feat[f * STAGE_CAP + slot] = xf[u][f];
+                for (int f = 0; f < NF; ++f) s_feat[f * SM::FEAT_STRIDE + slot] = xf[u][f];
             }
             nst += __popc(kept[u]);
         }

@@ -12,7 +12,7 @@ namespace tiga {
 
 struct LjMsg {
     static constexpr int CAP = 256, STAGED = 0, OUT = 4, WARPS = 28;
-    static constexpr float OUTSIDE = 1.0e30f;
+    static constexpr float OUTSIDE = INFINITY;             // reciprocal 0: no force, no energy
     float s2, force, energy;
     __device__ __forceinline__ explicit LjMsg(const RadiusParams& p) : s2(p.p1 * p.p1), force(24.f * p.p0), energy(2.f * p.p0) {}
     __device__ __forceinline__ void pair(f32x2 (&acc)[4], const float da, const float db, const f32x2 dx, const f32x2 dy, const f32x2 dz,

@@ -173,6 +173,42 @@ def test_runs_of_sparse_cells(tiga, cells, F):
         _check_gauss(tiga, pos, x, gy, r, box, [periodic] * 3, np.float32(0.5), use_cells=True, backward=F >= 4)
 
 
+@pytest.mark.parametrize("sigma", [1e14, 1e20, np.inf])
+@pytest.mark.parametrize("F", [1, 2, 3, 4, 8])
+def test_gaussian_as_wide_as_fp32_allows(tiga, F, sigma):
+    """Every accepted pair weighs one: the message becomes a plain neighbour sum (the oracle's with a weight that is one
+    to the last bit).  Cutoff of a lattice spacing's multiple, so that pairs sit on the cutoff and are refused in fp64."""
+    i = np.arange(12, dtype=np.float32) * np.float32(0.08) + np.float32(0.05)
+    pos = np.stack([t.reshape(-1) for t in np.meshgrid(i, i, i, indexing="ij")], 1)
+    pos = np.concatenate([pos, gen.uniform_points(1777, 33)]).astype(np.float32)
+    x = gen.normal_features(len(pos), F, 34)
+    ones = np.ones(3, np.float32)
+    r = np.float32(0.08)
+    y, A, cnt = oracle.radius_forward(pos, x, r, ones, [0, 0, 0], oracle.MSG_GAUSS, p0=1e9)
+    out, count, _ = tiga.tiga_apply_radius(dev(pos, torch), dev(x, torch), r, ones, [0, 0, 0], tiga.MSG_GAUSS, p0=sigma, want_count=True)
+    assert np.array_equal(host(count), cnt) and rel_err(host(out), y, A) <= SUM_TOL
+
+
+@pytest.mark.parametrize("message", ["gauss", "dist"])
+@pytest.mark.parametrize("F", [1, 2, 3, 4])
+def test_infinite_features_reach_their_neighbours_only(tiga, F, message):
+    """A row with an infinite source among its neighbours is that infinity, any other row is what it is without it."""
+    pos, x = gen.uniform_points(2000, 35), gen.normal_features(2000, F, 36)
+    ones, r, per = np.ones(3, np.float32), np.float32(0.11), [1, 1, 1]
+    kind = tiga.MSG_GAUSS if message == "gauss" else tiga.MSG_DIST
+    P = dev(pos, torch)
+    plain = host(tiga.tiga_apply_radius(P, dev(x, torch), r, ones, per, kind, p0=0.1)[0])
+    x[1234] = np.inf
+    got = host(tiga.tiga_apply_radius(P, dev(x, torch), r, ones, per, kind, p0=0.1)[0])
+    d = pos.astype(np.float64) - pos[1234].astype(np.float64)
+    d2 = ((d - np.rint(d)) ** 2).sum(1)
+    assert abs(d2 - np.float64(r) ** 2).min() > 1e-7          # no pair of this point is near the cutoff
+    near = d2 <= np.float64(r) ** 2
+    near[1234] = False
+    assert 3 < near.sum() < 30
+    assert np.all(got[near] == np.inf) and np.array_equal(got[~near], plain[~near])
+
+
 def test_few_cells_mixed_periodicity_and_anisotropic_box(tiga):
     # the paper's tiny radius shape: 128 points, cutoff 0.35 (two cells per dimension)
     pos = gen.uniform_points(128, 7)
@@ -256,6 +292,18 @@ def test_lennard_jones_lattices(tiga):
     d = np.linalg.norm(pos[:, None, :].astype(np.float64) - pos[None, :, :], axis=2) + np.eye(len(pos)) * 9
     keep[np.unique(np.nonzero(d < 0.7)[0])] = False          # no overlapping particles
     _check_lj(tiga, pos[keep], np.float32(2.0), np.full(3, 12.0, np.float32), [0, 0, 0], eps=1.5, s=0.8)
+
+
+def test_lennard_jones_at_any_unit_of_length(tiga):
+    """Lengths of 1e16 (squares beyond 1e30): the forces scale with eps / s, the energies and counts stay."""
+    c = gen.config("cfg3", m=10)
+    unit = np.float32(2.0 ** 53)                               # a power of two: every quotient of lengths stays the same bits
+    pos, r, box = c["pos"] * unit, np.float32(c["r"]) * unit, np.asarray(c["box"], np.float32) * unit
+    P = lambda a: dev(a, torch)
+    out, count, _ = tiga.tiga_apply_radius(P(c["pos"]), None, c["r"], c["box"], c["periodic"], tiga.MSG_LJ, p0=1.0, p1=1.0, want_count=True)
+    big, count2, _ = tiga.tiga_apply_radius(P(pos), None, r, box, c["periodic"], tiga.MSG_LJ, p0=1.0, p1=float(unit), want_count=True)
+    assert torch.equal(count, count2)
+    assert torch.equal(big[:, 3], out[:, 3]) and torch.equal(big[:, :3] * float(unit), out[:, :3])
 
 
 def test_lennard_jones_replica(tiga):
