@@ -284,7 +284,8 @@ tiga_status tiga_apply_radius(const float* pos, const float* feat, int64_t n, in
  *                                  (grad_out[k].feat[j] + grad_out[j].feat[k])
  *   grad_feat : fp32 [n, F] or NULL;  grad_pos : fp32 [n, 3] or NULL.  F must be a multiple of 4.
  *   reuse_plan != 0: ws still holds the bins of this very position snapshot (left there by
- *   tiga_apply_radius or tiga_radius_bin with the same n, r, box); otherwise it is rebuilt. */
+ *   tiga_apply_radius or tiga_radius_bin with the same n, r, box); otherwise it is rebuilt.  A reused plan is
+ *   only read, so calls on different streams may share it. */
 tiga_status tiga_apply_radius_backward(const float* pos, const float* feat, int64_t n, int32_t F,
                                        float r, const tiga_box* box, const tiga_msg* msg,
                                        const float* grad_out, float* grad_feat, float* grad_pos,

@@ -771,7 +771,6 @@ RadiusLayout carve_radius(RadiusParams* p, void* ws, int32_t** fill) {
     const int nblocks = (int)((nc + SCAN_BLOCK - 1) / SCAN_BLOCK);
     p->cnt = cv.take<int32_t>(2 * nc + 2 + 16);     // counts, then the scatter cursors, then the length of the dense-cell queue
     p->b_count = p->cnt + 2 * nc + 2;
-    p->ticket = p->b_count + 1;
     p->queue_n = p->b_count + 2;
     *fill = p->cnt + nc;
     p->cell = cv.take<int32_t>(n);

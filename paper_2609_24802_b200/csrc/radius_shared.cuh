@@ -58,7 +58,6 @@ struct RadiusParams {
     int unit;                 // points per warp (walk_unit)
     int dense, slice;         // a cell with more than `dense` points is cut into slices of `slice` queries
     int* queue_n;             // length of the kNN queue (zeroed with the counts)
-    int* ticket;              // unit counter of the edge network's backward (zeroed by that call)
     int32_t* b_items;         // cells with more than SORT_DENSE points (queued by the scan), and how many
     int* b_count;
     // optional user copies of the plan

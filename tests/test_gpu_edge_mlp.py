@@ -101,3 +101,29 @@ def test_every_split_of_lanes_and_staged_features(tiga, f_in, hidden):
     pos = (gen.uniform_points(n, 70 + f_in) * np.float32(0.35) + np.float32(0.8)) % np.float32(1.0)
     x, gy = gen.normal_features(n, f_in, 72, 31), gen.normal_features(n, 3, 72, 32)
     _check(tiga, pos, x, gy, np.float32(0.12), np.ones(3, np.float32), [1, 1, 1], gen.mlp_params(f_in, hidden, 3, 8), min_keep=0.5)
+
+
+@pytest.mark.parametrize("f_in,hidden", [(8, 32), (13, 16)])
+def test_backward_calls_share_a_plan(tiga, f_in, hidden):
+    """A reused plan is only read: two cotangents of the same points, on two streams at once, give what each gives alone."""
+    n = 30_000
+    pos, x = dev(gen.surface_points(n, 5), torch), dev(gen.normal_features(n, f_in, 6, 31), torch)
+    P = [dev(a, torch) for a in gen.mlp_params(f_in, hidden, 4, 7)]
+    r, ones = np.float32(0.016), np.ones(3, np.float32)
+    gys = [dev(gen.normal_features(n, 4, 8, 32 + i), torch) for i in range(2)]
+    _, _, ws = tiga.tiga_apply_radius_mlp(pos, x, r, ones, [0, 0, 0], *P)
+    plan = ws.clone()
+    alone = [tiga.tiga_apply_radius_mlp_backward(pos, x, gy, r, ones, [0, 0, 0], *P, ws=ws, reuse_plan=True) for gy in gys]
+    torch.cuda.synchronize()
+    assert torch.equal(ws, plan)
+    streams = [torch.cuda.Stream() for _ in gys]
+    for _ in range(5):
+        got = [None, None]
+        for i, s in enumerate(streams):
+            with torch.cuda.stream(s):
+                got[i] = tiga.tiga_apply_radius_mlp_backward(pos, x, gys[i], r, ones, [0, 0, 0], *P, ws=ws, reuse_plan=True)
+        torch.cuda.synchronize()
+        for a, b in zip(alone, got):
+            assert torch.equal(a["grad_feat"], b["grad_feat"]) and torch.equal(a["grad_pos"], b["grad_pos"])
+            for name in ("grad_W1", "grad_b1", "grad_W2", "grad_b2"):      # sums of 450 k pairs in any order
+                assert float((a[name] - b[name]).norm()) <= 1e-4 * float(a[name].norm()), name
