@@ -25,6 +25,7 @@
 // The displacement is formed from coordinates relative to the corner of the query's cell and the pre-activation as one chain
 // of fused multiply-adds (bias, displacement, features): a ReLU switches on the last bit of that sum.
 #include "radius_direct.cuh"
+#include <float.h>
 
 namespace tiga {
 
@@ -213,6 +214,16 @@ __global__ void __launch_bounds__(32 * mlp_warps<FQ>(BWD), (mlp_warps_per_sm<FQ,
                     for (int q = qa; q < qb; ++q) {                // the warp evaluates one query at a time
                         const int oq = __shfl_sync(FULL, qid, q * split.lpq), nq_in = __shfl_sync(FULL, nin, q * split.lpq);
                         const int off = s_off[q], end = s_end[q];
+                        if (nq_in == 0) {
+                            // no neighbour in this chunk: nothing is formed from the weights, the cotangent or the features (0 times
+                            // an infinite one would be NaN)
+                            if (first_chunk) {
+                                if (!BWD && lane < Fout) p.out[(size_t)oq * Fout + lane] = 0.f;
+                                if (BWD && p.gpos && lane < 3) p.gpos[3 * (size_t)oq + lane] = 0.f;
+                                if (BWD && p.gfeat && lane < Fin) p.gfeat[(size_t)oq * Fin + lane] = 0.f;
+                            }
+                            continue;
+                        }
                         float S = 0.f, comp = 0.f, cpos = 0.f, D0 = 0.f, D1 = 0.f, D2 = 0.f, G = 0.f, v = 0.f;
                         float xq[BWD ? NX : 1], gq[4];
                         if constexpr (BWD) {
@@ -267,7 +278,7 @@ __global__ void __launch_bounds__(32 * mlp_warps<FQ>(BWD), (mlp_warps_per_sm<FQ,
                                 // terms must not lose more there than summing the messages one by one would
                                 const float y = (in[0] ? fmaxf(h[0], 0.f) : 0.f) + (in[1] ? fmaxf(h[1], 0.f) : 0.f) - comp;
                                 const float sum = S + y;
-                                comp = (sum - S) - y;
+                                comp = fminf((sum - S) - y, FLT_MAX);       // NaN behind an infinite sum: any finite value will do
                                 S = sum;
                             }
                         }
@@ -293,7 +304,7 @@ __global__ void __launch_bounds__(32 * mlp_warps<FQ>(BWD), (mlp_warps_per_sm<FQ,
                                 *dst = first_chunk ? val : *dst + val;
                             }
                         } else {
-                            v = fmaf(w2[3], gq[3], fmaf(w2[2], gq[2], fmaf(w2[1], gq[1], w2[0] * gq[0])));
+                            v = cpos > 0.f ? fmaf(w2[3], gq[3], fmaf(w2[2], gq[2], fmaf(w2[1], gq[1], w2[0] * gq[0]))) : 0.f;
                             const float vc = v * cpos, Y = G - vc;
                             gW1[0] = fmaf(v, D0, gW1[0]); gW1[1] = fmaf(v, D1, gW1[1]); gW1[2] = fmaf(v, D2, gW1[2]);
 #pragma unroll

@@ -127,3 +127,61 @@ def test_backward_calls_share_a_plan(tiga, f_in, hidden):
             assert torch.equal(a["grad_feat"], b["grad_feat"]) and torch.equal(a["grad_pos"], b["grad_pos"])
             for name in ("grad_W1", "grad_b1", "grad_W2", "grad_b2"):      # sums of 450 k pairs in any order
                 assert float((a[name] - b[name]).norm()) <= 1e-4 * float(a[name].norm()), name
+
+
+def test_infinite_inputs_stay_where_they_belong(tiga):
+    """An infinite feature makes its neighbours' outputs infinite (not NaN: every first-layer feature weight and every
+    second-layer weight is positive); an isolated point with an infinite feature or cotangent adds nothing to any other
+    gradient and keeps zeros; a cotangent that is not finite does not reach the parameters of units that are off."""
+    n, f_in, hidden, f_out = 1500, 8, 16, 2
+    pos = gen.uniform_points(n, 44) * np.float32(0.8)
+    pos[:2] = [[0.95, 0.95, 0.95], [0.95, 0.05, 0.95]]
+    x, gy = gen.normal_features(n, f_in, 45, 31), gen.normal_features(n, f_out, 46, 32)
+    W1, b1, W2, b2 = gen.mlp_params(f_in, hidden, f_out, 7)
+    W1, W2 = np.abs(W1) + np.float32(0.01), np.abs(W2) + np.float32(0.01)
+    W1[5], b1[5] = 0, -1                                        # this unit is never on
+    P = [dev(a, torch) for a in (W1, b1, W2, b2)]
+    r, ones, per = np.float32(0.09), np.ones(3, np.float32), [0, 0, 0]
+
+    def both(x, gy):
+        X = dev(x, torch)
+        out, count, ws = tiga.tiga_apply_radius_mlp(dev(pos, torch), X, r, ones, per, *P, want_count=True)
+        g = tiga.tiga_apply_radius_mlp_backward(dev(pos, torch), X, dev(gy, torch), r, ones, per, *P, ws=ws, reuse_plan=True)
+        return host(out), host(count), {k: host(v) for k, v in g.items()}
+
+    out, count, g = both(x, gy)
+    assert count[0] == count[1] == 0 and count[7] > 2
+    d2 = ((pos.astype(np.float64) - pos[7].astype(np.float64)) ** 2).sum(1)
+    near = d2 <= np.float64(r) ** 2
+    near[7] = False
+    assert near.sum() == count[7]
+    far, lone, odd = x.copy(), x.copy(), gy.copy()
+    far[7] = np.inf
+    out2, _, _ = both(far, gy)
+    assert np.all(out2[near] == np.inf) and np.array_equal(out2[~near], out[~near])
+    lone[0] = np.inf
+    odd[1] = np.nan
+    out3, _, g3 = both(lone, odd)
+    assert np.array_equal(out3, out) and np.all(out3[:2] == 0)
+    for k in ("grad_feat", "grad_pos"):
+        assert np.array_equal(g3[k], g[k]) and np.all(g3[k][:2] == 0)
+    for k in ("grad_W1", "grad_b1", "grad_W2", "grad_b2"):      # added up in any order
+        assert np.allclose(g3[k], g[k], rtol=1e-4, atol=1e-4 * np.abs(g[k]).max()), k
+    odd = gy.copy()
+    odd[7] = np.inf
+    g4 = both(x, odd)[2]
+    assert np.all(g4["grad_W1"][5] == 0) and g4["grad_b1"][5] == 0
+    assert np.all(np.isinf(g4["grad_W1"][0, 3:]) | np.isnan(g4["grad_W1"][0, 3:]))
+
+
+@pytest.mark.parametrize("weight", ["W1", "b1", "W2", "b2"])
+def test_isolated_points_keep_the_zero_vector_for_any_weights(tiga, weight):
+    pos = (np.stack(np.meshgrid(*[np.arange(5)] * 3, indexing="ij"), -1).reshape(-1, 3) * 0.2 + 0.1).astype(np.float32)
+    n = len(pos)
+    params = dict(zip(("W1", "b1", "W2", "b2"), gen.mlp_params(3, 8, 2, 7)))
+    params[weight] = np.full_like(params[weight], np.inf)
+    P = [dev(a, torch) for a in params.values()]
+    X, G = dev(gen.normal_features(n, 3, 1, 31), torch), dev(gen.normal_features(n, 2, 1, 32), torch)
+    out, _, ws = tiga.tiga_apply_radius_mlp(dev(pos, torch), X, np.float32(0.1), np.ones(3, np.float32), [0, 0, 0], *P)
+    g = tiga.tiga_apply_radius_mlp_backward(dev(pos, torch), X, G, np.float32(0.1), np.ones(3, np.float32), [0, 0, 0], *P, ws=ws, reuse_plan=True)
+    assert not host(out).any() and not any(host(v).any() for v in g.values())
