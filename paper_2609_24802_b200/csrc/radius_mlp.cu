@@ -55,8 +55,8 @@ template <int FQ, bool BWD> __host__ __device__ constexpr int mlp_warps_per_sm()
 
 // Sums v[0..NV) over the L lanes of an aligned group by a halving exchange; afterwards lane l holds, in v[0..NV / min(NV, L)),
 // the totals of the entries from spread_first<NV, L>(l).
-template <int NV, int L>
-static __device__ __forceinline__ void spread_sum(float* v, const int l) {
+template <int NV, int L, typename T>
+static __device__ __forceinline__ void spread_sum(T* v, const int l) {
 #pragma unroll
     for (int j = 0; (1 << j) < L; ++j) {
         const int left = NV >> j;
@@ -64,7 +64,7 @@ static __device__ __forceinline__ void spread_sum(float* v, const int l) {
             const bool up = (l >> j) & 1;
 #pragma unroll
             for (int k = 0; k < left / 2; ++k) {
-                const float send = up ? v[k] : v[k + left / 2], keep = up ? v[k + left / 2] : v[k];
+                const T send = up ? v[k] : v[k + left / 2], keep = up ? v[k + left / 2] : v[k];
                 v[k] = keep + __shfl_xor_sync(0xffffffffu, send, 1 << j);
             }
         } else {
@@ -124,6 +124,13 @@ __global__ void __launch_bounds__(32 * mlp_warps<FQ>(BWD), (mlp_warps_per_sm<FQ,
         return (MI && mi) ? mi_delta(q, c4, p.len[d], 0.5f * p.len[d]) : q - c4;
     };
     const unsigned lt_mask = (1u << lane) - 1u;
+    // compensated: W2 S + |N| b2 and W1^T G cancel where the messages do, and a sum of hundreds of terms must not lose more
+    // there than adding the messages one by one would.  `lost` is added at the end, so the loop waits for one addition.
+    auto add = [](float& sum, float& lost, const float term) {
+        const float t = sum + term;
+        lost += term - (t - sum);
+        sum = t;
+    };
 
     auto slice = [&](const int (&cell)[3], const int run, const int qs0, const int qe0) {
         const RunFrame frame(p, cell, run);
@@ -224,7 +231,7 @@ __global__ void __launch_bounds__(32 * mlp_warps<FQ>(BWD), (mlp_warps_per_sm<FQ,
                             }
                             continue;
                         }
-                        float S = 0.f, comp = 0.f, cpos = 0.f, D0 = 0.f, D1 = 0.f, D2 = 0.f, G = 0.f, v = 0.f;
+                        float S = 0.f, lost = 0.f, cpos = 0.f, D0 = 0.f, D1 = 0.f, D2 = 0.f, G = 0.f, v = 0.f;
                         float xq[BWD ? NX : 1], gq[4];
                         if constexpr (BWD) {
 #pragma unroll
@@ -271,41 +278,41 @@ __global__ void __launch_bounds__(32 * mlp_warps<FQ>(BWD), (mlp_warps_per_sm<FQ,
 #pragma unroll
                                 for (int u = 0; u < 2; ++u) {
                                     if (in[u] && h[u] > 0.f) { S += h[u]; cpos += 1.f; D0 += e[u].x; D1 += e[u].y; D2 += e[u].z; }
-                                    if (in[u] && h2[u] > 0.f) G += vm[u];
+                                    if (!(in[u] && h2[u] > 0.f)) vm[u] = 0.f;
                                 }
+                                add(G, lost, vm[0] + vm[1]);
                             } else {
-                                // compensated: W2 S + |N| b2 cancels where the messages do, and a sum of hundreds of positive
-                                // terms must not lose more there than summing the messages one by one would
-                                const float y = (in[0] ? fmaxf(h[0], 0.f) : 0.f) + (in[1] ? fmaxf(h[1], 0.f) : 0.f) - comp;
-                                const float sum = S + y;
-                                comp = fminf((sum - S) - y, FLT_MAX);       // NaN behind an infinite sum: any finite value will do
-                                S = sum;
+                                add(S, lost, (in[0] ? fmaxf(h[0], 0.f) : 0.f) + (in[1] ? fmaxf(h[1], 0.f) : 0.f));
                             }
                         }
                         // sums over the groups of HID lanes
+                        double total = BWD ? G : S;
+                        if (fabsf(lost) <= FLT_MAX) total += lost;       // (not a number behind an infinite sum)
 #pragma unroll
                         for (int o = HID; o < 32; o <<= 1) {
-                            S += __shfl_xor_sync(FULL, S, o);
+                            total += __shfl_xor_sync(FULL, total, o);
                             if constexpr (BWD) {
-                                cpos += __shfl_xor_sync(FULL, cpos, o); G += __shfl_xor_sync(FULL, G, o);
+                                S += __shfl_xor_sync(FULL, S, o); cpos += __shfl_xor_sync(FULL, cpos, o);
                                 D0 += __shfl_xor_sync(FULL, D0, o); D1 += __shfl_xor_sync(FULL, D1, o); D2 += __shfl_xor_sync(FULL, D2, o);
                             }
                         }
                         if constexpr (!BWD) {
-                            float y[4];
+                            double y[4];
 #pragma unroll
-                            for (int o = 0; o < 4; ++o) y[o] = w2[o] * S;
+                            for (int o = 0; o < 4; ++o) y[o] = (double)w2[o] * total;
                             spread_sum<4, HID>(y, a);
                             const int o = spread_first<4, HID>(a);
                             const float bias = __shfl_sync(FULL, b2, o);
                             if (lane < 4 && o < Fout) {
                                 float* dst = p.out + (size_t)oq * Fout + o;
-                                const float val = fmaf((float)nq_in, bias, y[0]);
+                                const float val = (float)fma((double)nq_in, (double)bias, y[0]);
                                 *dst = first_chunk ? val : *dst + val;
                             }
                         } else {
+                            G = (float)total;
                             v = cpos > 0.f ? fmaf(w2[3], gq[3], fmaf(w2[2], gq[2], fmaf(w2[1], gq[1], w2[0] * gq[0]))) : 0.f;
-                            const float vc = v * cpos, Y = G - vc;
+                            const float vc = v * cpos;
+                            const double Y = total - (double)v * (double)cpos;
                             gW1[0] = fmaf(v, D0, gW1[0]); gW1[1] = fmaf(v, D1, gW1[1]); gW1[2] = fmaf(v, D2, gW1[2]);
 #pragma unroll
                             for (int f = 0; f < NX; ++f) gW1[3 + f] = fmaf(G, xq[f], gW1[3 + f]);
@@ -313,20 +320,28 @@ __global__ void __launch_bounds__(32 * mlp_warps<FQ>(BWD), (mlp_warps_per_sm<FQ,
 #pragma unroll
                             for (int o = 0; o < 4; ++o) gW2[o] = fmaf(gq[o], S, gW2[o]);
                             gb2 = fmaf((float)nq_in, lane == 0 ? gq[0] : lane == 1 ? gq[1] : lane == 2 ? gq[2] : gq[3], gb2);     // lanes 0..3
-                            constexpr int NV = KP <= 8 ? 8 : KP <= 16 ? 16 : 32;
+                            double pb[4];                          // the position gradient is the difference of the two sums
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) pb[k] = k < 3 ? (double)w[k] * Y : 0.0;
+                            spread_sum<4, HID>(pb, a);
+                            const int cp = spread_first<4, HID>(a);
+                            if (p.gpos && lane < 4 && cp < 3) {
+                                float* dst = p.gpos + 3 * (size_t)oq + cp;
+                                *dst = first_chunk ? (float)pb[0] : *dst + (float)pb[0];
+                            }
+                            constexpr int NV = NX <= 4 ? 4 : NX <= 8 ? 8 : 16;
                             float r[NV];
 #pragma unroll
-                            for (int k = 0; k < NV; ++k) r[k] = k < KP ? w[k < KP ? k : 0] * (k < 3 ? Y : G) : 0.f;
+                            for (int k = 0; k < NV; ++k) r[k] = k < NX ? w[k < NX ? 3 + k : 0] * G : 0.f;
                             spread_sum<NV, HID>(r, a);
                             constexpr int LEFT = NV > HID ? NV / HID : 1;
                             const int first = spread_first<NV, HID>(a);
-                            if (lane < (NV < HID ? NV : HID)) {
+                            if (p.gfeat && lane < (NV < HID ? NV : HID)) {
 #pragma unroll
                                 for (int k = 0; k < LEFT; ++k) {
-                                    const int c = first + k;
-                                    float* dst = c < 3 ? (p.gpos ? p.gpos + 3 * (size_t)oq + c : nullptr)
-                                                       : (c < K && p.gfeat ? p.gfeat + (size_t)oq * Fin + c - 3 : nullptr);
-                                    if (dst) *dst = first_chunk ? r[k] : *dst + r[k];
+                                    if (first + k >= Fin) continue;
+                                    float* dst = p.gfeat + (size_t)oq * Fin + first + k;
+                                    *dst = first_chunk ? r[k] : *dst + r[k];
                                 }
                             }
                         }
