@@ -1027,8 +1027,8 @@ static bool pick_shape(int nvec, int* G, int* VPL) {
 // 1.61 -> 1.48 ms with 1024; 2^30 edges the same with 1024 and 4096).
 static int row_huge_of(const tiga_csr* g) { return g->n_edges >= (1LL << 25) ? ROW_HUGE : ROW_HUGE_SMALL; }
 
-// tiles of a relation for a kernel's longest tile; without one, for the shortest of them (sizes workspaces, bounds grids)
-static long long num_tiles(const tiga_csr* g, int longest = CSR_TILE_MIN) {
+// tiles of a relation for a kernel's longest tile
+static long long num_tiles(const tiga_csr* g, int longest) {
     const long long items = g->n_dst + g->n_edges;
     const int tile = tile_length(items, longest);
     return (items + tile - 1) / tile;
@@ -1102,7 +1102,7 @@ static tiga_status launch_bwd_g(const CsrParams& p, int G, int VPL, cudaStream_t
 // entries of the per-tile / per-chunk workspace arrays: tiles of the tile kernels, or chunks of the row-class path
 // (at most E / chunk full chunks plus one partial chunk per chunked row, and a chunked row has more than a chunk)
 static size_t work_slots(const tiga_csr* g, bool narrow_rows) {
-    const size_t tiles = (size_t)num_tiles(g) + 1, chunks = (size_t)(2 * g->n_edges / row_huge_of(g)) + 2;
+    const size_t tiles = (size_t)tile_slots(g->n_dst + g->n_edges, CSR_TILE_MIN) + 1, chunks = (size_t)(2 * g->n_edges / row_huge_of(g)) + 2;
     return (narrow_rows && chunks > tiles) ? chunks : tiles;
 }
 
@@ -1114,7 +1114,7 @@ static tiga_status check_csr(const tiga_csr* g) {
     if (g->n_edges > 0 && (!g->col || !aligned16(g->col))) return TIGA_ERR_INVALID_ARG;
     if (g->rowptr_type == TIGA_I32 && g->n_edges > 0x7fffffffLL) return TIGA_ERR_INVALID_ARG;
     if (g->n_dst > 0x7fffffffLL || g->n_src > 0x7fffffffLL) return TIGA_ERR_UNSUPPORTED;
-    if (num_tiles(g) > 0x7fffffffLL) return TIGA_ERR_UNSUPPORTED;
+    if (tile_slots(g->n_dst + g->n_edges, CSR_TILE_MIN) > 0x7fffffffLL) return TIGA_ERR_UNSUPPORTED;
     return TIGA_OK;
 }
 

@@ -353,9 +353,10 @@ static tiga_status attention_check(const tiga_csr* g, int32_t D) {
 
 static size_t attention_carve(CsrParams* p, void* ws) {
     Carver cv(ws);
-    p->carry_row = cv.take<int32_t>((size_t)p->ntiles);
-    p->carry_ml = cv.take<float2>((size_t)p->ntiles);
-    p->carry_val = cv.take<float>((size_t)p->ntiles * p->F);
+    const size_t slots = (size_t)tile_slots(p->n_dst + p->n_edges, CSR_TILE_ATT);
+    p->carry_row = cv.take<int32_t>(slots);
+    p->carry_ml = cv.take<float2>(slots);
+    p->carry_val = cv.take<float>(slots * p->F);
     p->gw = cv.take<float>((size_t)p->n_dst + 1);            // lse of every row as stored by the tile it ends in
     return cv.off;
 }
@@ -367,9 +368,7 @@ using namespace tiga;
 extern "C" size_t tiga_csr_attention_workspace_bytes(const tiga_csr* g, int32_t D) {
     if (attention_check(g, D) != TIGA_OK) return 0;
     CsrParams p{};
-    p.n_dst = g->n_dst; p.n_edges = g->n_edges; p.n_src = g->n_src; p.F = D;
-    p.tile = tile_length(g->n_dst + g->n_edges, CSR_TILE_ATT);
-    p.ntiles = (g->n_dst + g->n_edges + p.tile - 1) / p.tile;
+    p.n_dst = g->n_dst; p.n_edges = g->n_edges; p.F = D;
     return attention_carve(&p, nullptr) + 256;
 }
 

@@ -86,9 +86,19 @@ struct CsrParams {
 
 // Items per tile: at most `longest` (what the kernel's shared memory holds), less where that would leave some of the 592
 // places (four CTAs per SM) empty, down to 256 (a tile's search and staging cost as much as a few hundred edges).
+constexpr int TILE_PLACES = 592, TILE_SHORTEST = 256;
 static inline int tile_length(long long items, int longest) {
-    const long long even = (items / 592 + 255) / 256 * 256;
-    return (int)(even < 256 ? 256 : even < longest ? even : longest);
+    const long long even = (items / TILE_PLACES + TILE_SHORTEST - 1) / TILE_SHORTEST * TILE_SHORTEST;
+    return (int)(even < TILE_SHORTEST ? TILE_SHORTEST : even < longest ? even : longest);
+}
+
+// Entries of the per-tile workspace arrays.  tile_length goes up in steps, so a smaller input may have more tiles than a
+// larger one; this bound on both never falls as the input grows: a workspace sized for a program's largest relation serves
+// the smaller ones.  (An input of less than 592 (tile + 1) items has at most 595 tiles of `tile`.)
+static inline long long tile_slots(long long items, int longest) {
+    const long long shortest = (items + TILE_SHORTEST - 1) / TILE_SHORTEST, most = (items + longest - 1) / longest;
+    const long long few = shortest < TILE_PLACES + 3 ? shortest : TILE_PLACES + 3;
+    return few > most ? few : most;
 }
 
 // host side, defined in csr_plan.cu: compact copy of the hot source rows, hot[r, :] = x[hot_id[r], :]

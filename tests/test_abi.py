@@ -114,6 +114,23 @@ def test_host_side_argument_errors(lib):
     assert cdll.tiga_apply_radius_backward(256, 256, 100, 6, r, ctypes.byref(b), ctypes.byref(_Msg(2, 0.1, 0.0)), 256, 256, 256, 256, big, 0, None) == 2
 
 
+def test_workspaces_grow_with_the_relation(lib):
+    """A program sizes one workspace for its largest relation and uses it for the smaller ones, and what fitted the built-in
+    array of 8 MiB goes on fitting: a relation of up to 592 * 1792 rows and edges needs at most 595 entries per array."""
+    cdll = lib.load_library()
+    from paper_2609_24802_b200.api import _Csr
+    items = sorted({int(s * 592 * t + d) for t in (1, 256, 512, 768, 1024, 1792, 2048, 4000) for s in (0.5, 1.0, 1.01) for d in (-1, 0, 1, 591, 592)})
+    csr = lambda n: ctypes.byref(_Csr(256, 0, 256, n // 9, n // 9, n - n // 9))
+    for F in (16, 64, 512):
+        for red in (0, 1, 2):
+            need = [cdll.tiga_csr_workspace_bytes(csr(n), F, 0, red, 0) for n in items]
+            assert need == sorted(need), (F, red)
+    need = [cdll.tiga_csr_attention_workspace_bytes(csr(n), 128) for n in items]
+    assert need == sorted(need)
+    widest = _Csr(256, 0, 256, 592 * 256, 592 * 256, 592 * 1536)
+    assert cdll.tiga_csr_workspace_bytes(ctypes.byref(widest), 1024, 1, 2, 0) <= 8 << 20       # F = 1024 fp16 with 64-bit positions
+
+
 def test_knn_and_attention_host_checks(lib):
     """Workspace sizing and argument checks of the widened entry points run on the host only."""
     cdll = lib.load_library()
