@@ -364,7 +364,13 @@ _BOX_OF = _Box.from_buffer_copy
 
 
 def _box(box, periodic):
-    return _BOX_OF(_BOX_BYTES.pack(box[0], box[1], box[2], int(periodic[0]), int(periodic[1]), int(periodic[2])))
+    try:
+        return _BOX_OF(_BOX_BYTES.pack(box[0], box[1], box[2], int(periodic[0]), int(periodic[1]), int(periodic[2])))
+    except (struct.error, OverflowError, TypeError):      # a number that fp32 or int32 does not hold, a text: as ctypes converts them
+        b = _Box()
+        for d in range(3):
+            b.len[d], b.periodic[d] = float(box[d]), int(periodic[d])
+        return b
 
 
 def tiga_radius_grid(n: int, r: float, box, periodic):

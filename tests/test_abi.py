@@ -157,6 +157,25 @@ def test_knn_and_attention_host_checks(lib):
     assert cdll.tiga_apply_csr_attention(ctypes.byref(g), None, None, None, 132, ctypes.c_float(1.0), None, None, None, 0, None) == 2
 
 
+@pytest.mark.parametrize("box,periodic", [((1e39, 1, 1), (0, 0, 0)), ((float("inf"), 1, 1), (0, 0, 0)), ((-1e39, 1, 1), (0, 0, 0)), ((float("nan"), 1, 1), (0, 0, 0))])
+def test_boxes_beyond_fp32_are_refused_by_the_library(lib, box, periodic):
+    """A length that fp32 does not hold is an infinite one: the calls refuse it with a status, the sizes are zero."""
+    with pytest.raises(lib.TigaError) as e:
+        lib.tiga_radius_grid(100, 0.1, box, periodic)
+    assert e.value.status == 1
+    assert lib.tiga_radius_workspace_bytes(100, 4, 0.1, box, periodic) == 0
+    assert lib.tiga_knn_workspace_bytes(100, 4, box) == 0
+
+
+def test_every_kind_of_number_makes_a_box(lib):
+    """Floats, integers, numpy and torch scalars, texts; any non-zero flag is periodic, whatever its size."""
+    import torch
+    want = lib.tiga_radius_grid(1000, 0.1, [1.0, 2.0, 3.0], [1, 0, 1])
+    for box in ([1, 2, 3], np.float32([1, 2, 3]), np.float64([1, 2, 3]), torch.tensor([1.0, 2.0, 3.0]), ["1.0", "2.0", "3.0"]):
+        for flag in (1, True, np.int64(1), torch.tensor(1), 2 ** 33 + 1):
+            assert lib.tiga_radius_grid(1000, 0.1, box, [flag, 0, flag]) == want
+
+
 def test_bench_probe_library_builds_and_checks_its_arguments(lib):
     """The benchmark's row-gather probe lives in a library of its own, outside the product ABI."""
     from paper_2609_24802_b200 import bench_probe
