@@ -157,8 +157,10 @@ _L = load_library()      # fail at import time, loudly, when the CUDA library is
 # A call on a small relation is bound by its marshalling, so the calls below avoid what costs a microsecond each:
 # the message structs of the stored relation are built once, a stream is looked up by its handle (no Stream object),
 # pointers are passed as plain integers, outputs are allocated with new_empty.
-_current_device = torch._C._cuda_getDevice
-_raw_stream = torch._C._cuda_getCurrentRawStream
+# (The two look-ups are torch's own shortcuts, not its documented interface: where a build of torch lacks them, a stream
+# object is asked.)
+_current_device = getattr(torch._C, "_cuda_getDevice", None)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def checked_status(reset: bool = True) -> int:
@@ -184,7 +186,9 @@ def _ptr(t):
 
 
 def _stream(stream):
-    return _raw_stream(_current_device()) if stream is None else stream.cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    return _raw_stream(_current_device()) if _raw_stream and _current_device else torch.cuda.current_stream().cuda_stream
 
 
 def _ok(st, where):

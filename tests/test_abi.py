@@ -176,6 +176,18 @@ def test_every_kind_of_number_makes_a_box(lib):
             assert lib.tiga_radius_grid(1000, 0.1, box, [flag, 0, flag]) == want
 
 
+def test_import_without_torch_shortcuts(lib):
+    """The two undocumented look-ups of torch that a call uses are optional."""
+    import subprocess
+    import sys
+    code = ("import torch\nfor n in ('_cuda_getDevice', '_cuda_getCurrentRawStream'):\n    if hasattr(torch._C, n): delattr(torch._C, n)\n"
+            "from paper_2609_24802_b200 import api\n"
+            "class S: cuda_stream = 7\n"
+            "torch.cuda.current_stream = lambda: S\nassert api._stream(None) == 7 and api._stream(S) == 7")
+    res = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
+    assert res.returncode == 0, res.stderr[-2000:]
+
+
 def test_bench_probe_library_builds_and_checks_its_arguments(lib):
     """The benchmark's row-gather probe lives in a library of its own, outside the product ABI."""
     from paper_2609_24802_b200 import bench_probe
