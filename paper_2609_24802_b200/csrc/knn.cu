@@ -185,13 +185,22 @@ static __device__ __forceinline__ void emit_row(const KnnParams& P, const int i,
         __syncwarp();
         if (sel) ids[place] = checked(id, P.rp.n, CHECK_POINT);
         __syncwarp();
-        const int lanes = F <= 8 ? 8 : F <= 16 ? 16 : 32, fl = lane & (lanes - 1), g = lane / lanes, step = 32 / lanes;
-        for (int f = fl; f - fl < F; f += lanes) {
+        // 8, 16 or 32 lanes span a row, the warp's groups take rows in turn; four rows in flight per lane (one at a time:
+        // F = 64, k = 16, 1 M points 2770 instead of 1633 us; F = 8 998 and 906)
+        const int lg = F <= 8 ? 3 : F <= 16 ? 4 : 5, fl = lane & ((1 << lg) - 1), g = lane >> lg, step = 32 >> lg;
+        for (int f = fl; f - fl < F; f += 1 << lg) {
+            const bool in = f < F;
             float acc = 0.f;
-            for (int t = g; t < m; t += step)
-                if (f < F) acc += __ldg(feat + (size_t)ids[t] * F + f);
-            for (int o = lanes; o < 32; o <<= 1) acc += __shfl_xor_sync(FULL, acc, o);
-            if (g == 0 && f < F) P.out[(size_t)i * F + f] = acc;
+            for (int t = g; t < m; t += 4 * step) {
+                float x[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) x[u] = in && t + u * step < m ? __ldg(feat + (size_t)ids[t + u * step] * F + f) : 0.f;
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (t + u * step < m) acc += x[u];
+            }
+            for (int o = 1 << lg; o < 32; o <<= 1) acc += __shfl_xor_sync(FULL, acc, o);
+            if (g == 0 && in) P.out[(size_t)i * F + f] = acc;
         }
     } else {
         const size_t row = sel ? (size_t)checked(id, P.rp.n, CHECK_POINT) * F : 0;
