@@ -224,11 +224,13 @@ static __device__ __forceinline__ void emit_sorted(const KnnParams& P, const int
 }
 
 // Selects and writes the row of query i from its list of n >= k entries, none farther than tau (squared).
-static __device__ __forceinline__ void select_and_emit(const KnnParams& P, const int i, float2* lq, int n, float tau, const int lane) {
+// tied: the warp's last query had equal distances, so this one is ordered by whole keys at once (points on a lattice: counting
+// first and then sorting, 64,000 points, k = 8 and 16, 105 and 95 us instead of 95 and 85 us).
+static __device__ __forceinline__ void select_and_emit(const KnnParams& P, const int i, float2* lq, int n, float tau, bool& tied, const int lane) {
     constexpr unsigned FULL = 0xffffffffu;
     const int k = P.k;
     if (k <= KNN_COUNT_K && n > KNN_TRIM) n = trim_list(lq, n, k, tau, lane);
-    if (k <= KNN_COUNT_K && n <= KNN_TRIM) {
+    if (k <= KNN_COUNT_K && n <= KNN_TRIM && !tied) {
         const float2 own = lane < n ? lq[lane] : make_float2(0.f, __int_as_float(0x7f800000));
         int place = 0;
         const float4* l4 = reinterpret_cast<const float4*>(lq);
@@ -245,12 +247,15 @@ static __device__ __forceinline__ void select_and_emit(const KnnParams& P, const
             return;
         }
     }
-    emit_sorted(P, i, select_sorted(lq, n, lane), k, reinterpret_cast<int*>(lq), lane);
+    const knn_key top = select_sorted(lq, n, lane);
+    const float before = __shfl_up_sync(FULL, key_dist(top), 1);
+    tied = __any_sync(FULL, lane > 0 && lane < n && key_dist(top) == before);
+    emit_sorted(P, i, top, k, reinterpret_cast<int*>(lq), lane);
 }
 
 // ------------------------------------------------------------------------------ cells kernel
 // queries [qs0, qe0) of one cell (the whole cell, or a slice of a dense one)
-__device__ __forceinline__ void knn_cell_slice(const KnnParams& P, const int (&c)[3], const int qs0, const int qe0, unsigned char* s_raw) {
+__device__ __forceinline__ void knn_cell_slice(const KnnParams& P, const int (&c)[3], const int qs0, const int qe0, bool& tied, unsigned char* s_raw) {
     const RadiusParams& p = P.rp;
     constexpr unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
@@ -423,7 +428,7 @@ __device__ __forceinline__ void knn_cell_slice(const KnnParams& P, const int (&c
             if (n < k) {
                 if (lane == 0) P.queue[atomicAdd(p.queue_n, 1)] = i;
             } else {
-                select_and_emit(P, i, list + q * KNN_QSTRIDE, n, s_tau[q], lane);
+                select_and_emit(P, i, list + q * KNN_QSTRIDE, n, s_tau[q], tied, lane);
             }
         }
     }
@@ -432,7 +437,8 @@ __device__ __forceinline__ void knn_cell_slice(const KnnParams& P, const int (&c
 // one warp per unit of points; cells are not joined (the search radius already gives a cell about k / 2 points)
 __global__ void __launch_bounds__(TRAV_THREADS, 32 / TRAV_WARPS) knn_cells_kernel(const __grid_constant__ KnnParams P) {
     extern __shared__ __align__(16) unsigned char s_raw[];
-    auto work = [&](const int (&cell)[3], int, const int qs, const int qe) { knn_cell_slice(P, cell, qs, qe, s_raw); };
+    bool tied = false;
+    auto work = [&](const int (&cell)[3], int, const int qs, const int qe) { knn_cell_slice(P, cell, qs, qe, tied, s_raw); };
     walk_unit(P.rp, blockIdx.x * TRAV_WARPS + (threadIdx.x >> 5), 1, work);
 }
 

@@ -164,3 +164,15 @@ def test_both_forms_of_selection(tiga, k):
 @pytest.mark.parametrize("n", [4095, 4096, 4097, 12500, 25000])
 def test_sizes_at_the_limits_of_slices_and_one_launch_binning(tiga, n):
     _check(tiga, gen.clustered_points(n, 17), gen.normal_features(n, 1, 96, 31), 8)
+
+
+@pytest.mark.parametrize("k", [8, 16, 24])
+def test_ties_that_come_and_go_within_a_warp(tiga, k):
+    """A warp whose last query had equal distances orders the next one by whole keys: rows of a lattice next to uniform
+    points, so that both kinds of query share cells and warps, compared key by key and index by index."""
+    i = np.arange(14, dtype=np.float32) / np.float32(32.0) + np.float32(0.03125)
+    z, y, x = np.meshgrid(i, i, i, indexing="ij")
+    lattice = np.stack([x.ravel(), y.ravel(), z.ravel()], 1)
+    pos = np.concatenate([lattice, gen.uniform_points(6000, 55)]).astype(np.float32)
+    pos = pos[np.random.default_rng(5).permutation(len(pos))]
+    _check(tiga, pos, gen.normal_features(len(pos), 2, 56, 31), k)
