@@ -255,6 +255,10 @@ static __device__ __forceinline__ void select_and_emit(const KnnParams& P, const
 
 // ------------------------------------------------------------------------------ cells kernel
 // queries [qs0, qe0) of one cell (the whole cell, or a slice of a dense one)
+// SU: groups of 32 candidates staged per step.  A step that no longer fits the stage is taken again, and above k = 20 the
+// stencil keeps more candidates (about 9 k) than the stage holds, for every batch of queries anew: short steps there (one
+// feature, 1 M points, k = 24, 25, 32: 1428, 1349, 1816 us with four groups, 1288, 1238, 1672 us with two; k = 16 783 and 816 us).
+template <int SU>
 __device__ __forceinline__ void knn_cell_slice(const KnnParams& P, const int (&c)[3], const int qs0, const int qe0, bool& tied, unsigned char* s_raw) {
     const RadiusParams& p = P.rp;
     constexpr unsigned FULL = 0xffffffffu;
@@ -293,7 +297,6 @@ __device__ __forceinline__ void knn_cell_slice(const KnnParams& P, const int (&c
     // ---- stages kept candidates starting at flattened stencil position v0 until the next step might not fit or the stencil
     //      ends; returns the next position, the kept count in ns.  `before` counts the ranges that began before v0 (-1 at 0).
     auto stage_from = [&](int v0, int& before, int& ns) -> int {
-        constexpr int SU = 4;                                 // groups of 32 candidates in flight
         static_assert(KNN_STAGE_CAP >= 32 * SU, "a step fits an empty stage");
         int nst = 0;
         while (v0 < total) {
@@ -435,10 +438,11 @@ __device__ __forceinline__ void knn_cell_slice(const KnnParams& P, const int (&c
 }
 
 // one warp per unit of points; cells are not joined (the search radius already gives a cell about k / 2 points)
+template <int SU>
 __global__ void __launch_bounds__(TRAV_THREADS, 32 / TRAV_WARPS) knn_cells_kernel(const __grid_constant__ KnnParams P) {
     extern __shared__ __align__(16) unsigned char s_raw[];
     bool tied = false;
-    auto work = [&](const int (&cell)[3], int, const int qs, const int qe) { knn_cell_slice(P, cell, qs, qe, tied, s_raw); };
+    auto work = [&](const int (&cell)[3], int, const int qs, const int qe) { knn_cell_slice<SU>(P, cell, qs, qe, tied, s_raw); };
     walk_unit(P.rp, blockIdx.x * TRAV_WARPS + (threadIdx.x >> 5), 1, work);
 }
 
@@ -624,8 +628,9 @@ extern "C" tiga_status tiga_apply_knn(const float* pos, const float* feat, int64
     st = run_binning(P.rp, fill, lay.nblocks, s);
     if (st != TIGA_OK) return st;
     constexpr int smem = KNN_PER_WARP * TRAV_WARPS;
-    TIGA_CUDA_TRY(cudaFuncSetAttribute(knn_cells_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    knn_cells_kernel<<<counted(unit_blocks(P.rp)), TRAV_THREADS, smem, s>>>(P);
+    auto cells = k > 20 ? knn_cells_kernel<2> : knn_cells_kernel<4>;
+    TIGA_CUDA_TRY(cudaFuncSetAttribute(cells, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    cells<<<counted(unit_blocks(P.rp)), TRAV_THREADS, smem, s>>>(P);
     knn_rings_kernel<<<counted(KNN_RING_BLOCKS), RING_THREADS, 0, s>>>(P);
     return launch_status();
 }

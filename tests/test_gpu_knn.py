@@ -150,7 +150,7 @@ def test_paper_size_131072_points(tiga):
     assert np.allclose(host(out)[:, 0], x[nb, 0].sum(1), rtol=1e-4, atol=1e-4)
 
 
-@pytest.mark.parametrize("k", [23, 24, 25, 31, 32])
+@pytest.mark.parametrize("k", [20, 21, 23, 24, 25, 31, 32])
 def test_both_forms_of_selection(tiga, k):
     """Rows are counted up to k = 24 and sorted above; lists of 32 / 33 entries are on either side of the trimming, and
     coincident points leave no distance that trims a list."""
