@@ -110,6 +110,18 @@ def test_one_launch_binning_of_anisotropic_boxes(tiga, n, r, box, cells):
     assert np.array_equal(host(nbr), idx) and np.array_equal(host(nd2), d2) and rel_err(host(out), y, A) <= SUM_TOL
 
 
+@pytest.mark.parametrize("counts", [(64, 65, 63, 0, 1, 128, 2), (4096,), (2000, 2001), (65,) * 63, (256, 257, 255, 1000, 66, 31, 32, 33), (64,) * 64])
+def test_one_launch_binning_of_dense_cells(tiga, counts):
+    """Cells on both sides of the 64 points that are ordered by counting, up to all points in one cell and as many denser cells
+    as there can be (63)."""
+    rng = np.random.default_rng(len(counts))
+    cell = rng.permutation(np.repeat(rng.permutation(64)[:len(counts)], counts))
+    corner = np.stack([cell % 4, cell // 4 % 4, cell // 16], 1)
+    pos = ((corner + rng.uniform(0.02, 0.98, corner.shape)) * 0.25).astype(np.float32)
+    assert tiga.tiga_radius_grid(len(pos), 0.24, np.ones(3, np.float32), [0, 0, 0])[0] == [4, 4, 4]
+    _check_bin(tiga, pos, np.float32(0.24), np.ones(3, np.float32), [0, 0, 0])
+
+
 def test_cfg0_tiny_forward_and_backward(tiga):
     c = gen.config("cfg0")
     _check_gauss(tiga, c["pos"], c["x"], c["gy"], c["r"], c["box"], c["periodic"], c["sigma"])
