@@ -658,7 +658,9 @@ __global__ void csr_fixup_kernel(const CsrParams p) {
     using AT = ArgT<RED>;
     const AT* carg = static_cast<const AT*>(p.carry_arg);
     AT a = RED ? carg[tile * p.F + f] : AT(0);
-    for (long long u0 = tile + 1; u0 < p.ntiles; u0 += 8) {      // eight carry-outs are requested at a time
+    // a row over several tiles requests eight carry-outs at a time; most rows end in the next tile, which has none of them
+    const bool several = tile + 1 < p.ntiles && p.carry_row[tile + 1] == row;
+    for (long long u0 = tile + 1; several && u0 < p.ntiles; u0 += 8) {
         int rr[8];
         float ov[8];
         AT oa[8];

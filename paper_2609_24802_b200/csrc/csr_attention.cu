@@ -296,8 +296,9 @@ __global__ void csr_attention_fixup_kernel(const CsrParams p) {
         m = M;
     };
     // a long row has one carry-out per tile: eight of them are requested at a time (one by one the longest row's chain of
-    // loads set the time of the launch)
-    for (long long u0 = tile + 1; u0 < p.ntiles; u0 += 8) {
+    // loads set the time of the launch); most rows end in the next tile, which has none of them
+    const bool several = tile + 1 < p.ntiles && p.carry_row[tile + 1] == row;
+    for (long long u0 = tile + 1; several && u0 < p.ntiles; u0 += 8) {
         int rr[8];
         float2 ml[8];
         float ov[8];
