@@ -1029,15 +1029,27 @@ static bool pick_shape(int nvec, int* G, int* VPL) {
 // 1.61 -> 1.48 ms with 1024; 2^30 edges the same with 1024 and 4096).
 static int row_huge_of(const tiga_csr* g) { return g->n_edges >= (1LL << 25) ? ROW_HUGE : ROW_HUGE_SMALL; }
 
-// tiles of a relation for a kernel's longest tile
-static long long num_tiles(const tiga_csr* g, int longest) {
-    const long long items = g->n_dst + g->n_edges;
-    const int tile = tile_length(items, longest);
-    return (items + tile - 1) / tile;
+static void set_tiles(CsrParams& p, const tiga_csr* g, int tile) {
+    p.tile = tile;
+    p.ntiles = (g->n_dst + g->n_edges + tile - 1) / tile;
 }
-static void set_tiles(CsrParams& p, const tiga_csr* g, int longest) {
-    p.tile = tile_length(g->n_dst + g->n_edges, longest);
-    p.ntiles = num_tiles(g, longest);
+
+// Forward.  Wide rows keep partial states of 512 VPL vectors, with their positions, in shared memory, and fewer than four CTAs
+// share an SM.  Tiles made for four (R-MAT, 680 k items: F = 256 with 64-bit positions 531 tiles on 444 places, F = 512
+// likewise) against tiles made for what fits: 222 and 175 us, 144 and 103 us; 20 k rows of 16, F = 1024 fp16 228 and 183 us.
+static int forward_tile(const tiga_csr* g, tiga_reducer reducer, int VPL, int vw) {
+    const int longest = reducer == TIGA_SUM ? CSR_TILE : CSR_TILE_MAX;
+    const int value = 4 + (reducer == TIGA_SUM ? 0 : reducer == TIGA_MAX ? 4 : 8);
+    const int smem = 12 * longest + 2 * CSR_THREADS * VPL * vw * value + 1536;
+    const int fit = 228 * 1024 / smem;
+    return tile_length(g->n_dst + g->n_edges, longest, 148 * (fit < 1 ? 1 : fit < 4 ? fit : 4));
+}
+
+// Backward (48 registers, five CTAs per SM; no per-tile arrays): whole waves of equal tiles.  60,000 rows of 32 edges are 1.49
+// waves of the longest tile, 60 us (F = 16) and 150 us (F = 64 fp16), against 52 and 130 us with two waves of 1344 items.
+static int backward_tile(const tiga_csr* g) {
+    const long long items = g->n_dst + g->n_edges, places = 148 * 5, wave = places * CSR_TILE_BWD;
+    return even_tile(items, CSR_TILE_BWD, (items > wave ? (items + wave - 1) / wave : 1) * places);
 }
 
 template <typename XT, int G, int VPL, int RED, typename IT>
@@ -1209,7 +1221,7 @@ extern "C" tiga_status tiga_apply_csr(const tiga_csr* g, const void* x, tiga_dty
     p.huge_count = cv.take<int>(1);
     p.huge_list = cv.take<int4>(slots);
     p.row_huge = row_huge_of(g);
-    set_tiles(p, g, reducer == TIGA_SUM ? CSR_TILE : CSR_TILE_MAX);      // the launch's tiles (the arrays hold at least as many)
+    set_tiles(p, g, forward_tile(g, reducer, VPL, x_dtype == TIGA_F32 ? 4 : 8));      // (the arrays hold at least as many)
 
     const bool i64 = g->rowptr_type == TIGA_I64;
     if (reducer == TIGA_MAX64) {
@@ -1368,7 +1380,7 @@ extern "C" tiga_status tiga_apply_csr_backward(const tiga_csr* g, const void* x,
     CsrParams p{};
     p.rowptr = g->rowptr; p.col = g->col; p.w = w; p.x = x; p.arg = const_cast<void*>(argmax);
     p.n_dst = g->n_dst; p.n_edges = g->n_edges; p.n_src = g->n_src; p.F = F; p.nvec = nvec;
-    set_tiles(p, g, CSR_TILE_BWD);
+    set_tiles(p, g, backward_tile(g));
     p.gy = grad_out; p.gx = grad_x; p.gw = grad_w;
     if (reducer == TIGA_SUM) {
         if (x_dtype == TIGA_F16)

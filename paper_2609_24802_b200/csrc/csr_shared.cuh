@@ -84,20 +84,24 @@ struct CsrParams {
     float2* carry_ml;        // [ntiles] (running maximum, mass) of a tile's carry-out
 };
 
-// Items per tile: at most `longest` (what the kernel's shared memory holds), less where that would leave some of the 592
-// places (four CTAs per SM) empty, down to 256 (a tile's search and staging cost as much as a few hundred edges).
+// Items per tile: at most `longest` (what the kernel's shared memory holds).  Shorter where that makes whole waves of the
+// `places` (CTAs that are resident together, four per SM unless a kernel holds fewer), as long as there are at most 592 tiles:
+// the per-tile arrays are sized for that many.  At least 256 (a tile's search and staging cost as much as a few hundred edges).
 constexpr int TILE_PLACES = 592, TILE_SHORTEST = 256;
-static inline int tile_length(long long items, int longest) {
-    const long long even = (items / TILE_PLACES + TILE_SHORTEST - 1) / TILE_SHORTEST * TILE_SHORTEST;
+static inline int even_tile(long long items, int longest, long long tiles) {
+    const long long even = (((items + tiles - 1) / tiles) + 31) / 32 * 32;
     return (int)(even < TILE_SHORTEST ? TILE_SHORTEST : even < longest ? even : longest);
 }
+static inline int tile_length(long long items, int longest, int places = TILE_PLACES) {
+    const long long wave = (long long)places * longest, tiles = (items > wave ? (items + wave - 1) / wave : 1) * places;
+    return tiles > TILE_PLACES ? longest : even_tile(items, longest, tiles);
+}
 
-// Entries of the per-tile workspace arrays.  tile_length goes up in steps, so a smaller input may have more tiles than a
-// larger one; this bound on both never falls as the input grows: a workspace sized for a program's largest relation serves
-// the smaller ones.  (An input of less than 592 (tile + 1) items has at most 595 tiles of `tile`.)
+// Entries of the per-tile workspace arrays: a bound on the tiles for any number of places that never falls as the input grows, so
+// that a workspace sized for a program's largest relation serves the smaller ones (the tiles themselves go up and down).
 static inline long long tile_slots(long long items, int longest) {
     const long long shortest = (items + TILE_SHORTEST - 1) / TILE_SHORTEST, most = (items + longest - 1) / longest;
-    const long long few = shortest < TILE_PLACES + 3 ? shortest : TILE_PLACES + 3;
+    const long long few = shortest < TILE_PLACES ? shortest : TILE_PLACES;
     return few > most ? few : most;
 }
 

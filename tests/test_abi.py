@@ -116,7 +116,7 @@ def test_host_side_argument_errors(lib):
 
 def test_workspaces_grow_with_the_relation(lib):
     """A program sizes one workspace for its largest relation and uses it for the smaller ones, and what fitted the built-in
-    array of 8 MiB goes on fitting: a relation of up to 592 * 1792 rows and edges needs at most 595 entries per array."""
+    array of 8 MiB goes on fitting: a relation of up to 592 * 1792 rows and edges needs at most 592 entries per array."""
     cdll = lib.load_library()
     from paper_2609_24802_b200.api import _Csr
     items = sorted({int(s * 592 * t + d) for t in (1, 256, 512, 768, 1024, 1792, 2048, 4000) for s in (0.5, 1.0, 1.01) for d in (-1, 0, 1, 591, 592)})

@@ -424,3 +424,19 @@ def test_tile_lengths_of_small_relations(tiga, items):
     x, w, gy = gen.normal_features(n, 12, 5, 31), gen.edge_weights(E, 6), gen.normal_features(n, 12, 5, 32)
     g, xd, wd, res = _check_forward(tiga, rowptr, col, x, w)
     _check_backward(tiga, rowptr, col, x, w, gy, g, xd, wd, res)
+
+
+@pytest.mark.parametrize("items,F", [(148 * 1792, 512), (148 * 1792 + 33, 512), (296 * 1792 + 1, 512), (444 * 1792 + 1, 256), (740 * 1792 + 1, 12)])
+def test_tiles_of_whole_waves(tiga, items, F):
+    """Wide rows leave room for one to three CTAs per SM and the backward for five: sizes at which one wave of the longest tiles
+    becomes two waves of shorter ones, with workspaces of exactly the reported size (all three reducers)."""
+    n = items // 9
+    E = items - n
+    rng = np.random.default_rng(F)
+    deg = np.bincount(np.minimum((n * rng.random(E) ** 3).astype(np.int64), n - 1), minlength=n)
+    rowptr = np.concatenate([[0], np.cumsum(deg)])
+    col = rng.integers(0, 2000, E).astype(np.int32)
+    x, w, gy = gen.normal_features(2000, F, 5, 31), gen.edge_weights(E, 6), gen.normal_features(n, F, 5, 32)
+    g, xd, wd, res = _check_forward(tiga, rowptr, col, x, w)
+    if F < 64:
+        _check_backward(tiga, rowptr, col, x, w, gy, g, xd, wd, res)
