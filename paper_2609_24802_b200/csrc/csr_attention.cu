@@ -5,11 +5,11 @@
 // an arbitrary CSR is graph attention).
 //
 // Same schedule as the sum / max reducers: merge-path tiles of "row ends + edges", one CTA per
-// tile, edges split evenly over workers of G lanes, each lane owning 16 bytes of the query, key
-// and value rows.  A worker walks its span in edge order with the streaming state of Section 5
-// in registers: running maximum m (in units of log 2), mass l, accumulator o.  Four edges are
-// taken per step: four key rows and four value rows are gathered at once, the four dot products
-// are reduced over the worker's lanes by shuffles, the state is rescaled once per step.  Partial
+// tile, edges split evenly over workers of G lanes, each lane owning 16 or 32 bytes of the query,
+// key and value rows.  A worker walks its span in edge order with the streaming state of Section 5
+// in registers: running maximum m (in units of log 2), mass l, accumulator o.  Four (two) edges are
+// taken per step: their key and value rows are gathered at once, the dot products are reduced
+// over the worker's lanes by shuffles, the state is rescaled once per step.  Partial
 // states at the ends of a span go to shared memory and are combined in edge order with the
 // paper's rule  m = max(ma, mb), l = e^(ma-m) la + e^(mb-m) lb, o likewise;  a tile's trailing
 // partial row is a carry-out in the workspace.  A finished row is stored finalised (o / l and
@@ -56,9 +56,14 @@ struct AttState {
 };
 
 // EXACT: the row fills the worker exactly (D == 4 G VPL): constant row stride, no lane predicates.
-// VPL vectors per lane: from 32 features on a lane owns two 16-byte pieces of every row and a worker takes two edges per step
-// instead of four, which keeps as many bytes in flight and halves the shuffles and exponentials per edge (R-MAT scale 20,
-// D = 64: 820 -> 743 us; 100 k rows, D = 128: 217 -> 172 us; causal, 4096 rows: 258 -> 239 us).
+// VPL vectors per lane: with rows of exactly 64 or 128 features a lane owns two 16-byte pieces of every row and a worker takes two
+// edges per step instead of four, which keeps as many bytes in flight and halves the shuffles and exponentials per edge (R-MAT
+// scale 20, 16 M edges: D = 64 847 -> 761 us, D = 128 1392 -> 1295 us; 100 k rows of 16, D = 64 126 -> 110 us; rows of 64
+// and more edges from small tables lose 2 to 8 %).  Narrower rows and rows that do not fill the worker keep one piece:
+// with two, 50,000 rows of 32 edges, D = 32, took 67 instead of 52 us, D = 20 71 instead of 54 us, R-MAT scale 20, D = 100,
+// 1516 instead of 1427 us (R-MAT of 100 k rows, D = 32, gained: 97 instead of 105 us).
+// Four CTAs per SM by the launch bound (64 registers): without it mesh of 30^3, D = 16, 36 instead of 28 us, R-MAT scale 20,
+// D = 16, 480 instead of 419 us.
 template <int G, int VPL, typename IT, bool EXACT>
 __global__ void __launch_bounds__(CSR_THREADS, 4) csr_attention_kernel(const CsrParams p) {
     constexpr int NW = CSR_THREADS / G;          // workers per CTA
@@ -335,9 +340,12 @@ static tiga_status launch_attention_t(const CsrParams& p, cudaStream_t s) {
 
 template <typename IT>
 static tiga_status launch_attention(const CsrParams& p, cudaStream_t s) {
+    // lanes per worker: the row's 16-byte vectors rounded up to a power of two, half of that where two per lane fill them (above)
     if (p.nvec <= 4) return launch_attention_t<4, 1, IT>(p, s);
-    if (p.nvec <= 8) return launch_attention_t<4, 2, IT>(p, s);
-    if (p.nvec <= 16) return launch_attention_t<8, 2, IT>(p, s);
+    if (p.nvec <= 8) return launch_attention_t<8, 1, IT>(p, s);
+    if (p.nvec < 16) return launch_attention_t<16, 1, IT>(p, s);
+    if (p.nvec == 16) return launch_attention_t<8, 2, IT>(p, s);
+    if (p.nvec < 32) return launch_attention_t<32, 1, IT>(p, s);
     return launch_attention_t<16, 2, IT>(p, s);
 }
 

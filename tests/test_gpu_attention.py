@@ -55,7 +55,7 @@ def test_causal_attention_example(tiga):
     assert np.allclose(host(out)[0], v[0], rtol=1e-6, atol=1e-7)      # token zero reads only itself
 
 
-@pytest.mark.parametrize("D", [4, 8, 16, 24, 32, 64, 100, 128])
+@pytest.mark.parametrize("D", [4, 8, 16, 20, 24, 32, 36, 60, 64, 68, 100, 124, 128])
 def test_widths_on_a_skewed_graph(tiga, D):
     c = gen.config("cfg1", 11, scale=12, F=4)                          # R-MAT: empty rows, one very long row
     q, k, v = _qkv(c["n"], c["n"], D, 12)
