@@ -136,10 +136,7 @@ struct Tile {
 };
 
 // Stage the tile: s_ptr[k] = clamp(rowptr[i0+k] - e0, -1, ne+1) for k = 0..nrows, col and w.
-// index with one pad word per 32: threads that read consecutive runs of 8 stay conflict free
-static __device__ __forceinline__ int pad32(int i) { return i + (i >> 5); }
-
-template <typename IT, bool PADDED = false>
+template <typename IT>
 __device__ Tile stage_tile(const CsrParams& p, int* s_ptr, int* s_col, float* s_w, long long* s_coord) {
     const IT* rowptr = static_cast<const IT*>(p.rowptr);
     const long long total = p.n_dst + p.n_edges;
@@ -171,12 +168,11 @@ __device__ Tile stage_tile(const CsrParams& p, int* s_ptr, int* s_col, float* s_
         s_ptr[k] = (int)v;
     }
     for (int k = threadIdx.x; k < t.ne; k += CSR_THREADS) {
-        const int kk = PADDED ? pad32(k) : k;
-        s_col[kk] = checked(ld_stream(p.col + t.e0 + k), p.n_src, CHECK_SOURCE);
-        s_w[kk] = p.w ? ld_stream(p.w + t.e0 + k) : 1.f;
+        s_col[k] = checked(ld_stream(p.col + t.e0 + k), p.n_src, CHECK_SOURCE);
+        s_w[k] = p.w ? ld_stream(p.w + t.e0 + k) : 1.f;
     }
     // a few valid entries behind the last edge: unrolled loops may load (never use) past their span
-    if (threadIdx.x < CSR_PAD) { s_col[(PADDED ? pad32(t.ne) : t.ne) + threadIdx.x] = 0; s_w[(PADDED ? pad32(t.ne) : t.ne) + threadIdx.x] = 0.f; }
+    if (threadIdx.x < CSR_PAD) { s_col[t.ne + threadIdx.x] = 0; s_w[t.ne + threadIdx.x] = 0.f; }
     __syncthreads();
     return t;
 }

@@ -8,7 +8,8 @@
 //   1. binning: cell id per point + per-cell counts, exclusive scan (reduce-then-scan, no
 //      inter-CTA waiting), scatter into cell order, per-cell rank sort by point id (which
 //      makes the scatter stable and therefore unique), sorted copy of the positions;
-//   2. traversal: one warp per query cell stages the 27 neighbouring cells (wrapped or
+//   2. traversal: a warp takes a share of the points in cell order (walk_unit) as runs of sparse
+//      cells, single cells and slices of dense ones; it stages the neighbouring cells (wrapped or
 //      clipped, contiguous ranges of the cell-ordered points) in shared memory, tests one
 //      staged candidate per lane against a batch of four or eight queries, compacts accepted
 //      (source, weight) pairs into one list per query and consumes the lists with groups of
@@ -341,9 +342,9 @@ __global__ void validate_points_kernel(const float* __restrict__ pos, long long 
 
 // ------------------------------------------------------------------------------ traversal
 
-// One warp per query cell.
-//   staging : the candidates of the 27-cell stencil (contiguous ranges of the cell-sorted
-//             positions) are copied once into shared memory in the frame of the query cell:
+// One warp per run of sparse cells, cell, or slice of a dense cell (walk_unit).
+//   staging : the candidates of the stencil (contiguous ranges of the cell-sorted
+//             positions) are copied once into shared memory in the frame of the run:
 //             original coordinates, except that in a dimension whose stencil wraps around a
 //             periodic face the points next to the upper face move down by the box length
 //             (exact).  The fp32 displacement of a pair is then accurate to half an ulp of the
@@ -377,7 +378,7 @@ template <int MODE> struct TravSmem {
 };
 
 // MODE 0: Gaussian (DIST = false) or distance-weighted (DIST = true) forward;
-// 2: Gaussian backward.  MI: some periodic dimension has a single cell (explicit minimum image).
+// 2: Gaussian backward.  MI: some periodic dimension has three cells or fewer (explicit minimum image).
 // VEC: 0 = scalar feature accesses (F % 4 != 0, forward only); 1 = 128-bit accesses, F % 4 == 0;
 // 2 = additionally F == 4 LF exactly, so the row stride is a compile-time constant.
 template <int MODE, int LF, bool DIST, bool MI, int VEC>
@@ -727,6 +728,10 @@ __device__ __forceinline__ void traverse_slice(const RadiusParams& p, const int 
     }
 }
 
+// Warps per SM that the registers must allow: 28 in the forward (72 registers, 12 to 56 bytes spilled), 16 in the backward (up to
+// 124, no spills).  28 / 24 / 20: 400 k points, 12 neighbours, F = 32 212 / 220 / 237 us, 50 k points, 45 neighbours 89 / 89 / 91 us,
+// 20 k clustered points 235 / 220 / 218 us, lattice of 8 points a cell, F = 128, 112 / 112 / 101 us.  16 / 20 / 12: F = 32 282 / 286 /
+// 343 us, F = 128 533 / 600 / 533 us.
 template <int MODE, int LF, bool DIST, bool MI, int VEC = 1>
 __global__ void __launch_bounds__(TRAV_THREADS, (MODE == 0 ? 28 : 16) / TRAV_WARPS) radius_traverse_kernel(const __grid_constant__ RadiusParams p) {
     extern __shared__ __align__(16) unsigned char s_raw[];
@@ -834,7 +839,7 @@ tiga_status fill_params(RadiusParams* p, long long n, float r, const tiga_box* b
     bool single_periodic = false;      // some periodic dimension uses the explicit minimum image (two roundings more)
     for (int d = 0; d < 3; ++d) {
         p->nc[d] = nc[d]; p->invh[d] = invh[d];
-        p->len[d] = box->len[d]; p->inv_len[d] = 1.f / box->len[d];
+        p->len[d] = box->len[d];
         p->hcell[d] = box->len[d] / (float)nc[d];
         p->periodic[d] = box->periodic[d] ? 1 : 0;
         if (p->periodic[d] && nc[d] <= 3) single_periodic = true;

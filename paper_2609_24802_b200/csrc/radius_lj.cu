@@ -2,7 +2,7 @@
 // energy, sum reducer (radius_direct.cuh).
 //
 // Every row walks its full neighbourhood, which forms each unordered pair twice but needs no atomics, no memset and no
-// list, and is reproducible.  Bound by instruction issue (75 % of the slots): per cell of 12.6 particles 1430 warp
+// list, and is reproducible.  Bound by instruction issue (73.5 % of the slots): per cell of 12.6 particles 1430 warp
 // instructions stage 340 candidates (195 survive the pruning), 760 test them, 1280 form the forces, 300 add up and store.
 // 4.1 M particles 1467 -> 1321 us against the earlier form (every unordered pair once through per-query lists, the
 // opposite force added with a vector atomic); 28 warps per SM measured fastest (24 1350, 32 1343 us).

@@ -35,7 +35,6 @@ struct RadiusParams {
     float r2_mid, r2_band;    // its centre and half width
     double r2_exact;          // (double)r * (double)r
     float len[3];
-    float inv_len[3];
     int periodic[3];
     int nc[3];
     float invh[3];

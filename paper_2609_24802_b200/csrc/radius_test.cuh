@@ -5,7 +5,7 @@
 // per component and forms both squared distances with packed instructions.  Every query of the run gets
 // LPQ = 32 / queries lanes.  A lane keeps its query in registers, walks the candidate pairs sub, sub + LPQ, ... and
 // shifts one sign bit per candidate into a mask, which costs about seven instructions per 32 tests; only accepted
-// candidates (one in four at the usual density) are looked at again, one at a time per lane.
+// candidates (one in four at the usual density) are looked at again, two at a time per lane.
 #pragma once
 #include "radius_shared.cuh"
 
