@@ -96,7 +96,8 @@ def test_every_split_of_lanes_and_staged_features(tiga, f_in, hidden):
     """32 / hidden pairs advance together and features are staged four at a time: every combination, on a cloud of 30 to
     250 neighbours that spans slices, several stage chunks (144 candidates), list batches (176 pairs) and wrapped
     faces.  (No query has only a few neighbours: a single message, or a single pair's gradient, may cancel to nearly
-    nothing, and a tolerance relative to it would test the rounding of the terms it is formed from.)"""
+    nothing, and a tolerance relative to it would test the rounding of the terms it is formed from.  The thin background of
+    test_messages_that_cancel_lose_no_precision has such queries, in a norm over all rows.)"""
     n = 1500
     pos = (gen.uniform_points(n, 70 + f_in) * np.float32(0.35) + np.float32(0.8)) % np.float32(1.0)
     x, gy = gen.normal_features(n, f_in, 72, 31), gen.normal_features(n, 3, 72, 32)
