@@ -5,7 +5,7 @@
 // instead, which keeps the result exact (keys are compared, never approximated) and removes the
 // quadratic scan on inputs of roughly even density:
 //
-//   knn_cells_kernel  one warp per cell.  The points are binned with a cell edge a little above a
+//   knn_cells_kernel  a warp per share of the points in cell order, a cell (a slice of a dense one) at a time.  The points are binned with a cell edge a little above a
 //                     search radius h chosen so that a ball of radius h holds about 2k points on
 //                     average.  Every point closer than h to a query of the cell lies in the
 //                     27-cell stencil, so a query that finds k keys <= h^2 there is finished: no
@@ -27,8 +27,7 @@
 // list's length, counts grow with the cube of the distance, and corrected by counting ballots); then every lane
 // counts the entries closer than its own, which is that entry's place in the row.  Equal distances and k > 24 go
 // through the general form, a bitonic network of shuffles over 32 keys at a time and merges, which orders
-// whole keys.  (Sorting every list took 225 of 520 warp instructions per query at k = 16, counting takes about 90; a
-// full list is trimmed for 60 instructions where sorting it took 500.)
+// whole keys.
 #include "radius_test.cuh"
 #include <type_traits>
 
