@@ -20,7 +20,7 @@
 // Bound by instruction issue (57 % of the slots, 28 and 49 M warp instructions) and the tail of the work units.  35,947 surface
 // points, 15.6 neighbours, 8 features, HID = 32: forward 121 -> 55 us, backward 512 -> 86 us against one lane per pair with
 // the weights read from shared memory (the earlier form, some 600 shared-memory reads per 32 pairs); 300 k uniform points,
-// 32 neighbours, HID = 16: 455 -> 383 and 1750 -> 603 us.
+// 32 neighbours, HID = 16: 455 -> 383 and 1750 -> 603 us.  (Sums that keep their precision, below, add 5 % to the surface's two passes.)
 //
 // The displacement is formed from coordinates relative to the corner of the query's cell and the pre-activation as one chain
 // of fused multiply-adds (bias, displacement, features): a ReLU switches on the last bit of that sum.
