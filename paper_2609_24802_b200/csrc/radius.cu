@@ -23,7 +23,7 @@
 // coordinates; a cell whose stencil wraps around a periodic face moves the points next to the
 // upper face down by the box length, which is exact in fp32, so every displacement is one
 // rounded subtraction of two stored coordinates, for wrapped pairs as for interior ones.
-#include "radius_direct.cuh"
+#include "radius_group_direct.cuh"
 #include <type_traits>
 
 namespace tiga {
@@ -245,7 +245,7 @@ __global__ void __launch_bounds__(SMALL_THREADS) bin_small_kernel(const RadiusPa
     constexpr int PP = SMALL_POINTS / SMALL_THREADS, PC = SMALL_CELLS / SMALL_THREADS;
     const int tid = threadIdx.x;
     for (int k = tid; k < p.ncells; k += SMALL_THREADS) s_start[k] = 0;
-    if (tid == 0) { s_ndense = 0; *p.queue_n = 0; }
+    if (tid == 0) { s_ndense = 0; *p.queue_n = 0; *p.failed = 0; }
     __syncthreads();
     float v[PP][3];
     int c[PP], slot[PP];
@@ -742,18 +742,18 @@ __global__ void __launch_bounds__(TRAV_THREADS, (MODE == 0 ? 28 : 16) / TRAV_WAR
 // ------------------------------------------------------------------------------ at most four features
 // Forward with NF <= 4 features per point (the distance-weighted scalar sum among them).  A gather by groups of
 // lanes would leave most of the warp idle on such rows, so nothing is gathered: the features are staged with
-// the candidates and summed where a pair is accepted (radius_direct.cuh).
+// the candidates and summed where a pair is accepted (radius_group_direct.cuh; figures of the cells' form, radius_direct.cuh, here).
 // Bound by instruction issue and by the latency of the staging loads.  Against the list kernel below four features:
 // F = 4, n = 1M, 32 neighbours 616 -> 393 us; F = 1, n = 131072, distance-weighted 108 -> 58 us; F = 2, n = 300k,
 // 8 neighbours 218 -> 100 us.  Warps per SM measured: F = 1 28 / 24 / 20: 57 / 61 / 65 us; F = 3 401 / 394 / 381 us.
 template <int NF, bool DIST>
 struct SumMsg {
-    static constexpr int CAP = 256, STAGED = NF, OUT = NF, WARPS = NF <= 2 ? 28 : 20;
+    static constexpr int CAP = 256, STAGED = NF, OUT = NF, WARPS = NF <= 2 ? 28 : 20, GROUP_CAP = 384, GROUP_WARPS = NF <= 2 ? 20 : 16;
     static constexpr float OUTSIDE = 1.f;                  // any weight that is finite for every sigma
-    static constexpr int FEAT_STRIDE = CAP + 4;
     float neg_c2;
     // exp(-d2/(2 s^2)) = 2^(d2 * neg_c2)
     __device__ __forceinline__ explicit SumMsg(const RadiusParams& p) : neg_c2(!DIST ? -1.4426950408889634f / (2.f * p.p0 * p.p0) : 0.f) {}
+    template <int FEAT_STRIDE>
     __device__ __forceinline__ void pair(f32x2 (&acc)[NF], const float da, const float db, f32x2, f32x2, f32x2, const float* xa, const float* xb) const {
         const f32x2 val = DIST ? pack2(sqrtf(da), sqrtf(db)) : pack2(fast_exp2(da * neg_c2), fast_exp2(db * neg_c2));
 #pragma unroll
@@ -794,6 +794,7 @@ RadiusLayout carve_radius(RadiusParams* p, void* ws, int32_t** fill) {
     p->cnt = cv.take<int32_t>(2 * nc + 2 + 16);     // counts, then the scatter cursors, then the length of the dense-cell queue
     p->b_count = p->cnt + 2 * nc + 2;
     p->queue_n = p->b_count + 2;
+    p->failed = p->b_count + 3;
     *fill = p->cnt + nc;
     p->cell = cv.take<int32_t>(n);
     p->cell_start = cv.take<int32_t>(nc + 1);
@@ -810,9 +811,13 @@ RadiusLayout carve_radius(RadiusParams* p, void* ws, int32_t** fill) {
 // neighbours: 139 -> 48 and 209 -> 78 us; nothing is joined at 32 neighbours).
 // Cells along x that are joined at most: enough for about RUN_QUERIES / 2 points at the mean density; a run's stencil must
 // not meet itself around a periodic face (the frame shift needs two cells between).
+static int run_room(const RadiusParams& p, const int most) {
+    const int room = !p.periodic[0] ? most : p.nc[0] < 4 ? 1 : p.nc[0] - 3;
+    return room < most ? room : most;
+}
 static int run_length(const RadiusParams& p) {
     long long r = p.n > 0 ? (long long)p.ncells * (RUN_QUERIES / 2) / p.n : 1;
-    const long long room = !p.periodic[0] ? RUN_CELLS : p.nc[0] < 4 ? 1 : p.nc[0] - 3;
+    const long long room = run_room(p, RUN_CELLS);
     r = r > room ? room : r;
     r = r > RUN_CELLS ? RUN_CELLS : r;
     return r < 1 ? 1 : (int)r;
@@ -847,6 +852,7 @@ tiga_status fill_params(RadiusParams* p, long long n, float r, const tiga_box* b
     p->ncells = nc[0] * nc[1] * nc[2];
     p->run = run_length(*p);
     p->unit = unit_length(*p);
+    p->group_run = run_room(*p, GROUP_RUN);
     // (slices of 16 from cells above 64 points, the earlier rule, against this one: 40 k clustered points, F = 8, forward +
     // backward 1972 -> 594 us; 4 k, F = 16, 330 -> 109 us; 30 k uniform points with 45 neighbours 155 -> 140 us)
     cut_cells(*p, 148 * 42);

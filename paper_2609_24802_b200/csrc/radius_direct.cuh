@@ -2,14 +2,14 @@
 // lane adds the messages of its accepted candidates in registers.  No lists, no gathers, no atomics.
 //
 // Msg supplies the message:
-//   CAP             candidates the stage holds
+//   CAP, WARPS      candidates the stage holds, and warps per SM
 //   STAGED          features per point that are staged with the candidates
 //   OUT             sums per query
 //   OUTSIDE         squared distance given to a half that adds nothing (an absent or refused candidate); its features read as
 //                   zero, and the message of that distance times zero must be zero (no decay with the distance is assumed:
 //                   a Gaussian as wide as fp32 allows gives every distance the weight one)
 //   Msg(p)          constants
-//   pair(...)       adds the messages of two accepted candidates to acc[OUT], one per half
+//   pair<STRIDE>(...)  adds the messages of two accepted candidates to acc[OUT], one per half; STRIDE between staged features
 //   scale(f, v)     the stored value of sum f
 #pragma once
 #include "radius_test.cuh"
@@ -119,7 +119,7 @@ __device__ __forceinline__ void direct_slice(const RadiusParams& p, const int (&
                     if (two && db > p.r2_mid - p.r2_band && !exact_pair(p, qid, stage.id[sb])) { db = Msg::OUTSIDE; fb = STAGE_CAP; --cnt; }
                 }
                 if (!two) db = Msg::OUTSIDE;
-                msg.pair(acc2, da, db, dx, dy, dz, s_feat + fa, s_feat + fb);
+                msg.template pair<SM::FEAT_STRIDE>(acc2, da, db, dx, dy, dz, s_feat + fa, s_feat + fb);
             }
             float acc[OUT];
 #pragma unroll
@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(TRAV_THREADS, Msg::WARPS / TRAV_WARPS) radius_
 }
 
 template <typename Msg, bool MI>
-static tiga_status launch_direct_t(const RadiusParams& p, cudaStream_t s) {
+static tiga_status launch_direct_slices(const RadiusParams& p, cudaStream_t s) {
     constexpr int smem = DirectSmem<Msg>::PER_WARP * TRAV_WARPS;
     auto kern = radius_direct_kernel<Msg, MI>;
     if (smem > 48 * 1024) TIGA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));

@@ -1,0 +1,163 @@
+// Traversal that consumes a pair where it is accepted, by groups of queries (radius_group.cuh): the lanes of a query add the
+// messages of its accepted candidates in registers.  Nothing is gathered, no atomics.  The messages are those of
+// radius_direct.cuh, with GROUP_CAP and GROUP_WARPS in the places of CAP and WARPS where cells hold several points.
+#pragma once
+#include "radius_direct.cuh"
+#include "radius_group.cuh"
+#include <type_traits>
+
+namespace tiga {
+
+template <typename Msg, bool SPARSE> struct GroupDirectSmem {
+    using Stage = std::conditional_t<SPARSE, GroupStage<256, 560>, GroupStage<Msg::GROUP_CAP, 1088>>;
+    static constexpr int WARPS = SPARSE ? 24 : Msg::GROUP_WARPS;
+    static constexpr int STAGED = Msg::STAGED, STAGE_BYTES = Stage::BYTES;
+    static constexpr int FEAT_STRIDE = Stage::SLOTS;                        // the entry of the far slot stays zero
+    static constexpr int PER_WARP = STAGE_BYTES + STAGED * FEAT_STRIDE * 4;
+    static_assert(PER_WARP % 16 == 0, "the stage is accessed as 16-byte vectors");
+};
+
+// MI: some periodic dimension has three cells or fewer and uses the explicit minimum image.
+// COUNT: the numbers of neighbours are wanted.
+template <typename Msg, bool SPARSE, bool MI, bool COUNT>
+__device__ __forceinline__ bool direct_group(const RadiusParams& p, typename GroupDirectSmem<Msg, SPARSE>::Stage& st, float* s_feat, const int (&cell)[3], const int run, const int qs, const int nq) {
+    using SM = GroupDirectSmem<Msg, SPARSE>;
+    constexpr int OUT = Msg::OUT, NF = Msg::STAGED;
+    constexpr unsigned FULL = 0xffffffffu;
+    using Stage = typename SM::Stage;
+    const int lane = threadIdx.x & 31;
+    const Msg msg(p);
+    Group<MI, Stage> grp(p, st, cell, run, qs, nq);
+
+    // the lane's query and its sums
+    const int q = lane >> grp.lsh, lpq = 1 << grp.lsh, sub = lane & (lpq - 1);
+    const float4 qv = grp.query(q < nq ? q : 0);
+    const f32x2 qx2 = dup2(qv.x), qy2 = dup2(qv.y), qz2 = dup2(qv.z);
+    f32x2 acc2[OUT];
+    int cnt = 0;
+#pragma unroll
+    for (int f = 0; f < OUT; ++f) acc2[f] = 0ull;
+
+    for (int k0 = 0; k0 < grp.sten.total; k0 += Stage::CAPACITY) {
+        const int ns = grp.stage(k0);
+        if (ns == 0) return false;
+        if constexpr (NF > 0) {
+            for (int b = lane; b - lane < ns; b += 128) {          // four rows in flight
+                float x[4][NF];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int id = b + 32 * u < ns ? __float_as_int(grp.st.c[b + 32 * u].w) : -1;
+#pragma unroll
+                    for (int f = 0; f < NF; ++f) x[u][f] = 0.f;
+                    if (id < 0) continue;
+                    const float* xr = p.feat + (size_t)(unsigned)checked(id, p.n, CHECK_POINT) * NF;
+                    if constexpr (NF == 4) {
+                        const float4 x4 = __ldg(reinterpret_cast<const float4*>(xr));
+                        x[u][0] = x4.x; x[u][1] = x4.y; x[u][2] = x4.z; x[u][3] = x4.w;
+                    } else {
+#pragma unroll
+                        for (int f = 0; f < NF; ++f) x[u][f] = __ldg(xr + f);
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    if (b + 32 * u >= ns) continue;
+#pragma unroll
+                    for (int f = 0; f < NF; ++f) s_feat[f * SM::FEAT_STRIDE + b + 32 * u] = x[u][f];
+                }
+            }
+        }
+        GroupMask<Stage::WORDS> mask;
+        grp.test(ns, k0, mask);
+        grp.lists(ns, mask, [&](const int first, const int end) {
+            for (int j = first + 2 * sub; j < end; j += 2 * lpq) {
+                const unsigned two = *reinterpret_cast<const unsigned*>(grp.st.list + j);
+                unsigned sa = two & 0xffffu, sb = two >> 16;
+                const float4 ca = *reinterpret_cast<const float4*>(reinterpret_cast<const unsigned char*>(st.c) + sa);
+                const float4 cb = *reinterpret_cast<const float4*>(reinterpret_cast<const unsigned char*>(st.c) + sb);
+                f32x2 dx, dy, dz;
+                if constexpr (!MI) {
+                    dx = sub2(qx2, pack2(ca.x, cb.x));
+                    dy = sub2(qy2, pack2(ca.y, cb.y));
+                    dz = sub2(qz2, pack2(ca.z, cb.z));
+                } else {
+                    dx = pack2(grp.delta(0, qv.x, ca.x), grp.delta(0, qv.x, cb.x));
+                    dy = pack2(grp.delta(1, qv.y, ca.y), grp.delta(1, qv.y, cb.y));
+                    dz = pack2(grp.delta(2, qv.z, ca.z), grp.delta(2, qv.z, cb.z));
+                }
+                float da, db;
+                unpack2(fma2(dz, dz, fma2(dy, dy, mul2(dx, dx))), da, db);
+                bool in_a = da <= p.r2_mid, in_b = db <= p.r2_mid;
+                const float ea = fabsf(da - p.r2_mid), eb = fabsf(db - p.r2_mid);
+                if (fminf(ea, eb) <= p.r2_band) {                  // within the fp32 error band around the cutoff: decided in fp64
+                    if (ea <= p.r2_band) in_a = exact_pair(p, __float_as_int(qv.w), __float_as_int(ca.w));
+                    if (eb <= p.r2_band) in_b = exact_pair(p, __float_as_int(qv.w), __float_as_int(cb.w));
+                }
+                if (!in_a) { da = Msg::OUTSIDE; sa = 16 * Stage::FAR; }
+                if (!in_b) { db = Msg::OUTSIDE; sb = 16 * Stage::FAR; }
+                if (COUNT) cnt += (int)in_a + (int)in_b;
+                msg.template pair<SM::FEAT_STRIDE>(acc2, da, db, dx, dy, dz, reinterpret_cast<const float*>(reinterpret_cast<const unsigned char*>(s_feat) + (sa >> 2)),
+                         reinterpret_cast<const float*>(reinterpret_cast<const unsigned char*>(s_feat) + (sb >> 2)));
+            }
+        });
+    }
+    float acc[OUT];
+#pragma unroll
+    for (int f = 0; f < OUT; ++f) { float lo, hi; unpack2(acc2[f], lo, hi); acc[f] = lo + hi; }
+    for (int o = 1; o < lpq; o <<= 1) {
+#pragma unroll
+        for (int f = 0; f < OUT; ++f) acc[f] += __shfl_xor_sync(FULL, acc[f], o);
+        if (COUNT) cnt += __shfl_xor_sync(FULL, cnt, o);
+    }
+    if (q < nq && sub == 0) {
+        const int qid = checked(__float_as_int(qv.w), p.n, CHECK_POINT);
+#pragma unroll
+        for (int f = 0; f < OUT; ++f) acc[f] = msg.scale(f, acc[f]);
+        float* o = p.out + (size_t)qid * OUT;
+        if constexpr (OUT == 4) {
+            *reinterpret_cast<float4*>(o) = make_float4(acc[0], acc[1], acc[2], acc[3]);
+        } else {
+#pragma unroll
+            for (int f = 0; f < OUT; ++f) o[f] = acc[f];
+        }
+        if (COUNT) p.count[qid] = cnt;
+    }
+    return true;
+}
+
+template <typename Msg, bool SPARSE, bool MI, bool COUNT>
+__global__ void __launch_bounds__(32, (GroupDirectSmem<Msg, SPARSE>::WARPS)) radius_group_kernel(const __grid_constant__ RadiusParams p, const int unit) {
+    using SM = GroupDirectSmem<Msg, SPARSE>;
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    float* s_feat = reinterpret_cast<float*>(s_raw + SM::STAGE_BYTES);                   // [STAGED][FEAT_STRIDE]
+    if (threadIdx.x < SM::STAGED) s_feat[threadIdx.x * SM::FEAT_STRIDE + SM::Stage::FAR] = 0.f;
+    typename SM::Stage st(s_raw);
+    walk_groups(p, blockIdx.x, unit, [&](const int (&cell)[3], const int run, const int qs, const int nq) {
+        const bool ok = direct_group<Msg, SPARSE, MI, COUNT>(p, st, s_feat, cell, run, qs, nq);
+        if (!ok) group_failed(p, st);
+        return ok;
+    });
+}
+
+template <typename Msg, bool SPARSE, bool MI>
+static tiga_status launch_direct_group(const RadiusParams& p, cudaStream_t s) {
+    constexpr int smem = GroupDirectSmem<Msg, SPARSE>::PER_WARP;
+    static_assert(smem <= 48 * 1024, "no attribute needed");
+    auto kern = p.count ? radius_group_kernel<Msg, SPARSE, MI, true> : radius_group_kernel<Msg, SPARSE, MI, false>;
+    const int unit = group_unit(p.n);
+    kern<<<counted((unsigned)(((long long)p.n + unit - 1) / unit)), 32, smem, s>>>(p, unit);
+    return launch_status();
+}
+
+// Groups or cells and slices (radius_direct.cuh).  Groups need points that fill them: where cells hold less than 0.7 points on average
+// the input is a surface or clustered, and cells win (us, cells / groups: 100 k surface points, 16 neighbours 73 / 77; 40 k clustered
+// points 231 / 272).  Uniform points: 1 M, 32 neighbours, F = 1 392 / 367, F = 4 458 / 378; 4 neighbours, F = 1 288 / 239; 300 k,
+// 8 neighbours, F = 3 151 / 121; 30 k, 45 neighbours, F = 3 63 / 47.  Inputs that leave the machine half empty either way: 4 k, 16
+// neighbours, F = 1 24.3 / 25.2, but dense ones gain (Lennard-Jones, 1728 particles 24.9 / 23.7).
+template <typename Msg, bool MI>
+static tiga_status launch_direct_t(const RadiusParams& p, cudaStream_t s) {
+    if (10LL * p.n < 7LL * p.ncells || (p.n < 8192 && p.n < 8LL * p.ncells)) return launch_direct_slices<Msg, MI>(p, s);
+    return group_sparse(p) ? launch_direct_group<Msg, true, MI>(p, s) : launch_direct_group<Msg, false, MI>(p, s);
+}
+
+}  // namespace tiga

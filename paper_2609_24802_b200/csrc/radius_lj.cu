@@ -1,20 +1,22 @@
 // Lennard-Jones over the generated radius relation (paper Section 4.9): fused cell-list traversal, pair force and
-// energy, sum reducer (radius_direct.cuh).
+// energy, sum reducer (radius_group_direct.cuh).
 //
 // Every row walks its full neighbourhood, which forms each unordered pair twice but needs no atomics, no memset and no
-// list, and is reproducible.  Bound by instruction issue (73.5 % of the slots): per cell of 12.6 particles 1430 warp
-// instructions stage 340 candidates (195 survive the pruning), 760 test them, 1280 form the forces, 300 add up and store.
-// 4.1 M particles 1467 -> 1321 us against the earlier form (every unordered pair once through per-query lists, the
-// opposite force added with a vector atomic); 28 warps per SM measured fastest (24 1350, 32 1343 us).
-#include "radius_direct.cuh"
+// list in memory, and is reproducible.  Bound by instruction issue (two thirds of the slots): per group of 15.7 particles about 880 warp
+// instructions find and stage 470 candidates, 720 test them, 670 gather the accepted ones into lists, 830 form the forces.
+// 4.1 M particles with binning 1456 -> 1238 us against cells of 12.6 particles tested with packed fp32 instructions (300 instead of 200
+// warp instructions per particle); 20 warps per SM (what the stage allows) measured faster than 24 with 80 registers (1272 us),
+// units of 32 points faster than 16 (1262 us).
+#include "radius_group_direct.cuh"
 
 namespace tiga {
 
 struct LjMsg {
-    static constexpr int CAP = 256, STAGED = 0, OUT = 4, WARPS = 28;
+    static constexpr int CAP = 256, STAGED = 0, OUT = 4, WARPS = 28, GROUP_CAP = 512, GROUP_WARPS = 20;
     static constexpr float OUTSIDE = INFINITY;             // reciprocal 0: no force, no energy
     float s2, force, energy;
     __device__ __forceinline__ explicit LjMsg(const RadiusParams& p) : s2(p.p1 * p.p1), force(24.f * p.p0), energy(2.f * p.p0) {}
+    template <int>
     __device__ __forceinline__ void pair(f32x2 (&acc)[4], const float da, const float db, const f32x2 dx, const f32x2 dy, const f32x2 dz,
                                          const float*, const float*) const {
         const f32x2 inv = pack2(fast_rcp(da), fast_rcp(db));

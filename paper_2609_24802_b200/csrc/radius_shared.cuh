@@ -17,6 +17,7 @@ constexpr int QSLICE = 16;              // most queries of a slice of a dense ce
 constexpr int QDENSE = QSLICE + QSLICE / 2;   // most queries of one piece of work
 constexpr int UNIT_MAX = 32;            // most points per unit of work (at most 32: a lane each)
 constexpr int RUN_CELLS = 8;            // longest run of cells along x that one warp covers
+constexpr int GROUP_RUN = 16;           // most cells along x a group of queries spans
 constexpr int RUN_QUERIES = 16;         // points a warp joins cells for
 constexpr int SORT_DENSE = 256;         // a cell with more points than this is ordered by a sorting network, not by rank counting
 
@@ -55,10 +56,12 @@ struct RadiusParams {
     int32_t* blocksum;
     int run;                  // cells along x that a warp joins at most
     int unit;                 // points per warp (walk_unit)
+    int group_run;            // cells along x that a group of queries spans at most (walk_groups)
     int dense, slice;         // a cell with more than `dense` points is cut into slices of `slice` queries
     int* queue_n;             // length of the kNN queue (zeroed with the counts)
     int32_t* b_items;         // cells with more than SORT_DENSE points (queued by the scan), and how many
     int* b_count;
+    int* failed;              // set when a traversal's staged copies did not arrive (zeroed with the counts)
     // optional user copies of the plan
     int32_t* u_cell;
     int32_t* u_cell_start;

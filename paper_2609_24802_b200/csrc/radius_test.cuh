@@ -48,13 +48,19 @@ struct RunFrame {
 // The run's stencil: lanes 0..8 hold the (y, z) rows over the run's x range, lanes 9..17 the cell that row reaches
 // around a periodic x face.  begin: flattened position of the lane's range; s_delta maps a position to its source.
 struct RunStencil {
-    int begin, len, total;
-    __device__ __forceinline__ RunStencil(const RadiusParams& p, const int (&c)[3], const int run, int* s_delta) {
+    int begin, len, total, cs;             // cs: source of the lane's first position
+    __device__ __forceinline__ RunStencil(const RadiusParams& p, const int (&c)[3], const int run, int* s_delta) : RunStencil(p, c, run) {
+        const unsigned some = __ballot_sync(0xffffffffu, len > 0);
+        if (len > 0) s_delta[__popc(some & ((1u << (threadIdx.x & 31)) - 1u))] = cs - begin;
+        __syncwarp();
+    }
+    __device__ __forceinline__ RunStencil(const RadiusParams& p, const int (&c)[3], const int run) {
         constexpr unsigned FULL = 0xffffffffu;
         const int lane = threadIdx.x & 31;
         const int row = lane < 9 ? lane : lane - 9;
-        const int oy = row % 3 - 1, oz = row / 3 - 1;
-        int y = c[1] + oy, z = c[2] + oz, cs = 0;
+        const int oz = row >= 6 ? 1 : row >= 3 ? 0 : -1, oy = row - 3 * oz - 4;
+        int y = c[1] + oy, z = c[2] + oz;
+        cs = 0;
         bool ok = lane < 18;
         if (p.nc[1] == 1) { ok = ok && oy == 0; y = 0; }
         else if (y < 0) { if (p.periodic[1]) y += p.nc[1]; else ok = false; }
@@ -82,9 +88,6 @@ struct RunStencil {
         }
         total = __shfl_sync(FULL, begin, 31);
         begin -= len;
-        const unsigned some = __ballot_sync(FULL, len > 0);
-        if (len > 0) s_delta[__popc(some & ((1u << lane) - 1u))] = cs - begin;
-        __syncwarp();
     }
     // source of flattened position k0 + lane; `before` counts the ranges that began before k0 (start with -1).  The
     // ranges that begin in this window of 32 positions set one bit each: the bits at and below a lane count up to

@@ -537,3 +537,42 @@ def test_clustered_points_are_spread_over_many_warps(tiga):
     print(f"clustered: {p_c} pairs in {t_c:.3f} ms; uniform: {p_u} pairs in {t_u:.3f} ms")
     assert 0.7 * p_c < p_u < 1.4 * p_c
     assert t_c < 5.0 * t_u
+
+
+# (points, cutoff, box, periodic): units of 4, 8 and 16 points, sparse and dense cells on both sides of the two stages (fewer and more than
+# three points per cell), rows of cells that end inside a group, a run that nearly closes around the box (4 and 5 cells), explicit
+# minimum image (3 cells), more accepted candidates than the lists hold, a stencil of many stages (one cell, all points), lengths
+# far from one
+_GROUPS = [(8192, 0.05, (1, 1, 1), [0, 0, 0]), (11841, 0.05, (1, 1, 1), [0, 1, 1]), (24001, 0.035, (1, 1, 1), [0, 0, 0]),
+           (24001, 0.045, (1, 1, 1), [1, 1, 1]), (24001, 0.05, (1, 1, 1), [1, 0, 1]), (24001, 0.19, (1, 1, 1), [1, 1, 1]),
+           (11999, 0.24, (1, 1, 1), [1, 1, 1]), (11999, 0.3, (1, 1, 1), [1, 0, 1]), (8192, 0.9, (1, 1, 1), [0, 0, 0]),
+           (30011, 0.05, (4, 0.5, 0.5), [1, 1, 0]), (30011, 0.05, (0.23, 4, 1), [1, 0, 1]),
+           (24001, 50.0, (1024, 1024, 1024), [1, 1, 1]), (24001, 0.04 / 4096, (1 / 4096,) * 3, [0, 1, 0])]
+
+
+@pytest.mark.parametrize("n,r,box,periodic", _GROUPS)
+@pytest.mark.parametrize("F", [1, 4])
+def test_groups_of_queries(tiga, F, n, r, box, periodic):
+    box = np.asarray(box, np.float32)
+    pos = np.minimum(gen.uniform_points(n, 71) * box, np.nextafter(box, np.float32(0))).astype(np.float32)
+    x = gen.normal_features(n, F, 71, 31)
+    for kind in (tiga.MSG_GAUSS, tiga.MSG_DIST):
+        _check_gauss(tiga, pos, x, None, np.float32(r), box, periodic, np.float32(r) / 2, kind=kind, use_cells=r < 0.2 * box.min(), backward=False)
+
+
+@pytest.mark.parametrize("m", [21, 29])
+def test_groups_decide_pairs_at_the_cutoff_exactly(tiga, m):
+    """Lattices whose neighbours lie exactly at the cutoff, just inside and just outside."""
+    h = np.float32(1.0 / 32.0)
+    grid = (np.stack(np.meshgrid(*[np.arange(m)] * 3, indexing="ij"), -1).reshape(-1, 3) * h).astype(np.float32)
+    box = np.full(3, m, np.float32) * h
+    x = gen.normal_features(len(grid), 2, 5, 31)
+    for r in (h, np.nextafter(h, np.float32(0)), np.nextafter(h, np.float32(1)), np.float32(np.sqrt(2.0)) * h, 2 * h):
+        for periodic in ([0, 0, 0], [1, 1, 1]):
+            _check_gauss(tiga, grid, x, None, r, box, periodic, r, use_cells=True, backward=False)
+
+
+@pytest.mark.parametrize("n", [8, 9, 15, 16, 17, 33, 700])
+def test_lennard_jones_in_one_cell(tiga, n):
+    pos = _separated_points(n, np.full(3, 6.0, np.float32), 9, 0.45)
+    _check_lj(tiga, pos, np.float32(5.9), np.full(3, 6.0, np.float32), [0, 0, 0])
