@@ -176,3 +176,23 @@ def test_ties_that_come_and_go_within_a_warp(tiga, k):
     pos = np.concatenate([lattice, gen.uniform_points(6000, 55)]).astype(np.float32)
     pos = pos[np.random.default_rng(5).permutation(len(pos))]
     _check(tiga, pos, gen.normal_features(len(pos), 2, 56, 31), k)
+
+
+@pytest.mark.parametrize("k", [1, 7, 32])
+@pytest.mark.parametrize("shape", ["line", "corner", "two"])
+def test_queries_far_from_their_neighbours(tiga, shape, k):
+    """Neighbours several shells of cells away: on a line, around one dense corner, in two blobs at opposite faces."""
+    rng = np.random.default_rng(3)
+    n = 3001
+    if shape == "line":
+        pos = np.zeros((n, 3)) + 0.5
+        pos[:, 0] = rng.random(n) ** 3
+    elif shape == "corner":
+        pos = rng.random((n, 3)) ** 6
+    else:
+        pos = rng.random((n, 3)) * 0.01 + np.where(rng.random((n, 1)) < 0.998, 0.0, 0.98)
+    pos = np.minimum(pos, 1.0 - 2.0 ** -24).astype(np.float32)
+    x = gen.normal_features(n, 3, 5, 31)
+    idx, d2, y, A = oracle.knn(pos, x, k)
+    out, nbr, nd2, _ = tiga.tiga_apply_knn(dev(pos, torch), dev(x, torch), k, np.ones(3, np.float32))
+    assert np.array_equal(host(nbr), idx) and np.array_equal(host(nd2), d2) and rel_err(host(out), y, A) <= SUM_TOL
