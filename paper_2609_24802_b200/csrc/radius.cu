@@ -32,6 +32,7 @@ constexpr int RAD_THREADS = 256;
 constexpr int SCAN_BLOCK = 2048;   // elements per CTA in the scan passes
 constexpr int SMALL_POINTS = 4096, SMALL_CELLS = 8192, SMALL_THREADS = 1024;     // inputs binned by one CTA in one launch
 constexpr int SMALL_DENSE = 64;        // there, longest cell ordered by counting
+constexpr int SCAN_FOLD_CHUNKS = 2048; // up to this many chunks every CTA of the last pass adds up the totals before its own
 constexpr int SCAN_SMALL_CHUNKS = 4;   // up to this many chunks are scanned by one CTA in one launch
 
 // ------------------------------------------------------------------------------ binning
@@ -87,7 +88,7 @@ __global__ void scan_reduce_kernel(const RadiusParams p) {
     if (threadIdx.x == 0) p.blocksum[blockIdx.x] = total;
 }
 
-// pass B: one CTA turns the totals into exclusive offsets (sequential over chunks)
+// pass B, above SCAN_FOLD_CHUNKS chunks: one CTA turns the totals into exclusive offsets (sequential over chunks)
 __global__ void scan_blocksums_kernel(const RadiusParams p, int nblocks) {
     __shared__ int s_warp[33];
     __shared__ int s_carry;
@@ -136,10 +137,20 @@ static __device__ void scan_finish(const RadiusParams& p) {
     if (p.u_cell_start) p.u_cell_start[p.ncells] = p.n;
 }
 
-// pass C: exclusive scan inside every CTA's chunk plus its offset -> cell_start
-__global__ void scan_apply_kernel(const RadiusParams p) {
+// pass C: exclusive scan inside every CTA's chunk plus its offset -> cell_start.  totals: the CTA adds up the totals of the chunks
+// before its own, which pass B has not turned into offsets.  (A launch less: 131 k points, scalar sum 85.8 -> 81.7 us;
+// 30 k points, F = 8 49 -> 45 us.)
+__global__ void scan_apply_kernel(const RadiusParams p, const bool totals) {
     __shared__ int s_warp[33];
-    scan_chunk(p, blockIdx.x, p.blocksum[blockIdx.x], s_warp);
+    int offset = 0;
+    if (totals) {
+        int v = 0;
+        for (int k = threadIdx.x; k < (int)blockIdx.x; k += blockDim.x) v += p.blocksum[k];
+        block_exclusive_scan(v, s_warp, &offset);
+    } else {
+        offset = p.blocksum[blockIdx.x];
+    }
+    scan_chunk(p, blockIdx.x, offset, s_warp);
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == blockDim.x - 1) scan_finish(p);
 }
 
@@ -883,8 +894,9 @@ tiga_status run_binning(RadiusParams& p, int32_t* fill, int nblocks, cudaStream_
         scan_small_kernel<<<counted(1), RAD_THREADS, 0, s>>>(p, nblocks);
     } else {
         scan_reduce_kernel<<<counted(nblocks), RAD_THREADS, 0, s>>>(p);
-        scan_blocksums_kernel<<<counted(1), 1024, 0, s>>>(p, nblocks);
-        scan_apply_kernel<<<counted(nblocks), RAD_THREADS, 0, s>>>(p);
+        const bool totals = nblocks <= SCAN_FOLD_CHUNKS;
+        if (!totals) scan_blocksums_kernel<<<counted(1), 1024, 0, s>>>(p, nblocks);
+        scan_apply_kernel<<<counted(nblocks), RAD_THREADS, 0, s>>>(p, totals);
     }
     bin_scatter_kernel<<<counted(pb), 256, 0, s>>>(p, fill);
     const long long dense_cells = (long long)p.n / SORT_DENSE + 1;          // at most this many cells can be dense

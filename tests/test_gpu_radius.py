@@ -576,3 +576,9 @@ def test_groups_decide_pairs_at_the_cutoff_exactly(tiga, m):
 def test_lennard_jones_in_one_cell(tiga, n):
     pos = _separated_points(n, np.full(3, 6.0, np.float32), 9, 0.45)
     _check_lj(tiga, pos, np.float32(5.9), np.full(3, 6.0, np.float32), [0, 0, 0])
+
+
+@pytest.mark.parametrize("n", [8200, 40_000, 500_000, 600_000])
+def test_binning_at_every_form_of_the_scan(tiga, n):
+    """Cells as fine as the grid allows: 32, 154, 1926 and 2316 chunks of cells (the last above the limit of the folded totals)."""
+    _check_bin(tiga, gen.uniform_points(n, 17), np.float32(1e-4), np.ones(3, np.float32), [0, 0, 0])
