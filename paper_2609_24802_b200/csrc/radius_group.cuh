@@ -4,8 +4,8 @@
 // 15 to 16 queries a group at every density, where cells taken one at a time (7.6 or 12.6 points) leave a quarter to a half of
 // the lanes without a query and stage 340 candidates for 12.6 queries instead of 470 for 16.
 //
-// The whole stencil is staged, one float4 per candidate as it lies in memory (coordinates, point id).  With q and c relative to an
-// origin among the queries
+// The whole stencil is staged, one float4 per candidate as it lies in memory (coordinates, point id).  With q and c relative to
+// the middle of the group's cells
 //     |q - c|^2 - T = (|q|^2 - T) + (-2 q, 0, 1, 1, 1, 0) . (c, -, c^2, -),
 // so one mma of 16 queries by 8 candidates with K = 8 forms 128 tests, whose signs are the answer: 40 instructions per
 // 512 tests against 96 with packed fp32 instructions (and the tests are cheap enough not to sort out the candidates that are far
@@ -132,7 +132,9 @@ struct Group {
 #pragma unroll
         for (int d = 0; d < 3; ++d) mi[d] = MI && p.periodic[d] && p.nc[d] <= 3;
         lsh = nq <= 4 ? 3 : nq <= 8 ? 2 : 1;
-        origin = query(nq >> 1);
+        // origin: the middle of the group's cells, not a point (one coordinate that is not finite would take the others' tests with it)
+        origin = make_float4((cell[0] + 0.5f * run) * p.hcell[0], (cell[1] + 0.5f) * p.hcell[1], (cell[2] + 0.5f) * p.hcell[2], 0.f);
+        frame.shift(p, origin);
         const float4 qa = query(g < nq ? g : 0), qb = query(g + 8 < nq ? g + 8 : 0);
         const float na = norm(qa), nb = norm(qb);
         ot = t == 0 ? origin.x : t == 1 ? origin.y : origin.z;

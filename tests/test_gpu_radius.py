@@ -560,6 +560,26 @@ def test_groups_of_queries(tiga, F, n, r, box, periodic):
         _check_gauss(tiga, pos, x, None, np.float32(r), box, periodic, np.float32(r) / 2, kind=kind, use_cells=r < 0.2 * box.min(), backward=False)
 
 
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
+@pytest.mark.parametrize("message", ["sum1", "sum4", "lj"])
+def test_a_coordinate_that_is_not_finite_affects_its_own_point_only(tiga, message, bad):
+    """What a diverging simulation hands over: every other point has the neighbours that it has without the bad ones."""
+    c = gen.config("cfg3", m=21)
+    r, box, periodic = (c["r"], c["box"], c["periodic"]) if message == "lj" else (np.float32(0.08), np.ones(3, np.float32), [0, 0, 0])
+    pos = c["pos"].copy() if message == "lj" else gen.uniform_points(24001, 72)
+    n, F = len(pos), 1 if message == "sum1" else 4
+    x = gen.normal_features(n, F, 72, 31)
+    which = np.sort(gen.rng(72, 3).choice(n, 300, replace=False))
+    pos[which, np.arange(300) % 3] = bad
+    good = np.delete(np.arange(n), which)
+    kind, p0, p1 = (tiga.MSG_LJ, 1.0, 1.0) if message == "lj" else (tiga.MSG_DIST, 0.0, 0.0)
+    y, A, cnt = oracle.radius_forward(pos[good], None if message == "lj" else x[good], r, box, periodic, kind, p0, p1, use_cells=True)
+    out, count, _ = tiga.tiga_apply_radius(dev(pos, torch), None if message == "lj" else dev(x, torch), r, box, periodic, kind, p0=p0, p1=p1, want_count=True)
+    assert np.array_equal(host(count)[good], cnt)
+    assert rel_err(host(out)[good], y, A) <= SUM_TOL
+    assert not host(count)[which].any() and not host(out)[which].any()
+
+
 @pytest.mark.parametrize("m", [21, 29])
 def test_groups_decide_pairs_at_the_cutoff_exactly(tiga, m):
     """Lattices whose neighbours lie exactly at the cutoff, just inside and just outside."""

@@ -22,7 +22,7 @@ def test_no_neighbour_fails_the_filter(unit, extent, place):
         d *= (1.0 - rng.random((16, 64, 1)) ** 4 * 0.01) * unit / np.linalg.norm(d, axis=2, keepdims=True)      # close to the cutoff
         c = (q[:, None, :] + d).astype(F32)
         near = ((q[:, None, :].astype(np.float64) - c) ** 2).sum(2) <= float(r) ** 2
-        o = q[8]
+        o = (np.array([place, place, place]) * unit).astype(F32)                      # the middle of the cells
         ql, cl = q - o, c - o
         norm = (ql * ql).sum(1, dtype=F32)
         far = np.sqrt(norm.max())
