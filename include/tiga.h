@@ -274,7 +274,9 @@ tiga_status tiga_radius_bin(const float* pos, int64_t n, float r, const tiga_box
  *                  F_i = sum_j 24 eps (2 (s/d)^12 - (s/d)^6) (p_i - p_j) / d^2 and
  *                  e_i = (1/2) sum_j 4 eps ((s/d)^12 - (s/d)^6)
  *   count        : int32 [n] number of neighbours of every point, or NULL
- * A point without neighbours gets the zero vector. */
+ * A point without neighbours gets the zero vector.
+ * Some kernels stage points with asynchronous copies and wait about a second for them at most: should a copy not
+ * arrive, the points it was for get NaN in every sum and -1 as their count, and all others their results. */
 tiga_status tiga_apply_radius(const float* pos, const float* feat, int64_t n, int32_t F,
                               float r, const tiga_box* box, const tiga_msg* msg,
                               float* out, int32_t* count, void* ws, size_t ws_bytes, void* stream);

@@ -24,6 +24,7 @@
 // upper face down by the box length, which is exact in fp32, so every displacement is one
 // rounded subtraction of two stored coordinates, for wrapped pairs as for interior ones.
 #include "radius_group_direct.cuh"
+#include <stdlib.h>
 #include <type_traits>
 
 namespace tiga {
@@ -256,7 +257,7 @@ __global__ void __launch_bounds__(SMALL_THREADS) bin_small_kernel(const RadiusPa
     constexpr int PP = SMALL_POINTS / SMALL_THREADS, PC = SMALL_CELLS / SMALL_THREADS;
     const int tid = threadIdx.x;
     for (int k = tid; k < p.ncells; k += SMALL_THREADS) s_start[k] = 0;
-    if (tid == 0) { s_ndense = 0; *p.queue_n = 0; *p.failed = 0; }
+    if (tid == 0) { s_ndense = 0; *p.queue_n = 0; }
     __syncthreads();
     float v[PP][3];
     int c[PP], slot[PP];
@@ -805,7 +806,6 @@ RadiusLayout carve_radius(RadiusParams* p, void* ws, int32_t** fill) {
     p->cnt = cv.take<int32_t>(2 * nc + 2 + 16);     // counts, then the scatter cursors, then the length of the dense-cell queue
     p->b_count = p->cnt + 2 * nc + 2;
     p->queue_n = p->b_count + 2;
-    p->failed = p->b_count + 3;
     *fill = p->cnt + nc;
     p->cell = cv.take<int32_t>(n);
     p->cell_start = cv.take<int32_t>(nc + 1);
@@ -874,6 +874,10 @@ tiga_status fill_params(RadiusParams* p, long long n, float r, const tiga_box* b
     p->r2_mid = r2;
     p->r2_band = r2 * beta * 1.25f;      // a little wider than [r2_lo, r2_hi]: nothing near the cutoff escapes the exact test
     p->r2_exact = (double)r * (double)r;
+#ifdef TIGA_CHECKED
+    const char* tries = getenv("TIGA_CHECKED_COPY_TRIES");       // 0: every staged copy counts as late
+    p->copy_tries = tries ? atoi(tries) : COPY_TRIES;
+#endif
     return TIGA_OK;
 }
 

@@ -85,15 +85,16 @@ template <int CAP, int LIST> struct GroupStage {
         }
         __syncwarp();
     }
-    // true when all bytes of the phase have arrived; false if they do not within a second or so
-    __device__ __forceinline__ bool wait() {
-        for (int k = 0; k < 1 << 20; ++k) {
-            unsigned done;
+    // whether all bytes of the phase have arrived, the same for all lanes; false if they have not after `tries` looks of up to a
+    // microsecond each.  The phase is over only when every lane has seen it: another wait after a failed one waits for the same bytes
+    __device__ __forceinline__ bool wait(const int tries) {
+        unsigned done = 0u;
+        for (int k = 0; k < tries && !done; ++k)
             asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                         : "=r"(done) : "r"(arrived), "r"(phase), "r"(1000u) : "memory");      // (up to a microsecond at a time)
-            if (done) { phase ^= 1u; return true; }
-        }
-        return false;
+                         : "=r"(done) : "r"(arrived), "r"(phase), "r"(1000u) : "memory");
+        if (__any_sync(0xffffffffu, !done)) return false;
+        phase ^= 1u;
+        return true;
     }
 };
 
@@ -182,7 +183,7 @@ struct Group {
         }
         const int ns = (n + 31) & ~31;
         if (n + lane < ns) st.c[n + lane] = make_float4(FAR_AWAY, FAR_AWAY, FAR_AWAY, __int_as_float(-1));
-        if (__any_sync(0xffffffffu, !st.wait())) return 0;
+        if (!st.wait(copy_tries(p))) return 0;
         __syncwarp();
         if (frame.face) {                                      // warp uniform
             for (int k = lane; k < n; k += 32) frame.shift(p, st.c[k]);
@@ -317,11 +318,14 @@ struct Group {
     }
 };
 
-// Copies that did not arrive in time: the plan's failure word is set and the warp ends, once they have arrived or another limit is over.
-template <typename Stage>
-static __device__ __forceinline__ void group_failed(const RadiusParams& p, Stage& st) {
-    if ((threadIdx.x & 31) == 0) atomicExch(p.failed, 1);
-    st.wait();
+// Copies that did not arrive in time: points [from, end) in cell order, which the warp leaves undone, get sums that are not a number and counts
+// of -1.  (Never seen; a caller who looks at the results cannot take them for sums.)
+static __device__ __noinline__ void give_up(const RadiusParams& p, const int sums, const int from, const int end) {
+    for (int i = from + (int)(threadIdx.x & 31); i < end; i += 32) {
+        const int id = checked(__float_as_int(p.spos[i].w), p.n, CHECK_POINT);
+        for (int f = 0; f < sums; ++f) p.out[(size_t)id * sums + f] = __int_as_float(0x7fffffff);
+        if (p.count) p.count[id] = -1;
+    }
 }
 
 }  // namespace tiga

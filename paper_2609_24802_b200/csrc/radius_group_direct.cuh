@@ -132,10 +132,12 @@ __global__ void __launch_bounds__(32, (GroupDirectSmem<Msg, SPARSE>::WARPS)) rad
     float* s_feat = reinterpret_cast<float*>(s_raw + SM::STAGE_BYTES);                   // [STAGED][FEAT_STRIDE]
     if (threadIdx.x < SM::STAGED) s_feat[threadIdx.x * SM::FEAT_STRIDE + SM::Stage::FAR] = 0.f;
     typename SM::Stage st(s_raw);
+    const int end = p.n - (int)blockIdx.x * unit < unit ? p.n : (int)(blockIdx.x + 1) * unit;
     walk_groups(p, blockIdx.x, unit, [&](const int (&cell)[3], const int run, const int qs, const int nq) {
-        const bool ok = direct_group<Msg, SPARSE, MI, COUNT>(p, st, s_feat, cell, run, qs, nq);
-        if (!ok) group_failed(p, st);
-        return ok;
+        if (direct_group<Msg, SPARSE, MI, COUNT>(p, st, s_feat, cell, run, qs, nq)) return true;
+        st.wait(COPY_TRIES);                                       // no copy outlives the warp, unless another limit is over
+        give_up(p, Msg::OUT, qs, end);
+        return false;
     });
 }
 

@@ -19,6 +19,7 @@ constexpr int UNIT_MAX = 32;            // most points per unit of work (at most
 constexpr int RUN_CELLS = 8;            // longest run of cells along x that one warp covers
 constexpr int GROUP_RUN = 16;           // most cells along x a group of queries spans
 constexpr int RUN_QUERIES = 16;         // points a warp joins cells for
+constexpr int COPY_TRIES = 1 << 20;     // looks at a staged copy, up to a microsecond each, before a traversal gives up
 constexpr int SORT_DENSE = 256;         // a cell with more points than this is ordered by a sorting network, not by rank counting
 
 struct RadiusParams {
@@ -61,12 +62,20 @@ struct RadiusParams {
     int* queue_n;             // length of the kNN queue (zeroed with the counts)
     int32_t* b_items;         // cells with more than SORT_DENSE points (queued by the scan), and how many
     int* b_count;
-    int* failed;              // set when a traversal's staged copies did not arrive (zeroed with the counts)
     // optional user copies of the plan
     int32_t* u_cell;
     int32_t* u_cell_start;
     int32_t* u_order;
+#ifdef TIGA_CHECKED
+    int copy_tries;           // in the place of COPY_TRIES
+#endif
 };
+
+#ifdef TIGA_CHECKED
+static __device__ __forceinline__ int copy_tries(const RadiusParams& p) { return p.copy_tries; }
+#else
+static __device__ __forceinline__ int copy_tries(const RadiusParams&) { return COPY_TRIES; }
+#endif
 
 struct RadiusLayout {
     size_t bytes;

@@ -6,7 +6,8 @@ when the binding is imported.
 Part 1: well-formed inputs through the main entry points; results match the oracle and the status
 word stays 0.  Part 2: relations whose index arrays hold a few out-of-range entries; the status word
 names the violation, nothing faults, and the result equals the oracle's for the same relation with the
-bad entries pointing at element 0 (which is where the checked build sends them)."""
+bad entries pointing at element 0 (which is where the checked build sends them).  Part 3: asynchronous
+copies that the checked build is told to take for late (TIGA_CHECKED_COPY_TRIES=0)."""
 import os
 import sys
 
@@ -126,6 +127,22 @@ def main():
         T.tiga_apply_csr_backward(g, dev(x, torch), dev(w, torch), dev(gy, torch), T.MAX, argmax=am_bad)
         st = T.checked_status()
         assert st & 2, f"status word {st}: an out-of-range edge position must set bit 2"
+
+    # ---- part 3: staged copies that count as late (the wait gives up at once and the copies are then waited for): the
+    # points that were not computed say so, nothing faults, and the next call is whole again
+    n = 9001
+    pos, x = dev(gen.uniform_points(n, 63), torch), dev(gen.normal_features(n, 4, 63, 31), torch)
+    for late in (True, False):
+        if late:
+            os.environ["TIGA_CHECKED_COPY_TRIES"] = "0"
+        for message, feat, r in ((T.MSG_DIST, x[:, :1].contiguous(), 0.08), (T.MSG_GAUSS, x, 0.05), (T.MSG_LJ, None, 0.08)):
+            out, count, _ = T.tiga_apply_radius(pos, feat, r, ones, [0, 0, 0], message, p0=r, p1=1e-3, want_count=True)
+            if late:
+                assert bool(torch.isnan(out).all()) and bool((count == -1).all())
+            else:
+                assert not bool(torch.isnan(out).any()) and int(count.min()) >= 0 and int(count.sum()) > n
+        os.environ.pop("TIGA_CHECKED_COPY_TRIES", None)
+    assert T.checked_status() == 0
     torch.cuda.synchronize()
     print("checked build: all cases passed")
 
