@@ -54,6 +54,12 @@ static inline int group_unit(const long long n) {
     return n >= 3 * 32 * places ? 32 : n >= 8 * places ? 16 : n >= 4 * places ? 8 : 4;
 }
 
+// The groups fill their stage up with the far slot: it has to lie outside the box and beyond every cutoff.  (At the small end nothing is lost:
+// squares are cut downwards, which lets more pairs through, and the tensor cores keep products below the normal numbers.)
+static inline bool group_lengths(const RadiusParams& p) {
+    return fmaxf(fmaxf(p.len[0], p.len[1]), p.len[2]) < 0.25f * FAR_AWAY && p.r < FAR_AWAY;
+}
+
 // Few points per cell: the stencil of 16 queries has fewer than 256 candidates, and a smaller stage lets more warps share an SM.
 static inline bool group_sparse(const RadiusParams& p) { return (long long)p.n < 3LL * p.ncells; }
 

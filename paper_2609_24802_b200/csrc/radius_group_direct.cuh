@@ -158,6 +158,7 @@ static tiga_status launch_direct_group(const RadiusParams& p, cudaStream_t s) {
 // neighbours, F = 1 24.3 / 25.2, but dense ones gain (Lennard-Jones, 1728 particles 24.9 / 23.7).
 template <typename Msg, bool MI>
 static tiga_status launch_direct_t(const RadiusParams& p, cudaStream_t s) {
+    if (!group_lengths(p)) return launch_direct_slices<Msg, MI>(p, s);
     if (10LL * p.n < 7LL * p.ncells || (p.n < 8192 && p.n < 8LL * p.ncells)) return launch_direct_slices<Msg, MI>(p, s);
     return group_sparse(p) ? launch_direct_group<Msg, true, MI>(p, s) : launch_direct_group<Msg, false, MI>(p, s);
 }

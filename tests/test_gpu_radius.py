@@ -560,6 +560,18 @@ def test_groups_of_queries(tiga, F, n, r, box, periodic):
         _check_gauss(tiga, pos, x, None, np.float32(r), box, periodic, np.float32(r) / 2, kind=kind, use_cells=r < 0.2 * box.min(), backward=False)
 
 
+@pytest.mark.parametrize("L", [4e18, 2e17, 1e-14, 1e-17])
+@pytest.mark.parametrize("F", [1, 3])
+def test_narrow_features_at_lengths_near_the_ends_of_fp32(tiga, F, L):
+    """A box that holds the place of the padding, one just short of it, squared cutoffs near and below the smallest normal number."""
+    box = np.full(3, L, np.float32)
+    pos = np.minimum(gen.uniform_points(24001, 73) * box, np.nextafter(box, np.float32(0))).astype(np.float32)
+    x = gen.normal_features(len(pos), F, 73, 31)
+    r = np.float32(0.045 * L)
+    for kind in (tiga.MSG_GAUSS, tiga.MSG_DIST):
+        _check_gauss(tiga, pos, x, None, r, box, [0, 0, 0], r / np.float32(2), kind=kind, use_cells=True, backward=False)
+
+
 @pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
 @pytest.mark.parametrize("message", ["sum1", "sum4", "lj"])
 def test_a_coordinate_that_is_not_finite_affects_its_own_point_only(tiga, message, bad):
