@@ -678,7 +678,10 @@ __device__ __forceinline__ void traverse_slice(const RadiusParams& p, const int 
         __syncwarp();
     };
 
-    const RunStencil sten(p, c, run, s_delta);
+    // Forward of rows of 16 to 64 features: a division costs less than the 12 to 24 bytes more that are spilled without one (1 M points, 32 neighbours,
+    // F = 32 607 / 617 us; 30 k, 45 neighbours, F = 64 81 / 85); narrower and wider rows gain from its absence (40 k clustered points, F = 8
+    // 300 / 289; 300 k, 8 neighbours, F = 128 213 / 209).
+    const RunStencil sten(p, c, run, s_delta, !(MODE == 0 && (LF == 2 || LF == 32)));
     const int total = sten.total;
 
     // bounding box of the queries (in the frame): a candidate farther than the cutoff from this box cannot be a
@@ -740,7 +743,7 @@ __device__ __forceinline__ void traverse_slice(const RadiusParams& p, const int 
     }
 }
 
-// Warps per SM that the registers must allow: 28 in the forward (72 registers, 12 to 56 bytes spilled), 16 in the backward (up to
+// Warps per SM that the registers must allow: 28 in the forward (72 registers, 0 to 68 bytes spilled), 16 in the backward (up to
 // 124, no spills).  28 / 24 / 20: 400 k points, 12 neighbours, F = 32 212 / 220 / 237 us, 50 k points, 45 neighbours 89 / 89 / 91 us,
 // 20 k clustered points 235 / 220 / 218 us, lattice of 8 points a cell, F = 128, 112 / 112 / 101 us.  16 / 20 / 12: F = 32 282 / 286 /
 // 343 us, F = 128 533 / 600 / 533 us.

@@ -116,6 +116,12 @@ template <int WORDS> struct GroupMask {
     unsigned a[2 * WORDS], b[2 * WORDS];
 };
 
+// The stencil by lane: cs is the source of the lane's first position.
+struct GroupStencil {
+    int begin, len, total, cs;
+    __device__ __forceinline__ GroupStencil(const RadiusParams& p, const int (&c)[3], const int run) { cs = stencil_range(p, c, run, false, begin, len, total); }
+};
+
 // The group: frame, stencil, the lane's operands of the test.
 // MI: some periodic dimension has three cells or fewer and uses the explicit minimum image; its tests are scalar.
 template <bool MI, typename Stage>
@@ -124,7 +130,7 @@ struct Group {
     Stage& st;
     const int qs, nq;
     const RunFrame frame;
-    const RunStencil sten;
+    const GroupStencil sten;
     bool mi[3];
     float4 origin;
     float ot;                              // the lane's component of the origin

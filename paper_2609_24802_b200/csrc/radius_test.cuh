@@ -45,49 +45,55 @@ struct RunFrame {
     }
 };
 
-// The run's stencil: lanes 0..8 hold the (y, z) rows over the run's x range, lanes 9..17 the cell that row reaches
-// around a periodic x face.  begin: flattened position of the lane's range; s_delta maps a position to its source.
-struct RunStencil {
-    int begin, len, total, cs;             // cs: source of the lane's first position
-    __device__ __forceinline__ RunStencil(const RadiusParams& p, const int (&c)[3], const int run, int* s_delta) : RunStencil(p, c, run) {
-        const unsigned some = __ballot_sync(0xffffffffu, len > 0);
-        if (len > 0) s_delta[__popc(some & ((1u << (threadIdx.x & 31)) - 1u))] = cs - begin;
-        __syncwarp();
+// The run's stencil: lanes 0..8 hold the (y, z) rows over the run's x range, lanes 9..17 the cell that row
+// reaches around a periodic x face.  begin: flattened position of the lane's range.  Returns the source of its first position.
+// divide: how the row is found.  Without a division is shorter, but the compiler then shares the 72 registers of the list kernels out in another way
+// (see there).
+static __device__ __forceinline__ int stencil_range(const RadiusParams& p, const int (&c)[3], const int run, const bool divide, int& begin, int& len, int& total) {
+    constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const int row = lane < 9 ? lane : lane - 9;
+    const int oz = divide ? row / 3 - 1 : row >= 6 ? 1 : row >= 3 ? 0 : -1, oy = divide ? row % 3 - 1 : row - 3 * oz - 4;
+    int y = c[1] + oy, z = c[2] + oz, cs = 0;
+    bool ok = lane < 18;
+    if (p.nc[1] == 1) { ok = ok && oy == 0; y = 0; }
+    else if (y < 0) { if (p.periodic[1]) y += p.nc[1]; else ok = false; }
+    else if (y >= p.nc[1]) { if (p.periodic[1]) y -= p.nc[1]; else ok = false; }
+    if (p.nc[2] == 1) { ok = ok && oz == 0; z = 0; }
+    else if (z < 0) { if (p.periodic[2]) z += p.nc[2]; else ok = false; }
+    else if (z >= p.nc[2]) { if (p.periodic[2]) z -= p.nc[2]; else ok = false; }
+    const int lo = c[0] - 1, hi = c[0] + run, top = p.nc[0] - 1;
+    int xa = lo > 0 ? lo : 0, xb = hi < top ? hi : top;
+    if (lane >= 9) {
+        xa = xb = lo < 0 ? top : 0;
+        ok = ok && p.periodic[0] && top > 0 && (lo < 0 || hi > top);
     }
-    __device__ __forceinline__ RunStencil(const RadiusParams& p, const int (&c)[3], const int run) {
-        constexpr unsigned FULL = 0xffffffffu;
-        const int lane = threadIdx.x & 31;
-        const int row = lane < 9 ? lane : lane - 9;
-        const int oz = row >= 6 ? 1 : row >= 3 ? 0 : -1, oy = row - 3 * oz - 4;
-        int y = c[1] + oy, z = c[2] + oz;
-        cs = 0;
-        bool ok = lane < 18;
-        if (p.nc[1] == 1) { ok = ok && oy == 0; y = 0; }
-        else if (y < 0) { if (p.periodic[1]) y += p.nc[1]; else ok = false; }
-        else if (y >= p.nc[1]) { if (p.periodic[1]) y -= p.nc[1]; else ok = false; }
-        if (p.nc[2] == 1) { ok = ok && oz == 0; z = 0; }
-        else if (z < 0) { if (p.periodic[2]) z += p.nc[2]; else ok = false; }
-        else if (z >= p.nc[2]) { if (p.periodic[2]) z -= p.nc[2]; else ok = false; }
-        const int lo = c[0] - 1, hi = c[0] + run, top = p.nc[0] - 1;
-        int xa = lo > 0 ? lo : 0, xb = hi < top ? hi : top;
-        if (lane >= 9) {
-            xa = xb = lo < 0 ? top : 0;
-            ok = ok && p.periodic[0] && top > 0 && (lo < 0 || hi > top);
-        }
-        len = 0;
-        if (ok) {
-            const int id = (z * p.nc[1] + y) * p.nc[0];
-            cs = p.cell_start[id + xa];
-            len = p.cell_start[id + xb + 1] - cs;
-        }
-        begin = len;
+    len = 0;
+    if (ok) {
+        const int id = (z * p.nc[1] + y) * p.nc[0];
+        cs = p.cell_start[id + xa];
+        len = p.cell_start[id + xb + 1] - cs;
+    }
+    begin = len;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(FULL, begin, o);
-            if (lane >= o) begin += t;
-        }
-        total = __shfl_sync(FULL, begin, 31);
-        begin -= len;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(FULL, begin, o);
+        if (lane >= o) begin += t;
+    }
+    total = __shfl_sync(FULL, begin, 31);
+    begin -= len;
+    return cs;
+}
+
+// The stencil by position: s_delta maps a flattened position to its source.
+struct RunStencil {
+    int begin, len, total;
+    __device__ __forceinline__ RunStencil(const RadiusParams& p, const int (&c)[3], const int run, int* s_delta, const bool divide = false) {
+        const int lane = threadIdx.x & 31;
+        const int cs = stencil_range(p, c, run, divide, begin, len, total);
+        const unsigned some = __ballot_sync(0xffffffffu, len > 0);
+        if (len > 0) s_delta[__popc(some & ((1u << lane) - 1u))] = cs - begin;
+        __syncwarp();
     }
     // source of flattened position k0 + lane; `before` counts the ranges that began before k0 (start with -1).  The
     // ranges that begin in this window of 32 positions set one bit each: the bits at and below a lane count up to
