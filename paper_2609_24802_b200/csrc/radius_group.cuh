@@ -123,15 +123,13 @@ struct GroupStencil {
 };
 
 // The group: frame, stencil, the lane's operands of the test.
-// MI: some periodic dimension has three cells or fewer and uses the explicit minimum image; its tests are scalar.
-template <bool MI, typename Stage>
+template <typename Stage>
 struct Group {
     const RadiusParams& p;
     Stage& st;
     const int qs, nq;
     const RunFrame frame;
     const GroupStencil sten;
-    bool mi[3];
     float4 origin;
     float ot;                              // the lane's component of the origin
     unsigned mask;                         // TF32 bits of the lane's component, nothing of the fourth
@@ -142,8 +140,6 @@ struct Group {
     __device__ __forceinline__ Group(const RadiusParams& p_, Stage& st_, const int (&cell)[3], const int run, const int qs_, const int nq_)
         : p(p_), st(st_), qs(qs_), nq(nq_), frame(p_, cell, run), sten(p_, cell, run) {
         const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-#pragma unroll
-        for (int d = 0; d < 3; ++d) mi[d] = MI && p.periodic[d] && p.nc[d] <= 3;
         lsh = nq <= 4 ? 3 : nq <= 8 ? 2 : 1;
         // origin: the middle of the group's cells, not a point (one coordinate that is not finite would take the others' tests with it)
         origin = make_float4((cell[0] + 0.5f * run) * p.hcell[0], (cell[1] + 0.5f) * p.hcell[1], (cell[2] + 0.5f) * p.hcell[2], 0.f);
@@ -172,9 +168,6 @@ struct Group {
     __device__ __forceinline__ float norm(const float4& v) const {
         const float x = v.x - origin.x, y = v.y - origin.y, z = v.z - origin.z;
         return fmaf(z, z, fmaf(y, y, x * x));
-    }
-    __device__ __forceinline__ float delta(const int d, const float q, const float c) const {
-        return MI && mi[d] ? mi_delta(q, c, p.len[d], 0.5f * p.len[d]) : q - c;
     }
 
     // Stages positions [k0, k0 + CAPACITY) of the flattened stencil, the last step of 32 filled up with far candidates; returns the slots
@@ -208,8 +201,6 @@ struct Group {
     __device__ __forceinline__ void test(const int ns, const int k0, GroupMask<Stage::WORDS>& m) const {
         const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
         const float* s = reinterpret_cast<const float*>(st.c) + lane;      // component t of slot g
-        float4 qa, qb;
-        if (MI) { qa = query(g < nq ? g : 0); qb = query(g + 8 < nq ? g + 8 : 0); }
 #pragma unroll
         for (int w = 0; w < Stage::WORDS; ++w) {
             const int eights = ns - 256 * w >= 256 ? 32 : ns > 256 * w ? (ns - 256 * w) >> 3 : 0;      // multiple of four
@@ -218,19 +209,8 @@ struct Group {
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     float d[4];
-                    if constexpr (!MI) {
-                        const float v = s[32 * j] - ot;
-                        mma_16x8x8(d, a, __float_as_uint(v) & mask, __float_as_uint(v * v) & mask, c0, c1);
-                    } else {
-#pragma unroll
-                        for (int b = 0; b < 2; ++b) {
-                            const float4 c = st.c[256 * w + 8 * (k + j) + 2 * t + b];
-                            const float ax = delta(0, qa.x, c.x), ay = delta(1, qa.y, c.y), az = delta(2, qa.z, c.z);
-                            const float bx = delta(0, qb.x, c.x), by = delta(1, qb.y, c.y), bz = delta(2, qb.z, c.z);
-                            d[b] = g < nq ? fmaf(az, az, fmaf(ay, ay, fmaf(ax, ax, -p.r2_hi))) : 1.f;
-                            d[2 + b] = g + 8 < nq ? fmaf(bz, bz, fmaf(by, by, fmaf(bx, bx, -p.r2_hi))) : 1.f;
-                        }
-                    }
+                    const float v = s[32 * j] - ot;
+                    mma_16x8x8(d, a, __float_as_uint(v) & mask, __float_as_uint(v * v) & mask, c0, c1);
                     m0 = __funnelshift_l(__float_as_uint(d[0]), m0, 1);
                     m1 = __funnelshift_l(__float_as_uint(d[1]), m1, 1);
                     m2 = __funnelshift_l(__float_as_uint(d[2]), m2, 1);

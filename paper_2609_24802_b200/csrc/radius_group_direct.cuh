@@ -17,9 +17,8 @@ template <typename Msg, bool SPARSE> struct GroupDirectSmem {
     static_assert(PER_WARP % 16 == 0, "the stage is accessed as 16-byte vectors");
 };
 
-// MI: some periodic dimension has three cells or fewer and uses the explicit minimum image.
 // COUNT: the numbers of neighbours are wanted.
-template <typename Msg, bool SPARSE, bool MI, bool COUNT>
+template <typename Msg, bool SPARSE, bool COUNT>
 __device__ __forceinline__ bool direct_group(const RadiusParams& p, typename GroupDirectSmem<Msg, SPARSE>::Stage& st, float* s_feat, const int (&cell)[3], const int run, const int qs, const int nq) {
     using SM = GroupDirectSmem<Msg, SPARSE>;
     constexpr int OUT = Msg::OUT, NF = Msg::STAGED;
@@ -27,7 +26,7 @@ __device__ __forceinline__ bool direct_group(const RadiusParams& p, typename Gro
     using Stage = typename SM::Stage;
     const int lane = threadIdx.x & 31;
     const Msg msg(p);
-    Group<MI, Stage> grp(p, st, cell, run, qs, nq);
+    Group<Stage> grp(p, st, cell, run, qs, nq);
 
     // the lane's query and its sums
     const int q = lane >> grp.lsh, lpq = 1 << grp.lsh, sub = lane & (lpq - 1);
@@ -93,16 +92,7 @@ __device__ __forceinline__ bool direct_group(const RadiusParams& p, typename Gro
                 unsigned sa = two & 0xffffu, sb = two >> 16;
                 const float4 ca = *reinterpret_cast<const float4*>(reinterpret_cast<const unsigned char*>(st.c) + sa);
                 const float4 cb = *reinterpret_cast<const float4*>(reinterpret_cast<const unsigned char*>(st.c) + sb);
-                f32x2 dx, dy, dz;
-                if constexpr (!MI) {
-                    dx = sub2(qx2, pack2(ca.x, cb.x));
-                    dy = sub2(qy2, pack2(ca.y, cb.y));
-                    dz = sub2(qz2, pack2(ca.z, cb.z));
-                } else {
-                    dx = pack2(grp.delta(0, qv.x, ca.x), grp.delta(0, qv.x, cb.x));
-                    dy = pack2(grp.delta(1, qv.y, ca.y), grp.delta(1, qv.y, cb.y));
-                    dz = pack2(grp.delta(2, qv.z, ca.z), grp.delta(2, qv.z, cb.z));
-                }
+                const f32x2 dx = sub2(qx2, pack2(ca.x, cb.x)), dy = sub2(qy2, pack2(ca.y, cb.y)), dz = sub2(qz2, pack2(ca.z, cb.z));
                 float da, db;
                 unpack2(fma2(dz, dz, fma2(dy, dy, mul2(dx, dx))), da, db);
                 bool in_a = da <= p.r2_mid, in_b = db <= p.r2_mid;
@@ -148,7 +138,7 @@ __device__ __forceinline__ bool direct_group(const RadiusParams& p, typename Gro
     return true;
 }
 
-template <typename Msg, bool SPARSE, bool MI, bool COUNT>
+template <typename Msg, bool SPARSE, bool COUNT>
 __global__ void __launch_bounds__(32, (GroupDirectSmem<Msg, SPARSE>::WARPS)) radius_group_kernel(const __grid_constant__ RadiusParams p, const int unit) {
     using SM = GroupDirectSmem<Msg, SPARSE>;
     extern __shared__ __align__(16) unsigned char s_raw[];
@@ -157,18 +147,18 @@ __global__ void __launch_bounds__(32, (GroupDirectSmem<Msg, SPARSE>::WARPS)) rad
     typename SM::Stage st(s_raw);
     const int end = p.n - (int)blockIdx.x * unit < unit ? p.n : (int)(blockIdx.x + 1) * unit;
     walk_groups(p, blockIdx.x, unit, [&](const int (&cell)[3], const int run, const int qs, const int nq) {
-        if (direct_group<Msg, SPARSE, MI, COUNT>(p, st, s_feat, cell, run, qs, nq)) return true;
+        if (direct_group<Msg, SPARSE, COUNT>(p, st, s_feat, cell, run, qs, nq)) return true;
         st.wait(COPY_TRIES);                                       // no copy outlives the warp, unless another limit is over
         give_up(p, Msg::OUT, qs, end);
         return false;
     });
 }
 
-template <typename Msg, bool SPARSE, bool MI>
+template <typename Msg, bool SPARSE>
 static tiga_status launch_direct_group(const RadiusParams& p, cudaStream_t s) {
     constexpr int smem = GroupDirectSmem<Msg, SPARSE>::PER_WARP;
     static_assert(smem <= 48 * 1024, "no attribute needed");
-    auto kern = p.count ? radius_group_kernel<Msg, SPARSE, MI, true> : radius_group_kernel<Msg, SPARSE, MI, false>;
+    auto kern = p.count ? radius_group_kernel<Msg, SPARSE, true> : radius_group_kernel<Msg, SPARSE, false>;
     const int unit = group_unit(p.n);
     kern<<<counted((unsigned)(((long long)p.n + unit - 1) / unit)), 32, smem, s>>>(p, unit);
     return launch_status();
@@ -179,11 +169,15 @@ static tiga_status launch_direct_group(const RadiusParams& p, cudaStream_t s) {
 // points 231 / 272).  Uniform points: 1 M, 32 neighbours, F = 1 392 / 367, F = 4 458 / 378; 4 neighbours, F = 1 288 / 239; 300 k,
 // 8 neighbours, F = 3 151 / 121; 30 k, 45 neighbours, F = 3 63 / 47.  Inputs that leave the machine half empty either way: 4 k, 16
 // neighbours, F = 1 24.3 / 25.2, but dense ones gain (Lennard-Jones, 1728 particles 24.9 / 23.7).
+// Inputs with the explicit minimum image take cells: their tests are scalar either way, and groups sort no candidate out first (1 k points in three
+// cells a side, F = 1 78 / 162, Lennard-Jones 80 / 158; 8 k 695 / 1319; only 24 k points in one cell gained, 4287 / 3628).
 template <typename Msg, bool MI>
 static tiga_status launch_direct_t(const RadiusParams& p, cudaStream_t s) {
-    if (!group_lengths(p)) return launch_direct_slices<Msg, MI>(p, s);
-    if (10LL * p.n < 7LL * p.ncells || (p.n < 8192 && p.n < 8LL * p.ncells)) return launch_direct_slices<Msg, MI>(p, s);
-    return group_sparse(p) ? launch_direct_group<Msg, true, MI>(p, s) : launch_direct_group<Msg, false, MI>(p, s);
+    if constexpr (!MI) {
+        if (group_lengths(p) && 10LL * p.n >= 7LL * p.ncells && (p.n >= 8192 || p.n >= 8LL * p.ncells))
+            return group_sparse(p) ? launch_direct_group<Msg, true>(p, s) : launch_direct_group<Msg, false>(p, s);
+    }
+    return launch_direct_slices<Msg, MI>(p, s);
 }
 
 }  // namespace tiga
