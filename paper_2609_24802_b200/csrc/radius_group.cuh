@@ -252,9 +252,9 @@ struct Group {
     }
 
     // Calls consume(first, end) with the list of the lane's query (lane >> lsh), st.list[first, end), in whole steps of two entries per
-    // lane; several times when the accepted slots do not fit.
-    template <typename Consume>
-    __device__ __forceinline__ void lists(const int ns, const GroupMask<Stage::WORDS>& m, Consume consume) const {
+    // lane; several times, with between() after all but the last, when the accepted slots do not fit.
+    template <typename Consume, typename Between>
+    __device__ __forceinline__ void lists(const int ns, const GroupMask<Stage::WORDS>& m, Consume consume, Between between) const {
         constexpr unsigned FULL = 0xffffffffu;
         constexpr int WORDS = Stage::WORDS, NW = 2 * WORDS, WINDOW = Stage::WINDOW;
         const int lane = threadIdx.x & 31, t = lane & 3;
@@ -306,6 +306,7 @@ struct Group {
             consume(first, q < nq ? first + (q < 8 ? f0 & 0xffff : f0 >> 16) : first);
             __syncwarp();
             if (whole || 8 * WINDOW * ++win >= ns) break;
+            between();
         }
     }
 };

@@ -38,10 +38,10 @@ __device__ __forceinline__ bool direct_group(const RadiusParams& p, typename Gro
     for (int f = 0; f < OUT; ++f) acc2[f] = 0ull;
     // A list's terms are added up by themselves, and so are the sums of eight lists: however long the stencil, no partial sum runs
     // long (rms error over 24 k positive terms 0.6e-7 of their magnitude; 5.7e-7 with one running sum per lane and half, 1.4e-7 in cells).
-    // Most groups have one list per query; the others keep these sums in local memory (4.1 M Lennard-Jones particles 1232 -> 1239 us, and 1307
-    // with the sums in registers, which spills in the loop below).
+    // Most groups have one list per query; the others keep these sums in local memory, as registers are short, and add them up behind a list (4.1 M
+    // Lennard-Jones particles 1232 us with and without; in front of it 1239; in registers, which spills in the loop below, 1307).
     volatile f32x2 sum8[OUT], sums[OUT];
-    int folds = -1;
+    int folds = 0;
     auto fold = [&]() {
 #pragma unroll
         for (int f = 0; f < OUT; ++f) {
@@ -51,6 +51,7 @@ __device__ __forceinline__ bool direct_group(const RadiusParams& p, typename Gro
             else sums[f] = folds > 7 ? add2(sums[f], s) : s;
             acc2[f] = 0ull;
         }
+        ++folds;
     };
 
     for (int k0 = 0; k0 < grp.sten.total; k0 += Stage::CAPACITY) {
@@ -85,8 +86,6 @@ __device__ __forceinline__ bool direct_group(const RadiusParams& p, typename Gro
         GroupMask<Stage::WORDS> mask;
         grp.test(ns, k0, mask);
         grp.lists(ns, mask, [&](const int first, const int end) {
-            if (folds >= 0) fold();
-            ++folds;
             for (int j = first + 2 * sub; j < end; j += 2 * lpq) {
                 const unsigned two = *reinterpret_cast<const unsigned*>(grp.st.list + j);
                 unsigned sa = two & 0xffffu, sb = two >> 16;
@@ -107,7 +106,8 @@ __device__ __forceinline__ bool direct_group(const RadiusParams& p, typename Gro
                 msg.template pair<SM::FEAT_STRIDE>(acc2, da, db, dx, dy, dz, reinterpret_cast<const float*>(reinterpret_cast<const unsigned char*>(s_feat) + (sa >> 2)),
                          reinterpret_cast<const float*>(reinterpret_cast<const unsigned char*>(s_feat) + (sb >> 2)));
             }
-        });
+        }, fold);
+        if (grp.sten.total - k0 > Stage::CAPACITY + 128) fold();   // (a short last stage adds little: to the piece before)
     }
 #pragma unroll
     for (int f = 0; f < OUT; ++f) {
