@@ -761,9 +761,11 @@ __global__ void __launch_bounds__(TRAV_THREADS, (MODE == 0 ? 28 : 16) / TRAV_WAR
 // Bound by instruction issue and by the latency of the staging loads.  Against the list kernel below four features:
 // F = 4, n = 1M, 32 neighbours 616 -> 393 us; F = 1, n = 131072, distance-weighted 108 -> 58 us; F = 2, n = 300k,
 // 8 neighbours 218 -> 100 us.  Warps per SM measured: F = 1 28 / 24 / 20: 57 / 61 / 65 us; F = 3 401 / 394 / 381 us.
+// Candidates that a group's stage holds, 384 / 512 (1 M points, 32 and 45 neighbours): F = 1 340 / 330 and 414 / 385, F = 2 376 / 383 and 457 / 448
+// (16 and 60 neighbours: 289 / 303, 564 / 596).
 template <int NF, bool DIST>
 struct SumMsg {
-    static constexpr int CAP = 256, STAGED = NF, OUT = NF, WARPS = NF <= 2 ? 28 : 20, GROUP_CAP = 384, GROUP_WARPS = NF <= 2 ? 20 : 16;
+    static constexpr int CAP = 256, STAGED = NF, OUT = NF, WARPS = NF <= 2 ? 28 : 20, GROUP_CAP = NF == 1 ? 512 : 384, GROUP_WARPS = NF <= 2 ? 18 : 16;
     static constexpr float OUTSIDE = 1.f;                  // any weight that is finite for every sigma
     float neg_c2;
     // exp(-d2/(2 s^2)) = 2^(d2 * neg_c2)
