@@ -21,32 +21,53 @@
 namespace tiga {
 
 constexpr int GROUP = 16;                  // queries of a group: rows of the mma
+// A unit of a sparse input with a point in a cell of more than this many is done as slices of cells: the input is clustered there, and what the
+// slices sort out beforehand is worth more than cheap tests (us, cells / groups / either by unit; 200 k clustered points, one point per
+// cell on average, F = 1 1131 / 1265 / 1003, F = 4 1298 / 1580 / 1191, Lennard-Jones 1255 / 1353 / 1076; 40 k, F = 1 214 / 284 / 199).  20: the
+// fullest cell of 1 M uniform points at three per cell holds 16.  12 / 20: 40 k clustered points, F = 4 224 / 247, but a slab of eight points
+// a cell, 400 k points, F = 1 191 / 160.  The look costs uniform points 0 to 2 % (1 M, 4 neighbours, F = 1 222 / 226).
+constexpr int FULL_CELL = 20;
 
-// Unit u: points [u p.unit, (u + 1) p.unit) in cell order, cut into groups where the row of cells changes, at GROUP queries and
-// at p.group_run cells.  work(first cell, cells, first query, queries) returns whether to go on
-template <typename Work>
-static __device__ __forceinline__ void walk_groups(const RadiusParams& p, const int u, const int unit, Work work) {
-    constexpr unsigned FULL = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    const int i = u * unit + lane;
-    const bool valid = lane < unit && (unsigned)i < (unsigned)p.n;
-    int at = 0;                                                 // cell of the lane's point, ten bits per coordinate
-    if (valid) {
-        const float4 v = p.spos[i];
-        at = cell_coordinate(p, v.x, 0) | cell_coordinate(p, v.y, 1) << 10 | cell_coordinate(p, v.z, 2) << 20;
+// Unit u: points [u unit, (u + 1) unit) in cell order, a lane each.
+struct GroupUnit {
+    int begin, at;                         // first point; cell of the lane's point, ten bits per coordinate
+    bool valid;
+    __device__ __forceinline__ GroupUnit(const RadiusParams& p, const int u, const int unit) : begin(u * unit), at(0) {
+        const int lane = threadIdx.x & 31, i = begin + lane;
+        valid = lane < unit && (unsigned)i < (unsigned)p.n;
+        if (valid) {
+            const float4 v = p.spos[i];
+            at = cell_coordinate(p, v.x, 0) | cell_coordinate(p, v.y, 1) << 10 | cell_coordinate(p, v.z, 2) << 20;
+        }
     }
-    unsigned left = __ballot_sync(FULL, valid);
-    while (left) {
-        const int a = __ffs(left) - 1;
-        const int first = __shfl_sync(FULL, at, a);
-        const unsigned in = __ballot_sync(FULL, (left >> lane) & 1u && ((at ^ first) >> 10) == 0 && at - first < p.group_run && lane - a < GROUP);
-        const int last = __shfl_sync(FULL, at, 31 - __clz(in));
-        left &= ~in;
-        const int cell[3] = {first & 1023, (first >> 10) & 1023, first >> 20};
-        if (!work(cell, last - first + 1, u * unit + a, __popc(in))) return;
-        __syncwarp();
+    // whether a point lies in a cell of more than FULL_CELL points
+    __device__ __forceinline__ bool full(const RadiusParams& p) const {
+        int count = 0;
+        if (valid) {
+            const int* start = p.cell_start + ((at >> 20) * p.nc[1] + ((at >> 10) & 1023)) * p.nc[0] + (at & 1023);
+            count = start[1] - start[0];
+        }
+        return __any_sync(0xffffffffu, count > FULL_CELL);
     }
-}
+    // The points, cut into groups where the row of cells changes, at GROUP queries and at p.group_run cells.
+    // work(first cell, cells, first query, queries) returns whether to go on
+    template <typename Work>
+    __device__ __forceinline__ void walk(const RadiusParams& p, Work work) const {
+        constexpr unsigned FULL = 0xffffffffu;
+        const int lane = threadIdx.x & 31;
+        unsigned left = __ballot_sync(FULL, valid);
+        while (left) {
+            const int a = __ffs(left) - 1;
+            const int first = __shfl_sync(FULL, at, a);
+            const unsigned in = __ballot_sync(FULL, (left >> lane) & 1u && ((at ^ first) >> 10) == 0 && at - first < p.group_run && lane - a < GROUP);
+            const int last = __shfl_sync(FULL, at, 31 - __clz(in));
+            left &= ~in;
+            const int cell[3] = {first & 1023, (first >> 10) & 1023, first >> 20};
+            if (!work(cell, last - first + 1, begin + a, __popc(in))) return;
+            __syncwarp();
+        }
+    }
+};
 
 // Points per warp.
 static inline int group_unit(const long long n) {

@@ -15,6 +15,7 @@ template <typename Msg, bool SPARSE> struct GroupDirectSmem {
     static constexpr int FEAT_STRIDE = Stage::SLOTS;                        // the entry of the far slot stays zero
     static constexpr int PER_WARP = STAGE_BYTES + STAGED * FEAT_STRIDE * 4;
     static_assert(PER_WARP % 16 == 0, "the stage is accessed as 16-byte vectors");
+    static_assert(!SPARSE || DirectSmem<Msg>::PER_WARP <= PER_WARP, "units of full cells take the cells' form");
 };
 
 // COUNT: the numbers of neighbours are wanted.
@@ -142,11 +143,19 @@ template <typename Msg, bool SPARSE, bool COUNT>
 __global__ void __launch_bounds__(32, (GroupDirectSmem<Msg, SPARSE>::WARPS)) radius_group_kernel(const __grid_constant__ RadiusParams p, const int unit) {
     using SM = GroupDirectSmem<Msg, SPARSE>;
     extern __shared__ __align__(16) unsigned char s_raw[];
+    const GroupUnit work(p, blockIdx.x, unit);
+    if (SPARSE && work.full(p)) {
+        work.walk(p, [&](const int (&cell)[3], const int run, const int qs, const int nq) {
+            direct_slice<Msg, false>(p, cell, run, qs, qs + nq, s_raw);
+            return true;
+        });
+        return;
+    }
     float* s_feat = reinterpret_cast<float*>(s_raw + SM::STAGE_BYTES);                   // [STAGED][FEAT_STRIDE]
     if (threadIdx.x < SM::STAGED) s_feat[threadIdx.x * SM::FEAT_STRIDE + SM::Stage::FAR] = 0.f;
     typename SM::Stage st(s_raw);
-    const int end = p.n - (int)blockIdx.x * unit < unit ? p.n : (int)(blockIdx.x + 1) * unit;
-    walk_groups(p, blockIdx.x, unit, [&](const int (&cell)[3], const int run, const int qs, const int nq) {
+    const int end = p.n - work.begin < unit ? p.n : work.begin + unit;
+    work.walk(p, [&](const int (&cell)[3], const int run, const int qs, const int nq) {
         if (direct_group<Msg, SPARSE, COUNT>(p, st, s_feat, cell, run, qs, nq)) return true;
         st.wait(COPY_TRIES);                                       // no copy outlives the warp, unless another limit is over
         give_up(p, Msg::OUT, qs, end);

@@ -588,6 +588,28 @@ def test_long_sums_are_added_up_in_pieces(tiga):
     assert err <= 2.2e-7
 
 
+# (points, cutoff, periodic, shape): inputs of less than three points per cell on average whose points crowd together: units of full cells (above 20
+# points) beside units of groups, more accepted candidates than the sparse stage's lists hold (a slab of about 8 points a cell), every unit length
+_CROWDED = [(8192, 0.05, [0, 0, 0], "blobs"), (15001, 0.04, [1, 1, 0], "blobs"), (24001, 0.035, [0, 0, 0], "blobs"), (24001, 0.0341, [0, 0, 0], "slab"),
+            (24001, 0.0341, [1, 1, 1], "slab"), (300_007, 0.014, [1, 0, 1], "blobs"), (300_007, 0.0152, [0, 1, 0], "slab")]
+
+
+@pytest.mark.parametrize("n,r,periodic,shape", _CROWDED)
+@pytest.mark.parametrize("message", ["sum1", "sum4", "lj"])
+def test_groups_and_full_cells_side_by_side(tiga, message, n, r, periodic, shape):
+    ones = np.ones(3, np.float32)
+    pos = gen.clustered_points(n, 75) if shape == "blobs" else gen.uniform_points(n, 75) * np.array([1.0, 1.0, 0.1], np.float32)
+    grid, _ = tiga.tiga_radius_grid(n, r, ones, periodic)
+    cell = np.minimum((pos * np.float32(grid)).astype(np.int64), np.array(grid) - 1)
+    held = np.bincount((cell[:, 2] * grid[1] + cell[:, 1]) * grid[0] + cell[:, 0])
+    assert 0.7 <= n / np.prod(grid) < 3 and (held > 20).any() and ((held > 0) & (held <= 20)).any()
+    if message == "lj":
+        _check_lj(tiga, pos * np.float32(300.0), np.float32(300.0 * r), np.full(3, 300.0, np.float32), periodic, eps=1e-3, s=0.001, use_cells=True)
+    else:
+        x = gen.normal_features(n, 1 if message == "sum1" else 4, 75, 31)
+        _check_gauss(tiga, pos, x, None, np.float32(r), ones, periodic, np.float32(r) / 2, kind=tiga.MSG_DIST, use_cells=True, backward=False)
+
+
 @pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
 @pytest.mark.parametrize("message", ["sum1", "sum4", "lj"])
 def test_a_coordinate_that_is_not_finite_affects_its_own_point_only(tiga, message, bad):
