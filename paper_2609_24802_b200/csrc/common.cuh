@@ -52,6 +52,12 @@ __device__ __forceinline__ I checked(I idx, long long n, unsigned code) {
     if ((long long)idx < 0 || (long long)idx >= n) { atomicOr(&g_check_status, code); return I(0); }
     return idx;
 }
+// whether [first, first + len) lies within n entries; a range that does not is for the caller to read entry by entry, through checked()
+__device__ __forceinline__ bool checked_range(int first, int len, long long n, unsigned code) {
+    const bool whole = len <= 0 || (first >= 0 && (long long)first + len <= n);
+    if (!whole) atomicOr(&g_check_status, code);
+    return whole;
+}
 static inline unsigned read_check_status(bool reset) {
     unsigned v = 0, z = 0;
     if (cudaMemcpyFromSymbol(&v, g_check_status, sizeof(v)) != cudaSuccess) return 0x80000000u;
@@ -61,6 +67,7 @@ static inline unsigned read_check_status(bool reset) {
 #else
 template <typename I>
 __device__ __forceinline__ I checked(I idx, long long, unsigned) { return idx; }
+__device__ __forceinline__ bool checked_range(int, int, long long, unsigned) { return true; }
 static inline unsigned read_check_status(bool) { return 0u; }
 #endif
 // one reader per translation unit (defined at the end of every .cu file), combined by tiga_checked_status

@@ -10,7 +10,8 @@
 // so one mma of 16 queries by 8 candidates with K = 8 forms 128 tests, whose signs are the answer: 40 instructions per
 // 512 tests against 96 with packed fp32 instructions (and the tests are cheap enough not to sort out the candidates that are far
 // from all queries, which cost more).  The operands have TF32 precision, so this is a filter: T lies above the squared cutoff by
-// the bound of the product's error, about 1 % more pairs pass than are neighbours, and every pair that passes is decided in fp32
+// the bound of the product's error, 2^-8 |q| (|q| + r) with |q| up to half the length of the group: 2 % more pairs pass than are
+// neighbours at 8 points per cell, 7 % at 3, a third at one, where 16 points span 14 cells.  Every pair that passes is decided in fp32
 // from the coordinates and, near the cutoff, in fp64.  (mma.sync and not tcgen05: a warp's 16 x 8 results are looked at by the lanes
 // that hold them, one instruction later; a tcgen05 tile has 64 rows or more and its results go through tensor memory.)
 //
@@ -21,6 +22,9 @@
 namespace tiga {
 
 constexpr int GROUP = 16;                  // queries of a group: rows of the mma
+constexpr float FILTER_PRODUCT = 3.95e-3f; // margin of the test (Group): of the products, in |q| |c|;
+constexpr float FILTER_REACH = 1.001f;     // |c| of a neighbour exceeds |q| by this many cutoffs at most;
+constexpr float FILTER_SUMS = 4e-6f;       // of the sums, in |c|^2
 // A unit of a sparse input with a point in a cell of more than this many is done as slices of cells: the input is clustered there, and what the
 // slices sort out beforehand is worth more than cheap tests (us, cells / groups / either by unit; 200 k clustered points, one point per
 // cell on average, F = 1 1131 / 1265 / 1003, F = 4 1298 / 1580 / 1191, Lennard-Jones 1255 / 1353 / 1076; 40 k, F = 1 214 / 284 / 199).  20: the
@@ -175,8 +179,8 @@ struct Group {
         a[2] = a[3] = t == 3 ? 0u : __float_as_uint(1.f);
         // |q . c - (q . c of the operands)| <= |q| |c| (2^-10 + 2^-10 + 2^-20), |c| <= |q| + r for a neighbour; the squares are rounded
         // down; the rounding of the fp32 sums stays below 2^-18 of their largest term
-        const float far = sqrtf(warp_max(fmaxf(na, nb))), reach = far + 1.001f * p.r;
-        const float thr = p.r2_hi + 3.95e-3f * far * reach + 4e-6f * reach * reach;
+        const float far = sqrtf(warp_max(fmaxf(na, nb))), reach = far + FILTER_REACH * p.r;
+        const float thr = p.r2_hi + FILTER_PRODUCT * far * reach + FILTER_SUMS * reach * reach;
         c0 = g < nq ? na - thr : INFINITY;
         c1 = g + 8 < nq ? nb - thr : INFINITY;
     }
@@ -199,11 +203,16 @@ struct Group {
         const int n = sten.total - k0 < Stage::CAPACITY ? sten.total - k0 : Stage::CAPACITY;
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");       // what was read and written here before
         __syncwarp();
-        if (lane == 0) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(st.arrived), "r"(16 * n) : "memory");
         const int from = sten.begin > k0 ? sten.begin : k0, end = sten.begin + sten.len < k0 + n ? sten.begin + sten.len : k0 + n;
-        if (from < end) {
-            const int src = sten.cs + from - sten.begin;
-            checked(src + end - from - 1, p.n, CHECK_SLOT);
+        const int src = sten.cs + from - sten.begin;
+        const bool whole = checked_range(src, end - from, p.n, CHECK_SLOT);
+        int copied = n;
+#ifdef TIGA_CHECKED
+        if (!whole) for (int k = 0; k < end - from; ++k) st.c[from - k0 + k] = p.spos[checked(src + k, p.n, CHECK_SLOT)];
+        copied -= __reduce_add_sync(0xffffffffu, whole ? 0 : end - from);
+#endif
+        if (lane == 0) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(st.arrived), "r"(16 * copied) : "memory");
+        if (from < end && whole) {
             asm volatile("cp.async.bulk.shared::cta.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                          ::"r"((unsigned)__cvta_generic_to_shared(st.c + (from - k0))), "l"(p.spos + src), "r"(16 * (end - from)), "r"(st.arrived) : "memory");
         }
