@@ -28,7 +28,7 @@ struct RunFrame {
         face = false;
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-            thr[d] = FAR_AWAY;
+            thr[d] = INFINITY;
             const int last = d == 0 ? c[0] + run - 1 : c[d];
             if (p.periodic[d] && p.nc[d] >= 4) {
                 if (c[d] == 0) { thr[d] = ((float)(last - c[d]) + 2.5f) * p.hcell[d]; face = true; }

@@ -652,3 +652,46 @@ def test_lennard_jones_in_one_cell(tiga, n):
 def test_binning_at_every_form_of_the_scan(tiga, n):
     """Cells as fine as the grid allows: 32, 154, 1926 and 2316 chunks of cells (the last above the limit of the folded totals)."""
     _check_bin(tiga, gen.uniform_points(n, 17), np.float32(1e-4), np.ones(3, np.float32), [0, 0, 0])
+
+
+@pytest.mark.parametrize("n,r", [(9001, 0.05), (9001, 0.12), (24001, 0.9)])
+@pytest.mark.parametrize("F", [1, 2, 3, 4])
+def test_groups_with_infinite_features_and_widest_gaussian(tiga, F, n, r):
+    """Sparse and dense stages, many stages: a row with an infinite source among its neighbours is that infinity, any other row is what it is
+    without it; with a Gaussian that gives every distance the weight one the sums are the plain neighbour sums."""
+    pos, x = gen.uniform_points(n, 76), gen.normal_features(n, F, 77)
+    ones, r, per = np.ones(3, np.float32), np.float32(r), [0, 0, 0]
+    rows = np.sort(gen.rng(76, 1).choice(n, 512, replace=False))
+    y, A, cnt = oracle.radius_forward(pos, x, r, ones, per, oracle.MSG_GAUSS, p0=1e9, rows=rows)
+    P = dev(pos, torch)
+    for sigma in (1e14, np.inf):
+        out, count, _ = tiga.tiga_apply_radius(P, dev(x, torch), r, ones, per, tiga.MSG_GAUSS, p0=sigma, want_count=True)
+        assert np.array_equal(host(count)[rows], cnt) and rel_err(host(out)[rows], y, A) <= SUM_TOL
+    d2 = ((pos.astype(np.float64) - pos[1234].astype(np.float64)) ** 2).sum(1)
+    near = d2 <= np.float64(r) ** 2
+    near[1234] = False
+    sure = abs(d2 - np.float64(r) ** 2) > 1e-7
+    x[1234] = 0.0
+    plain = {kind: host(tiga.tiga_apply_radius(P, dev(x, torch), r, ones, per, kind, p0=0.1)[0]) for kind in (tiga.MSG_GAUSS, tiga.MSG_DIST)}
+    x[1234] = np.inf
+    for kind in plain:
+        got = host(tiga.tiga_apply_radius(P, dev(x, torch), r, ones, per, kind, p0=0.1)[0])
+        assert np.all(got[near & sure] == np.inf) and np.array_equal(got[~near & sure], plain[kind][~near & sure])
+
+
+@pytest.mark.parametrize("F,n,r,periodic", [(1, 300_007, 0.0294, [0, 0, 0]), (4, 300_007, 0.0294, [1, 1, 1]), (4, 300_007, 0.0147, [1, 0, 1])])
+def test_groups_in_units_of_32_points(tiga, F, n, r, periodic):
+    pos, x = gen.uniform_points(n, 78), gen.normal_features(n, F, 78, 31)
+    for kind in (tiga.MSG_GAUSS, tiga.MSG_DIST):
+        _check_gauss(tiga, pos, x, None, np.float32(r), np.ones(3, np.float32), periodic, np.float32(r) / 2, kind=kind, use_cells=True, backward=False)
+
+
+@pytest.mark.parametrize("per_cell", [22, 24, 25, 27, 40])
+def test_narrow_features_in_slices_of_sixteen(tiga, per_cell):
+    """Cells' form (the box holds the place of the padding) with more than 100 k points: slices of 16 queries, cells cut above 24."""
+    cells, L = 17, 4e18
+    n = per_cell * cells ** 3
+    box = np.full(3, L, np.float32)
+    pos = np.minimum(gen.uniform_points(n, 90 + per_cell) * box, np.nextafter(box, np.float32(0))).astype(np.float32)
+    r = np.float32(L / cells / 1.002)
+    _check_gauss(tiga, pos, gen.normal_features(n, 3, 91, 31), None, r, box, [1, 1, 1], r / np.float32(2), use_cells=True, backward=False)
