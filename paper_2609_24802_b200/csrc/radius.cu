@@ -126,6 +126,7 @@ static __device__ int scan_chunk(const RadiusParams& p, const int chunk, const i
         if (base + k < p.ncells) {
             p.cell_start[base + k] = ex;
             if (p.u_cell_start) p.u_cell_start[base + k] = ex;
+            if (v[k] > p.full) atomicAdd(p.crowded, v[k]);
             if (v[k] > SORT_DENSE) p.b_items[atomicAdd(p.b_count, 1)] = base + k;
         }
         ex += v[k];
@@ -257,7 +258,7 @@ __global__ void __launch_bounds__(SMALL_THREADS) bin_small_kernel(const RadiusPa
     constexpr int PP = SMALL_POINTS / SMALL_THREADS, PC = SMALL_CELLS / SMALL_THREADS;
     const int tid = threadIdx.x;
     for (int k = tid; k < p.ncells; k += SMALL_THREADS) s_start[k] = 0;
-    if (tid == 0) { s_ndense = 0; *p.queue_n = 0; }
+    if (tid == 0) { s_ndense = 0; *p.queue_n = 0; *p.crowded = 0; }
     __syncthreads();
     float v[PP][3];
     int c[PP], slot[PP];
@@ -288,6 +289,7 @@ __global__ void __launch_bounds__(SMALL_THREADS) bin_small_kernel(const RadiusPa
             s_start[base + k] = ex;
             p.cell_start[base + k] = ex;
             if (p.u_cell_start) p.u_cell_start[base + k] = ex;
+            if (m[k] > p.full) atomicAdd(p.crowded, m[k]);
             if (m[k] > SMALL_DENSE) s_dense[atomicAdd(&s_ndense, 1)] = base + k;
         }
         ex += m[k];
@@ -811,6 +813,7 @@ RadiusLayout carve_radius(RadiusParams* p, void* ws, int32_t** fill) {
     p->cnt = cv.take<int32_t>(2 * nc + 2 + 16);     // counts, then the scatter cursors, then the length of the dense-cell queue
     p->b_count = p->cnt + 2 * nc + 2;
     p->queue_n = p->b_count + 2;
+    p->crowded = p->b_count + 3;
     *fill = p->cnt + nc;
     p->cell = cv.take<int32_t>(n);
     p->cell_start = cv.take<int32_t>(nc + 1);
@@ -849,6 +852,13 @@ static int unit_length(const RadiusParams& p) {
     return per > UNIT_MAX ? UNIT_MAX : per < 2 ? 2 : per;
 }
 
+// Cells of a uniform cloud hold the mean and a few roots of it: among 10^6 cells the fullest holds 36 points at a mean of 13, 75 at 40.  Below 48 points
+// (a surface or a slab has up to that many where its mean is 3) groups gain as often as they lose.
+static int full_cell(const RadiusParams& p) {
+    const double mean = (double)p.n / p.ncells, most = mean + 6.0 * sqrt(mean) + 6.0;
+    return most < 48.0 ? 48 : most < 1e9 ? (int)most : 1000000000;
+}
+
 tiga_status fill_params(RadiusParams* p, long long n, float r, const tiga_box* box) {
     int nc[3];
     float invh[3];
@@ -869,6 +879,7 @@ tiga_status fill_params(RadiusParams* p, long long n, float r, const tiga_box* b
     p->run = run_length(*p);
     p->unit = unit_length(*p);
     p->group_run = run_room(*p, GROUP_RUN);
+    p->full = full_cell(*p);
     // (slices of 16 from cells above 64 points, the earlier rule, against this one: 40 k clustered points, F = 8, forward +
     // backward 1972 -> 594 us; 4 k, F = 16, 330 -> 109 us; 30 k uniform points with 45 neighbours 155 -> 140 us)
     cut_cells(*p, 148 * 42);

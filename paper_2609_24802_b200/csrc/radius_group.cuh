@@ -21,17 +21,18 @@
 
 namespace tiga {
 
+constexpr int GROUP_PLACES = 148 * 20;     // warps of groups that run at once, about
 constexpr int GROUP = 16;                  // queries of a group: rows of the mma
 constexpr float FILTER_PRODUCT = 3.95e-3f; // margin of the test (Group): of the products, in |q| |c|;
 constexpr float FILTER_REACH = 1.001f;     // |c| of a neighbour exceeds |q| by this many cutoffs at most;
 constexpr float FILTER_SUMS = 4e-6f;       // of the sums, in |c|^2
-// A unit of a sparse input with a point in a cell of more than this many is done as slices of cells: the input is clustered there, and what the
-// slices sort out beforehand is worth more than cheap tests (us, cells / groups / either by unit; 200 k clustered points, one point per
-// cell on average, F = 1 1131 / 1265 / 1003, F = 4 1298 / 1580 / 1191, Lennard-Jones 1255 / 1353 / 1076; 40 k, F = 1 214 / 284 / 199).  20: the
-// fullest cell of 1 M uniform points at three per cell holds 16.  12 / 20: 40 k clustered points, F = 4 224 / 247, but a slab of eight points
-// a cell, 400 k points, F = 1 191 / 160.  The look costs uniform points 0 to 2 % (1 M, 4 neighbours, F = 1 222 / 226).
-constexpr int FULL_CELL = 20;
 
+// A unit of a large sparse input with a point in a cell of more than this many is done as slices of cells: the input is clustered there, and what the
+// slices sort out beforehand is worth more than cheap tests (us, cells / groups / either by unit above 20; 200 k clustered points, one point per
+// cell on average, F = 1 1131 / 1265 / 1003, F = 4 1298 / 1580 / 1191, Lennard-Jones 1255 / 1353 / 1076).  Above 20 / 40 points (200 k): clustered,
+// two per cell on average, F = 4 2377 / 2464; a slab of 20 points a cell 266 / 234 (cells 209).  The look costs uniform points 0 to 2 % (1 M, 4
+// neighbours, F = 1 222 / 226).
+constexpr int FULL_CELL = 40;
 // Unit u: points [u unit, (u + 1) unit) in cell order, a lane each.
 struct GroupUnit {
     int begin, at;                         // first point; cell of the lane's point, ten bits per coordinate
@@ -75,7 +76,7 @@ struct GroupUnit {
 
 // Points per warp.
 static inline int group_unit(const long long n) {
-    const long long places = 148 * 20;
+    const long long places = GROUP_PLACES;
     return n >= 3 * 32 * places ? 32 : n >= 8 * places ? 16 : n >= 4 * places ? 8 : 4;
 }
 

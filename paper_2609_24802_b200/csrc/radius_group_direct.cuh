@@ -15,7 +15,7 @@ template <typename Msg, bool SPARSE> struct GroupDirectSmem {
     static constexpr int FEAT_STRIDE = Stage::SLOTS;                        // the entry of the far slot stays zero
     static constexpr int PER_WARP = STAGE_BYTES + STAGED * FEAT_STRIDE * 4;
     static_assert(PER_WARP % 16 == 0, "the stage is accessed as 16-byte vectors");
-    static_assert(!SPARSE || DirectSmem<Msg>::PER_WARP <= PER_WARP, "units of full cells take the cells' form");
+    static_assert(DirectSmem<Msg>::PER_WARP <= PER_WARP, "crowded cells take the cells' form");
 };
 
 // COUNT: the numbers of neighbours are wanted.
@@ -139,17 +139,38 @@ __device__ __forceinline__ bool direct_group(const RadiusParams& p, typename Gro
     return true;
 }
 
-template <typename Msg, bool SPARSE, bool COUNT>
+// What a kernel of groups does with clustered inputs.  Slices sort candidates out beforehand, and short ones spread over more warps than units of
+// groups do; but of these kernels fewer warps run at once than of the one for slices alone.  (us, cells / groups, full units as slices where sparse /
+// this rule, F = 1: 40 k clustered points, one per cell on average 256 / 431 / 260, eight 418 / 518 / 446.  200 k, one 1861 / 1738, eight 3144 / 3540;
+// as cells and slices in this kernel 1843 and 3780.  A surface of 50 k points, 32 a cell, 82 / 102.)
+enum class Clustered {
+    Groups,        // nothing: many dense units, whose groups keep the machine busy, lose less than slices at this occupancy
+    Units,         // many sparse units: those with a full cell as slices
+    Cells,         // fewer units than two rounds of the machine: the whole input as cells and slices, by units of that form, when more than a quarter of
+                   // the points lie in cells that stand out (RadiusParams::full; a sixteenth: a slab of 40 points a cell, 20 k points, 70 -> 87 us)
+};
+
+template <typename Msg, bool SPARSE, Clustered MODE, bool COUNT>
 __global__ void __launch_bounds__(32, (GroupDirectSmem<Msg, SPARSE>::WARPS)) radius_group_kernel(const __grid_constant__ RadiusParams p, const int unit) {
     using SM = GroupDirectSmem<Msg, SPARSE>;
     extern __shared__ __align__(16) unsigned char s_raw[];
+    if constexpr (MODE == Clustered::Cells) {
+        if (*p.crowded > p.n >> 2) {
+            auto slice = [&](const int (&cell)[3], const int run, const int qs, const int qe) { direct_slice<Msg, false>(p, cell, run, qs, qe, s_raw); };
+            if (blockIdx.x * (long long)p.unit < p.n) walk_unit(p, blockIdx.x, p.run, slice);
+            return;
+        }
+        if (blockIdx.x * (long long)unit >= p.n) return;
+    }
     const GroupUnit work(p, blockIdx.x, unit);
-    if (SPARSE && work.full(p)) {
-        work.walk(p, [&](const int (&cell)[3], const int run, const int qs, const int nq) {
-            direct_slice<Msg, false>(p, cell, run, qs, qs + nq, s_raw);
-            return true;
-        });
-        return;
+    if constexpr (MODE == Clustered::Units) {
+        if (work.full(p)) {
+            work.walk(p, [&](const int (&cell)[3], const int run, const int qs, const int nq) {
+                direct_slice<Msg, false>(p, cell, run, qs, qs + nq, s_raw);
+                return true;
+            });
+            return;
+        }
     }
     float* s_feat = reinterpret_cast<float*>(s_raw + SM::STAGE_BYTES);                   // [STAGED][FEAT_STRIDE]
     if (threadIdx.x < SM::STAGED) s_feat[threadIdx.x * SM::FEAT_STRIDE + SM::Stage::FAR] = 0.f;
@@ -163,13 +184,17 @@ __global__ void __launch_bounds__(32, (GroupDirectSmem<Msg, SPARSE>::WARPS)) rad
     });
 }
 
-template <typename Msg, bool SPARSE>
+template <typename Msg, bool SPARSE, Clustered MODE>
 static tiga_status launch_direct_group(const RadiusParams& p, cudaStream_t s) {
     constexpr int smem = GroupDirectSmem<Msg, SPARSE>::PER_WARP;
     static_assert(smem <= 48 * 1024, "no attribute needed");
-    auto kern = p.count ? radius_group_kernel<Msg, SPARSE, true> : radius_group_kernel<Msg, SPARSE, false>;
+    auto kern = p.count ? radius_group_kernel<Msg, SPARSE, MODE, true> : radius_group_kernel<Msg, SPARSE, MODE, false>;
     const int unit = group_unit(p.n);
-    kern<<<counted((unsigned)(((long long)p.n + unit - 1) / unit)), 32, smem, s>>>(p, unit);
+    RadiusParams q = p;
+    // (half of the groups' unit at least: warps without work cost 30 k uniform points a microsecond)
+    if (MODE == Clustered::Cells) q.unit = p.unit < unit / 2 ? unit / 2 : p.unit < unit ? p.unit : unit;
+    else q.unit = unit;
+    kern<<<counted(unit_count(q)), 32, smem, s>>>(q, unit);
     return launch_status();
 }
 
@@ -183,8 +208,11 @@ static tiga_status launch_direct_group(const RadiusParams& p, cudaStream_t s) {
 template <typename Msg, bool MI>
 static tiga_status launch_direct_t(const RadiusParams& p, cudaStream_t s) {
     if constexpr (!MI) {
-        if (group_lengths(p) && 10LL * p.n >= 7LL * p.ncells && (p.n >= 8192 || p.n >= 8LL * p.ncells))
-            return group_sparse(p) ? launch_direct_group<Msg, true>(p, s) : launch_direct_group<Msg, false>(p, s);
+        if (group_lengths(p) && 10LL * p.n >= 7LL * p.ncells && (p.n >= 8192 || p.n >= 8LL * p.ncells)) {
+            if (p.n <= 2LL * GROUP_PLACES * GROUP)
+                return group_sparse(p) ? launch_direct_group<Msg, true, Clustered::Cells>(p, s) : launch_direct_group<Msg, false, Clustered::Cells>(p, s);
+            return group_sparse(p) ? launch_direct_group<Msg, true, Clustered::Units>(p, s) : launch_direct_group<Msg, false, Clustered::Groups>(p, s);
+        }
     }
     return launch_direct_slices<Msg, MI>(p, s);
 }

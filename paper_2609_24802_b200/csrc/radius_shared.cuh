@@ -60,6 +60,8 @@ struct RadiusParams {
     int group_run;            // cells along x that a group of queries spans at most (walk_groups)
     int dense, slice;         // a cell with more than `dense` points is cut into slices of `slice` queries
     int* queue_n;             // length of the kNN queue (zeroed with the counts)
+    int full;                 // a cell with more points than this stands out from the mean (full_cell)
+    int* crowded;             // points in such cells (zeroed with the counts)
     int32_t* b_items;         // cells with more than SORT_DENSE points (queued by the scan), and how many
     int* b_count;
     // optional user copies of the plan

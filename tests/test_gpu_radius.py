@@ -695,3 +695,25 @@ def test_narrow_features_in_slices_of_sixteen(tiga, per_cell):
     pos = np.minimum(gen.uniform_points(n, 90 + per_cell) * box, np.nextafter(box, np.float32(0))).astype(np.float32)
     r = np.float32(L / cells / 1.002)
     _check_gauss(tiga, pos, gen.normal_features(n, 3, 91, 31), None, r, box, [1, 1, 1], r / np.float32(2), use_cells=True, backward=False)
+
+
+@pytest.mark.parametrize("n,mean,periodic", [(1500, 9.0, [0, 0, 0]), (8192, 3.2, [0, 1, 0]), (24001, 1.0, [1, 1, 1]), (24001, 5.0, [0, 0, 0]), (94719, 3.5, [0, 0, 0]), (94721, 3.5, [1, 0, 0])])
+@pytest.mark.parametrize("message", ["sum1", "sum4", "lj"])
+def test_clustered_inputs_on_both_sides_of_the_rule(tiga, message, n, mean, periodic):
+    """Sparse and dense on average, up to the size (94,720 points) that is done as cells and slices when more than a quarter of the points lie in cells
+    that stand out from the mean, and above it; the smallest goes through the one-launch binning."""
+    ones, r = np.ones(3, np.float32), float((mean / n) ** (1 / 3) / 1.002)
+    pos = gen.clustered_points(n, 79)
+    grid, _ = tiga.tiga_radius_grid(n, np.float32(r), ones, periodic)
+    cell = np.minimum((pos * np.float32(grid)).astype(np.int64), np.array(grid) - 1)
+    held = np.bincount((cell[:, 2] * grid[1] + cell[:, 1]) * grid[0] + cell[:, 0])
+    per = n / np.prod(grid)
+    assert 0.7 <= per and held[held > max(48, per + 6 * per ** 0.5 + 6)].sum() > n / 4 and min(grid) > 3
+    rows = np.sort(gen.rng(79, 1).choice(n, 512, replace=False))
+    kind = tiga.MSG_LJ if message == "lj" else tiga.MSG_DIST
+    x = None if message == "lj" else gen.normal_features(n, 1 if message == "sum1" else 4, 79, 31)
+    s = 2e-6 if message == "lj" else 0.0                      # below the smallest distance
+    y, A, cnt = oracle.radius_forward(pos, x, np.float32(r), ones, periodic, kind, 1e-3, s, rows=rows)
+    out, count, _ = tiga.tiga_apply_radius(dev(pos, torch), None if x is None else dev(x, torch), np.float32(r), ones, periodic, kind, p0=1e-3, p1=s, want_count=True)
+    assert np.array_equal(host(count)[rows], cnt)
+    assert rel_err(host(out)[rows], y, A) <= SUM_TOL
