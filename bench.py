@@ -152,7 +152,7 @@ def input_hashes(snaps):
 # DRAM traffic per unit measured with ncu on reduced replicas (profiles/*.md), used to scale
 # `traffic` to a full launch: bytes per particle / point / edge of one launch of the row's kernels.
 TRAFFIC_PER_UNIT = {
-    "radius_lj_fwd": ("particle", 33.6),          # profiles/radius_direct_lj_1M.md: 17.6 B measured + the 16-byte row that leaves L2 at full size
+    "radius_lj_fwd": ("particle", 32.4),          # profiles/radius_group_lj_1M.md: 16.4 B measured + the 16-byte row that leaves L2 at full size
     "radius_gauss_fwd": ("point", 186.7),         # profiles/radius_traverse_gaussian_300k.md
     "radius_gauss_bwd": ("point", 364.6),
     "csr_sum_fwd": ("edge", 21.3),                # profiles/csr_kernels_rmat_scale18.md

@@ -27,7 +27,7 @@
 // list's length, counts grow with the cube of the distance, and corrected by counting ballots); then every lane
 // counts the entries closer than its own, which is that entry's place in the row.  Equal distances and k > 24 go
 // through the general form, a bitonic network of shuffles over 32 keys at a time and merges, which orders
-// whole keys.  (131,072 uniform points, k = 16, one feature: 555 warp instructions per query here and 50 in the rings kernel.)
+// whole keys.  (131,072 uniform points, k = 16, one feature: 552 warp instructions per query here and 40 in the rings kernel.)
 #include "radius_test.cuh"
 #include <type_traits>
 
